@@ -1385,12 +1385,24 @@ static int ensure_build_buffers(kdfmm_tree_s* t, int64_t n) {
   return KDFMM_OK;
 }
 
+// Queue entries and dynamic shared memory of the subtree kernel for trees of
+// the given leaf size.
+static int subtree_qcap(int n_leaf) { return kSubtreeMax / (n_leaf + 1) + 2; }
+static size_t subtree_smem_for(int qcap) {
+  return 4 * kSubtreeMax * sizeof(double) + 3 * kSubtreeMax * sizeof(float) +
+         2 * kSubtreeMax * sizeof(uint16_t) + 4 * (size_t)qcap * sizeof(int4);
+}
+
 // Launch sizes of the persistent subtree kernel (host calls only; made once
-// per handle and shared-memory size, outside any stream capture).
+// per handle and shared-memory size, outside any stream capture).  The
+// kernel's shared-memory limit is one value for all handles of the process,
+// so it is set to the size of the smallest leaves (1), which no handle
+// exceeds: a limit set to this handle's own size would fail the next launch
+// of a handle with smaller leaves.
 static int subtree_setup(kdfmm_tree_s* t, size_t smem) {
   if (t->subtree_smem == smem) return KDFMM_OK;
   int rc = check_cuda(cudaFuncSetAttribute(k_subtree, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem),
+                                           (int)subtree_smem_for(subtree_qcap(1))),
                       "subtree smem attribute");
   if (rc) return rc;
   int per_sm = 0, sms = 0;
@@ -1498,9 +1510,8 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
   S.buf1 = t->buf[1];
   S.out = t->tp;
   S.segB = t->segB;
-  S.qcap = kSubtreeMax / (t->min_nleaf + 1) + 2;
-  const size_t smem = 4 * kSubtreeMax * sizeof(double) + 3 * kSubtreeMax * sizeof(float) +
-                      2 * kSubtreeMax * sizeof(uint16_t) + 4 * (size_t)S.qcap * sizeof(int4);
+  S.qcap = subtree_qcap(t->min_nleaf);
+  const size_t smem = subtree_smem_for(S.qcap);
   if ((rc = subtree_setup(t, smem))) return rc;
   const int gsub = deferred ? t->subtree_grid : std::max(1, std::min(t->subtree_grid, hc[C_NB]));
   k_subtree<<<gsub, kSubtreeThreads, smem, s>>>(S);
