@@ -200,8 +200,9 @@ int kdfmm_fmm_accel(kdfmm_tree t, double* a, double* phi, void* stream);
  * mixed mode forms the M2L r-derivatives and the P2P pair terms in float32
  * (as its evaluation does) from float64 differences, with float64 sums.  Cell
  * cotangents and the P2P source-side terms are summed with float64 atomics,
- * so the last bits may vary run to run.  Allocates its scratch (88 bytes per
- * particle, 160 per leaf, 80 per cell) with cudaMallocAsync on `stream`.  Errors:
+ * so the last bits may vary run to run.  Its scratch (at most 144 bytes per
+ * particle, 180 per leaf, 80 per cell, 4 per near-list entry) stays with the
+ * handle; a call on a capturing stream takes it with cudaMallocAsync.  Errors:
  * KDFMM_ERR_INVALID_ARG before any evaluation or for non-device pointers,
  * KDFMM_ERR_CUDA on allocation or launch failure. */
 int kdfmm_fmm_accel_vjp(kdfmm_tree t, const double* a_bar, double* x_bar, double* m_bar,

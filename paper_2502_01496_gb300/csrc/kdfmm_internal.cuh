@@ -214,6 +214,9 @@ struct kdfmm_tree_s {
     int64_t nfar = 0, nnear = 0;         // entries (both directions)
   } dual;
 
+  void* vjp_buf = nullptr;         // scratch of the adjoint
+  size_t vjp_cap = 0;              // its bytes
+
   // captured evaluation (kdfmm_fmm_accel_batched): valid for the arguments
   // and buffers it was captured with
   struct GraphKey {
@@ -274,6 +277,38 @@ __device__ __forceinline__ float trunc_to_float(double v) {
   if (e >= 255) return __uint_as_float(sign | 0x7f800000u);
   const unsigned mant = ((hi & 0xfffffu) << 3) | (lo >> 29);
   return __uint_as_float(sign | ((unsigned)e << 23) | mant);
+}
+
+// Reciprocal square root, flush-to-zero form of the hardware approximation
+// (relative error below 2^-22) for arguments that are 0 or far above the
+// subnormal range.
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// 1 / sqrt(v) in float64 with four operations on the float64 pipe (1/64 of the
+// float32 rate here: each costs as much as ~75 float32 or integer ones).  The
+// float32 estimate y of the mantissa's reciprocal root is moved to float64
+// with integer operations, and one step of Householder's third-order
+// iteration, y (1 + e/2 + 3/8 e^2) with e = 1 - v y^2, leaves the rounding of
+// e and of the result (|e| < 2^-21, so the remainder is below 2^-64).  The
+// 3/8 e^2 term, below 2^-43, is formed in float32.  Zero, subnormal, negative,
+// infinite and NaN arguments take the library's function.
+__device__ __forceinline__ double rsqrt64(double v) {
+  const int hi = __double2hiint(v), lo = __double2loint(v);
+  if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return rsqrt(v);
+  const int ex = (hi >> 20) - 1023;
+  const float m = __int_as_float(((127 + (ex & 1)) << 23) | ((hi & 0xfffff) << 3) |
+                                 (int)((unsigned)lo >> 29));
+  const int yb = __float_as_int(rsqrt_ftz(m));             // in (1/2, 1]
+  const double y = __hiloint2double((yb >> 3) + ((896 - (ex >> 1)) << 20), yb << 29);
+  const double e = fma(-(v * y), y, 1.0);
+  const float ef = trunc_to_float(e);
+  const int cb = __float_as_int(0.375f * ef * ef);         // (0 becomes 2^-127: far below rounding)
+  const double c = __hiloint2double((cb >> 3) + (896 << 20), cb << 29);
+  return fma(y, fma(0.5, e, c), y);
 }
 
 // Bound on |d_float32 - d| for a distance d whose coordinates and centre lie

@@ -87,16 +87,6 @@ __device__ __forceinline__ double m4_pot_d(double q, double qi) {
   return 1.6 + q2 * (-4.0 / 3.0 + q * (1.0 + q * (-0.3 + q * (1.0 / 30.0)))) - qi * (1.0 / 15.0);
 }
 
-// Reciprocal square root, flush-to-zero form of the hardware approximation
-// (relative error below 2^-22).  Its arguments here are 0 (coincident
-// particles, selected away) or far above the subnormal range, where the
-// flush changes nothing and the subnormal fix-up of rsqrtf is dead weight.
-__device__ __forceinline__ float rsqrt_ftz(float x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // Interaction of one target with one source, float32, accumulated into f*.
 template <int SOFT>
 __device__ __forceinline__ void pair32(float rx, float ry, float rz, float mj, const float4& hi,

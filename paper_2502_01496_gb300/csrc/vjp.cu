@@ -67,19 +67,20 @@ __device__ __forceinline__ DualT<S> rsqrt_dual(const DualT<S>& a) {
   return DualT<S>{r, {dr * a.d[0], dr * a.d[1], dr * a.d[2]}};
 }
 
+// A scalar as the coefficients' type (a dual number with zero derivatives).
 template <class T>
-__device__ __forceinline__ T tc(double v);
-template <>
-__device__ __forceinline__ double tc<double>(double v) { return v; }
-template <>
-__device__ __forceinline__ float tc<float>(double v) { return (float)v; }
-template <>
-__device__ __forceinline__ DualT<double> tc<DualT<double>>(double v) {
-  return DualT<double>{v, {0.0, 0.0, 0.0}};
-}
-template <>
-__device__ __forceinline__ DualT<float> tc<DualT<float>>(double v) {
-  return DualT<float>{(float)v, {0.0f, 0.0f, 0.0f}};
+struct Lift {
+  __device__ static __forceinline__ T of(T v) { return v; }
+  using Scalar = T;
+};
+template <class S>
+struct Lift<DualT<S>> {
+  __device__ static __forceinline__ DualT<S> of(S v) { return DualT<S>{v, {S(0), S(0), S(0)}}; }
+  using Scalar = S;
+};
+template <class T>
+__device__ __forceinline__ T tc(double v) {
+  return Lift<T>::of((typename Lift<T>::Scalar)v);
 }
 
 __device__ __forceinline__ double rs(double v) { return rsq(v); }
@@ -114,10 +115,13 @@ __device__ __forceinline__ T c3e(int a, int b, int c, const T R[3], const T u[3]
 // STD: the standard p = 3 series -- the quadrupole keeps only its C0 and C1
 // terms (as in m2l.cu).
 template <class T, bool STD>
-__device__ T m2l_contract(const T R[3], double M, const double Q[6], const double w[20]) {
-  const T Qm[3][3] = {{tc<T>(Q[0]), tc<T>(Q[1]), tc<T>(Q[2])},
-                      {tc<T>(Q[1]), tc<T>(Q[3]), tc<T>(Q[4])},
-                      {tc<T>(Q[2]), tc<T>(Q[4]), tc<T>(Q[5])}};
+__device__ T m2l_contract(const T R[3], typename Lift<T>::Scalar M,
+                          const typename Lift<T>::Scalar Q[6],
+                          const typename Lift<T>::Scalar w[20]) {
+  using L = Lift<T>;
+  const T Qm[3][3] = {{L::of(Q[0]), L::of(Q[1]), L::of(Q[2])},
+                      {L::of(Q[1]), L::of(Q[3]), L::of(Q[4])},
+                      {L::of(Q[2]), L::of(Q[4]), L::of(Q[5])}};
   const T R2 = R[0] * R[0] + R[1] * R[1] + R[2] * R[2];
   const T g0 = rs(R2);
   const T i2 = g0 * g0;
@@ -130,11 +134,11 @@ __device__ T m2l_contract(const T R[3], double M, const double Q[6], const doubl
   for (int i = 0; i < 3; ++i) u[i] = Qm[i][0] * R[0] + Qm[i][1] * R[1] + Qm[i][2] * R[2];
   const T q = R[0] * u[0] + R[1] * u[1] + R[2] * u[2];
   const T qs = q * tc<T>(1.0 / 6.0);
-  const T Mt = tc<T>(M);
+  const T Mt = L::of(M);
   const T s1 = -(Mt * g1) - g3 * qs;
   const T t2 = g2 * tc<T>(-1.0 / 3.0);
-  T acc = tc<T>(w[0]) * (-(Mt * g0) - g2 * qs);
-  for (int i = 0; i < 3; ++i) acc += tc<T>(w[1 + i]) * (s1 * R[i] + t2 * u[i]);
+  T acc = L::of(w[0]) * (-(Mt * g0) - g2 * qs);
+  for (int i = 0; i < 3; ++i) acc += L::of(w[1 + i]) * (s1 * R[i] + t2 * u[i]);
   const T s1h = STD ? -(Mt * g1) : s1;
   const T s2 = STD ? -(Mt * g2) : -(Mt * g2) - g4 * qs;
   const T s3 = STD ? -(Mt * g3) : -(Mt * g3) - g5 * qs;
@@ -144,28 +148,13 @@ __device__ T m2l_contract(const T R[3], double M, const double Q[6], const doubl
   const int c2a[6] = {0, 0, 0, 1, 1, 2}, c2b[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
   for (int k = 0; k < 6; ++k)
-    acc += tc<T>(w[4 + k]) * c2e<T>(c2a[k], c2b[k], R, u, Qm, s1h, s2, t2h, t3);
+    acc += L::of(w[4 + k]) * c2e<T>(c2a[k], c2b[k], R, u, Qm, s1h, s2, t2h, t3);
   const int c3a[10] = {0, 0, 0, 0, 0, 0, 1, 1, 1, 2}, c3b[10] = {0, 0, 0, 1, 1, 2, 1, 1, 2, 2},
             c3c[10] = {0, 1, 2, 1, 2, 2, 1, 2, 2, 2};
 #pragma unroll
   for (int k = 0; k < 10; ++k)
-    acc += tc<T>(w[10 + k]) * c3e<T>(c3a[k], c3b[k], c3c[k], R, u, Qm, s2, s3, t3, t4);
+    acc += L::of(w[10 + k]) * c3e<T>(c3a[k], c3b[k], c3c[k], R, u, Qm, s2, s3, t3, t4);
   return acc;
-}
-
-// index of the compact C2 entry (a, b) and C3 entry (a, b, c)
-__device__ __forceinline__ int c2i(int a, int b) {
-  if (a > b) { int t = a; a = b; b = t; }
-  return a == 0 ? 4 + b : (a == 1 ? 6 + b : 9);
-}
-__device__ __forceinline__ int c3i(int a, int b, int c) {
-  // sort a <= b <= c
-  if (a > b) { int t = a; a = b; b = t; }
-  if (b > c) { int t = b; b = c; c = t; }
-  if (a > b) { int t = a; a = b; b = t; }
-  if (a == 0) return b == 0 ? 10 + c : (b == 1 ? 12 + c : 15);
-  if (a == 1) return b == 1 ? 15 + c : 18;
-  return 19;
 }
 
 // ---------------------------------------------------------------------------
@@ -174,7 +163,6 @@ __device__ __forceinline__ int c3i(int a, int b, int c) {
 struct VjpArgs {
   int64_t n;
   int nleaves, ncells;
-  int soft_kind;
   bool mixed;
   const int32_t* leaf_sys;
   const double* sys_eps;
@@ -182,12 +170,19 @@ struct VjpArgs {
   const int32_t* leaf_rank;
   Cells c;
   PCols tp;
+  const float4* ph;                     // (1/h, 1/h^3, h, (2h)^2) float32
   const float* lexp32;
   const double* lexp64;
   const int32_t *far_cnt, *far_idx, *near_cnt, *near_idx;
   const int64_t *far_off, *near_off;
   int64_t cap_far, cap_near;            // entries a list may hold
-  double* ab;                           // cotangent in tree order (N x 3)
+  double* ab;                           // cotangent in tree order (N x 3; FP64 mode)
+  double* hinv;                         // 1 / h in tree order (FP64 mode, M4 kernel)
+  const int32_t* sys_root;
+  // mixed mode, tree order: the position on three float32 grids (split_grid),
+  // q0 = (x0, m), q1 = (x1, 1 / h), q2 = (x2, first component of a_bar), q3 the other two
+  float4 *q0, *q1, *q2;
+  float2* q3;
   double* xbar;                         // tree order (N x 3)
   double* mbar;                         // tree order (N)
   double* xsrc;                         // P2P source-side part of x_bar (N x 3, atomics)
@@ -200,86 +195,152 @@ struct VjpArgs {
   const int32_t *seg_first, *seg_leaf;
   double* seg_part;
   int64_t seg_cap;
+  // transposed near lists: leaf ordinal r is a source of the target leaves
+  // tidx[toff[r] ...) (ordinals), tcnt[r] of them; cut into pieces of
+  // kSrcEntries, piece 0 the leaf's own work item, the others extra items
+  int32_t *tcnt, *tcur, *tidx;
+  int64_t* toff;
+  int64_t tcap;                         // entries of tidx
+  int32_t *tseg_leaf, *tseg_first;      // per extra item: its leaf; per leaf: its first extra item
+  int64_t tseg_cap;
+  unsigned long long* tctr;             // [0] entries reserved, [1] extra items
 };
 
-__global__ void k_gather_abar(const double* __restrict__ abar, VjpArgs V) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= V.n) return;
-  const int64_t i = V.tp.idx[p];
-  V.ab[3 * p] = abar[3 * i];
-  V.ab[3 * p + 1] = abar[3 * i + 1];
-  V.ab[3 * p + 2] = abar[3 * i + 2];
-  V.xbar[3 * p] = V.xbar[3 * p + 1] = V.xbar[3 * p + 2] = 0.0;
-  V.xsrc[3 * p] = V.xsrc[3 * p + 1] = V.xsrc[3 * p + 2] = 0.0;
-  V.mbar[p] = V.msrc[p] = 0.0;
+// A coordinate as x0 + x1 + x2 on the grids 2^(k-22), 2^(k-45) and 2^(k-68) of
+// its system (|x| <= 2^k): the difference of two coordinates is then three
+// exact float32 subtractions, and grid_diff their sum rounded to float32 -- the
+// float64 difference rounded to float32 -- without the float64 pipe (1/64 rate).
+struct GridScale {
+  double c0, c1, c2;                    // adding and subtracting rounds to the grid
+};
+__device__ __forceinline__ GridScale grid_scale(double bound) {
+  const int k = max(((__double2hiint(bound) >> 20) & 0x7ff) - 1022, -900);   // bound < 2^k
+  GridScale g;
+  g.c0 = __hiloint2double((min(k + 30, 1023) + 1023) << 20 | 0x80000, 0);     // 1.5 * 2^(k+30)
+  g.c1 = __hiloint2double((k + 7 + 1023) << 20 | 0x80000, 0);
+  g.c2 = __hiloint2double((k - 16 + 1023) << 20 | 0x80000, 0);
+  return g;
 }
-
-__device__ __forceinline__ void load_coeffs(const VjpArgs& V, int k, double C[20]) {
-  if (V.mixed) {
-    const float* f = V.lexp32 + 24 * (int64_t)k;
-    for (int j = 0; j < 20; ++j) C[j] = (double)f[j];
-    for (int j = 0; j < 4; ++j) C[j] += (double)f[20 + j];
-  } else {
-    const double* d = V.lexp64 + 20 * (int64_t)k;
-    for (int j = 0; j < 20; ++j) C[j] = d[j];
-  }
+__device__ __forceinline__ void split_grid(double x, const GridScale& g, float& x0, float& x1,
+                                           float& x2) {
+  const double a = __dsub_rn(__dadd_rn(x, g.c0), g.c0), r = __dsub_rn(x, a);
+  const double b = __dsub_rn(__dadd_rn(r, g.c1), g.c1), q = __dsub_rn(r, b);
+  x0 = (float)a;
+  x1 = (float)b;
+  x2 = (float)__dsub_rn(__dadd_rn(q, g.c2), g.c2);
+}
+__device__ __forceinline__ float grid_diff(float a0, float a1, float a2, float b0, float b1,
+                                           float b2) {
+  const float d0 = __fsub_rn(a0, b0), d1 = __fsub_rn(a1, b1), d2 = __fsub_rn(a2, b2);
+  const float s = __fadd_rn(d0, d1);
+  const float e = __fsub_rn(d1, __fsub_rn(s, d0));            // |d0| >= |d1| or d0 = 0
+  // s + e + d2 rounded once: the tail is cut off with its last bit set when
+  // anything was lost, so that it cannot make a tie of what is none
+  float r = __fadd_rz(e, d2);
+  if (__fsub_rn(d2, __fsub_rn(r, e)) != 0.0f) r = __int_as_float(__float_as_int(r) | 1);
+  return __fadd_rn(s, r);
 }
 
 // L2P reverse: warp per leaf, lane per particle.  a_i = -(C1 + C2 x + C3 x x / 2)
-// with x = x_i - com_alpha.
-__global__ void k_vjp_l2p(VjpArgs V) {
-  const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
+// with x = x_i - com_alpha.  Also brings the cotangent into tree order and
+// prepares the particle records of the P2P reverse.
+// Bound by the float64 pipe (1/64 rate): the lanes form the particles' 19
+// monomials b x x in parallel (29 float64 operations a warp), and lane j sums
+// monomial j over the leaf's particles from shared memory (11 additions a
+// leaf of 11), instead of butterflies over 23 values (115 additions).
+constexpr int kL2PWarps = 4;
+__global__ void __launch_bounds__(kL2PWarps * 32) k_vjp_l2p(const double* __restrict__ abar, VjpArgs V,
+                                                         bool m4) {
+  __shared__ double s_c[kL2PWarps][20];
+  __shared__ double s_v[kL2PWarps][22][33];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int k = blockIdx.x * kL2PWarps + w;
   if (k >= V.nleaves) return;
   const int a = V.leaf_cells[k];
   const int f = V.c.first[a], cnt = V.c.count[a];
-  double C[20];
-  load_coeffs(V, k, C);
-  double cb[20];
-  for (int j = 0; j < 20; ++j) cb[j] = 0.0;
-  double gx = 0.0, gy = 0.0, gz = 0.0;             // sum of (d a / d x)^T a_bar
+  double* C = s_c[w];
+  if (lane < 20) {
+    if (V.mixed) {
+      const float* e = V.lexp32 + 24 * (int64_t)k;
+      double v = (double)e[lane];
+      if (lane < 4) v += (double)e[20 + lane];
+      C[lane] = v;
+    } else {
+      C[lane] = V.lexp64[20 * (int64_t)k + lane];
+    }
+  }
+  __syncwarp();
+  double (*vals)[33] = s_v[w];
   if (lane < cnt) {
-    const int64_t p = (int64_t)f + lane;
-    const double x[3] = {V.tp.x[p] - V.c.cx[a], V.tp.y[p] - V.c.cy[a], V.tp.z[p] - V.c.cz[a]};
-    const double b[3] = {V.ab[3 * p], V.ab[3 * p + 1], V.ab[3 * p + 2]};
-    // (d a_i / d x_j) = -(C2_ij + C3_ijk x_k): g_j = sum_i b_i (d a_i / d x_j)
-    double g[3];
-    for (int jj = 0; jj < 3; ++jj) {
-      double s = 0.0;
-      for (int ii = 0; ii < 3; ++ii) {
-        double t = C[c2i(ii, jj)];
-        for (int kk = 0; kk < 3; ++kk) t += C[c3i(ii, jj, kk)] * x[kk];
-        s += b[ii] * t;
-      }
-      g[jj] = -s;
+    const int64_t p = (int64_t)f + lane, i = V.tp.idx[p];
+    const double x = V.tp.x[p] - V.c.cx[a], y = V.tp.y[p] - V.c.cy[a], z = V.tp.z[p] - V.c.cz[a];
+    const double b0 = abar[3 * i], b1 = abar[3 * i + 1], b2 = abar[3 * i + 2];
+    if (V.mixed) {
+      const int root = V.sys_root[V.leaf_sys[k]];
+      const GridScale g = grid_scale(
+          fmax(fabs(V.c.cx[root]), fmax(fabs(V.c.cy[root]), fabs(V.c.cz[root]))) + V.c.s[root]);
+      float4 u0, u1, u2;
+      split_grid(V.tp.x[p], g, u0.x, u1.x, u2.x);
+      split_grid(V.tp.y[p], g, u0.y, u1.y, u2.y);
+      split_grid(V.tp.z[p], g, u0.z, u1.z, u2.z);
+      u0.w = (float)V.tp.m[p];
+      u1.w = m4 ? 1.0f / (float)V.tp.h[p] : 0.0f;
+      u2.w = (float)b0;
+      V.q0[p] = u0;
+      V.q1[p] = u1;
+      V.q2[p] = u2;
+      V.q3[p] = make_float2((float)b1, (float)b2);
+    } else {
+      V.ab[3 * p] = b0;
+      V.ab[3 * p + 1] = b1;
+      V.ab[3 * p + 2] = b2;
+      if (m4) V.hinv[p] = 1.0 / V.tp.h[p];
     }
-    V.xbar[3 * p] += g[0];
-    V.xbar[3 * p + 1] += g[1];
-    V.xbar[3 * p + 2] += g[2];
-    gx = g[0]; gy = g[1]; gz = g[2];
+    // (d a_i / d x_j) = -N_ij, N_ij = C2_ij + C3_ijk x_k: g_j = -sum_i b_i N_ij
+    const double n00 = C[4] + C[10] * x + C[11] * y + C[12] * z;
+    const double n01 = C[5] + C[11] * x + C[13] * y + C[14] * z;
+    const double n02 = C[6] + C[12] * x + C[14] * y + C[15] * z;
+    const double n11 = C[7] + C[13] * x + C[16] * y + C[17] * z;
+    const double n12 = C[8] + C[14] * x + C[17] * y + C[18] * z;
+    const double n22 = C[9] + C[15] * x + C[18] * y + C[19] * z;
+    const double g0 = -(b0 * n00 + b1 * n01 + b2 * n02);
+    const double g1 = -(b0 * n01 + b1 * n11 + b2 * n12);
+    const double g2 = -(b0 * n02 + b1 * n12 + b2 * n22);
+    V.xbar[3 * p] = g0;
+    V.xbar[3 * p + 1] = g1;
+    V.xbar[3 * p + 2] = g2;
     // expansion cotangents: a_i depends on C1_i, C2_ij x_j, 1/2 C3_ijk x_j x_k
-    for (int ii = 0; ii < 3; ++ii) {
-      cb[1 + ii] -= b[ii];
-      for (int jj = 0; jj < 3; ++jj) {
-        cb[c2i(ii, jj)] -= b[ii] * x[jj];
-        for (int kk = 0; kk < 3; ++kk) cb[c3i(ii, jj, kk)] -= 0.5 * b[ii] * x[jj] * x[kk];
-      }
+    // (monomials here; their factors -1, -1/2 follow the sum)
+    const double xx = b0 * x, xy = b0 * y, xz = b0 * z, yx = b1 * x, yy = b1 * y, yz = b1 * z,
+                 zx = b2 * x, zy = b2 * y, zz = b2 * z;
+    const double sxy = xy + yx, sxz = xz + zx, syz = yz + zy;
+    vals[1][lane] = b0; vals[2][lane] = b1; vals[3][lane] = b2;
+    vals[4][lane] = xx; vals[5][lane] = sxy; vals[6][lane] = sxz;
+    vals[7][lane] = yy; vals[8][lane] = syz; vals[9][lane] = zz;
+    vals[10][lane] = xx * x;
+    vals[11][lane] = x * (sxy + xy);
+    vals[12][lane] = x * (sxz + xz);
+    vals[13][lane] = y * (sxy + yx);
+    vals[14][lane] = xy * z + x * syz;
+    vals[15][lane] = z * (sxz + zx);
+    vals[16][lane] = yy * y;
+    vals[17][lane] = y * (syz + yz);
+    vals[18][lane] = z * (syz + zy);
+    vals[19][lane] = zz * z;
+    vals[0][lane] = g0; vals[20][lane] = g1; vals[21][lane] = g2;
+  }
+  __syncwarp();
+  if (lane < 22) {
+    double s = 0.0;
+    for (int j = 0; j < cnt; ++j) s += vals[lane][j];
+    if (lane >= 1 && lane < 20) {
+      const double scale = lane < 10 || lane == 14 ? -1.0 : -0.5;
+      V.cbar[20 * (int64_t)k + lane] = scale * s;
+    } else {
+      // x = x_i - com_alpha: the com receives minus the particles' share
+      if (lane == 0) V.cbar[20 * (int64_t)k] = 0.0;
+      atomicAdd(&V.cell_bar[10 * (int64_t)a + (lane == 0 ? 1 : lane - 18)], -s);
     }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    for (int j = 0; j < 20; ++j) cb[j] += __shfl_xor_sync(0xffffffffu, cb[j], o);
-    gx += __shfl_xor_sync(0xffffffffu, gx, o);
-    gy += __shfl_xor_sync(0xffffffffu, gy, o);
-    gz += __shfl_xor_sync(0xffffffffu, gz, o);
-  }
-  if (lane == 0) {
-    for (int j = 0; j < 20; ++j) V.cbar[20 * (int64_t)k + j] = cb[j];
-    // x = x_i - com_alpha: the com receives minus the particles' share
-    double* cbc = V.cell_bar + 10 * (int64_t)a;
-    atomicAdd(&cbc[1], -gx);
-    atomicAdd(&cbc[2], -gy);
-    atomicAdd(&cbc[3], -gz);
   }
 }
 
@@ -292,28 +353,29 @@ __global__ void k_vjp_m2l(VjpArgs V) {
   const int lane = threadIdx.x & 31;
   if (k >= V.nleaves) return;
   const int a = V.leaf_cells[k];
-  double cb[20];
-  for (int j = 0; j < 20; ++j) cb[j] = V.cbar[20 * (int64_t)k + j];
+  S cb[20];
+  for (int j = 0; j < 20; ++j) cb[j] = (S)V.cbar[20 * (int64_t)k + j];
   const double ax = V.c.cx[a], ay = V.c.cy[a], az = V.c.cz[a];
   double rx = 0.0, ry = 0.0, rz = 0.0;
   const int64_t off = V.far_off[k];
   const int nf = (int)min((int64_t)V.far_cnt[k], V.cap_far);
-  const double zq[6] = {0, 0, 0, 0, 0, 0};
+  const S zq[6] = {0, 0, 0, 0, 0, 0};
   for (int e = lane; e < nf; e += 32) {
     const int b = V.far_idx[off + e];
     const S r[3] = {(S)(ax - V.c.cx[b]), (S)(ay - V.c.cy[b]), (S)(az - V.c.cz[b])};
-    const double* Qb = V.c.Q + 6 * (int64_t)b;
+    S Qb[6];
+    for (int q = 0; q < 6; ++q) Qb[q] = (S)V.c.Q[6 * (int64_t)b + q];
     // r-derivatives of sum_j cb_j C_j by dual numbers; M and Q enter linearly
     const DualT<S> R[3] = {DualT<S>{r[0], {S(1), S(0), S(0)}}, DualT<S>{r[1], {S(0), S(1), S(0)}},
                            DualT<S>{r[2], {S(0), S(0), S(1)}}};
-    const DualT<S> cr = m2l_contract<DualT<S>, STD>(R, V.c.M[b], Qb, cb);
+    const DualT<S> cr = m2l_contract<DualT<S>, STD>(R, (S)V.c.M[b], Qb, cb);
     const double gr[3] = {(double)cr.d[0], (double)cr.d[1], (double)cr.d[2]};
-    const double mbar = (double)m2l_contract<S, STD>(r, 1.0, zq, cb);
+    const double mbar = (double)m2l_contract<S, STD>(r, S(1), zq, cb);
     double qbar[6];
     for (int qq = 0; qq < 6; ++qq) {
-      double eq[6] = {0, 0, 0, 0, 0, 0};
-      eq[qq] = 1.0;
-      qbar[qq] = (double)m2l_contract<S, STD>(r, 0.0, eq, cb);
+      S eq[6] = {0, 0, 0, 0, 0, 0};
+      eq[qq] = S(1);
+      qbar[qq] = (double)m2l_contract<S, STD>(r, S(0), eq, cb);
     }
     rx += gr[0]; ry += gr[1]; rz += gr[2];
     double* cbb = V.cell_bar + 10 * (int64_t)b;
@@ -337,145 +399,558 @@ __global__ void k_vjp_m2l(VjpArgs V) {
   }
 }
 
-// Pair kernel K (a_i += m_j K(d), d = x_i - x_j) and (J b) for J = dK/dd.
-// M4 mass fraction F(q) for 1 <= q < 2, and 4 pi w(q) (the M4 kernel times 4 pi).
-template <class S>
-__device__ __forceinline__ S m4_F_outer(S q) {
-  const S t = S(2) - q;
-  return S(1) - t * t * t * t * (S(1) - S(0.8) * t + t * t / S(6));
+// ---------------------------------------------------------------------------
+// Transposed near lists.  The leaf-only walk is one-sided (b near a does not
+// imply a near b), so the target leaves of a source leaf are collected from
+// the near lists: counts, room reserved per leaf, fill.  A source then sums
+// its own cotangents in registers; with the pairs walked by target alone they
+// took four float64 atomics per (target leaf, source) and butterflies over
+// the leaf's targets per pair (47 ms of the 2^20 Plummer sphere's adjoint).
+// ---------------------------------------------------------------------------
+constexpr int kSrcEntries = 128;        // target leaves per source work item
+
+// The entries of a work item: a leaf's first near segment, or an extra one.
+__device__ __forceinline__ int near_item(const VjpArgs& V, int item, int* k, int64_t* e0) {
+  const bool seg = item >= V.nleaves;
+  const int g = item - V.nleaves;
+  *k = seg ? V.seg_leaf[g] : item;
+  if (*k < 0) return 0;
+  const int64_t sidx = seg ? (int64_t)(g - V.seg_first[*k] + 1) : 0;
+  *e0 = V.near_off[*k] + sidx * kSegEntries;
+  return (int)(min(min((int64_t)V.near_cnt[*k], V.cap_near), (sidx + 1) * kSegEntries) -
+               sidx * kSegEntries);
 }
-template <class S>
-__device__ __forceinline__ S m4_w4pi(S q) {
-  if (q < S(1)) return S(4) * (S(1) - S(1.5) * q * q + S(0.75) * q * q * q);
-  if (q < S(2)) { const S t = S(2) - q; return t * t * t; }
-  return S(0);
+
+__global__ void k_tr_count(VjpArgs V) {
+  const int lane = threadIdx.x & 31;
+  const int nitems = V.nleaves + (int)min((int64_t)V.counters[C_SEGS], V.seg_cap);
+  for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
+       item += (int)((gridDim.x * blockDim.x) >> 5)) {
+    int k;
+    int64_t e0 = 0;
+    const int nn = near_item(V, item, &k, &e0);
+    for (int e = lane; e < nn; e += 32) atomicAdd(&V.tcnt[V.leaf_rank[V.near_idx[e0 + e]]], 1);
+  }
 }
-// K(d) = -f(r) d with J = dK/dd = -f I - g d d^T, g = f'(r) / r.  Plummer:
-// f = (r^2 + eps^2)^(-3/2), g = -3 (r^2 + eps^2)^(-5/2).  M4 (Eq. 13,
-// symmetrised): the mean of the two sides' terms; one side, q = r/h:
+
+// Room for each leaf's entries and extra items (any order), reserved once per warp.
+__global__ void k_tr_plan(VjpArgs V) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r - lane >= V.nleaves) return;
+  const int cnt = r < V.nleaves ? V.tcnt[r] : 0;
+  const int extra = cnt > kSrcEntries ? (cnt - 1) / kSrcEntries : 0;
+  long long ic = cnt;
+  int ie = extra;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long uc = __shfl_up_sync(full, ic, o);
+    const int ue = __shfl_up_sync(full, ie, o);
+    if (lane >= o) { ic += uc; ie += ue; }
+  }
+  unsigned long long bc = 0, be = 0;
+  if (lane == 31) {
+    bc = atomicAdd(&V.tctr[0], (unsigned long long)ic);
+    be = ie ? atomicAdd(&V.tctr[1], (unsigned long long)ie) : 0;
+  }
+  bc = __shfl_sync(full, bc, 31);
+  be = __shfl_sync(full, be, 31);
+  if (r >= V.nleaves) return;
+  V.toff[r] = (int64_t)bc + ic - cnt;
+  const int64_t first = (int64_t)be + ie - extra;
+  V.tseg_first[r] = (int32_t)first;
+  for (int q = 0; q < extra; ++q)
+    if (first + q < V.tseg_cap) V.tseg_leaf[first + q] = r;
+}
+
+__global__ void k_tr_fill(VjpArgs V) {
+  const int lane = threadIdx.x & 31;
+  const int nitems = V.nleaves + (int)min((int64_t)V.counters[C_SEGS], V.seg_cap);
+  for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
+       item += (int)((gridDim.x * blockDim.x) >> 5)) {
+    int k;
+    int64_t e0 = 0;
+    const int nn = near_item(V, item, &k, &e0);
+    for (int e = lane; e < nn; e += 32) {
+      const int r = V.leaf_rank[V.near_idx[e0 + e]];
+      const int64_t at = V.toff[r] + atomicAdd(&V.tcur[r], 1);
+      if (at < V.tcap) V.tidx[at] = k;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// P2P reverse.  Pair kernel K (a_i += m_j K(d), d = x_i - x_j), K = -f(r) d,
+// J = dK/dd = -f I - g d d^T, g = f'(r) / r.  Plummer: f = (r^2 + eps^2)^(-3/2),
+// g = -3 (r^2 + eps^2)^(-5/2).  M4 (Eq. 13, symmetrised): the mean of the two
+// sides' terms; one side, q = r/h:
 //   q < 1:       f = (4/3 - 6/5 q^2 + q^3/2) / h^3,   g = (-12/5 + 3/2 q) / h^5
 //   1 <= q < 2:  f = F(q) / (q^3 h^3),  g = (F'(q) q - 3 F(q)) / (q^5 h^5), F' = 4 pi w q^2
 //   q >= 2:      f = 1 / r^3,           g = -3 / r^5
 // (the q < 1 forms are the polynomials themselves, finite at r = 0, where g
-// multiplies d = 0).
-template <class S>
-__device__ __forceinline__ void pair_fg(int kind, S r2, S eps2, S hi, S hj, S& f, S& g) {
-  if (kind == KDFMM_SOFT_PLUMMER) {
-    const S inv = rsq(r2 + eps2);
-    const S inv3 = inv * inv * inv;
-    f = inv3;
-    g = S(-3) * inv3 * inv * inv;
-    return;
-  }
-  const S r = sqrt(r2);
-  S fs = S(0), gs = S(0);
-  const S hs[2] = {hi, hj};
-  for (int side = 0; side < 2; ++side) {
-    const S h = hs[side];
-    const S hinv = S(1) / h;
-    const S q = r * hinv;
-    const S h3inv = hinv * hinv * hinv;
-    if (q >= S(2)) {
-      const S rinv = S(1) / r;
-      const S r3inv = rinv * rinv * rinv;
-      fs += r3inv;
-      gs += S(-3) * r3inv * rinv * rinv;
-    } else if (q < S(1)) {
-      fs += (S(4) / S(3) + q * q * (S(-1.2) + S(0.5) * q)) * h3inv;
-      gs += (S(-2.4) + S(1.5) * q) * h3inv * hinv * hinv;
-    } else {
-      const S q2 = q * q, F = m4_F_outer(q);
-      fs += F / (q2 * q) * h3inv;
-      gs += (m4_w4pi(q) * q2 * q - S(3) * F) / (q2 * q2 * q) * h3inv * hinv * hinv;
-    }
-  }
-  f = S(0.5) * fs;
-  g = S(0.5) * gs;
+// multiplies d = 0).  F: M4 mass fraction for 1 <= q < 2; 4 pi w(q) = t^3
+// there, t = 2 - q.
+// Target side:  x_bar_i += sum_j m_j J(d) a_bar_i;
+// source side:  x_bar_j -= m_j sum_i J(d) a_bar_i,  m_bar_j += sum_i K(d).a_bar_i.
+// ---------------------------------------------------------------------------
+// The rounding order of a pair's terms is fixed, so that both sides of a pair
+// (and any version of these kernels) form the same float32 values.
+__device__ __forceinline__ float dot_rn(float a0, float b0, float a1, float b1, float a2, float b2) {
+  return __fmaf_rn(a2, b2, __fmaf_rn(a0, b0, __fmul_rn(a1, b1)));
+}
+// One component of J b = -f b - g d (d.b).
+__device__ __forceinline__ float jb_term(float f, float b, float g, float d, float db) {
+  return __fmaf_rn(-f, b, -__fmul_rn(__fmul_rn(g, d), db));
 }
 
-// P2P reverse, warp per target leaf, lanes = (target, slice) as in the
-// forward: the target side x_bar_i += sum_j m_j J(d) a_bar_i stays in the
-// lane; the source side (x_bar_j -= m_j J(d) a_bar_i, m_bar_j += K(d).a_bar_i)
-// is summed over the leaf's targets by shuffles and added with one float64
-// atomic per source into separate arrays.
-// S: arithmetic of the pair terms (float in mixed mode); differences of
-// positions are formed in float64 first and every sum is kept in float64.
-template <class S>
-__global__ void k_vjp_p2p(VjpArgs V) {
+__device__ __forceinline__ float m4_F_outer(float q) {
+  const float t = 2.0f - q;
+  return 1.0f - t * t * t * t * (1.0f - 0.8f * t + t * t / 6.0f);
+}
+
+template <int SOFT>
+__device__ __forceinline__ void pair_fg32(float r2, float eps2, float hinv_i, float hinv_j, float& f,
+                                          float& g) {
+  if (SOFT == KDFMM_SOFT_PLUMMER) {
+    const float inv = rsq(__fadd_rn(r2, eps2));
+    const float inv3 = __fmul_rn(__fmul_rn(inv, inv), inv);
+    f = inv3;
+    g = -3.0f * inv3 * inv * inv;
+    return;
+  }
+  const float r = sqrtf(r2);
+  float fs = 0.0f, gs = 0.0f;
+  const float hs[2] = {hinv_i, hinv_j};
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    const float hinv = hs[side];
+    const float q = r * hinv;
+    const float h3inv = hinv * hinv * hinv;
+    if (q >= 2.0f) {
+      const float rinv = 1.0f / r;
+      const float r3inv = rinv * rinv * rinv;
+      fs += r3inv;
+      gs += -3.0f * r3inv * rinv * rinv;
+    } else if (q < 1.0f) {
+      fs += (4.0f / 3.0f + q * q * (-1.2f + 0.5f * q)) * h3inv;
+      gs += (-2.4f + 1.5f * q) * h3inv * hinv * hinv;
+    } else {
+      const float q2 = q * q, F = m4_F_outer(q);
+      const float t = 2.0f - q;
+      fs += F / (q2 * q) * h3inv;
+      gs += (t * t * t * q2 * q - 3.0f * F) / (q2 * q2 * q) * h3inv * hinv * hinv;
+    }
+  }
+  f = 0.5f * fs;
+  g = 0.5f * gs;
+}
+
+// The leaves of a batch of up to 32 list entries, one per lane, in shared memory.
+struct LeafBatch {
+  int first[32], count[32];
+};
+
+constexpr int kVjpWarps = 4;
+
+// Mixed mode, target side: warp per target leaf (or segment of a long near
+// list), lanes = (target, slice) as in the forward; a leaf's sources are read
+// by broadcast (a warp instruction touches the slices' few records).  Terms in
+// float32, the same operations as the source side's; each is added to a
+// (high, low) float32 pair, 48 bits, which takes the place of a float64 sum
+// (three float64 additions a pair would keep the 1/64-rate pipe busy for
+// longer than the rest of the pair).  2^20 Plummer sphere, 1.17e9 pairs: 4.7 ms
+// here and 5.7 ms on the source side, against 47.3 ms for the two together
+// when one kernel walked the pairs by target.
+template <int SOFT>
+__global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target32(VjpArgs V) {
+  __shared__ LeafBatch s_batch[kVjpWarps];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  LeafBatch& B = s_batch[threadIdx.x >> 5];
+  const int nitems = V.nleaves + (int)min((int64_t)V.counters[C_SEGS], V.seg_cap);
+  for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
+       item += (int)((gridDim.x * blockDim.x) >> 5)) {
+    const bool seg = item >= V.nleaves;
+    const int gi = item - V.nleaves;
+    int k;
+    int64_t e0 = 0;
+    const int nn = near_item(V, item, &k, &e0);
+    if (k < 0) continue;
+    const int a = V.leaf_cells[k];
+    const int fa = V.c.first[a], nt = V.c.count[a];
+    const int K = 32 / nt, t = lane % nt, sl = lane / nt;
+    const bool act = sl < K;
+    const int pi = fa + t;
+    const float4 o0 = V.q0[pi], o1 = V.q1[pi], o2 = V.q2[pi];
+    const float2 o3 = V.q3[pi];
+    const float3 b = make_float3(o2.w, o3.x, o3.y);
+    const double eps = V.sys_eps[V.leaf_sys[k]];
+    float eps2 = (float)(eps * eps);
+    asm("" : "+f"(eps2));
+    float gxh = 0.f, gxl = 0.f, gyh = 0.f, gyl = 0.f, gzh = 0.f, gzl = 0.f;
+    for (int eb = 0; eb < nn; eb += 32) {
+      __syncwarp();
+      if (eb + lane < nn) {
+        const int bc = V.near_idx[e0 + eb + lane];
+        B.first[lane] = V.c.first[bc];
+        B.count[lane] = V.c.count[bc];
+      }
+      __syncwarp();
+      const int m = min(32, nn - eb);
+      for (int q = 0; act && q < m; ++q) {
+        const int fb = B.first[q], nb = B.count[q];
+        for (int j = sl; j < nb; j += K) {
+          const int pj = fb + j;
+          const float4 s0 = V.q0[pj], s1 = V.q1[pj], s2 = V.q2[pj];
+          if (pj == pi) continue;
+          const float d0 = grid_diff(o0.x, o1.x, o2.x, s0.x, s1.x, s2.x),
+                      d1 = grid_diff(o0.y, o1.y, o2.y, s0.y, s1.y, s2.y),
+                      d2 = grid_diff(o0.z, o1.z, o2.z, s0.z, s1.z, s2.z);
+          const float r2 = dot_rn(d0, d0, d1, d1, d2, d2);
+          float f, g;
+          pair_fg32<SOFT>(r2, eps2, o1.w, s1.w, f, g);
+          const float db = dot_rn(d0, b.x, d1, b.y, d2, b.z);
+          // J b = -f b - (f'/r) d (d.b)
+          const float jx = jb_term(f, b.x, g, d0, db);
+          const float jy = jb_term(f, b.y, g, d1, db);
+          const float jz = jb_term(f, b.z, g, d2, db);
+          df_add(gxh, gxl, __fmul_rn(s0.w, jx));
+          df_add(gyh, gyl, __fmul_rn(s0.w, jy));
+          df_add(gzh, gzl, __fmul_rn(s0.w, jz));
+        }
+      }
+    }
+    double gx = (double)gxh + (double)gxl, gy = (double)gyh + (double)gyl,
+           gz = (double)gzh + (double)gzl;
+    for (int s = 1; s < K; ++s) {
+      const int src = t + s * nt;
+      const double ox = __shfl_sync(full, gx, src), oy = __shfl_sync(full, gy, src),
+                   oz = __shfl_sync(full, gz, src);
+      if (sl == 0) { gx += ox; gy += oy; gz += oz; }
+    }
+    if (act && sl == 0) {
+      if (seg) {
+        double* P = V.seg_part + (int64_t)gi * 128 + 4 * t;
+        P[0] = gx; P[1] = gy; P[2] = gz;
+      } else {
+        V.xbar[3 * (int64_t)pi] += gx;
+        V.xbar[3 * (int64_t)pi + 1] += gy;
+        V.xbar[3 * (int64_t)pi + 2] += gz;
+      }
+    }
+  }
+}
+
+// Mixed mode, source side: warp per source leaf (or piece of a long
+// transposed list), lanes = (source, slice), a slice taking every K-th target
+// leaf.  A leaf's terms are summed over its targets in float32 as a perfect
+// binary tree (four at a time, then a carry stack), then added to a (high,
+// low) float32 pair; one float64 atomic per source and item at the end.
+template <int SOFT>
+__global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source32(VjpArgs V) {
+  __shared__ LeafBatch s_batch[kVjpWarps];
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  LeafBatch& B = s_batch[threadIdx.x >> 5];
+  const int nitems = V.nleaves + (int)min((int64_t)V.tctr[1], V.tseg_cap);
+  for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
+       item += (int)((gridDim.x * blockDim.x) >> 5)) {
+    const bool seg = item >= V.nleaves;
+    const int r = seg ? V.tseg_leaf[item - V.nleaves] : item;
+    const int piece = seg ? item - V.nleaves - V.tseg_first[r] + 1 : 0;
+    const int a = V.leaf_cells[r];
+    const int fa = V.c.first[a], ns = V.c.count[a];
+    const int K = 32 / ns, j = lane % ns, sl = lane / ns;
+    const bool act = sl < K;
+    const int pj = fa + j;
+    const float4 o0 = V.q0[pj], o1 = V.q1[pj], o2 = V.q2[pj];
+    const float mj = o0.w;
+    const double eps = V.sys_eps[V.leaf_sys[r]];
+    float eps2 = (float)(eps * eps);
+    asm("" : "+f"(eps2));
+    float sh[4] = {0.f, 0.f, 0.f, 0.f}, slo[4] = {0.f, 0.f, 0.f, 0.f};
+    const int64_t e0 = V.toff[r] + (int64_t)piece * kSrcEntries;
+    const int nn = min(V.tcnt[r] - piece * kSrcEntries, kSrcEntries);
+    for (int eb = 0; eb < nn; eb += 32) {
+      __syncwarp();
+      if (eb + lane < nn) {
+        const int bc = V.leaf_cells[V.tidx[e0 + eb + lane]];
+        B.first[lane] = V.c.first[bc];
+        B.count[lane] = V.c.count[bc];
+      }
+      __syncwarp();
+      const int m = min(32, nn - eb);
+      if (!act) continue;
+      for (int q = sl; q < m; q += K) {
+        const int fb = B.first[q], nb = B.count[q];
+        float h1[4], h2[4], h3[4], acc[4];
+        for (int i0 = 0; i0 < nb; i0 += 4) {
+          float s[4][4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int pi = fb + i0 + u;
+            s[u][0] = s[u][1] = s[u][2] = s[u][3] = 0.0f;
+            if (i0 + u < nb && pi != pj) {
+              const float4 t0 = V.q0[pi], t1 = V.q1[pi], t2 = V.q2[pi];
+              const float2 t3 = V.q3[pi];
+              const float3 b = make_float3(t2.w, t3.x, t3.y);
+              const float d0 = grid_diff(t0.x, t1.x, t2.x, o0.x, o1.x, o2.x),
+                          d1 = grid_diff(t0.y, t1.y, t2.y, o0.y, o1.y, o2.y),
+                          d2 = grid_diff(t0.z, t1.z, t2.z, o0.z, o1.z, o2.z);
+              const float r2 = dot_rn(d0, d0, d1, d1, d2, d2);
+              float f, g;
+              pair_fg32<SOFT>(r2, eps2, t1.w, o1.w, f, g);
+              const float db = dot_rn(d0, b.x, d1, b.y, d2, b.z);
+              const float jx = jb_term(f, b.x, g, d0, db);
+              const float jy = jb_term(f, b.y, g, d1, db);
+              const float jz = jb_term(f, b.z, g, d2, db);
+              s[u][0] = __fmul_rn(-mj, jx);
+              s[u][1] = __fmul_rn(-mj, jy);
+              s[u][2] = __fmul_rn(-mj, jz);
+              s[u][3] = __fmul_rn(-f, db);    // K(d) . a_bar_i
+            }
+          }
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            float v = __fadd_rn(__fadd_rn(s[0][c], s[1][c]), __fadd_rn(s[2][c], s[3][c]));
+            const int blk = i0 >> 2;
+            const bool last = i0 + 4 >= nb;
+            // the tree over the blocks of four: odd blocks join the one held
+            // below; what is held is joined at the end
+            if (blk & 1) {
+              v = __fadd_rn(h1[c], v);
+              if (blk & 2) {
+                v = __fadd_rn(h2[c], v);
+                if (blk & 4) v = __fadd_rn(h3[c], v); else h3[c] = v;
+              } else {
+                h2[c] = v;
+              }
+            } else {
+              h1[c] = v;
+            }
+            if (last) {
+              if (!(blk & 1)) {
+                if (blk & 2) v = __fadd_rn(h2[c], v);
+                if (blk & 4) v = __fadd_rn(h3[c], v);
+              } else if (!(blk & 2)) {
+                if (blk & 4) v = __fadd_rn(h3[c], v);
+              }
+              acc[c] = v;
+            }
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) df_add(sh[c], slo[c], acc[c]);
+      }
+    }
+    double g[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) g[c] = (double)sh[c] + (double)slo[c];
+    for (int s = 1; s < K; ++s) {
+      const int src = j + s * ns;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const double o = __shfl_sync(full, g[c], src);
+        if (sl == 0) g[c] += o;
+      }
+    }
+    if (act && sl == 0) {
+      atomicAdd(&V.xsrc[3 * (int64_t)pj], g[0]);
+      atomicAdd(&V.xsrc[3 * (int64_t)pj + 1], g[1]);
+      atomicAdd(&V.xsrc[3 * (int64_t)pj + 2], g[2]);
+      atomicAdd(&V.msrc[pj], g[3]);
+    }
+  }
+}
+
+// Float64 f and g of the M4 pair, r2 > 0 or = 0 (finite: the q < 1 form).
+__device__ __forceinline__ void m4_fg64(double r2, double hinv_i, double hinv_j, double& f, double& g) {
+  const double inv = rsqrt64(fmax(r2, 1e-290));
+  const double r = r2 * inv;
+  const double inv2 = inv * inv, inv3 = inv2 * inv, inv5 = inv3 * inv2;
+  const double hs[2] = {hinv_i, hinv_j};
+  f = g = 0.0;
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    const double hinv = hs[side], q = r * hinv;
+    if (q < 1.0) {
+      const double h2inv = hinv * hinv, h3inv = h2inv * hinv;
+      f += (4.0 / 3.0 + q * q * (-1.2 + 0.5 * q)) * h3inv;
+      g += (-2.4 + 1.5 * q) * (h3inv * h2inv);
+    } else {
+      const double t = fmax(2.0 - q, 0.0);
+      const double t3 = t * t * t;
+      const double F = 1.0 - t3 * t * (1.0 + t * (-0.8 + t * (1.0 / 6.0)));
+      f += F * inv3;
+      g += (t3 * (q * q * q) - 3.0 * F) * inv5;
+    }
+  }
+  f *= 0.5;
+  g *= 0.5;
+}
+
+// Whether a pair may lie inside either smoothing kernel's support: float32
+// test with a margin, h2 = (2 h)^2 of each side (true where the squared
+// distance leaves the float range; the kernel's formulas hold outside too).
+__device__ __forceinline__ bool maybe_inside(double r2, float h2i, float h2j) {
+  const float r2f = trunc_to_float(r2);
+  return !(r2f >= fmaxf(h2i, h2j) * 1.000001f && r2f < __int_as_float(0x7f800000));
+}
+
+// FP64 mode, target side (as k_vjp_target32, in float64).  x_bar_i gets
+// -(a_bar_i sum m f + sum m g (d.a_bar_i) d).  M4: pairs outside both supports
+// first (f = r^-3, g = -3 r^-5), those that may be inside are marked and
+// follow with the kernel, so that a warp does not run both paths per pair.
+template <int SOFT>
+__global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target64(VjpArgs V) {
+  constexpr bool M4 = SOFT == KDFMM_SOFT_M4;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int nitems = V.nleaves + (int)min((int64_t)V.counters[C_SEGS], V.seg_cap);
   for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
        item += (int)((gridDim.x * blockDim.x) >> 5)) {
-  const bool seg = item >= V.nleaves;
-  const int g = item - V.nleaves;
-  const int k = seg ? V.seg_leaf[g] : item;
-  if (k < 0) continue;
-  const int a = V.leaf_cells[k];
-  const int fa = V.c.first[a], nt = V.c.count[a];
-  const int K = 32 / nt, t = lane % nt, sl = lane / nt;
-  const bool act = sl < K;
-  const int64_t pi = (int64_t)fa + t;
-  const double xi = V.tp.x[pi], yi = V.tp.y[pi], zi = V.tp.z[pi], hi = V.tp.h[pi];
-  const S bS[3] = {(S)V.ab[3 * pi], (S)V.ab[3 * pi + 1], (S)V.ab[3 * pi + 2]};
-  const double eps = V.sys_eps[V.leaf_sys[k]], eps2 = eps * eps;
-  double gx = 0.0, gy = 0.0, gz = 0.0;
-  const int64_t nall = min((int64_t)V.near_cnt[k], V.cap_near);
-  const int64_t sidx = seg ? (int64_t)(g - V.seg_first[k] + 1) : 0;
-  const int64_t e0 = V.near_off[k] + sidx * kSegEntries;
-  const int nn = (int)(min(nall, (sidx + 1) * kSegEntries) - sidx * kSegEntries);
-  for (int e = 0; e < nn; ++e) {
-    const int bc = V.near_idx[e0 + e];
-    const int fb = V.c.first[bc], nb = V.c.count[bc];
-    const int iters = (nb + K - 1) / K;
-    for (int it = 0; it < iters; ++it) {
-      const int j = sl + K * it;
-      const int64_t pj = (int64_t)fb + j;
-      S sx = S(0), sy = S(0), sz = S(0), sm = S(0);
-      if (act && j < nb && pj != pi) {
-        const S d[3] = {(S)(xi - V.tp.x[pj]), (S)(yi - V.tp.y[pj]), (S)(zi - V.tp.z[pj])};
-        const S r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-        S f, g;
-        pair_fg<S>(V.soft_kind, r2, (S)eps2, (S)hi, (S)V.tp.h[pj], f, g);
-        const S db = d[0] * bS[0] + d[1] * bS[1] + d[2] * bS[2];
-        const S mj = (S)V.tp.m[pj];
-        // J b = -f b - (f'/r) d (d.b)
-        const S jx = -f * bS[0] - g * d[0] * db;
-        const S jy = -f * bS[1] - g * d[1] * db;
-        const S jz = -f * bS[2] - g * d[2] * db;
-        gx += (double)(mj * jx); gy += (double)(mj * jy); gz += (double)(mj * jz);
-        sx = -mj * jx; sy = -mj * jy; sz = -mj * jz;
-        sm = -f * db;                                          // K(d) . a_bar_i
+    const bool seg = item >= V.nleaves;
+    const int gi = item - V.nleaves;
+    int k;
+    int64_t e0 = 0;
+    const int nn = near_item(V, item, &k, &e0);
+    if (k < 0) continue;
+    const int a = V.leaf_cells[k];
+    const int fa = V.c.first[a], nt = V.c.count[a];
+    const int K = 32 / nt, t = lane % nt, sl = lane / nt;
+    const bool act = sl < K;
+    const int64_t pi = (int64_t)fa + t;
+    const double xi = V.tp.x[pi], yi = V.tp.y[pi], zi = V.tp.z[pi];
+    const double b0 = V.ab[3 * pi], b1 = V.ab[3 * pi + 1], b2 = V.ab[3 * pi + 2];
+    const float h2i = M4 ? V.ph[pi].w : 0.0f;
+    const double hinv_i = M4 ? V.hinv[pi] : 0.0;
+    const double eps = V.sys_eps[V.leaf_sys[k]], eps2 = M4 ? 0.0 : eps * eps;
+    double sf = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
+    for (int e = 0; act && e < nn; ++e) {
+      const int bc = V.near_idx[e0 + e];
+      const int fb = V.c.first[bc], nb = V.c.count[bc];
+      unsigned in = 0u;
+      for (int j = sl; j < nb; j += K) {
+        const int64_t pj = (int64_t)fb + j;
+        if (pj == pi) continue;
+        const double d0 = xi - V.tp.x[pj], d1 = yi - V.tp.y[pj], d2 = zi - V.tp.z[pj];
+        const double r2 = fma(d2, d2, fma(d1, d1, fma(d0, d0, eps2)));
+        if (M4 && maybe_inside(r2, h2i, V.ph[pj].w)) { in |= 1u << j; continue; }
+        const double inv = rsqrt64(r2), inv2 = inv * inv;
+        const double mf = V.tp.m[pj] * (inv2 * inv);
+        const double db = d0 * b0 + d1 * b1 + d2 * b2;
+        const double u = -3.0 * (mf * inv2) * db;
+        sf += mf;
+        gx = fma(u, d0, gx); gy = fma(u, d1, gy); gz = fma(u, d2, gz);
       }
-      for (int o = 1; o < nt; o <<= 1) {                       // over the slice's targets
-        const S ox = __shfl_down_sync(full, sx, o), oy = __shfl_down_sync(full, sy, o);
-        const S oz = __shfl_down_sync(full, sz, o), om = __shfl_down_sync(full, sm, o);
-        if (t + o < nt) { sx += ox; sy += oy; sz += oz; sm += om; }
+      while (M4 && in != 0u) {
+        const int j = __ffs(in) - 1;
+        in &= in - 1u;
+        const int64_t pj = (int64_t)fb + j;
+        const double d0 = xi - V.tp.x[pj], d1 = yi - V.tp.y[pj], d2 = zi - V.tp.z[pj];
+        double f, g;
+        m4_fg64(d0 * d0 + d1 * d1 + d2 * d2, hinv_i, V.hinv[pj], f, g);
+        const double mj = V.tp.m[pj];
+        const double u = mj * g * (d0 * b0 + d1 * b1 + d2 * b2);
+        sf = fma(mj, f, sf);
+        gx = fma(u, d0, gx); gy = fma(u, d1, gy); gz = fma(u, d2, gz);
       }
-      if (t == 0 && act && j < nb) {
-        atomicAdd(&V.xsrc[3 * pj], (double)sx);
-        atomicAdd(&V.xsrc[3 * pj + 1], (double)sy);
-        atomicAdd(&V.xsrc[3 * pj + 2], (double)sz);
-        atomicAdd(&V.msrc[pj], (double)sm);
+    }
+    gx = -fma(sf, b0, gx); gy = -fma(sf, b1, gy); gz = -fma(sf, b2, gz);
+    for (int s = 1; s < K; ++s) {
+      const int src = t + s * nt;
+      const double ox = __shfl_sync(full, gx, src), oy = __shfl_sync(full, gy, src),
+                   oz = __shfl_sync(full, gz, src);
+      if (sl == 0) { gx += ox; gy += oy; gz += oz; }
+    }
+    if (act && sl == 0) {
+      if (seg) {
+        double* P = V.seg_part + (int64_t)gi * 128 + 4 * t;
+        P[0] = gx; P[1] = gy; P[2] = gz;
+      } else {
+        V.xbar[3 * pi] += gx;
+        V.xbar[3 * pi + 1] += gy;
+        V.xbar[3 * pi + 2] += gz;
       }
     }
   }
-  for (int s = 1; s < K; ++s) {
-    const int src = t + s * nt;
-    const double ox = __shfl_sync(full, gx, src), oy = __shfl_sync(full, gy, src),
-                 oz = __shfl_sync(full, gz, src);
-    if (sl == 0) { gx += ox; gy += oy; gz += oz; }
-  }
-  if (act && sl == 0) {
-    if (seg) {
-      double* P = V.seg_part + (int64_t)g * 128 + 4 * t;
-      P[0] = gx; P[1] = gy; P[2] = gz;
-    } else {
-      V.xbar[3 * pi] += gx;
-      V.xbar[3 * pi + 1] += gy;
-      V.xbar[3 * pi + 2] += gz;
+}
+
+// FP64 mode, source side (as k_vjp_source32, in float64):
+// x_bar_j += m_j sum_i (f a_bar_i + g (d.a_bar_i) d), m_bar_j -= sum_i f d.a_bar_i.
+template <int SOFT>
+__global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source64(VjpArgs V) {
+  constexpr bool M4 = SOFT == KDFMM_SOFT_M4;
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int nitems = V.nleaves + (int)min((int64_t)V.tctr[1], V.tseg_cap);
+  for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
+       item += (int)((gridDim.x * blockDim.x) >> 5)) {
+    const bool seg = item >= V.nleaves;
+    const int r = seg ? V.tseg_leaf[item - V.nleaves] : item;
+    const int piece = seg ? item - V.nleaves - V.tseg_first[r] + 1 : 0;
+    const int a = V.leaf_cells[r];
+    const int fa = V.c.first[a], ns = V.c.count[a];
+    const int K = 32 / ns, js = lane % ns, sl = lane / ns;
+    const bool act = sl < K;
+    const int64_t pj = (int64_t)fa + js;
+    const double xj = V.tp.x[pj], yj = V.tp.y[pj], zj = V.tp.z[pj];
+    const float h2j = M4 ? V.ph[pj].w : 0.0f;
+    const double hinv_j = M4 ? V.hinv[pj] : 0.0;
+    const double eps = V.sys_eps[V.leaf_sys[r]], eps2 = M4 ? 0.0 : eps * eps;
+    double g[4] = {0.0, 0.0, 0.0, 0.0};
+    const int64_t e0 = V.toff[r] + (int64_t)piece * kSrcEntries;
+    const int nn = min(V.tcnt[r] - piece * kSrcEntries, kSrcEntries);
+    for (int e = 0; act && e < nn; ++e) {
+      const int bc = V.leaf_cells[V.tidx[e0 + e]];
+      const int fb = V.c.first[bc], nb = V.c.count[bc];
+      unsigned in = 0u;
+      for (int i = sl; i < nb; i += K) {
+        const int64_t pi = (int64_t)fb + i;
+        if (pi == pj) continue;
+        const double d0 = V.tp.x[pi] - xj, d1 = V.tp.y[pi] - yj, d2 = V.tp.z[pi] - zj;
+        const double r2 = fma(d2, d2, fma(d1, d1, fma(d0, d0, eps2)));
+        if (M4 && maybe_inside(r2, h2j, V.ph[pi].w)) { in |= 1u << i; continue; }
+        const double b0 = V.ab[3 * pi], b1 = V.ab[3 * pi + 1], b2 = V.ab[3 * pi + 2];
+        const double inv = rsqrt64(r2), inv2 = inv * inv, f = inv2 * inv;
+        const double fdb = f * (d0 * b0 + d1 * b1 + d2 * b2);
+        const double u = -3.0 * inv2 * fdb;
+        g[0] = fma(f, b0, fma(u, d0, g[0]));
+        g[1] = fma(f, b1, fma(u, d1, g[1]));
+        g[2] = fma(f, b2, fma(u, d2, g[2]));
+        g[3] -= fdb;
+      }
+      while (M4 && in != 0u) {
+        const int i = __ffs(in) - 1;
+        in &= in - 1u;
+        const int64_t pi = (int64_t)fb + i;
+        const double d0 = V.tp.x[pi] - xj, d1 = V.tp.y[pi] - yj, d2 = V.tp.z[pi] - zj;
+        const double b0 = V.ab[3 * pi], b1 = V.ab[3 * pi + 1], b2 = V.ab[3 * pi + 2];
+        double f, gg;
+        m4_fg64(d0 * d0 + d1 * d1 + d2 * d2, V.hinv[pi], hinv_j, f, gg);
+        const double db = d0 * b0 + d1 * b1 + d2 * b2, u = gg * db;
+        g[0] = fma(f, b0, fma(u, d0, g[0]));
+        g[1] = fma(f, b1, fma(u, d1, g[1]));
+        g[2] = fma(f, b2, fma(u, d2, g[2]));
+        g[3] = fma(-f, db, g[3]);
+      }
     }
-  }
+    for (int s = 1; s < K; ++s) {
+      const int src = js + s * ns;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const double o = __shfl_sync(full, g[c], src);
+        if (sl == 0) g[c] += o;
+      }
+    }
+    if (act && sl == 0) {
+      const double mj = V.tp.m[pj];
+      atomicAdd(&V.xsrc[3 * pj], mj * g[0]);
+      atomicAdd(&V.xsrc[3 * pj + 1], mj * g[1]);
+      atomicAdd(&V.xsrc[3 * pj + 2], mj * g[2]);
+      atomicAdd(&V.msrc[pj], g[3]);
+    }
   }
 }
 
@@ -561,28 +1036,35 @@ __global__ void k_scatter_bar(VjpArgs V, double* __restrict__ x_bar, double* __r
 
 }  // namespace
 
+// Scratch of the adjoint, kept with the handle (grows only; freed with it).
+static int ensure_vjp_scratch(kdfmm_tree_s* t, size_t bytes) {
+  if (t->vjp_cap >= bytes) return KDFMM_OK;
+  cudaFree(t->vjp_buf);
+  t->vjp_buf = nullptr;
+  t->vjp_cap = 0;
+  const int rc = check_cuda(cudaMalloc(&t->vjp_buf, bytes), "adjoint scratch");
+  if (!rc) t->vjp_cap = bytes;
+  else cudaGetLastError();
+  return rc;
+}
+
 int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, cudaStream_t s) {
   const int64_t n = t->n;
   const int nl = t->nleaves, nc = t->ncells;
-  // scratch: a_bar, x_bar (two parts), m_bar (two parts) in tree order, then
-  // the leaves' expansion cotangents and the cells' moment cotangents
-  const size_t bytes = (size_t)n * 11 * sizeof(double) + (size_t)nl * 20 * sizeof(double) +
-                       (size_t)nc * 10 * sizeof(double);
-  char* buf = nullptr;
-  int rc = check_cuda(cudaMallocAsync((void**)&buf, bytes, s), "adjoint scratch");
-  if (rc) return rc;
+  const int64_t nnear = t->host_stats[KDFMM_STAT_NNEAR];
   VjpArgs V{};
   V.n = n;
   V.nleaves = nl;
   V.ncells = nc;
-  V.soft_kind = t->p.soft_kind;
   V.leaf_sys = t->leaf_sys;
+  V.sys_root = t->sys_root;
   V.sys_eps = t->sys_eps;
   V.mixed = t->p.precision == KDFMM_MIXED;
   V.leaf_cells = t->leaf_cells;
   V.leaf_rank = t->leaf_rank;
   V.c = t->c;
   V.tp = t->tp;
+  V.ph = t->ph;
   V.lexp32 = t->lexp32;
   V.lexp64 = t->lexp64;
   V.far_cnt = t->L.far_cnt; V.far_idx = t->L.far_idx;
@@ -595,34 +1077,91 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
   V.seg_leaf = t->L.seg_leaf;
   V.seg_part = t->L.seg_part;
   V.seg_cap = t->L.seg_cap;
-  double* dp = reinterpret_cast<double*>(buf);
-  V.ab = dp; dp += 3 * n;
-  V.xbar = dp; dp += 3 * n;
-  V.xsrc = dp; dp += 3 * n;
-  V.mbar = dp; dp += n;
-  V.msrc = dp; dp += n;
-  V.cbar = dp; dp += 20 * (int64_t)nl;
-  V.cell_bar = dp;
-  cudaMemsetAsync(V.cell_bar, 0, (size_t)nc * 10 * sizeof(double), s);
-  k_gather_abar<<<blocks_for(n, 256), 256, 0, s>>>(a_bar, V);
-  k_vjp_l2p<<<blocks_for((int64_t)nl * 32, 128), 128, 0, s>>>(V);
+  V.tcap = nnear;
+  V.tseg_cap = nnear / kSrcEntries + 1;
+  // scratch, in two parts: what starts at zero first (one memset), then the
+  // rest; every array on a 16-byte boundary
+  size_t at = 0, zeroed = 0;
+  auto take = [&](size_t bytes) {
+    const size_t was = at;
+    at += (bytes + 15) / 16 * 16;
+    return was;
+  };
+  const size_t o_cell = take((size_t)nc * 10 * 8), o_xsrc = take((size_t)n * 3 * 8),
+               o_msrc = take((size_t)n * 8), o_mbar = take((size_t)n * 8),
+               o_tcnt = take((size_t)nl * 4), o_tcur = take((size_t)nl * 4), o_tctr = take(16);
+  zeroed = at;
+  const size_t o_xbar = take((size_t)n * 3 * 8), o_cbar = take((size_t)nl * 20 * 8),
+               o_toff = take((size_t)nl * 8), o_tfirst = take((size_t)nl * 4),
+               o_tidx = take((size_t)nnear * 4), o_tseg = take((size_t)V.tseg_cap * 4);
+  const size_t o_q = V.mixed ? take((size_t)n * 56) : take((size_t)n * 32);
+  // a call that is being captured takes its scratch from the stream's pool (a
+  // graph must not refer to memory that the handle may replace)
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  int rc = check_cuda(cudaStreamIsCapturing(s, &capturing), "adjoint stream");
+  if (rc) return rc;
+  const bool pooled = capturing != cudaStreamCaptureStatusNone;
+  char* buf = nullptr;
+  if (pooled) rc = check_cuda(cudaMallocAsync((void**)&buf, at, s), "adjoint scratch");
+  else if (!(rc = ensure_vjp_scratch(t, at))) buf = static_cast<char*>(t->vjp_buf);
+  if (rc) return rc;
+  V.cell_bar = (double*)(buf + o_cell);
+  V.xsrc = (double*)(buf + o_xsrc);
+  V.msrc = (double*)(buf + o_msrc);
+  V.mbar = (double*)(buf + o_mbar);
+  V.tcnt = (int32_t*)(buf + o_tcnt);
+  V.tcur = (int32_t*)(buf + o_tcur);
+  V.tctr = (unsigned long long*)(buf + o_tctr);
+  V.xbar = (double*)(buf + o_xbar);
+  V.cbar = (double*)(buf + o_cbar);
+  V.toff = (int64_t*)(buf + o_toff);
+  V.tseg_first = (int32_t*)(buf + o_tfirst);
+  V.tidx = (int32_t*)(buf + o_tidx);
+  V.tseg_leaf = (int32_t*)(buf + o_tseg);
+  V.q0 = (float4*)(buf + o_q);
+  V.q1 = V.q0 + n;
+  V.q2 = V.q1 + n;
+  V.q3 = (float2*)(V.q2 + n);
+  V.ab = (double*)(buf + o_q);
+  V.hinv = V.ab + 3 * n;
+  cudaMemsetAsync(buf, 0, zeroed, s);
+  const bool m4 = t->p.soft_kind == KDFMM_SOFT_M4;
   const unsigned gw = blocks_for((int64_t)nl * 32, 128);
+  k_vjp_l2p<<<gw, kL2PWarps * 32, 0, s>>>(a_bar, V, m4);
   const bool std_exp = t->p.expansion == KDFMM_EXPANSION_STANDARD;
   if (V.mixed) {
     if (std_exp) k_vjp_m2l<true, float><<<gw, 128, 0, s>>>(V);
     else k_vjp_m2l<false, float><<<gw, 128, 0, s>>>(V);
-    k_vjp_p2p<float><<<gw, 128, 0, s>>>(V);
   } else {
     if (std_exp) k_vjp_m2l<true, double><<<gw, 128, 0, s>>>(V);
     else k_vjp_m2l<false, double><<<gw, 128, 0, s>>>(V);
-    k_vjp_p2p<double><<<gw, 128, 0, s>>>(V);
+  }
+  k_tr_count<<<grid_blocks(), 256, 0, s>>>(V);
+  k_tr_plan<<<blocks_for(nl, 128), 128, 0, s>>>(V);
+  k_tr_fill<<<grid_blocks(), 256, 0, s>>>(V);
+  if (V.mixed) {
+    if (m4) {
+      k_vjp_target32<KDFMM_SOFT_M4><<<gw, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_source32<KDFMM_SOFT_M4><<<gw, kVjpWarps * 32, 0, s>>>(V);
+    } else {
+      k_vjp_target32<KDFMM_SOFT_PLUMMER><<<gw, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_source32<KDFMM_SOFT_PLUMMER><<<gw, kVjpWarps * 32, 0, s>>>(V);
+    }
+  } else {
+    if (m4) {
+      k_vjp_target64<KDFMM_SOFT_M4><<<gw, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_source64<KDFMM_SOFT_M4><<<gw, kVjpWarps * 32, 0, s>>>(V);
+    } else {
+      k_vjp_target64<KDFMM_SOFT_PLUMMER><<<gw, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_source64<KDFMM_SOFT_PLUMMER><<<gw, kVjpWarps * 32, 0, s>>>(V);
+    }
   }
   k_vjp_seg_combine<<<grid_blocks(2), 256, 0, s>>>(V);
   k_vjp_moments<<<blocks_for(nl, 128), 128, 0, s>>>(V);
   k_scatter_bar<<<blocks_for(n, 256), 256, 0, s>>>(V, x_bar, m_bar);
-  t->launches += 7;
+  t->launches += 10;
   rc = check_cuda(cudaGetLastError(), "adjoint launch");
-  cudaFreeAsync(buf, s);
+  if (pooled) cudaFreeAsync(buf, s);
   return rc;
 }
 
