@@ -57,7 +57,6 @@ __device__ __forceinline__ DualT<S> operator*(const DualT<S>& a, const DualT<S>&
 template <class S>
 __device__ __forceinline__ DualT<S>& operator+=(DualT<S>& a, const DualT<S>& b) { return a = a + b; }
 
-__device__ __forceinline__ double rsq(double v) { return 1.0 / sqrt(v); }
 __device__ __forceinline__ float rsq(float v) { return rsqrtf(v); }
 
 template <class S>
@@ -83,7 +82,6 @@ __device__ __forceinline__ T tc(double v) {
   return Lift<T>::of((typename Lift<T>::Scalar)v);
 }
 
-__device__ __forceinline__ double rs(double v) { return rsq(v); }
 __device__ __forceinline__ float rs(float v) { return rsq(v); }
 template <class S>
 __device__ __forceinline__ DualT<S> rs(const DualT<S>& v) { return rsqrt_dual(v); }
@@ -344,46 +342,365 @@ __global__ void __launch_bounds__(kL2PWarps * 32) k_vjp_l2p(const double* __rest
   }
 }
 
-// M2L reverse: warp per sink leaf, lanes over its far cells.  S: arithmetic
-// of the coefficients (float in mixed mode, as in the forward); r is formed
-// in float64 and every sum is kept in float64.
-template <bool STD, class S>
-__global__ void k_vjp_m2l(VjpArgs V) {
+// M2L reverse: warp per sink leaf, lanes over its far cells.  Mixed mode is bound
+// by float32 issue (some 2500 instructions a pair, three quarters of them the
+// dual numbers): the cotangents of M and Q, which needed seven contractions with
+// mostly zero terms (15.8 ms on the 2^20 Plummer sphere, 1.32e8 pairs; 12.0 now), are
+// written without those terms.  A far cell's ten
+// cotangents (M_bar, com_bar, Q_bar) go to float64 atomics through shared
+// memory, so that a warp instruction adds 32 consecutive values (about three
+// cells) instead of one value of 32 scattered cells.
+constexpr int kM2LWarps = 4;
+struct CellBuf {
+  double v[32 * 11];                    // 10 per lane, stride 11 against bank conflicts
+  int cell[32];
+};
+__device__ __forceinline__ void cell_buf_add(const VjpArgs& V, CellBuf& B, int lane, int n) {
+  __syncwarp();
+  for (int i = lane; i < 10 * n; i += 32) {
+    const int c = i / 10, q = i - 10 * c;
+    atomicAdd(&V.cell_bar[10 * (int64_t)B.cell[c] + q], B.v[11 * c + q]);
+  }
+  __syncwarp();
+}
+
+// The cotangent of M: sum_j w_j C_j for M = 1, Q = 0, in the operations and
+// the order of m2l_contract (float32) without its terms that are exactly zero.
+struct GTerms {
+  float g[6];                           // g_n of R
+  float t2, t3, t4;
+};
+__device__ __forceinline__ GTerms g_terms(const float R[3]) {
+  GTerms G;
+  const float R2 = __fadd_rn(__fadd_rn(__fmul_rn(R[0], R[0]), __fmul_rn(R[1], R[1])),
+                             __fmul_rn(R[2], R[2]));
+  G.g[0] = rsqrtf(R2);
+  const float i2 = __fmul_rn(G.g[0], G.g[0]);
+  G.g[1] = -__fmul_rn(G.g[0], i2);
+#pragma unroll
+  for (int n = 2; n < 6; ++n) G.g[n] = __fmul_rn(__fmul_rn((float)(1 - 2 * n), G.g[n - 1]), i2);
+  const float third = (float)(-1.0 / 3.0);
+  G.t2 = __fmul_rn(G.g[2], third);
+  G.t3 = __fmul_rn(G.g[3], third);
+  G.t4 = __fmul_rn(G.g[4], third);
+  return G;
+}
+
+constexpr int kC2[6][2] = {{0, 0}, {0, 1}, {0, 2}, {1, 1}, {1, 2}, {2, 2}};
+constexpr int kC3[10][3] = {{0, 0, 0}, {0, 0, 1}, {0, 0, 2}, {0, 1, 1}, {0, 1, 2},
+                            {0, 2, 2}, {1, 1, 1}, {1, 1, 2}, {1, 2, 2}, {2, 2, 2}};
+
+// s3 R_a R_b R_c + s2 (d_ab R_c + d_ac R_b + d_bc R_a)
+template <int a, int b, int c>
+__device__ __forceinline__ float c3_radial(const float R[3], float s2, float s3) {
+  const float p = __fmul_rn(__fmul_rn(s3, R[a]), R[b]);
+  if constexpr (a == b && b == c) {
+    return __fmaf_rn(s2, __fadd_rn(__fadd_rn(R[a], R[a]), R[a]), __fmul_rn(p, R[c]));
+  } else if constexpr (a == b || b == c) {
+    return __fmaf_rn(s2, a == b ? R[c] : R[a], __fmul_rn(p, R[c]));
+  } else {
+    return __fmul_rn(p, R[c]);
+  }
+}
+
+template <int K>
+__device__ __forceinline__ float mass_c2(const float R[3], float s1, float s2, const float* w, float acc) {
+  constexpr int a = kC2[K][0], b = kC2[K][1];
+  float v = __fmul_rn(__fmul_rn(s2, R[a]), R[b]);
+  if (a == b) v = __fadd_rn(v, s1);
+  return __fmaf_rn(w[4 + K], v, acc);
+}
+template <int K>
+__device__ __forceinline__ float mass_c3(const float R[3], float s2, float s3, const float* w, float acc) {
+  return __fmaf_rn(w[10 + K], c3_radial<kC3[K][0], kC3[K][1], kC3[K][2]>(R, s2, s3), acc);
+}
+__device__ __forceinline__ float mass_cotangent(const float R[3], const GTerms& G, const float w[20]) {
+  const float s1 = -G.g[1], s2 = -G.g[2], s3 = -G.g[3];
+  float acc = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) acc = __fmaf_rn(w[1 + i], __fmul_rn(s1, R[i]), acc);
+  acc = mass_c2<0>(R, s1, s2, w, acc); acc = mass_c2<1>(R, s1, s2, w, acc);
+  acc = mass_c2<2>(R, s1, s2, w, acc); acc = mass_c2<3>(R, s1, s2, w, acc);
+  acc = mass_c2<4>(R, s1, s2, w, acc); acc = mass_c2<5>(R, s1, s2, w, acc);
+  acc = mass_c3<0>(R, s2, s3, w, acc); acc = mass_c3<1>(R, s2, s3, w, acc);
+  acc = mass_c3<2>(R, s2, s3, w, acc); acc = mass_c3<3>(R, s2, s3, w, acc);
+  acc = mass_c3<4>(R, s2, s3, w, acc); acc = mass_c3<5>(R, s2, s3, w, acc);
+  acc = mass_c3<6>(R, s2, s3, w, acc); acc = mass_c3<7>(R, s2, s3, w, acc);
+  acc = mass_c3<8>(R, s2, s3, w, acc); acc = mass_c3<9>(R, s2, s3, w, acc);
+  return acc;
+}
+
+// The cotangent of Q_ij (i = A, j = B, A <= B): sum_j w_j C_j for M = 0 and the
+// unit Q_ij = Q_ji = 1, likewise.  u = Q R has u_A = R_B, u_B = R_A.
+template <int A, int B>
+struct UnitQ {
+  // u_i is R[ui(i)], or zero (-1)
+  __host__ __device__ static constexpr int ui(int i) { return i == A ? B : (i == B ? A : -1); }
+  __host__ __device__ static constexpr bool q(int i, int j) {
+    return (i == A && j == B) || (i == B && j == A);
+  }
+};
+// sum of the non-zero of two terms x y, contracted as fma(x0, y0, x1 y1)
+template <bool Z0, bool Z1>
+__device__ __forceinline__ float sum2(float x0, float y0, float x1, float y1) {
+  if constexpr (Z0 && Z1) return 0.0f;
+  else if constexpr (Z0) return __fmul_rn(x1, y1);
+  else if constexpr (Z1) return __fmul_rn(x0, y0);
+  else return __fmaf_rn(x0, y0, __fmul_rn(x1, y1));
+}
+template <int A, int B, int K>
+__device__ __forceinline__ float q_c2(const float R[3], const GTerms& G, float s1, float s2,
+                                      const float* w, float acc) {
+  using U = UnitQ<A, B>;
+  constexpr int a = kC2[K][0], b = kC2[K][1], ua = U::ui(a), ub = U::ui(b);
+  const float p = __fmul_rn(s2, R[a]);
+  float v;
+  if constexpr (ua < 0 && ub < 0) {
+    v = __fmul_rn(p, R[b]);
+  } else {
+    const float in = sum2<(ub < 0), (ua < 0)>(R[a], R[ub < 0 ? 0 : ub], R[b], R[ua < 0 ? 0 : ua]);
+    v = __fmaf_rn(p, R[b], __fmul_rn(G.t3, in));
+  }
+  if (U::q(a, b)) v = __fadd_rn(v, G.t2);
+  if (a == b) v = __fadd_rn(v, s1);
+  return __fmaf_rn(w[4 + K], v, acc);
+}
+template <int A, int B, int K>
+__device__ __forceinline__ float q_c3(const float R[3], const GTerms& G, float s2, float s3,
+                                      const float* w, float acc) {
+  using U = UnitQ<A, B>;
+  constexpr int a = kC3[K][0], b = kC3[K][1], c = kC3[K][2];
+  constexpr int ua = U::ui(a), ub = U::ui(b), uc = U::ui(c);
+  float v = c3_radial<a, b, c>(R, s2, s3);
+  if constexpr (ua >= 0 || ub >= 0 || uc >= 0) {
+    float x = sum2<(ua < 0), (ub < 0)>(__fmul_rn(R[b], R[c]), R[ua < 0 ? 0 : ua],
+                                       __fmul_rn(R[a], R[c]), R[ub < 0 ? 0 : ub]);
+    if constexpr (uc >= 0) {
+      if constexpr (ua < 0 && ub < 0) x = __fmul_rn(__fmul_rn(R[a], R[b]), R[uc]);
+      else x = __fmaf_rn(__fmul_rn(R[a], R[b]), R[uc], x);
+    }
+    v = __fmaf_rn(G.t4, x, v);
+  }
+  constexpr bool e0 = U::q(b, c), e1 = U::q(a, c), e2 = U::q(a, b);
+  constexpr bool d0 = a == b && uc >= 0, d1 = a == c && ub >= 0, d2 = b == c && ua >= 0;
+  if constexpr (e0 || e1 || e2 || d0 || d1 || d2) {
+    float y = 0.0f, du = 0.0f;
+    if constexpr (e0) y = R[a];
+    if constexpr (e1) y = __fadd_rn(y, R[b]);
+    if constexpr (e2) y = __fadd_rn(y, R[c]);
+    if constexpr (d0) du = R[uc];
+    if constexpr (d1) du = __fadd_rn(du, R[ub]);
+    if constexpr (d2) du = __fadd_rn(du, R[ua]);
+    v = __fmaf_rn(G.t3, __fadd_rn(y, du), v);
+  }
+  return __fmaf_rn(w[10 + K], v, acc);
+}
+template <int A, int B, bool STD>
+__device__ __forceinline__ float q_cotangent(const float R[3], const GTerms& G, const float w[20]) {
+  using U = UnitQ<A, B>;
+  const float q = A == B ? __fmul_rn(R[A], R[A]) : __fmaf_rn(R[A], R[B], __fmul_rn(R[A], R[B]));
+  const float qs = __fmul_rn(q, (float)(1.0 / 6.0));
+  const float s1 = -__fmul_rn(G.g[3], qs);
+  float acc = 0.0f;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    float t = __fmul_rn(s1, R[i]);
+    if (U::ui(i) >= 0) t = __fmaf_rn(s1, R[i], __fmul_rn(G.t2, R[U::ui(i) < 0 ? 0 : U::ui(i)]));
+    acc = __fmaf_rn(w[1 + i], t, acc);
+  }
+  if constexpr (!STD) {
+    const float s2 = -__fmul_rn(G.g[4], qs), s3 = -__fmul_rn(G.g[5], qs);
+    acc = q_c2<A, B, 0>(R, G, s1, s2, w, acc); acc = q_c2<A, B, 1>(R, G, s1, s2, w, acc);
+    acc = q_c2<A, B, 2>(R, G, s1, s2, w, acc); acc = q_c2<A, B, 3>(R, G, s1, s2, w, acc);
+    acc = q_c2<A, B, 4>(R, G, s1, s2, w, acc); acc = q_c2<A, B, 5>(R, G, s1, s2, w, acc);
+    acc = q_c3<A, B, 0>(R, G, s2, s3, w, acc); acc = q_c3<A, B, 1>(R, G, s2, s3, w, acc);
+    acc = q_c3<A, B, 2>(R, G, s2, s3, w, acc); acc = q_c3<A, B, 3>(R, G, s2, s3, w, acc);
+    acc = q_c3<A, B, 4>(R, G, s2, s3, w, acc); acc = q_c3<A, B, 5>(R, G, s2, s3, w, acc);
+    acc = q_c3<A, B, 6>(R, G, s2, s3, w, acc); acc = q_c3<A, B, 7>(R, G, s2, s3, w, acc);
+    acc = q_c3<A, B, 8>(R, G, s2, s3, w, acc); acc = q_c3<A, B, 9>(R, G, s2, s3, w, acc);
+  }
+  return acc;
+}
+
+// Mixed mode: coefficients in float32 (as in the forward), r formed in
+// float64, sums in float64 (atomics) or (high, low) float32 pairs.
+template <bool STD>
+__global__ void __launch_bounds__(kM2LWarps * 32) k_vjp_m2l32(VjpArgs V) {
+  __shared__ CellBuf s_buf[kM2LWarps];
   const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (k >= V.nleaves) return;
+  CellBuf& B = s_buf[threadIdx.x >> 5];
   const int a = V.leaf_cells[k];
-  S cb[20];
-  for (int j = 0; j < 20; ++j) cb[j] = (S)V.cbar[20 * (int64_t)k + j];
+  const float mine = lane < 20 ? (float)V.cbar[20 * (int64_t)k + lane] : 0.0f;
+  float cb[20];
+#pragma unroll
+  for (int j = 0; j < 20; ++j) cb[j] = __shfl_sync(0xffffffffu, mine, j);
+  const double ax = V.c.cx[a], ay = V.c.cy[a], az = V.c.cz[a];
+  float rh[3] = {0.f, 0.f, 0.f}, rl[3] = {0.f, 0.f, 0.f};
+  const int64_t off = V.far_off[k];
+  const int nf = (int)min((int64_t)V.far_cnt[k], V.cap_far);
+  for (int e0 = 0; e0 < nf; e0 += 32) {
+    const int n = min(32, nf - e0);
+    if (lane < n) {
+      const int b = V.far_idx[off + e0 + lane];
+      const double* s64 = V.c.src64 + 10 * (int64_t)b;
+      const float r[3] = {(float)(ax - s64[0]), (float)(ay - s64[1]), (float)(az - s64[2])};
+      const float4 q0 = V.c.src32[4 * (int64_t)b + 2], q1 = V.c.src32[4 * (int64_t)b + 3];
+      const float Qb[6] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y};
+      // r-derivatives of sum_j cb_j C_j by dual numbers; M and Q enter linearly
+      const DualT<float> R[3] = {DualT<float>{r[0], {1.f, 0.f, 0.f}}, DualT<float>{r[1], {0.f, 1.f, 0.f}},
+                                 DualT<float>{r[2], {0.f, 0.f, 1.f}}};
+      const DualT<float> cr =
+          m2l_contract<DualT<float>, STD>(R, V.c.src32[4 * (int64_t)b].w, Qb, cb);
+      double* v = B.v + 11 * lane;
+      B.cell[lane] = b;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        df_add(rh[i], rl[i], cr.d[i]);
+        v[1 + i] = -(double)cr.d[i];
+      }
+      const GTerms G = g_terms(r);
+      v[0] = (double)mass_cotangent(r, G, cb);
+      v[4] = (double)q_cotangent<0, 0, STD>(r, G, cb);
+      v[5] = (double)q_cotangent<0, 1, STD>(r, G, cb);
+      v[6] = (double)q_cotangent<0, 2, STD>(r, G, cb);
+      v[7] = (double)q_cotangent<1, 1, STD>(r, G, cb);
+      v[8] = (double)q_cotangent<1, 2, STD>(r, G, cb);
+      v[9] = (double)q_cotangent<2, 2, STD>(r, G, cb);
+    }
+    cell_buf_add(V, B, lane, n);
+  }
+  double rx = (double)rh[0] + (double)rl[0], ry = (double)rh[1] + (double)rl[1],
+         rz = (double)rh[2] + (double)rl[2];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    rx += __shfl_xor_sync(0xffffffffu, rx, o);
+    ry += __shfl_xor_sync(0xffffffffu, ry, o);
+    rz += __shfl_xor_sync(0xffffffffu, rz, o);
+  }
+  if (lane < 3)
+    atomicAdd(&V.cell_bar[10 * (int64_t)a + 1 + lane], lane == 0 ? rx : (lane == 1 ? ry : rz));
+}
+
+// FP64 mode.  With W1, W2, W3 the leaf's cotangents as symmetric tensors, their
+// traces removed (1/R is harmonic), A(R) = W1.D1 + W2:D2 + W3:D3 of 1/R is
+//   A = g1 l1 + g2 l2 + g3 l3,  l1 = W1.R, l2 = R.W2.R, l3 = W3 R R R,
+// harmonic and homogeneous in each l_n, and the sum of the coefficients is
+// -M A - Q:(grad grad A) / 6.  So M_bar = -A, Q_bar = -(grad grad A) / 6 (an
+// isotropic part, which a traceless Q does not see, left out) and r_bar =
+// -M grad A - grad(Q:grad grad A) / 6, with grad g_n = g_(n+1) R, v = W2 R,
+// Y = W3 R, z = Y R, u = Q R: some 200 float64 operations a pair where the
+// dual numbers and the seven contractions took 3000.
+struct LeafW {
+  double w1[3], w2[6], w3[10];          // compact: xx xy xz yy yz zz; xxx xxy xxz xyy xyz xzz yyy yyz yzz zzz
+};
+template <bool STD>
+__global__ void __launch_bounds__(kM2LWarps * 32) k_vjp_m2l64(VjpArgs V) {
+  __shared__ CellBuf s_buf[kM2LWarps];
+  const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (k >= V.nleaves) return;
+  CellBuf& B = s_buf[threadIdx.x >> 5];
+  const int a = V.leaf_cells[k];
+  LeafW W;
+  {
+    const double* cb = V.cbar + 20 * (int64_t)k;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) W.w1[i] = cb[1 + i];
+    const double tr = (cb[4] + cb[7] + cb[9]) * (1.0 / 3.0);
+    W.w2[0] = cb[4] - tr; W.w2[3] = cb[7] - tr; W.w2[5] = cb[9] - tr;
+    W.w2[1] = 0.5 * cb[5]; W.w2[2] = 0.5 * cb[6]; W.w2[4] = 0.5 * cb[8];
+    const double third = 1.0 / 3.0;
+    double x[10] = {cb[10], cb[11] * third, cb[12] * third, cb[13] * third, cb[14] * (1.0 / 6.0),
+                    cb[15] * third, cb[16], cb[17] * third, cb[18] * third, cb[19]};
+    const double t0 = 0.2 * (x[0] + x[3] + x[5]), t1 = 0.2 * (x[1] + x[6] + x[8]),
+                 t2 = 0.2 * (x[2] + x[7] + x[9]);
+    W.w3[0] = x[0] - 3.0 * t0; W.w3[1] = x[1] - t1; W.w3[2] = x[2] - t2; W.w3[3] = x[3] - t0;
+    W.w3[4] = x[4]; W.w3[5] = x[5] - t0; W.w3[6] = x[6] - 3.0 * t1; W.w3[7] = x[7] - t2;
+    W.w3[8] = x[8] - t1; W.w3[9] = x[9] - 3.0 * t2;
+  }
   const double ax = V.c.cx[a], ay = V.c.cy[a], az = V.c.cz[a];
   double rx = 0.0, ry = 0.0, rz = 0.0;
   const int64_t off = V.far_off[k];
   const int nf = (int)min((int64_t)V.far_cnt[k], V.cap_far);
-  const S zq[6] = {0, 0, 0, 0, 0, 0};
-  for (int e = lane; e < nf; e += 32) {
-    const int b = V.far_idx[off + e];
-    const S r[3] = {(S)(ax - V.c.cx[b]), (S)(ay - V.c.cy[b]), (S)(az - V.c.cz[b])};
-    S Qb[6];
-    for (int q = 0; q < 6; ++q) Qb[q] = (S)V.c.Q[6 * (int64_t)b + q];
-    // r-derivatives of sum_j cb_j C_j by dual numbers; M and Q enter linearly
-    const DualT<S> R[3] = {DualT<S>{r[0], {S(1), S(0), S(0)}}, DualT<S>{r[1], {S(0), S(1), S(0)}},
-                           DualT<S>{r[2], {S(0), S(0), S(1)}}};
-    const DualT<S> cr = m2l_contract<DualT<S>, STD>(R, (S)V.c.M[b], Qb, cb);
-    const double gr[3] = {(double)cr.d[0], (double)cr.d[1], (double)cr.d[2]};
-    const double mbar = (double)m2l_contract<S, STD>(r, S(1), zq, cb);
-    double qbar[6];
-    for (int qq = 0; qq < 6; ++qq) {
-      S eq[6] = {0, 0, 0, 0, 0, 0};
-      eq[qq] = S(1);
-      qbar[qq] = (double)m2l_contract<S, STD>(r, S(0), eq, cb);
+  constexpr int s3[3][6] = {{0, 1, 2, 3, 4, 5}, {1, 3, 4, 6, 7, 8}, {2, 4, 5, 7, 8, 9}};   // W3 slice of an axis
+  for (int e0 = 0; e0 < nf; e0 += 32) {
+    const int n = min(32, nf - e0);
+    if (lane < n) {
+      const int b = V.far_idx[off + e0 + lane];
+      const double* s = V.c.src64 + 10 * (int64_t)b;
+      const double R[3] = {ax - s[0], ay - s[1], az - s[2]};
+      const double M = s[3];
+      const double Q[6] = {s[4], s[5], s[6], s[7], s[8], s[9]};
+      const double g0 = rsqrt64(R[0] * R[0] + R[1] * R[1] + R[2] * R[2]);
+      const double i2 = g0 * g0, g1 = -g0 * i2, g2 = -3.0 * g1 * i2, g3 = -5.0 * g2 * i2,
+                   g4 = -7.0 * g3 * i2, g5 = -9.0 * g4 * i2, g6 = -11.0 * g5 * i2;
+      auto mul = [](const double S[6], const double x[3], double out[3]) {
+        out[0] = S[0] * x[0] + S[1] * x[1] + S[2] * x[2];
+        out[1] = S[1] * x[0] + S[3] * x[1] + S[4] * x[2];
+        out[2] = S[2] * x[0] + S[4] * x[1] + S[5] * x[2];
+      };
+      auto dot = [](const double x[3], const double y[3]) { return x[0] * y[0] + x[1] * y[1] + x[2] * y[2]; };
+      auto con = [](const double S[6], const double T[6]) {
+        return S[0] * T[0] + S[3] * T[3] + S[5] * T[5] + 2.0 * (S[1] * T[1] + S[2] * T[2] + S[4] * T[4]);
+      };
+      double v[3], Y[6], z[3], u[3];
+      mul(W.w2, R, v);
+#pragma unroll
+      for (int q = 0; q < 6; ++q)
+        Y[q] = W.w3[s3[0][q]] * R[0] + W.w3[s3[1][q]] * R[1] + W.w3[s3[2][q]] * R[2];
+      mul(Y, R, z);
+      mul(Q, R, u);
+      const double l1 = dot(W.w1, R), l2 = dot(v, R), l3 = dot(z, R), q = dot(u, R);
+      const double S2 = g2 * l1 + g3 * l2 + g4 * l3;
+      // the quadrupole sees all orders, or the first alone (standard series)
+      double P[3], P4[3], H[6], K[6], dA[3];
+      const double S4 = STD ? g3 * l1 : g3 * l1 + g4 * l2 + g5 * l3;
+      const double S5 = STD ? g4 * l1 : g4 * l1 + g5 * l2 + g6 * l3;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        dA[i] = S2 * R[i] + g1 * W.w1[i] + 2.0 * (g2 * v[i]) + 3.0 * (g3 * z[i]);
+        P[i] = STD ? g2 * W.w1[i] : g2 * W.w1[i] + 2.0 * (g3 * v[i]) + 3.0 * (g4 * z[i]);
+        P4[i] = STD ? g3 * W.w1[i] : g3 * W.w1[i] + 2.0 * (g4 * v[i]) + 3.0 * (g5 * z[i]);
+      }
+#pragma unroll
+      for (int c = 0; c < 6; ++c) {
+        H[c] = STD ? 0.0 : 2.0 * (g2 * W.w2[c]) + 6.0 * (g3 * Y[c]);
+        K[c] = STD ? 0.0 : 2.0 * (g3 * W.w2[c]) + 6.0 * (g4 * Y[c]);
+      }
+      double QP[3], Ku[3], WQ[3] = {0.0, 0.0, 0.0};
+      mul(Q, P, QP);
+      mul(K, u, Ku);
+      if (!STD) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          const double T[6] = {W.w3[s3[i][0]], W.w3[s3[i][1]], W.w3[s3[i][2]],
+                               W.w3[s3[i][3]], W.w3[s3[i][4]], W.w3[s3[i][5]]};
+          WQ[i] = 6.0 * g3 * con(Q, T);
+        }
+      }
+      const double cR = q * S5 + 2.0 * dot(u, P4) + con(Q, K);
+      double* out = B.v + 11 * lane;
+      B.cell[lane] = b;
+      out[0] = -(g1 * l1 + g2 * l2 + g3 * l3);
+      double gr[3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const double t = cR * R[i] + 2.0 * (S4 * u[i] + QP[i] + Ku[i]) + q * P4[i] + WQ[i];
+        gr[i] = -(M * dA[i]) - t * (1.0 / 6.0);
+        out[1 + i] = -gr[i];
+      }
+      rx += gr[0]; ry += gr[1]; rz += gr[2];
+      const double sx = S4 * R[0], sy = S4 * R[1], sz = S4 * R[2];
+      out[4] = (sx * R[0] + 2.0 * (R[0] * P[0]) + H[0]) * (-1.0 / 6.0);
+      out[5] = (sx * R[1] + (R[0] * P[1] + R[1] * P[0]) + H[1]) * (-1.0 / 3.0);
+      out[6] = (sx * R[2] + (R[0] * P[2] + R[2] * P[0]) + H[2]) * (-1.0 / 3.0);
+      out[7] = (sy * R[1] + 2.0 * (R[1] * P[1]) + H[3]) * (-1.0 / 6.0);
+      out[8] = (sy * R[2] + (R[1] * P[2] + R[2] * P[1]) + H[4]) * (-1.0 / 3.0);
+      out[9] = (sz * R[2] + 2.0 * (R[2] * P[2]) + H[5]) * (-1.0 / 6.0);
     }
-    rx += gr[0]; ry += gr[1]; rz += gr[2];
-    double* cbb = V.cell_bar + 10 * (int64_t)b;
-    atomicAdd(&cbb[0], mbar);
-    atomicAdd(&cbb[1], -gr[0]);
-    atomicAdd(&cbb[2], -gr[1]);
-    atomicAdd(&cbb[3], -gr[2]);
-    for (int q = 0; q < 6; ++q) atomicAdd(&cbb[4 + q], qbar[q]);
+    cell_buf_add(V, B, lane, n);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -391,12 +708,8 @@ __global__ void k_vjp_m2l(VjpArgs V) {
     ry += __shfl_xor_sync(0xffffffffu, ry, o);
     rz += __shfl_xor_sync(0xffffffffu, rz, o);
   }
-  if (lane == 0) {
-    double* cba = V.cell_bar + 10 * (int64_t)a;
-    atomicAdd(&cba[1], rx);
-    atomicAdd(&cba[2], ry);
-    atomicAdd(&cba[3], rz);
-  }
+  if (lane < 3)
+    atomicAdd(&V.cell_bar[10 * (int64_t)a + 1 + lane], lane == 0 ? rx : (lane == 1 ? ry : rz));
 }
 
 // ---------------------------------------------------------------------------
@@ -1130,11 +1443,11 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
   k_vjp_l2p<<<gw, kL2PWarps * 32, 0, s>>>(a_bar, V, m4);
   const bool std_exp = t->p.expansion == KDFMM_EXPANSION_STANDARD;
   if (V.mixed) {
-    if (std_exp) k_vjp_m2l<true, float><<<gw, 128, 0, s>>>(V);
-    else k_vjp_m2l<false, float><<<gw, 128, 0, s>>>(V);
+    if (std_exp) k_vjp_m2l32<true><<<gw, kM2LWarps * 32, 0, s>>>(V);
+    else k_vjp_m2l32<false><<<gw, kM2LWarps * 32, 0, s>>>(V);
   } else {
-    if (std_exp) k_vjp_m2l<true, double><<<gw, 128, 0, s>>>(V);
-    else k_vjp_m2l<false, double><<<gw, 128, 0, s>>>(V);
+    if (std_exp) k_vjp_m2l64<true><<<gw, kM2LWarps * 32, 0, s>>>(V);
+    else k_vjp_m2l64<false><<<gw, kM2LWarps * 32, 0, s>>>(V);
   }
   k_tr_count<<<grid_blocks(), 256, 0, s>>>(V);
   k_tr_plan<<<blocks_for(nl, 128), 128, 0, s>>>(V);
