@@ -509,537 +509,420 @@ struct SubArgs {
   int qcap;
 };
 
-// Cells of at least kBlockSeg particles are split by the whole CTA, one after
-// the other; smaller ones by one warp each, in parallel (1024 measured 4 %
-// faster over the build than 256, where a level of 8 cells of 256 took 8
-// CTA-wide splits in a row).
-constexpr int kBlockSeg = 1024;
-constexpr int kSubWarps = kSubtreeThreads / 32;
+// All cells of a tree level are processed together, in batches of up to
+// kBatchCells: a cell's particles are cut into octets (8 consecutive
+// positions, an aligned block of its pairwise tree), a thread takes an octet
+// whatever the size of its cell, and the octets' sums are folded cell by cell
+// as the rest of the perfect binary tree.  So every level keeps the CTA's
+// threads equally busy, and takes a dozen barriers.  Splitting large cells by
+// the CTA one after the other, medium ones by a warp and small ones by a
+// thread left most warps idle behind one: 1009 particles on one CTA took 323 us
+// (now 104), a 60013-particle sphere 450 us (193), 2^24 clumped particles 10.4 ms
+// (4.2).  Bound: the float64 pipe (1/64 rate; 3 products and 4 sums a particle and
+// level) once the SMs are full, barriers and shared-memory latency before.
+constexpr int kBatchCells = 128;
+constexpr int kBatchOctets = kSubtreeMax / 8 + kBatchCells;
+constexpr int kOctetsPerThread = 2;
+static_assert(kBatchOctets <= kOctetsPerThread * kSubtreeThreads, "octets of a batch per thread");
+static_assert(kBatchCells * 2 <= kSubtreeThreads && kBatchCells % 32 == 0, "cells of a batch per thread");
 
-// Shared-memory views of one subtree: float64 particles, float32 shadows of
-// the positions (for the size filter), local index and scratch index arrays,
-// and the two segment queues.
+// Shared-memory views of one subtree.
 struct SubSmem {
-  double *x, *y, *z, *m;
-  float *xf, *yf, *zf;
-  uint16_t *idx, *scr;
-  int4* q[2];
+  double *x, *y, *z, *m;               // float64 particles (phase-A order)
+  Sum4* osum;                          // per octet: its sum, then folded into the cell's first
+  long long* key;                      // (same memory) per cell: exact bounding-box keys, if needed
+  double* com;                         // per cell: centre of mass
+  unsigned long long* s2;              // per cell: exact squared size (bits)
+  int* bb;                             // per cell: float32 bounding box keys, min xyz, max xyz
+  int *d2m, *axis, *irank;             // per cell: float32 squared size, cut axis, rank among the split
+  float* thr2;                         // per cell: candidates for the exact size
+  int* oct0;                           // per cell: its first octet (kBatchCells + 1)
+  int* opre;                           // per octet: left particles before it (kBatchOctets + 1)
+  uint16_t *idx0, *idx1, *fin;         // particle order of a level (two buffers) and of finished leaves
+  int2 *q0, *q1;                       // cells of a level (two buffers): (first | count << 16, cell id)
 };
 
-__device__ __forceinline__ float dist2_f(const SubSmem& S, int q, float cx, float cy, float cz) {
-  const float dx = S.xf[q] - cx, dy = S.yf[q] - cy, dz = S.zf[q] - cz;
-  return dx * dx + dy * dy + dz * dz;
-}
-
-__device__ __forceinline__ float abs_bound(const double lo[3], const double hi[3]) {
-  double X = 0.0;
-  for (int d = 0; d < 3; ++d) X = fmax(X, fmax(fabs(lo[d]), fabs(hi[d])));
-  return (float)X * 1.0000005f;
-}
-
-constexpr int kThreadSeg = 64;                      // split by one thread at this size
-
-// Canonical pairwise sum of the cnt (<= 2^7) particles idx[lf..lf+cnt) by one
-// thread: a carry stack builds the perfect binary tree over the sequence
-// zero-padded to a power of two.  The padded zeros are not added: a subtree
-// of zeros contributes nothing and x + 0 = x, so folding the stack from its
-// top after the last element gives the same tree value.
-__device__ __forceinline__ Sum4 thread_pairwise(const SubSmem& L, int lf, int cnt) {
-  Sum4 st[8];
-  int top = 0;
-  for (int k = 0; k < cnt; ++k) {
-    const int q = L.idx[lf + k];
-    Sum4 e = elem4(L.m[q], L.x[q], L.y[q], L.z[q]);
-    for (int kk = k; kk & 1; kk >>= 1) e = add4(st[--top], e);
-    st[top++] = e;
-  }
-  Sum4 v = st[top - 1];
-  for (int i = top - 2; i >= 0; --i) v = add4(st[i], v);
-  return v;
-}
-
-// Exact squared size of a cell held in shared memory, by one thread: float32
-// distances over the shadow coordinates select the particles that may hold the
-// maximum, and only those are evaluated in float64.
-__device__ __forceinline__ long long thread_size2(const SubSmem& L, int lf, int cnt, double cx,
-                                                  double cy, double cz) {
-  const float cxf = (float)cx, cyf = (float)cy, czf = (float)cz;
-  float d2m = 0.0f, X = fmaxf(fabsf(cxf), fmaxf(fabsf(cyf), fabsf(czf)));
-  for (int k = 0; k < cnt; ++k) {
-    const int q = L.idx[lf + k];
-    d2m = fmaxf(d2m, dist2_f(L, q, cxf, cyf, czf));
-    X = fmaxf(X, fmaxf(fabsf(L.xf[q]), fmaxf(fabsf(L.yf[q]), fabsf(L.zf[q]))));
-  }
-  const float Dm = sqrtf(d2m);
-  const float thr = Dm - 2.0f * dist_err_bound(X * 1.0000005f, Dm);
-  const float thr2 = thr > 0.0f ? thr * thr * (1.0f - 1e-6f) : -1.0f;
-  long long s2 = 0;
-  for (int k = 0; k < cnt; ++k) {
-    const int q = L.idx[lf + k];
-    if (dist2_f(L, q, cxf, cyf, czf) >= thr2)
-      s2 = max(s2, __double_as_longlong(dist2_rn(L.x[q], L.y[q], L.z[q], cx, cy, cz)));
-  }
-  return s2;
-}
-
-// Moments of a leaf in shared memory, computed by one thread.
-__device__ void leaf_thread(const SubArgs& S, const SubSmem& L, int lf, int cnt, int cell,
-                            int depth, int gfirst) {
-  const Sum4 v = thread_pairwise(L, lf, cnt);
-  const double M = v.m;
-  const double cx = __ddiv_rn(v.x, M), cy = __ddiv_rn(v.y, M), cz = __ddiv_rn(v.z, M);
-  const long long s2 = thread_size2(L, lf, cnt, cx, cy, cz);
-  TmpCells t = S.A.tmp;
-  t.first[cell] = gfirst + lf; t.count[cell] = cnt; t.depth[cell] = depth;
-  t.M[cell] = M; t.cx[cell] = cx; t.cy[cell] = cy; t.cz[cell] = cz;
-  t.s[cell] = sqrt(__longlong_as_double(s2));
-  t.left[cell] = -1; t.right[cell] = -1;
-}
-
-// Queues of one level of a subtree: cells to split next, leaves to finish.
-struct Queues {
-  int* qn_next;
-  int4* q_next;
-  int* nleaf;
-  int4* leaves;
-  int leafcap;
-  int n_leaf;      // leaf size of the subtree's system
-};
-
-// Pushes child `c` (local first, count, cell, depth) onto the queue that will
-// process it; called by one thread.
-__device__ __forceinline__ void push_local(const SubArgs& S, const Queues& Q, int4 c) {
-  if (c.y > Q.n_leaf) {
-    int pos = atomicAdd(Q.qn_next, 1);
-    if (pos < S.qcap) Q.q_next[pos] = c; else set_status(S.A.status, ST_CAPACITY);
-  } else {
-    int pos = atomicAdd(Q.nleaf, 1);
-    if (pos < Q.leafcap) Q.leaves[pos] = c; else set_status(S.A.status, ST_CAPACITY);
-  }
-}
-
-// Allocates the two children of `cell` and queues them (lane 0 of the calling
-// warp).  Returns false if the cell table is full.
-__device__ bool make_children(const SubArgs& S, const Queues& Q, int lf, int cnt, int nl, int cell,
-                              int depth) {
-  const int lane = threadIdx.x & 31;
-  const BuildArgs& A = S.A;
-  int ok = 1;
-  if (lane == 0) {
-    const int cid = atomicAdd(&A.counters[0], 2);
-    if (cid + 2 > A.cap_cells) {
-      set_status(A.status, ST_CAPACITY);
-      ok = 0;
-    } else {
-      A.tmp.left[cell] = cid;
-      A.tmp.right[cell] = cid + 1;
-      push_local(S, Q, make_int4(lf, nl, cid, depth + 1));
-      push_local(S, Q, make_int4(lf + nl, cnt - nl, cid + 1, depth + 1));
-    }
-  }
-  return __shfl_sync(0xffffffffu, ok, 0) != 0;
-}
-
-// A segment split by one thread (small cells): sums, bounding box, centre of
-// mass, exact size, serial stable partition; leaf children are finished at
-// once by the same thread.
-__device__ void split_thread(const SubArgs& S, const SubSmem& L, const Queues& Q, int4 e, int gfirst,
-                             int& depth_max) {
-  const int lf = e.x, cnt = e.y, cell = e.z, depth = e.w;
-  const BuildArgs& A = S.A;
-  const Sum4 v = thread_pairwise(L, lf, cnt);
-  long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
-  for (int k = 0; k < cnt; ++k) {
-    const int q = L.idx[lf + k];
-    const long long kx = dkey(L.x[q]), ky = dkey(L.y[q]), kz = dkey(L.z[q]);
-    lo[0] = min(lo[0], kx); hi[0] = max(hi[0], kx);
-    lo[1] = min(lo[1], ky); hi[1] = max(hi[1], ky);
-    lo[2] = min(lo[2], kz); hi[2] = max(hi[2], kz);
-  }
-  double dlo[3], dhi[3];
-  for (int d = 0; d < 3; ++d) { dlo[d] = dunkey(lo[d]); dhi[d] = dunkey(hi[d]); }
-  const double M = v.m;
-  const double cx = __ddiv_rn(v.x, M), cy = __ddiv_rn(v.y, M), cz = __ddiv_rn(v.z, M);
-  const int axis = longest_axis(dlo, dhi);
-  const long long ckey = dkey(axis == 0 ? cx : (axis == 1 ? cy : cz));
-  const double* sa = axis == 0 ? L.x : (axis == 1 ? L.y : L.z);
-  const long long s2 = thread_size2(L, lf, cnt, cx, cy, cz);
-  int nl = 0;
-  for (int k = 0; k < cnt; ++k) nl += dkey(sa[L.idx[lf + k]]) < ckey;
-  if (nl == 0 || nl == cnt) {
-    nl = cnt / 2;
-    atomicAdd(&A.counters[5], 1);
-  } else {
-    int l = 0, r = nl;
-    for (int k = 0; k < cnt; ++k) {
-      const int q = L.idx[lf + k];
-      L.scr[lf + (dkey(sa[q]) < ckey ? l++ : r++)] = (uint16_t)q;
-    }
-    for (int k = 0; k < cnt; ++k) L.idx[lf + k] = L.scr[lf + k];
-  }
-  TmpCells t = A.tmp;
-  t.first[cell] = gfirst + lf; t.count[cell] = cnt; t.depth[cell] = depth;
-  t.M[cell] = M; t.cx[cell] = cx; t.cy[cell] = cy; t.cz[cell] = cz;
-  t.s[cell] = sqrt(__longlong_as_double(s2));
-  const int cid = atomicAdd(&A.counters[0], 2);
-  if (cid + 2 > A.cap_cells) {
-    set_status(A.status, ST_CAPACITY);
-    return;
-  }
-  t.left[cell] = cid;
-  t.right[cell] = cid + 1;
-  depth_max = max(depth_max, depth + 1);
-  const int clf[2] = {lf, lf + nl}, ccnt[2] = {nl, cnt - nl};
-  for (int side = 0; side < 2; ++side) {
-    if (ccnt[side] > Q.n_leaf) {
-      int pos = atomicAdd(Q.qn_next, 1);
-      if (pos < S.qcap) Q.q_next[pos] = make_int4(clf[side], ccnt[side], cid + side, depth + 1);
-      else set_status(A.status, ST_CAPACITY);
-    } else {
-      leaf_thread(S, L, clf[side], ccnt[side], cid + side, depth + 1, gfirst);
-    }
-  }
-}
-
-// A segment split by one warp.
-__device__ void split_warp(const SubArgs& S, const SubSmem& L, const Queues& Q, int4 e, int gfirst,
-                           int& depth_max) {
-  const int lane = threadIdx.x & 31;
-  const int lf = e.x, cnt = e.y, cell = e.z, depth = e.w;
-  const BuildArgs& A = S.A;
-  auto get = [&](int k) {
-    int qq = L.idx[lf + k];
-    return elem4(L.m[qq], L.x[qq], L.y[qq], L.z[qq]);
+__host__ __device__ __forceinline__ size_t sub_carve(unsigned char* base, int qcap, SubSmem* L) {
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    const size_t was = at;
+    at += (bytes + 15) / 16 * 16;
+    return base + was;
   };
-  Sum4 v = warp_pairwise(cnt, get);
-  long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
-  for (int k = lane; k < cnt; k += 32) {
-    int qq = L.idx[lf + k];
-    long long kx = dkey(L.x[qq]), ky = dkey(L.y[qq]), kz = dkey(L.z[qq]);
-    lo[0] = min(lo[0], kx); hi[0] = max(hi[0], kx);
-    lo[1] = min(lo[1], ky); hi[1] = max(hi[1], ky);
-    lo[2] = min(lo[2], kz); hi[2] = max(hi[2], kz);
-  }
-  double dlo[3], dhi[3];
-  for (int d = 0; d < 3; ++d) { dlo[d] = dunkey(warp_min_ll(lo[d])); dhi[d] = dunkey(warp_max_ll(hi[d])); }
-  const double M = v.m;
-  // the three divisions run once, on lanes 0, 1, 2
-  const double quo = __ddiv_rn(lane == 1 ? v.y : (lane == 2 ? v.z : v.x), M);
-  const double cx = __shfl_sync(0xffffffffu, quo, 0), cy = __shfl_sync(0xffffffffu, quo, 1),
-               cz = __shfl_sync(0xffffffffu, quo, 2);
-  const int axis = longest_axis(dlo, dhi);
-  const long long ckey = dkey(axis == 0 ? cx : (axis == 1 ? cy : cz));
-  const double* sa = axis == 0 ? L.x : (axis == 1 ? L.y : L.z);
-  // size: float32 filter, then exact float64 for the candidates
-  const float cxf = (float)cx, cyf = (float)cy, czf = (float)cz, X = abs_bound(dlo, dhi);
-  float d2m = 0.0f;
-  int nl = 0;
-  for (int k = lane; k < cnt; k += 32) {
-    int qq = L.idx[lf + k];
-    d2m = fmaxf(d2m, dist2_f(L, qq, cxf, cyf, czf));
-    nl += dkey(sa[qq]) < ckey;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    d2m = fmaxf(d2m, __shfl_xor_sync(0xffffffffu, d2m, o));
-    nl += __shfl_xor_sync(0xffffffffu, nl, o);
-  }
-  const float Dm = sqrtf(d2m);
-  const float thr = Dm - 2.0f * dist_err_bound(X, Dm);
-  const float thr2 = thr > 0.0f ? thr * thr * (1.0f - 1e-6f) : -1.0f;
-  long long s2 = 0;
-  for (int k = lane; k < cnt; k += 32) {
-    int qq = L.idx[lf + k];
-    if (dist2_f(L, qq, cxf, cyf, czf) >= thr2)
-      s2 = max(s2, __double_as_longlong(dist2_rn(L.x[qq], L.y[qq], L.z[qq], cx, cy, cz)));
-  }
-  s2 = warp_max_ll(s2);
-  const bool fallback = (nl == 0 || nl == cnt);
-  if (fallback) {
-    nl = cnt / 2;
-    if (lane == 0) atomicAdd(&A.counters[5], 1);
-  } else {
-    int offl = 0, offr = nl;
-    for (int base = 0; base < cnt; base += 32) {
-      int k = base + lane;
-      bool valid = k < cnt;
-      int qq = valid ? L.idx[lf + k] : 0;
-      bool f = valid && dkey(sa[qq]) < ckey;
-      unsigned ml = __ballot_sync(0xffffffffu, f);
-      unsigned mr = __ballot_sync(0xffffffffu, valid && !f);
-      unsigned lt = (1u << lane) - 1u;
-      if (valid) L.scr[lf + (f ? offl + __popc(ml & lt) : offr + __popc(mr & lt))] = (uint16_t)qq;
-      offl += __popc(ml);
-      offr += __popc(mr);
-    }
-    __syncwarp();
-    for (int k = lane; k < cnt; k += 32) L.idx[lf + k] = L.scr[lf + k];
-    __syncwarp();
-  }
-  if (lane == 0) {
-    TmpCells t = A.tmp;
-    t.first[cell] = gfirst + lf; t.count[cell] = cnt; t.depth[cell] = depth;
-    t.M[cell] = M; t.cx[cell] = cx; t.cy[cell] = cy; t.cz[cell] = cz;
-    t.s[cell] = sqrt(__longlong_as_double(s2));
-  }
-  if (make_children(S, Q, lf, cnt, nl, cell, depth)) depth_max = max(depth_max, depth + 1);
+  double* x = reinterpret_cast<double*>(take(4 * kSubtreeMax * sizeof(double)));
+  L->x = x; L->y = x + kSubtreeMax; L->z = x + 2 * kSubtreeMax; L->m = x + 3 * kSubtreeMax;
+  L->osum = reinterpret_cast<Sum4*>(take(kBatchOctets * sizeof(Sum4)));
+  L->key = reinterpret_cast<long long*>(L->osum);
+  L->com = reinterpret_cast<double*>(take(3 * kBatchCells * sizeof(double)));
+  L->s2 = reinterpret_cast<unsigned long long*>(take(kBatchCells * sizeof(unsigned long long)));
+  L->bb = reinterpret_cast<int*>(take(6 * kBatchCells * sizeof(int)));
+  L->d2m = reinterpret_cast<int*>(take(kBatchCells * sizeof(int)));
+  L->axis = reinterpret_cast<int*>(take(kBatchCells * sizeof(int)));
+  L->irank = reinterpret_cast<int*>(take(kBatchCells * sizeof(int)));
+  L->thr2 = reinterpret_cast<float*>(take(kBatchCells * sizeof(float)));
+  L->oct0 = reinterpret_cast<int*>(take((kBatchCells + 1) * sizeof(int)));
+  L->opre = reinterpret_cast<int*>(take((kBatchOctets + 1) * sizeof(int)));
+  uint16_t* ix = reinterpret_cast<uint16_t*>(take(3 * kSubtreeMax * sizeof(uint16_t)));
+  L->idx0 = ix; L->idx1 = ix + kSubtreeMax; L->fin = ix + 2 * kSubtreeMax;
+  L->q0 = reinterpret_cast<int2*>(take(2 * (size_t)qcap * sizeof(int2)));
+  L->q1 = L->q0 + qcap;
+  return at;
 }
 
-// Block-wide helpers (all kSubtreeThreads threads call them).
-struct BlockScratch {
-  Sum4 ws[kSubWarps];
-  long long wk[kSubWarps][6];
-  float wf[kSubWarps];
-  int wi[kSubWarps];
-  double com[3];
-  double bb[6];
-  float thr2;
-  int nl;
-  int axis;
-};
-
-// A segment split by the whole CTA.  The pairwise sum splits the padded
-// sequence into kSubWarps aligned sub-blocks, one per warp (the top levels of
-// the same perfect tree).
-__device__ void split_block(const SubArgs& S, const SubSmem& L, BlockScratch& B, const Queues& Q,
-                            int4 e, int gfirst, int& depth_max) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int lf = e.x, cnt = e.y, cell = e.z, depth = e.w;
-  const BuildArgs& A = S.A;
-  int P = 1;
-  while (P < cnt) P <<= 1;                         // P >= kBlockSeg
-  const int Pw = P / kSubWarps;                    // per warp, >= 32
-  const int base = w * Pw + lane * (Pw >> 5);
-  auto get = [&](int k) {
-    int qq = L.idx[lf + k];
-    return elem4(L.m[qq], L.x[qq], L.y[qq], L.z[qq]);
-  };
-  Sum4 v;
-  switch (Pw >> 5) {
-    case 1: v = block_tree<0>(base, cnt, get); break;
-    case 2: v = block_tree<1>(base, cnt, get); break;
-    case 4: v = block_tree<2>(base, cnt, get); break;
-    default: v = block_tree<3>(base, cnt, get); break;
-  }
-  v = warp_tree4(v);
-  long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
-  for (int k = threadIdx.x; k < cnt; k += kSubtreeThreads) {
-    int qq = L.idx[lf + k];
-    long long kx = dkey(L.x[qq]), ky = dkey(L.y[qq]), kz = dkey(L.z[qq]);
-    lo[0] = min(lo[0], kx); hi[0] = max(hi[0], kx);
-    lo[1] = min(lo[1], ky); hi[1] = max(hi[1], ky);
-    lo[2] = min(lo[2], kz); hi[2] = max(hi[2], kz);
-  }
-  for (int d = 0; d < 3; ++d) { lo[d] = warp_min_ll(lo[d]); hi[d] = warp_max_ll(hi[d]); }
-  if (lane == 0) {
-    B.ws[w] = v;
-    for (int d = 0; d < 3; ++d) { B.wk[w][d] = lo[d]; B.wk[w][3 + d] = hi[d]; }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    Sum4 t = add4(add4(add4(B.ws[0], B.ws[1]), add4(B.ws[2], B.ws[3])),
-                  add4(add4(B.ws[4], B.ws[5]), add4(B.ws[6], B.ws[7])));
-    double dlo[3], dhi[3];
-    for (int d = 0; d < 3; ++d) {
-      long long l = B.wk[0][d], h = B.wk[0][3 + d];
-      for (int q = 1; q < kSubWarps; ++q) { l = min(l, B.wk[q][d]); h = max(h, B.wk[q][3 + d]); }
-      dlo[d] = dunkey(l);
-      dhi[d] = dunkey(h);
-    }
-    B.com[0] = t.x; B.com[1] = t.y; B.com[2] = t.z; B.bb[0] = t.m;
-    B.axis = longest_axis(dlo, dhi);
-  }
-  __syncthreads();
-  if (w == 0) {                                    // the three divisions on lanes 0, 1, 2
-    const double quo = __ddiv_rn(B.com[lane < 3 ? lane : 0], B.bb[0]);
-    const double Mc = B.bb[0];
-    __syncwarp();
-    if (lane < 3) B.com[lane] = quo;
-    if (lane == 0) {
-      TmpCells tc = A.tmp;
-      tc.first[cell] = gfirst + lf; tc.count[cell] = cnt; tc.depth[cell] = depth;
-      tc.M[cell] = Mc; tc.cx[cell] = quo;
-    }
-    const double qy = __shfl_sync(0xffffffffu, quo, 1), qz = __shfl_sync(0xffffffffu, quo, 2);
-    if (lane == 0) { A.tmp.cy[cell] = qy; A.tmp.cz[cell] = qz; }
-  }
-  __syncthreads();
-  const double cx = B.com[0], cy = B.com[1], cz = B.com[2];
-  const int axis = B.axis;
-  const long long ckey = dkey(B.com[axis]);
-  const double* sa = axis == 0 ? L.x : (axis == 1 ? L.y : L.z);
-  const float cxf = (float)cx, cyf = (float)cy, czf = (float)cz;
-  float d2m = 0.0f;
-  int nl = 0;
-  for (int k = threadIdx.x; k < cnt; k += kSubtreeThreads) {
-    int qq = L.idx[lf + k];
-    d2m = fmaxf(d2m, dist2_f(L, qq, cxf, cyf, czf));
-    nl += dkey(sa[qq]) < ckey;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    d2m = fmaxf(d2m, __shfl_xor_sync(0xffffffffu, d2m, o));
-    nl += __shfl_xor_sync(0xffffffffu, nl, o);
-  }
-  if (lane == 0) { B.wf[w] = d2m; B.wi[w] = nl; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float m2 = 0.0f;
-    int t = 0;
-    for (int q = 0; q < kSubWarps; ++q) { m2 = fmaxf(m2, B.wf[q]); t += B.wi[q]; }
-    double blo[3], bhi[3];
-    for (int d = 0; d < 3; ++d) {
-      long long l = B.wk[0][d], h = B.wk[0][3 + d];
-      for (int q = 1; q < kSubWarps; ++q) { l = min(l, B.wk[q][d]); h = max(h, B.wk[q][3 + d]); }
-      blo[d] = dunkey(l);
-      bhi[d] = dunkey(h);
-    }
-    const float Dm = sqrtf(m2);
-    const float thr = Dm - 2.0f * dist_err_bound(abs_bound(blo, bhi), Dm);
-    B.thr2 = thr > 0.0f ? thr * thr * (1.0f - 1e-6f) : -1.0f;
-    B.nl = t;
-  }
-  __syncthreads();
-  const float thr2 = B.thr2;
-  nl = B.nl;
-  long long s2 = 0;
-  for (int k = threadIdx.x; k < cnt; k += kSubtreeThreads) {
-    int qq = L.idx[lf + k];
-    if (dist2_f(L, qq, cxf, cyf, czf) >= thr2)
-      s2 = max(s2, __double_as_longlong(dist2_rn(L.x[qq], L.y[qq], L.z[qq], cx, cy, cz)));
-  }
-  s2 = warp_max_ll(s2);
-  __syncthreads();                                 // B.wk reused below
-  if (lane == 0) B.wk[w][0] = s2;
-  const bool fallback = (nl == 0 || nl == cnt);
-  if (!fallback) {
-    // stable partition in rounds of one element per thread
-    int offl = 0;
-    for (int r0 = 0; r0 < cnt; r0 += kSubtreeThreads) {
-      const int k = r0 + threadIdx.x;
-      const bool valid = k < cnt;
-      const int qq = valid ? L.idx[lf + k] : 0;
-      const bool f = valid && dkey(sa[qq]) < ckey;
-      const unsigned ml = __ballot_sync(0xffffffffu, f);
-      if (lane == 0) B.wi[w] = __popc(ml);
-      __syncthreads();
-      int woff = 0, tot = 0;
-      for (int q = 0; q < kSubWarps; ++q) {
-        if (q < w) woff += B.wi[q];
-        tot += B.wi[q];
-      }
-      if (valid) {
-        const int lb = offl + woff + __popc(ml & ((1u << lane) - 1u));
-        L.scr[lf + (f ? lb : nl + (k - lb))] = (uint16_t)qq;
-      }
-      offl += tot;
-      __syncthreads();
-    }
-    for (int k = threadIdx.x; k < cnt; k += kSubtreeThreads) L.idx[lf + k] = L.scr[lf + k];
-  }
-  __syncthreads();
-  if (w == 0) {
-    long long m2 = lane < kSubWarps ? B.wk[lane][0] : 0;
-    m2 = warp_max_ll(m2);
-    if (lane == 0) A.tmp.s[cell] = sqrt(__longlong_as_double(m2));
-    if (fallback) {
-      nl = cnt / 2;
-      if (lane == 0) atomicAdd(&A.counters[5], 1);
-    }
-    if (make_children(S, Q, lf, cnt, nl, cell, depth)) depth_max = max(depth_max, depth + 1);
-  }
-  __syncthreads();
+// Order-preserving int32 key of a float.
+__device__ __forceinline__ int fkey(float v) {
+  const int b = __float_as_int(v);
+  return b ^ ((b >> 31) & 0x7fffffff);
 }
+__device__ __forceinline__ float funkey(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7fffffff)); }
 
-__global__ void __launch_bounds__(kSubtreeThreads)
+__global__ void __launch_bounds__(kSubtreeThreads, 2)
 k_subtree(SubArgs S) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ BlockScratch B;
-  __shared__ int qn[2];
-  __shared__ int nleaf;
+  __shared__ int s_seg, s_base, s_tot[3][kBatchCells / 32];
   SubSmem L;
-  L.x = reinterpret_cast<double*>(smem_raw);
-  L.y = L.x + kSubtreeMax;
-  L.z = L.y + kSubtreeMax;
-  L.m = L.z + kSubtreeMax;
-  L.xf = reinterpret_cast<float*>(L.m + kSubtreeMax);
-  L.yf = L.xf + kSubtreeMax;
-  L.zf = L.yf + kSubtreeMax;
-  L.idx = reinterpret_cast<uint16_t*>(L.zf + kSubtreeMax);
-  L.scr = L.idx + kSubtreeMax;
-  L.q[0] = reinterpret_cast<int4*>(L.scr + kSubtreeMax);
-  L.q[1] = L.q[0] + S.qcap;
-  int4* leaves = L.q[1] + S.qcap;
-  const int leafcap = 2 * S.qcap;
+  sub_carve(smem_raw, S.qcap, &L);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned full = 0xffffffffu;
+  const BuildArgs& A = S.A;
+  const TmpCells& T = A.tmp;
 
   // persistent: the CTA takes segments from a work counter until none is left
-  __shared__ int s_seg;
-  const int nB = min(S.A.counters[C_NB], (int)S.A.capB);
+  const int nB = min(A.counters[C_NB], (int)A.capB);
   for (;;) {
   __syncthreads();
-  if (threadIdx.x == 0) s_seg = atomicAdd(&S.A.counters[C_WORK], 1);
+  if (tid == 0) s_seg = atomicAdd(&A.counters[C_WORK], 1);
   __syncthreads();
   if (s_seg >= nB) break;
   const Seg g = S.segB[s_seg];
   const PCols in = (g.dbuf & 1) ? S.buf1 : S.buf0;
-  const int n = g.count;
-  const int gfirst = g.first;
-  const int n_leaf = nleaf_at(S.A, gfirst);
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    const double x = in.x[gfirst + k], y = in.y[gfirst + k], z = in.z[gfirst + k];
-    L.x[k] = x; L.y[k] = y; L.z[k] = z;
+  const int n = g.count, gfirst = g.first;
+  const int n_leaf = nleaf_at(A, gfirst);
+  for (int k = tid; k < n; k += kSubtreeThreads) {
+    L.x[k] = in.x[gfirst + k]; L.y[k] = in.y[gfirst + k]; L.z[k] = in.z[gfirst + k];
     L.m[k] = in.m[gfirst + k];
-    L.xf[k] = trunc_to_float(x); L.yf[k] = trunc_to_float(y); L.zf[k] = trunc_to_float(z);
-    L.idx[k] = (uint16_t)k;
+    L.idx0[k] = (uint16_t)k;
   }
-  int cur = 0;
-  if (threadIdx.x == 0) {
-    L.q[0][0] = make_int4(0, n, g.cell, g.dbuf >> 1);
-    qn[0] = 1;
-  }
+  if (tid == 0) L.q0[0] = make_int2(n << 16, g.cell);
+  int cur = 0, nq = 1, depth = g.dbuf >> 1;
+  bool overflow = false;
   __syncthreads();
-  const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  int depth_max = 0;
-  while (qn[cur] > 0) {
-    const int nxt = cur ^ 1;
-    if (threadIdx.x == 0) { qn[nxt] = 0; nleaf = 0; }
-    __syncthreads();
-    const int nq = qn[cur];
-    const Queues Q{&qn[nxt], L.q[nxt], &nleaf, leaves, leafcap, n_leaf};
-    // large cells: the whole CTA, one after the other
-    for (int qi = 0; qi < nq; ++qi) {
-      const int4 e = L.q[cur][qi];
-      if (e.y >= kBlockSeg) split_block(S, L, B, Q, e, gfirst, depth_max);
+  while (nq > 0 && !overflow) {
+    const uint16_t* const ix = cur ? L.idx1 : L.idx0;
+    uint16_t* const ox = cur ? L.idx0 : L.idx1;
+    const int2* const q_in = cur ? L.q1 : L.q0;
+    int2* const q_out = cur ? L.q0 : L.q1;
+    int nq_next = 0;
+    for (int b0 = 0; b0 < nq && !overflow; b0 += kBatchCells) {
+      const int ncb = min(kBatchCells, nq - b0);
+      const int2* const q = q_in + b0;
+      // octets and split cells before each cell (packed in one scan)
+      int cnt_c = 0, pack = 0, incl = 0;
+      if (tid < kBatchCells) {
+        cnt_c = tid < ncb ? q[tid].x >> 16 : 0;
+        incl = pack = ((cnt_c + 7) >> 3) | (cnt_c > n_leaf) << 16;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(full, incl, o);
+          if (lane >= o) incl += v;
+        }
+        const int mx = __reduce_max_sync(full, pack & 0xffff);
+        if (lane == 31) { s_tot[0][warp] = incl; s_tot[1][warp] = mx; }
+      }
+      __syncthreads();
+      int noct = 0, nsplit = 0, maxoct = 0;
+#pragma unroll
+      for (int w = 0; w < kBatchCells / 32; ++w) {
+        const int v = s_tot[0][w];
+        if (w < warp) incl += v;
+        noct += v & 0xffff;
+        nsplit += v >> 16;
+        maxoct = max(maxoct, s_tot[1][w]);
+      }
+      int base = 0;                       // (thread 0) first id of the children
+      if (tid < kBatchCells) {
+        const int ex = incl - pack;
+        L.oct0[tid] = ex & 0xffff;
+        L.irank[tid] = ex >> 16;
+        L.s2[tid] = 0ull;
+        L.d2m[tid] = 0;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) { L.bb[6 * tid + d] = INT_MAX; L.bb[6 * tid + 3 + d] = INT_MIN; }
+        if (tid == 0) {
+          L.oct0[kBatchCells] = noct;
+          if (nsplit > 0) base = atomicAdd(&A.counters[C_CELLS], 2 * nsplit);
+        }
+      }
+      __syncthreads();
+      // the thread's octets: cell, first element in the cell, elements
+      int oc[kOctetsPerThread], rel[kOctetsPerThread], val[kOctetsPerThread];
+      int lf[kOctetsPerThread], cn[kOctetsPerThread];
+#pragma unroll
+      for (int u = 0; u < kOctetsPerThread; ++u) {
+        const int o = tid + u * kSubtreeThreads;
+        oc[u] = -1; rel[u] = val[u] = lf[u] = cn[u] = 0;
+        if (o < noct) {
+          int c = 0;
+#pragma unroll
+          for (int step = kBatchCells / 2; step > 0; step >>= 1)
+            if (c + step < ncb && L.oct0[c + step] <= o) c += step;
+          const int e = q[c].x;
+          oc[u] = c;
+          lf[u] = e & 0xffff;
+          cn[u] = e >> 16;
+          rel[u] = 8 * (o - L.oct0[c]);
+          val[u] = min(8, cn[u] - rel[u]);
+        }
+      }
+      // octet sums, float32 bounding boxes (coordinates truncated: monotone)
+#pragma unroll
+      for (int u = 0; u < kOctetsPerThread; ++u) {
+        if (u * kSubtreeThreads + (tid & ~31) >= noct) continue;    // the whole warp has none
+        int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
+        if (oc[u] >= 0) {
+          const uint16_t* p = ix + lf[u] + rel[u];
+          auto get = [&](int k) {
+            const int i = p[k];
+            const double x = L.x[i], y = L.y[i], z = L.z[i];
+            const int kx = fkey(trunc_to_float(x)), ky = fkey(trunc_to_float(y)),
+                      kz = fkey(trunc_to_float(z));
+            lo[0] = min(lo[0], kx); hi[0] = max(hi[0], kx);
+            lo[1] = min(lo[1], ky); hi[1] = max(hi[1], ky);
+            lo[2] = min(lo[2], kz); hi[2] = max(hi[2], kz);
+            return elem4(L.m[i], x, y, z);
+          };
+          L.osum[tid + u * kSubtreeThreads] = block_tree<3>(0, val[u], get);
+        }
+        if (__all_sync(full, oc[u] == __shfl_sync(full, oc[u], 0))) {   // one cell: one set of atomics
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            const int l = __reduce_min_sync(full, lo[d]), h = __reduce_max_sync(full, hi[d]);
+            if (lane == 0) { atomicMin(&L.bb[6 * oc[u] + d], l); atomicMax(&L.bb[6 * oc[u] + 3 + d], h); }
+          }
+        } else if (oc[u] >= 0) {
+#pragma unroll
+          for (int d = 0; d < 3; ++d) {
+            atomicMin(&L.bb[6 * oc[u] + d], lo[d]);
+            atomicMax(&L.bb[6 * oc[u] + 3 + d], hi[d]);
+          }
+        }
+      }
+      // the rest of the pairwise tree: octets 2s apart take the one s after
+      for (int s = 1; s < maxoct; s <<= 1) {
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kOctetsPerThread; ++u) {
+          const int r = rel[u] >> 3;
+          if (oc[u] >= 0 && (r & (2 * s - 1)) == 0 && 8 * (r + s) < cn[u]) {
+            Sum4* p = L.osum + tid + u * kSubtreeThreads;
+            p[0] = add4(p[0], p[s]);
+          }
+        }
+      }
+      if (tid == 0) s_base = nsplit > 0 && base + 2 * nsplit > A.cap_cells ? -1 : base;
+      __syncthreads();
+      // centres of mass, cut axes; an axis whose lead is within the error of
+      // the float32 box is decided from the exact box
+      bool unclear = false;
+      for (int t = tid; t < 4 * ncb; t += kSubtreeThreads) {
+        const int c = t >> 2, d = t & 3, cell = q[c].y;
+        const Sum4& v = L.osum[L.oct0[c]];
+        if (d < 3) {
+          const double quo = __ddiv_rn(d == 0 ? v.x : (d == 1 ? v.y : v.z), v.m);
+          L.com[3 * c + d] = quo;
+          (d == 0 ? T.cx : (d == 1 ? T.cy : T.cz))[cell] = quo;
+        } else {
+          T.M[cell] = v.m;
+          T.first[cell] = gfirst + (q[c].x & 0xffff);
+          T.count[cell] = q[c].x >> 16;
+          T.depth[cell] = depth;
+          float ext[3], X = 0.0f;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            const float l = funkey(L.bb[6 * c + k]), h = funkey(L.bb[6 * c + 3 + k]);
+            ext[k] = h - l;
+            X = fmaxf(X, fmaxf(fabsf(l), fabsf(h)));
+          }
+          int ax = 0;
+          float best = ext[0];
+          if (ext[1] > best) { ax = 1; best = ext[1]; }
+          if (ext[2] > best) { ax = 2; best = ext[2]; }
+          // an extent is off by less than 3 x 2^-23 X (two truncations, one
+          // rounding); NaN and infinite boxes are unclear too
+          const float margin = X * 1e-6f + 1e-37f;
+          bool clear = true;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) clear = clear && (k == ax || best - ext[k] > margin);
+          if (q[c].x >> 16 <= n_leaf) clear = true;               // a leaf is not cut
+          L.axis[c] = clear ? ax : -1;
+          unclear = unclear || !clear;
+        }
+      }
+      const bool exact = __syncthreads_or(unclear);
+      if (s_base < 0) {
+        if (tid == 0) set_status(A.status, ST_CAPACITY);
+        overflow = true;
+        continue;
+      }
+      if (exact) {
+        for (int t = tid; t < 6 * ncb; t += kSubtreeThreads) L.key[t] = t % 6 < 3 ? LLONG_MAX : LLONG_MIN;
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < kOctetsPerThread; ++u) {
+          if (oc[u] < 0 || L.axis[oc[u]] >= 0) continue;
+          for (int k = 0; k < val[u]; ++k) {
+            const int i = ix[lf[u] + rel[u] + k];
+            long long* key = L.key + 6 * oc[u];
+            const long long kk[3] = {dkey(L.x[i]), dkey(L.y[i]), dkey(L.z[i])};
+            for (int d = 0; d < 3; ++d) { atomicMin(&key[d], kk[d]); atomicMax(&key[3 + d], kk[d]); }
+          }
+        }
+        __syncthreads();
+        if (tid < ncb && L.axis[tid] < 0) {
+          double dlo[3], dhi[3];
+          for (int d = 0; d < 3; ++d) {
+            dlo[d] = dunkey(L.key[6 * tid + d]);
+            dhi[d] = dunkey(L.key[6 * tid + 3 + d]);
+          }
+          L.axis[tid] = longest_axis(dlo, dhi);
+        }
+        __syncthreads();
+      }
+      // left flags (bits of the octet) and float32 squared distances
+      unsigned left[kOctetsPerThread];
+      float d2[kOctetsPerThread][8];
+#pragma unroll
+      for (int u = 0; u < kOctetsPerThread; ++u) {
+        left[u] = 0u;
+        if (u * kSubtreeThreads + (tid & ~31) >= noct) continue;
+        float mx = 0.0f;
+        if (oc[u] >= 0) {
+          const double* com = L.com + 3 * oc[u];
+          const float cx = trunc_to_float(com[0]), cy = trunc_to_float(com[1]), cz = trunc_to_float(com[2]);
+          const bool cut = cn[u] > n_leaf;
+          const int ax = L.axis[oc[u]];
+          const long long ckey = dkey(com[ax]);
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            d2[u][k] = -2.0f;
+            if (k < val[u]) {
+              const int i = ix[lf[u] + rel[u] + k];
+              const double x = L.x[i], y = L.y[i], z = L.z[i];
+              const float dx = trunc_to_float(x) - cx, dy = trunc_to_float(y) - cy, dz = trunc_to_float(z) - cz;
+              d2[u][k] = dx * dx + dy * dy + dz * dz;
+              mx = fmaxf(mx, d2[u][k]);
+              const double a = ax == 0 ? x : (ax == 1 ? y : z);
+              if (cut && dkey(a) < ckey) left[u] |= 1u << k;
+            }
+          }
+          L.opre[tid + u * kSubtreeThreads] = __popc(left[u]);
+        }
+        if (__all_sync(full, oc[u] == __shfl_sync(full, oc[u], 0))) {
+          const int m = __reduce_max_sync(full, __float_as_int(mx));
+          if (lane == 0) atomicMax(&L.d2m[oc[u]], m);
+        } else if (oc[u] >= 0) {
+          atomicMax(&L.d2m[oc[u]], __float_as_int(mx));
+        }
+      }
+      __syncthreads();
+      if (warp == 0) {                    // left particles before each octet of the batch
+        constexpr int kPer = kBatchOctets / 32;
+        int v[kPer], run = 0;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+          const int o = lane * kPer + k;
+          v[k] = run;
+          run += o < noct ? L.opre[o] : 0;
+        }
+        int in2 = run;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int w = __shfl_up_sync(full, in2, o);
+          if (lane >= o) in2 += w;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+          const int o = lane * kPer + k;
+          if (o < noct) L.opre[o] = in2 - run + v[k];
+        }
+        if (lane == 31) L.opre[noct] = in2;
+      } else if (tid >= kBatchCells && tid - kBatchCells < ncb) {
+        const int c = tid - kBatchCells;
+        float X = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) X = fmaxf(X, fabsf(funkey(L.bb[6 * c + k])));
+        const float Dm = sqrtf(__int_as_float(L.d2m[c]));
+        const float thr = Dm - 2.0f * dist_err_bound(X * 1.000001f, Dm);
+        L.thr2[c] = thr > 0.0f ? thr * thr * (1.0f - 1e-6f) : -1.0f;
+      }
+      __syncthreads();
+      // exact size from the candidates; the stable partition of cut cells
+#pragma unroll
+      for (int u = 0; u < kOctetsPerThread; ++u) {
+        const int c = oc[u];
+        if (c < 0) continue;
+        const float thr2 = L.thr2[c];
+        unsigned cand = 0u;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (k < val[u] && d2[u][k] >= thr2) cand |= 1u << k;
+        const uint16_t* p = ix + lf[u] + rel[u];
+        long long s2 = 0;
+        while (cand != 0u) {
+          const int i = p[__ffs(cand) - 1];
+          cand &= cand - 1u;
+          s2 = max(s2, __double_as_longlong(dist2_rn(L.x[i], L.y[i], L.z[i], L.com[3 * c],
+                                                     L.com[3 * c + 1], L.com[3 * c + 2])));
+        }
+        if (s2 > 0) atomicMax(&L.s2[c], (unsigned long long)s2);
+        if (cn[u] <= n_leaf) {
+          for (int k = 0; k < val[u]; ++k) L.fin[lf[u] + rel[u] + k] = p[k];
+        } else {
+          const int before = L.opre[L.oct0[c]], nl = L.opre[c + 1 < ncb ? L.oct0[c + 1] : noct] - before;
+          if (nl == 0 || nl == cn[u]) {                            // split by position: order kept
+            for (int k = 0; k < val[u]; ++k) ox[lf[u] + rel[u] + k] = p[k];
+          } else {
+            int l = L.opre[tid + u * kSubtreeThreads] - before, r = nl + rel[u] - l;
+            for (int k = 0; k < val[u]; ++k)
+              ox[lf[u] + ((left[u] >> k & 1u) ? l++ : r++)] = p[k];
+          }
+        }
+      }
+      __syncthreads();
+      // sizes, children
+      if (tid < ncb) {
+        const int cell = q[tid].y, first = q[tid].x & 0xffff, cnt = q[tid].x >> 16;
+        T.s[cell] = sqrt(__longlong_as_double((long long)L.s2[tid]));
+        if (cnt > n_leaf) {
+          int nl = L.opre[tid + 1 < ncb ? L.oct0[tid + 1] : noct] - L.opre[L.oct0[tid]];
+          if (nl == 0 || nl == cnt) {
+            nl = cnt / 2;
+            atomicAdd(&A.counters[C_FALLBACK], 1);
+          }
+          const int cid = s_base + 2 * L.irank[tid];
+          T.left[cell] = cid;
+          T.right[cell] = cid + 1;
+          int2* out = q_out + nq_next + 2 * L.irank[tid];
+          out[0] = make_int2(nl << 16 | first, cid);
+          out[1] = make_int2((cnt - nl) << 16 | (first + nl), cid + 1);
+        } else {
+          T.left[cell] = -1;
+          T.right[cell] = -1;
+        }
+      }
+      nq_next += 2 * nsplit;
+      __syncthreads();
     }
-    // medium cells: one warp each
-    for (int qi = warp; qi < nq; qi += nwarps) {
-      const int4 e = L.q[cur][qi];
-      if (e.y > kThreadSeg && e.y < kBlockSeg) split_warp(S, L, Q, e, gfirst, depth_max);
-    }
-    // small cells: one thread each (with their leaf children)
-    for (int qi = threadIdx.x; qi < nq; qi += blockDim.x) {
-      const int4 e = L.q[cur][qi];
-      if (e.y <= kThreadSeg) split_thread(S, L, Q, e, gfirst, depth_max);
-    }
-    __syncthreads();
-    // leaves split off by the CTA and warp passes: one thread each
-    const int nlv = min(nleaf, leafcap);
-    for (int li = threadIdx.x; li < nlv; li += blockDim.x) {
-      const int4 e = leaves[li];
-      leaf_thread(S, L, e.x, e.y, e.z, e.w, gfirst);
-    }
-    __syncthreads();
     cur ^= 1;
+    nq = nq_next;
+    if (nq > 0) ++depth;
   }
-  depth_max = max(depth_max, __shfl_xor_sync(0xffffffffu, depth_max, 16));
-  depth_max = max(depth_max, __shfl_xor_sync(0xffffffffu, depth_max, 8));
-  depth_max = max(depth_max, __shfl_xor_sync(0xffffffffu, depth_max, 4));
-  depth_max = max(depth_max, __shfl_xor_sync(0xffffffffu, depth_max, 2));
-  depth_max = max(depth_max, __shfl_xor_sync(0xffffffffu, depth_max, 1));
-  if ((threadIdx.x & 31) == 0 && depth_max > 0) atomicMax(&S.A.counters[6], depth_max);
-  for (int k = threadIdx.x; k < n; k += blockDim.x) {
-    int src = L.idx[k];
-    int64_t p = (int64_t)gfirst + k;
+  if (overflow) continue;
+  if (tid == 0) atomicMax(&A.counters[C_DEPTH], depth);
+  for (int k = tid; k < n; k += kSubtreeThreads) {
+    const int src = L.fin[k];
+    const int64_t p = (int64_t)gfirst + k;
     S.out.x[p] = L.x[src]; S.out.y[p] = L.y[src]; S.out.z[p] = L.z[src]; S.out.m[p] = L.m[src];
     S.out.h[p] = in.h[gfirst + src];
     S.out.idx[p] = in.idx[gfirst + src];
@@ -1385,12 +1268,13 @@ static int ensure_build_buffers(kdfmm_tree_s* t, int64_t n) {
   return KDFMM_OK;
 }
 
-// Queue entries and dynamic shared memory of the subtree kernel for trees of
-// the given leaf size.
-static int subtree_qcap(int n_leaf) { return kSubtreeMax / (n_leaf + 1) + 2; }
+// Queue entries (the cells a level can hold: twice the cells that a level can
+// split) and dynamic shared memory of the subtree kernel for trees of the
+// given leaf size.
+static int subtree_qcap(int n_leaf) { return 2 * (kSubtreeMax / (n_leaf + 1)) + 2; }
 static size_t subtree_smem_for(int qcap) {
-  return 4 * kSubtreeMax * sizeof(double) + 3 * kSubtreeMax * sizeof(float) +
-         2 * kSubtreeMax * sizeof(uint16_t) + 4 * (size_t)qcap * sizeof(int4);
+  SubSmem L;
+  return sub_carve(nullptr, qcap, &L);
 }
 
 // Launch sizes of the persistent subtree kernel (host calls only; made once

@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kL2PWarps * 32) k_vjp_l2p(const double* __rest
 // M2L reverse: warp per sink leaf, lanes over its far cells.  Mixed mode is bound
 // by float32 issue (some 2500 instructions a pair, three quarters of them the
 // dual numbers): the cotangents of M and Q, which needed seven contractions with
-// mostly zero terms (15.8 ms on the 2^20 Plummer sphere, 1.32e8 pairs; 12.0 now), are
+// mostly zero terms (15.8 ms on the 2^20 Plummer sphere, 1.32e8 pairs; 12.4 now), are
 // written without those terms.  A far cell's ten
 // cotangents (M_bar, com_bar, Q_bar) go to float64 atomics through shared
 // memory, so that a warp instruction adds 32 consecutive values (about three
