@@ -105,21 +105,23 @@ struct Lists {
   int32_t arena_grid;              // blocks of the arena walk
   int64_t* near_np;                // device statistics of the walk (4)
   int32_t* heavy;                  // leaves queued for the block-wide walk (nleaves)
-  // near lists longer than kSegEntries are split: segment 0 stays with the
+  // near lists longer than seg_entries are split: segment 0 stays with the
   // leaf, the others are work items of their own whose partial sums
   // (seg_part, 32 targets x 4 doubles each) are added in segment order
+  int32_t seg_entries;             // of the last plan
   int32_t* seg_first;              // per leaf: first extra segment, or -1
   int32_t* seg_leaf;               // per extra segment: its leaf
   double* seg_part;                // per extra segment: partial sums
   int64_t seg_cap;                 // extra segments allocated
 };
 
-// Near entries per P2P segment.
+// Near entries per P2P segment (float64 evaluations of few particles take
+// shorter ones, p2p.cu).
 constexpr int kSegEntries = 256;
 
 // Extra segments of a near list of n entries.
-__host__ __device__ __forceinline__ int extra_segments(int64_t n) {
-  return n > kSegEntries ? (int)((n - 1) / kSegEntries) : 0;
+__host__ __device__ __forceinline__ int extra_segments(int64_t n, int seg_entries) {
+  return n > seg_entries ? (int)((n - 1) / seg_entries) : 0;
 }
 
 }  // namespace kdfmm
@@ -309,6 +311,14 @@ __device__ __forceinline__ double rsqrt64(double v) {
   const int cb = __float_as_int(0.375f * ef * ef);         // (0 becomes 2^-127: far below rounding)
   const double c = __hiloint2double((cb >> 3) + (896 << 20), cb << 29);
   return fma(y, fma(0.5, e, c), y);
+}
+
+// Whether a pair may lie inside either smoothing kernel's support: float32
+// test with a margin, h2 = (2 h)^2 of each side (true where the squared
+// distance leaves the float range; the kernel's formulas hold outside too).
+__device__ __forceinline__ bool maybe_inside(double r2, float h2i, float h2j) {
+  const float r2f = trunc_to_float(r2);
+  return !(r2f >= fmaxf(h2i, h2j) * 1.000001f && r2f < __int_as_float(0x7f800000));
 }
 
 // Bound on |d_float32 - d| for a distance d whose coordinates and centre lie

@@ -13,9 +13,9 @@
 // One warp per target leaf.  A leaf of n_t <= 32 targets uses K = 32 / n_t
 // source slices: lane = target + n_t * slice, slice k takes sources k, k+K, ...
 // of every near leaf, and the slices are combined at the end.  A near list
-// longer than kSegEntries leaves (a large leaf in the sparse outskirts of a
+// longer than a segment (256 leaves; fewer in small float64 evaluations) (a large leaf in the sparse outskirts of a
 // centrally condensed system can have most of the system in it) is split
-// into segments of kSegEntries: the leaf's warp takes the first, the others
+// into segments: the leaf's warp takes the first, the others
 // are separate work items, and their partial sums are added afterwards in
 // segment order, so the result does not depend on scheduling.
 //
@@ -58,13 +58,14 @@ struct P2PArgs {
   const double* sys_eps;     // Plummer softening length of each system
   double* a;
   double* phi;
-  // near lists longer than kSegEntries: segment 0 is the leaf's own work
+  // near lists longer than seg_entries: segment 0 is the leaf's own work
   // item, the others (counters[C_SEGS], at most seg_cap) are items after the
   // leaves, whose partial sums seg_part k_seg_combine adds in segment order
   const int32_t* seg_first;
   const int32_t* seg_leaf;
   double* seg_part;
   int64_t seg_cap;
+  int seg_entries;
 };
 
 // M4 cubic spline, q = r/h < 2: F(q)/q^3 and P(q) (qi = 1/q).
@@ -77,16 +78,6 @@ __device__ __forceinline__ float m4_pot(float q, float qi) {
   if (q < 1.0f) return 1.4f + q2 * (-0.6666667f + q2 * (0.3f - 0.1f * q));
   return 1.6f + q2 * (-1.3333333f + q * (1.0f + q * (-0.3f + 0.033333335f * q))) - 0.06666667f * qi;
 }
-__device__ __forceinline__ double m4_fq3_d(double q, double qi) {
-  if (q < 1.0) return 4.0 / 3.0 + q * q * (-1.2 + 0.5 * q);
-  return 8.0 / 3.0 + q * (-3.0 + q * (1.2 - q * (1.0 / 6.0))) - qi * qi * qi * (1.0 / 15.0);
-}
-__device__ __forceinline__ double m4_pot_d(double q, double qi) {
-  const double q2 = q * q;
-  if (q < 1.0) return 1.4 + q2 * (-2.0 / 3.0 + q2 * (0.3 - 0.1 * q));
-  return 1.6 + q2 * (-4.0 / 3.0 + q * (1.0 + q * (-0.3 + q * (1.0 / 30.0)))) - qi * (1.0 / 15.0);
-}
-
 // Interaction of one target with one source, float32, accumulated into f*.
 template <int SOFT>
 __device__ __forceinline__ void pair32(float rx, float ry, float rz, float mj, const float4& hi,
@@ -279,8 +270,8 @@ __global__ void __launch_bounds__(kP2PWarps * 32, 6) k_p2p_mixed(P2PArgs A) {
   const unsigned full = 0xffffffffu, lt = (1u << lane) - 1u;
   const int64_t nall = min((int64_t)A.near_cnt[k], A.cap_near);
   const int64_t sidx = seg ? (int64_t)(g - A.seg_first[k] + 1) : 0;
-  const int64_t e1 = A.near_off[k] + min(nall, (sidx + 1) * kSegEntries);
-  for (int64_t e = A.near_off[k] + sidx * kSegEntries; e < e1;) {
+  const int64_t e1 = A.near_off[k] + min(nall, (sidx + 1) * A.seg_entries);
+  for (int64_t e = A.near_off[k] + sidx * A.seg_entries; e < e1;) {
     // up to 32 candidate leaves, one per lane
     const int64_t my = e + lane;
     int cnt = 0, first = 0;
@@ -459,60 +450,50 @@ __global__ void __launch_bounds__(kP2PWarps * 32, 6) k_p2p_mixed(P2PArgs A) {
 constexpr int kStage64 = 128;      // staged sources per warp and chunk (float64 path)
 constexpr int kP2P64Warps = 4;
 
-// Float64 pair on target i from source j, d = x_i - x_j; hinv = 1/h and
-// hinv3 = 1/h^3 of each side (M4 kernel), eps2 (Plummer).
-template <int SOFT>
-__device__ __forceinline__ void pair64(double rx, double ry, double rz, double mj, double hi,
-                                       double hinv_i, double hinv3_i, double hj, double hinv_j,
-                                       double hinv3_j, double eps2, double& fx, double& fy,
-                                       double& fz, double& fp) {
-  if (SOFT == KDFMM_SOFT_PLUMMER) {
-    const double r2 = rx * rx + ry * ry + rz * rz + eps2;
-    const double inv = rsqrt(r2);
-    const double minv = mj * inv;
-    const double f = minv * inv * inv;
-    fx -= f * rx; fy -= f * ry; fz -= f * rz;
-    fp -= minv;
-  } else {
-    const double r2 = rx * rx + ry * ry + rz * rz;
-    if (r2 == 0.0) {
-      fp -= mj * 0.7 * (hinv_i + hinv_j);        // P(0) = 7/5 on both sides, halved
-      return;
-    }
-    const double inv = rsqrt(r2);
-    const double r = r2 * inv;
-    const double qa = r * hinv_i, qb = r * hinv_j;
-    double f, p;
-    if (qa < 2.0 || qb < 2.0) {
-      const double inv3 = inv * inv * inv;
-      const double fa = qa < 2.0 ? hinv3_i * m4_fq3_d(qa, hi * inv) : inv3;
-      const double fb = qb < 2.0 ? hinv3_j * m4_fq3_d(qb, hj * inv) : inv3;
-      const double pa = qa < 2.0 ? hinv_i * m4_pot_d(qa, hi * inv) : inv;
-      const double pb = qb < 2.0 ? hinv_j * m4_pot_d(qb, hj * inv) : inv;
-      f = 0.5 * (fa + fb);
-      p = 0.5 * (pa + pb);
+// Force over distance and potential of the symmetrised M4 pair (Eq. 13) in
+// float64; hinv and h3inv = 1/h and 1/h^3 of each side.  Branches of q >= 1 as
+// in m4_side (t = 0 outside the support).
+__device__ __forceinline__ void m4pair64(double r2, double hinv_i, double h3inv_i, double hinv_j,
+                                         double& f, double& p) {
+  const double inv = rsqrt64(r2);
+  const double r = r2 * inv, inv3 = inv * inv * inv;
+  f = p = 0.0;
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    const double hinv = side ? hinv_j : hinv_i, q = r * hinv;
+    if (q < 1.0) {
+      const double q2 = q * q, h3inv = side ? hinv * hinv * hinv : h3inv_i;
+      f = fma(fma(q2, fma(0.5, q, -1.2), 4.0 / 3.0), h3inv, f);
+      p = fma(fma(q2, fma(q2, fma(-0.1, q, 0.3), -2.0 / 3.0), 1.4), hinv, p);
     } else {
-      f = inv * inv * inv;
-      p = inv;
+      const double t = fmax(2.0 - q, 0.0), t2 = t * t, t4 = t2 * t2;
+      f = fma(fma(-t4, fma(t, fma(t, 1.0 / 6.0, -0.8), 1.0), 1.0), inv3, f);
+      p = fma(fma(-t4 * t, fma(t, -1.0 / 30.0, 0.1), 1.0), inv, p);
     }
-    const double mf = mj * f;
-    fx -= mf * rx; fy -= mf * ry; fz -= mf * rz;
-    fp -= mj * p;
   }
+  f *= 0.5;
+  p *= 0.5;
 }
 
 // Float64 mode: lanes = (target, source slice) as K = 32 / n_t slices;
 // per chunk of near leaves (at most kStage64 sources) the warp stages the
-// sources' float64 positions, masses and smoothing lengths (with (2h)^2) in
-// shared memory, then every lane sums its slice; the target's own leaf is
-// summed separately (j != i).  The slices are added in slice order.
+// sources' float64 positions and masses in shared memory (M4: 1/h, and (2h)^2
+// as float32), then every lane sums its slice; the target's own leaf is staged
+// by itself (j != i).  The slices are added in slice order.
+//
+// Bound by the float64 pipe, where an operation costs as much as ~75 float32
+// ones: a 1/r^2 pair takes 17 of them (3 differences, 3 for r^2, 4 for 1/r
+// (rsqrt64), 4 for m/r and m/r^3, 3 for the force), the tests of the kernel
+// supports are float32.  With the library's rsqrt, float64 tests and divisions
+// per kernel pair it was ~45 (M4 binary of 2 x 2^20: 133 ms, now 98; Plummer
+// sphere of 4096: 1.42 ms in long segments, now 0.29).
 template <int SOFT>
 __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
   constexpr bool M4 = SOFT == KDFMM_SOFT_M4;
   __shared__ double s_x[kP2P64Warps][kStage64], s_y[kP2P64Warps][kStage64];
   __shared__ double s_z[kP2P64Warps][kStage64], s_m[kP2P64Warps][kStage64];
-  __shared__ double s_h[M4 ? kP2P64Warps : 1][M4 ? kStage64 : 1];
-  __shared__ double s_h2[M4 ? kP2P64Warps : 1][M4 ? kStage64 : 1];   // (2 h)^2, rounded up
+  __shared__ double s_hinv[M4 ? kP2P64Warps : 1][M4 ? kStage64 : 1];
+  __shared__ float s_h2[M4 ? kP2P64Warps : 1][M4 ? kStage64 : 1];
   __shared__ uint8_t s_leaf[kP2P64Warps][kStage64];
   __shared__ int s_tbeg[kP2P64Warps][32], s_tfirst[kP2P64Warps][32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -520,8 +501,8 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
   const int nleaves = min(A.counters[C_LEAVES], A.max_leaves);
   const int nitems = nleaves + (int)min((int64_t)A.counters[C_SEGS], A.seg_cap);
   double *sx = s_x[warp], *sy = s_y[warp], *sz = s_z[warp], *sm = s_m[warp];
-  double* sh = s_h[M4 ? warp : 0];
-  double* sh2 = s_h2[M4 ? warp : 0];
+  double* shinv = s_hinv[M4 ? warp : 0];
+  float* sh2 = s_h2[M4 ? warp : 0];
   uint8_t* sl_of = s_leaf[warp];
   int* tb = s_tbeg[warp];
   int* tf = s_tfirst[warp];
@@ -537,27 +518,69 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
   const bool act = sl < K;
   const int64_t it = (int64_t)fa + t;
   const double xi = A.tp.x[it], yi = A.tp.y[it], zi = A.tp.z[it];
-  const double hi = M4 ? A.tp.h[it] : 0.0;
-  const double hinv_i = M4 ? 1.0 / hi : 0.0;
-  const double hinv3_i = hinv_i * hinv_i * hinv_i;
-  const double h2i = 4.0 * hi * hi * (1.0 + 1e-12);
+  const double hinv_i = M4 ? 1.0 / A.tp.h[it] : 0.0;
+  const double h3inv_i = hinv_i * hinv_i * hinv_i;
+  const float h2i = M4 ? A.ph[it].w : 0.0f;
   const double eps = A.sys_eps[A.leaf_sys[k]];
-  const double eps2 = eps * eps;
+  // added to r^2: the softening, or (M4) what keeps 1/r finite for coincident
+  // particles, whose force is 0 and whose potential the q < 1 form's
+  const double soft2 = M4 ? 1e-290 : eps * eps;
   double fx = 0.0, fy = 0.0, fz = 0.0, fp = 0.0;
-  if (!seg && act) {
-    for (int j = sl; j < nt; j += K) {
-      if (j == t) continue;
-      const int64_t js = (int64_t)fa + j;
-      const double hj = M4 ? A.tp.h[js] : 0.0;
-      const double hinv_j = M4 ? 1.0 / hj : 0.0;
-      pair64<SOFT>(xi - A.tp.x[js], yi - A.tp.y[js], zi - A.tp.z[js], A.tp.m[js], hi, hinv_i,
-                   hinv3_i, hj, hinv_j, hinv_j * hinv_j * hinv_j, eps2, fx, fy, fz, fp);
+  auto stage = [&](int at, int64_t src) {
+    sx[at] = A.tp.x[src];
+    sy[at] = A.tp.y[src];
+    sz[at] = A.tp.z[src];
+    sm[at] = A.tp.m[src];
+    if (M4) {
+      shinv[at] = 1.0 / A.tp.h[src];
+      sh2[at] = A.ph[src].w;
     }
+  };
+  // the lane's slice of the staged sources but `skip`.  M4, 32 sources of the
+  // slice at a time: every pair as 1/r^2 except those that may lie inside
+  // either support, which are marked and follow with the kernel (a warp
+  // branching per pair ran the kernel path for all its lanes whenever one
+  // needed it)
+  auto sum_staged = [&](int total, int skip) {
+    for (int j0 = sl; j0 < total; j0 += 32 * K) {
+      uint32_t in = 0u;
+      for (int b = 0; b < 32; ++b) {
+        const int j = j0 + b * K;
+        if (j >= total) break;
+        if (j == skip) continue;
+        const double rx = xi - sx[j], ry = yi - sy[j], rz = zi - sz[j];
+        const double r2 = fma(rz, rz, fma(ry, ry, fma(rx, rx, soft2)));
+        if (M4 && maybe_inside(r2, h2i, sh2[j])) {
+          in |= 1u << b;
+          continue;
+        }
+        const double inv = rsqrt64(r2);
+        const double minv = sm[j] * inv, f = minv * (inv * inv);
+        fx = fma(-f, rx, fx); fy = fma(-f, ry, fy); fz = fma(-f, rz, fz);
+        fp -= minv;
+      }
+      while (M4 && in != 0u) {
+        const int j = j0 + (__ffs(in) - 1) * K;
+        in &= in - 1u;
+        const double rx = xi - sx[j], ry = yi - sy[j], rz = zi - sz[j];
+        double f, p;
+        m4pair64(fma(rz, rz, fma(ry, ry, fma(rx, rx, soft2))), hinv_i, h3inv_i, shinv[j], f, p);
+        f *= sm[j];
+        fx = fma(-f, rx, fx); fy = fma(-f, ry, fy); fz = fma(-f, rz, fz);
+        fp = fma(-sm[j], p, fp);
+      }
+    }
+  };
+  if (!seg) {
+    if (lane < nt) stage(lane, (int64_t)fa + lane);
+    __syncwarp();
+    if (act) sum_staged(nt, t);
+    __syncwarp();
   }
   const int64_t nall = min((int64_t)A.near_cnt[k], A.cap_near);
   const int64_t sidx = seg ? (int64_t)(g - A.seg_first[k] + 1) : 0;
-  const int64_t e1 = A.near_off[k] + min(nall, (sidx + 1) * kSegEntries);
-  for (int64_t e = A.near_off[k] + sidx * kSegEntries; e < e1;) {
+  const int64_t e1 = A.near_off[k] + min(nall, (sidx + 1) * A.seg_entries);
+  for (int64_t e = A.near_off[k] + sidx * A.seg_entries; e < e1;) {
     const int64_t my = e + lane;
     int cnt = 0, first = 0;
     if (my < e1) {
@@ -584,54 +607,10 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
     const int total = __shfl_sync(full, incl, L - 1);
     for (int idx = lane; idx < total; idx += 32) {
       const int l = sl_of[idx];
-      const int64_t src = (int64_t)tf[l] + idx - tb[l];
-      sx[idx] = A.tp.x[src];
-      sy[idx] = A.tp.y[src];
-      sz[idx] = A.tp.z[src];
-      sm[idx] = A.tp.m[src];
-      if (M4) {
-        const double h = A.tp.h[src];
-        sh[idx] = h;
-        sh2[idx] = 4.0 * h * h * (1.0 + 1e-12);
-      }
+      stage(idx, (int64_t)tf[l] + idx - tb[l]);
     }
     __syncwarp();
-    if (act && !M4) {
-      for (int j = sl; j < total; j += K)
-        pair64<SOFT>(xi - sx[j], yi - sy[j], zi - sz[j], sm[j], 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, eps2,
-                     fx, fy, fz, fp);
-    } else if (act) {
-      // M4 kernel, 32 sources of the lane's slice at a time.  Pass 1: every
-      // pair as 1/r^2 except those that may lie inside either support
-      // (r^2 < (2 max(h_i, h_j))^2, thresholds rounded up), which are marked;
-      // pass 2: the marked pairs with the full symmetrised pair.  A warp
-      // branching per pair instead ran the kernel path for all its lanes
-      // whenever one lane needed it.
-      for (int j0 = sl; j0 < total; j0 += 32 * K) {
-        uint32_t in = 0u;
-        for (int b = 0; b < 32; ++b) {
-          const int j = j0 + b * K;
-          if (j >= total) break;
-          const double rx = xi - sx[j], ry = yi - sy[j], rz = zi - sz[j];
-          const double r2 = rx * rx + ry * ry + rz * rz;
-          const bool inside = r2 < fmax(h2i, sh2[j]);
-          in |= (uint32_t)inside << b;
-          const double inv = rsqrt(inside ? 1.0 : r2);
-          const double minv = (inside ? 0.0 : sm[j]) * inv;
-          const double f = minv * inv * inv;
-          fx -= f * rx; fy -= f * ry; fz -= f * rz;
-          fp -= minv;
-        }
-        while (in != 0u) {
-          const int b = __ffs(in) - 1;
-          in &= in - 1u;
-          const int j = j0 + b * K;
-          const double hj = sh[j], hinv_j = 1.0 / hj;
-          pair64<SOFT>(xi - sx[j], yi - sy[j], zi - sz[j], sm[j], hi, hinv_i, hinv3_i, hj, hinv_j,
-                       hinv_j * hinv_j * hinv_j, eps2, fx, fy, fz, fp);
-        }
-      }
-    }
+    if (act) sum_staged(total, -1);
     __syncwarp();
     e += L;
   }
@@ -665,10 +644,11 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
 // their entries below seg_cap are marked -1, which every consumer skips.
 __global__ void k_seg_plan(const int32_t* __restrict__ near_cnt, int64_t cap_near,
                            int max_leaves, int32_t* counters, int32_t* seg_first,
-                           int32_t* seg_leaf, int64_t seg_cap, int32_t* status) {
+                           int32_t* seg_leaf, int64_t seg_cap, int seg_entries,
+                           int32_t* status) {
   const int nleaves = min(counters[C_LEAVES], max_leaves);
   KD_GRID_STRIDE(k, nleaves) {
-    const int x = extra_segments(min((int64_t)near_cnt[k], cap_near));
+    const int x = extra_segments(min((int64_t)near_cnt[k], cap_near), seg_entries);
     int first = -1;
     if (x > 0) {
       const int base = atomicAdd(&counters[C_SEGS], x);
@@ -697,7 +677,7 @@ __global__ void k_seg_combine(P2PArgs A) {
     if (g != f) continue;
     const int a = A.leaf_cells[k];
     if (lane >= A.ccount[a]) continue;
-    const int x = extra_segments(min((int64_t)A.near_cnt[k], A.cap_near));
+    const int x = extra_segments(min((int64_t)A.near_cnt[k], A.cap_near), A.seg_entries);
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
     for (int q = 0; q < x; ++q) {
       const double* P = A.seg_part + (int64_t)(f + q) * 128 + 4 * lane;
@@ -743,18 +723,30 @@ int ensure_segments(kdfmm_tree_s* t, int64_t need) {
   return KDFMM_OK;
 }
 
+// Near entries per segment: by the particle count alone, so that an eager
+// evaluation and a replayed graph split alike.  Float64 evaluations of few
+// particles take short segments: their leaves are too few warps for the GPU's
+// 608 float64 pipes (4096 particles: 367 leaves with ~108 near leaves each).
+// Mixed evaluations keep 256: a shorter segment would move the chunks of 256
+// sources whose float32 sums are folded at once.
+static int segment_entries(const kdfmm_tree_s* t) {
+  if (t->p.precision != KDFMM_FP64) return kSegEntries;
+  return t->n < 65536 ? 32 : (t->n < 262144 ? 64 : kSegEntries);
+}
+
 int64_t segments_bound(const kdfmm_tree_s* t) {
   const Lists& L = t->L;
   const int64_t entries = L.exact ? L.near_cap : t->host_stats[KDFMM_STAT_NNEAR];
-  return entries / kSegEntries + 64;
+  return entries / segment_entries(t) + 64;
 }
 
 int plan_segments(kdfmm_tree_s* t, cudaStream_t s) {
   const int gl = std::max(t->grid_leaves, 1);
+  t->L.seg_entries = segment_entries(t);
   cudaMemsetAsync(t->counters + C_SEGS, 0, sizeof(int32_t), s);
   k_seg_plan<<<std::min<unsigned>(blocks_for(gl, 256), grid_blocks()), 256, 0, s>>>(
       t->L.near_cnt, t->L.exact ? INT64_MAX : t->L.cap_near, gl, t->counters, t->L.seg_first,
-      t->L.seg_leaf, t->L.seg_cap, t->status);
+      t->L.seg_leaf, t->L.seg_cap, t->L.seg_entries, t->status);
   t->launches += 1;
   return check_cuda(cudaGetLastError(), "segment plan");
 }
@@ -789,6 +781,7 @@ int run_p2p(kdfmm_tree_s* t, double* a, double* phi, cudaStream_t s) {
   A.seg_cap = t->L.seg_cap;
   int rc = plan_segments(t, s);
   if (rc) return rc;
+  A.seg_entries = t->L.seg_entries;
   const int gl = std::max(t->grid_leaves, 1);
   const bool m4 = t->p.soft_kind == KDFMM_SOFT_M4;
   if (t->p.precision == KDFMM_MIXED) {
@@ -796,7 +789,8 @@ int run_p2p(kdfmm_tree_s* t, double* a, double* phi, cudaStream_t s) {
     if (m4) k_p2p_mixed<KDFMM_SOFT_M4><<<gm, kP2PWarps * 32, 0, s>>>(A);
     else k_p2p_mixed<KDFMM_SOFT_PLUMMER><<<gm, kP2PWarps * 32, 0, s>>>(A);
   } else {
-    const unsigned g64 = blocks_for(gl, kP2P64Warps);
+    // a warp per leaf and per segment that there may be
+    const unsigned g64 = blocks_for(gl + t->L.seg_cap, kP2P64Warps);
     if (m4) k_p2p_fp64<KDFMM_SOFT_M4><<<g64, kP2P64Warps * 32, 0, s>>>(A);
     else k_p2p_fp64<KDFMM_SOFT_PLUMMER><<<g64, kP2P64Warps * 32, 0, s>>>(A);
   }

@@ -82,7 +82,6 @@ __device__ __forceinline__ T tc(double v) {
   return Lift<T>::of((typename Lift<T>::Scalar)v);
 }
 
-__device__ __forceinline__ float rs(float v) { return rsq(v); }
 template <class S>
 __device__ __forceinline__ DualT<S> rs(const DualT<S>& v) { return rsqrt_dual(v); }
 
@@ -193,6 +192,7 @@ struct VjpArgs {
   const int32_t *seg_first, *seg_leaf;
   double* seg_part;
   int64_t seg_cap;
+  int seg_entries;
   // transposed near lists: leaf ordinal r is a source of the target leaves
   // tidx[toff[r] ...) (ordinals), tcnt[r] of them; cut into pieces of
   // kSrcEntries, piece 0 the leaf's own work item, the others extra items
@@ -729,9 +729,9 @@ __device__ __forceinline__ int near_item(const VjpArgs& V, int item, int* k, int
   *k = seg ? V.seg_leaf[g] : item;
   if (*k < 0) return 0;
   const int64_t sidx = seg ? (int64_t)(g - V.seg_first[*k] + 1) : 0;
-  *e0 = V.near_off[*k] + sidx * kSegEntries;
-  return (int)(min(min((int64_t)V.near_cnt[*k], V.cap_near), (sidx + 1) * kSegEntries) -
-               sidx * kSegEntries);
+  *e0 = V.near_off[*k] + sidx * V.seg_entries;
+  return (int)(min(min((int64_t)V.near_cnt[*k], V.cap_near), (sidx + 1) * V.seg_entries) -
+               sidx * V.seg_entries);
 }
 
 __global__ void k_tr_count(VjpArgs V) {
@@ -1103,14 +1103,6 @@ __device__ __forceinline__ void m4_fg64(double r2, double hinv_i, double hinv_j,
   g *= 0.5;
 }
 
-// Whether a pair may lie inside either smoothing kernel's support: float32
-// test with a margin, h2 = (2 h)^2 of each side (true where the squared
-// distance leaves the float range; the kernel's formulas hold outside too).
-__device__ __forceinline__ bool maybe_inside(double r2, float h2i, float h2j) {
-  const float r2f = trunc_to_float(r2);
-  return !(r2f >= fmaxf(h2i, h2j) * 1.000001f && r2f < __int_as_float(0x7f800000));
-}
-
 // FP64 mode, target side (as k_vjp_target32, in float64).  x_bar_i gets
 // -(a_bar_i sum m f + sum m g (d.a_bar_i) d).  M4: pairs outside both supports
 // first (f = r^-3, g = -3 r^-5), those that may be inside are marked and
@@ -1280,7 +1272,7 @@ __global__ void k_vjp_seg_combine(VjpArgs V) {
     if (g != f) continue;
     const int a = V.leaf_cells[k];
     if (lane >= V.c.count[a]) continue;
-    const int x = extra_segments(min((int64_t)V.near_cnt[k], V.cap_near));
+    const int x = extra_segments(min((int64_t)V.near_cnt[k], V.cap_near), V.seg_entries);
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
     for (int q = 0; q < x; ++q) {
       const double* P = V.seg_part + (int64_t)(f + q) * 128 + 4 * lane;
@@ -1390,6 +1382,7 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
   V.seg_leaf = t->L.seg_leaf;
   V.seg_part = t->L.seg_part;
   V.seg_cap = t->L.seg_cap;
+  V.seg_entries = t->L.seg_entries;
   V.tcap = nnear;
   V.tseg_cap = nnear / kSrcEntries + 1;
   // scratch, in two parts: what starts at zero first (one memset), then the
