@@ -224,7 +224,7 @@ k_chunk_reduce(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_s
 __global__ void k_decide(const Seg* __restrict__ segs, const int32_t* __restrict__ nA_dev, const int32_t* __restrict__ seg_off,
                          const double* __restrict__ csum, const long long* __restrict__ ckey,
                          TmpCells tmp, int32_t* __restrict__ seg_axis, double* __restrict__ seg_cut,
-                         float* __restrict__ seg_xb, long long* __restrict__ seg_s2) {
+                         float* __restrict__ seg_xb) {
   const int nA = *nA_dev;
   const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
@@ -273,12 +273,12 @@ __global__ void k_decide(const Seg* __restrict__ segs, const int32_t* __restrict
     const int c = g.cell;
     tmp.first[c] = g.first; tmp.count[c] = g.count; tmp.depth[c] = g.dbuf >> 1;
     tmp.M[c] = M; tmp.cx[c] = cx; tmp.cy[c] = cy; tmp.cz[c] = cz;
+    tmp.s[c] = 0.0;
     seg_axis[s] = axis;
     seg_cut[s] = axis == 0 ? cx : (axis == 1 ? cy : cz);
     double X = 0.0;
     for (int d = 0; d < 3; ++d) X = fmax(X, fmax(fabs(dlo[d]), fabs(dhi[d])));
     seg_xb[s] = (float)X * 1.000001f;
-    seg_s2[s] = 0;
   }
 }
 
@@ -404,7 +404,7 @@ k_chunk_scatter(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_
                 const int32_t* __restrict__ seg_off, const int32_t* __restrict__ counters, PCols src,
                 PCols dst, const int32_t* __restrict__ seg_axis, const double* __restrict__ seg_cut,
                 const int32_t* __restrict__ cloff, const int32_t* __restrict__ seg_nl,
-                TmpCells tmp, const float* __restrict__ seg_thr2, long long* __restrict__ seg_s2) {
+                TmpCells tmp, const float* __restrict__ seg_thr2) {
   const int b = blockIdx.x;
   if (b >= counters[4]) return;
   const int s = chunk_seg[b];
@@ -487,16 +487,9 @@ k_chunk_scatter(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_
   if (threadIdx.x == 0) {
     long long m2 = 0;
     for (int q = 0; q < kChunkThreads / 32; ++q) m2 = max(m2, ws2[q]);
-    if (m2 > 0) atomicMax(reinterpret_cast<unsigned long long*>(&seg_s2[s]), (unsigned long long)m2);
+    if (m2 > 0)
+      atomicMax(reinterpret_cast<unsigned long long*>(&tmp.s[g.cell]), (unsigned long long)m2);
   }
-}
-
-// Size of each phase-A cell from the exact squared maximum of its candidates.
-__global__ void k_seg_size(const Seg* __restrict__ segs, const int32_t* __restrict__ nA_dev, const long long* __restrict__ seg_s2,
-                           TmpCells tmp) {
-  const int nA = *nA_dev;
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < nA) tmp.s[segs[s].cell] = sqrt(__longlong_as_double(seg_s2[s]));
 }
 
 // ---------------------------------------------------------------------------
@@ -893,7 +886,7 @@ k_subtree(SubArgs S) {
       // sizes, children
       if (tid < ncb) {
         const int cell = q[tid].y, first = q[tid].x & 0xffff, cnt = q[tid].x >> 16;
-        T.s[cell] = sqrt(__longlong_as_double((long long)L.s2[tid]));
+        T.s[cell] = __longlong_as_double((long long)L.s2[tid]);
         if (cnt > n_leaf) {
           int nl = L.opre[tid + 1 < ncb ? L.oct0[tid + 1] : noct] - L.opre[L.oct0[tid]];
           if (nl == 0 || nl == cnt) {
@@ -965,171 +958,209 @@ __global__ void k_leaf_segs(SubArgs S, const Seg* __restrict__ segL) {
   const int c = g.cell;
   t.first[c] = g.first; t.count[c] = cnt; t.depth[c] = g.dbuf >> 1;
   t.M[c] = M; t.cx[c] = cx; t.cy[c] = cy; t.cz[c] = cz;
-  t.s[c] = sqrt(__longlong_as_double(s2));
+  t.s[c] = __longlong_as_double(s2);
   t.left[c] = -1; t.right[c] = -1;
   }
 }
 
 // ---------------------------------------------------------------------------
 // pre-order numbering: a cell's id is the number of cells starting before its
-// first particle plus its depth below the topmost cell starting there.
+// first particle plus its depth below the topmost cell starting there; a
+// leaf's ordinal the number of leaves starting before it.  One scan over the
+// particle positions counts both (cells in the low, leaves in the high half
+// of a 64-bit word).
 // ---------------------------------------------------------------------------
-__global__ void k_fill2(int32_t* a, int32_t va, int32_t* b, int32_t vb, int64_t n) {
+typedef unsigned long long Starts;
+__device__ __forceinline__ int cells_before(const Starts* off, int64_t p) { return (int)(unsigned)off[p]; }
+__device__ __forceinline__ int leaves_before(const Starts* off, int64_t p) { return (int)(off[p] >> 32); }
+
+__global__ void k_fill2(Starts* a, Starts va, int32_t* b, int32_t vb, int64_t n) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) { a[i] = va; b[i] = vb; }
 }
 
-__global__ void k_count_starts(TmpCells tmp, const int32_t* __restrict__ counters,
-                               int32_t* cnt_start, int32_t* min_depth) {
+__global__ void k_count_starts(TmpCells tmp, const int32_t* __restrict__ counters, Starts* cnt,
+                               int32_t* min_depth) {
   const int ncells = counters[C_CELLS];
   KD_GRID_STRIDE(c, ncells) {
     const int f = tmp.first[c];
-    atomicAdd(&cnt_start[f], 1);
+    atomicAdd(&cnt[f], tmp.left[c] < 0 ? (Starts(1) << 32 | 1) : Starts(1));
     atomicMin(&min_depth[f], tmp.depth[c]);
   }
 }
 
-__device__ __forceinline__ int preorder_id(const int32_t* start_off, const int32_t* min_depth,
-                                           int first, int depth) {
-  return start_off[first] + depth - min_depth[first];
+__device__ __forceinline__ int preorder_id(const Starts* off, const int32_t* min_depth, int first,
+                                           int depth) {
+  return cells_before(off, first) + depth - min_depth[first];
 }
 
-__global__ void k_remap(TmpCells tmp, const int32_t* __restrict__ counters, const int32_t* __restrict__ start_off,
-                        const int32_t* __restrict__ min_depth, Cells c, int32_t* status) {
+// Cells in pre-order, their sizes (the square root of the squared size), the
+// leaves with their systems, the systems' roots; the leaf count goes to
+// counters[C_LEAVES].
+__global__ void k_remap(TmpCells tmp, int32_t* counters, const Starts* __restrict__ off,
+                        const int32_t* __restrict__ min_depth, Cells c, int32_t* status, int64_t n,
+                        int32_t* leaf_rank, int32_t* leaf_cells, int32_t* leaf_sys,
+                        const int64_t* __restrict__ sys_off, int n_sys, int32_t* sys_root) {
   const int t_n = counters[C_CELLS];
+  if (blockIdx.x == 0 && threadIdx.x == 0) counters[C_LEAVES] = leaves_before(off, n);
+  KD_GRID_STRIDE(k, n_sys + 1) sys_root[k] = cells_before(off, sys_off[k]);
   KD_GRID_STRIDE(t, t_n) {
   const int f = tmp.first[t], cnt = tmp.count[t], d = tmp.depth[t];
-  const int id = preorder_id(start_off, min_depth, f, d);
+  const int id = preorder_id(off, min_depth, f, d);
   c.first[id] = f; c.count[id] = cnt; c.depth[id] = d;
-  c.skip[id] = start_off[f + cnt];
+  c.skip[id] = cells_before(off, f + cnt);
   c.M[id] = tmp.M[t]; c.cx[id] = tmp.cx[t]; c.cy[id] = tmp.cy[t]; c.cz[id] = tmp.cz[t];
-  c.s[id] = tmp.s[t];
+  c.s[id] = sqrt(tmp.s[t]);
+  c.ready[id] = 0;
   const int lt = tmp.left[t];
   if (lt >= 0) {
     const int rt = tmp.right[t];
-    const int idl = preorder_id(start_off, min_depth, tmp.first[lt], tmp.depth[lt]);
-    const int idr = preorder_id(start_off, min_depth, tmp.first[rt], tmp.depth[rt]);
+    const int idl = preorder_id(off, min_depth, tmp.first[lt], tmp.depth[lt]);
+    const int idr = preorder_id(off, min_depth, tmp.first[rt], tmp.depth[rt]);
     if (idl != id + 1) atomicOr(status, ST_INTERNAL);
     c.left[id] = idl; c.right[id] = idr;
     c.parent[idl] = id; c.parent[idr] = id;
+    leaf_rank[id] = -1;
   } else {
     c.left[id] = -1; c.right[id] = -1;
+    const int r = leaves_before(off, f);
+    leaf_rank[id] = r;
+    leaf_cells[r] = id;
+    leaf_sys[r] = system_of(sys_off, n_sys, f);
   }
   if (d == 0) c.parent[id] = -1;               // a system's root
   }
 }
 
-// Pre-order id of each system's root; sys_root[n_sys] = number of cells.
-__global__ void k_sys_roots(const int64_t* __restrict__ sys_off, int n_sys,
-                            const int32_t* __restrict__ start_off, int32_t* sys_root) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k <= n_sys) sys_root[k] = start_off[sys_off[k]];
+// Component q of a symmetric tensor xx xy xz yy yz zz.
+__device__ __forceinline__ int comp_i(int q) { return q < 3 ? 0 : (q < 5 ? 1 : 2); }
+__device__ __forceinline__ int comp_j(int q) { return q < 3 ? q : (q < 5 ? q - 2 : 2); }
+__device__ __forceinline__ double pick3(int i, double x, double y, double z) {
+  return i == 0 ? x : (i == 1 ? y : z);
 }
 
-// Leaves: h_max and Q (Eq. 7) from their particles (one thread per leaf);
-// then each parent, once its second child has finished, from its children
-// (parallel-axis shift of Q).  Every sum runs in a fixed order.
-__global__ void k_upward(Cells c, const int32_t* __restrict__ leaf_cells, const int32_t* __restrict__ counters, PCols tp) {
-  const int k_n = counters[C_LEAVES];
-  KD_GRID_STRIDE(k, k_n) {
-  const int t = leaf_cells[k];
-  double q[6], hm = 0.0;
-  {
-    // S_jk = sum m y_j y_k (9 float64 operations a particle), then
-    // Q = 3 S - tr(S) I (Eq. 7) once for the leaf
-    const int f = c.first[t], cnt = c.count[t];
-    const double cx = c.cx[t], cy = c.cy[t], cz = c.cz[t];
-    double S[6] = {0, 0, 0, 0, 0, 0};
-    for (int j = 0; j < cnt; ++j) {
-      const int64_t i = (int64_t)f + j;
-      const double m = tp.m[i];
-      const double y0 = tp.x[i] - cx, y1 = tp.y[i] - cy, y2 = tp.z[i] - cz;
-      const double my0 = m * y0, my1 = m * y1, my2 = m * y2;
-      S[0] = fma(my0, y0, S[0]); S[1] = fma(my0, y1, S[1]); S[2] = fma(my0, y2, S[2]);
-      S[3] = fma(my1, y1, S[3]); S[4] = fma(my1, y2, S[4]); S[5] = fma(my2, y2, S[5]);
-      hm = fmax(hm, tp.h[i]);
+// Upward pass: 8 lanes per leaf.  The lanes take the leaf's particles (their
+// float32 records on the way), sum S_jk = sum m y_j y_k (9 float64 operations a
+// particle) and scatter the sums over the lanes, lane q < 6 holding component
+// q: Q = 3 S - tr(S) I (Eq. 7).  Then the group climbs: the second child of a
+// cell to finish adds both children's Q, shifted to the parent's centre of mass
+// (parallel axes: + M (3 d d - |d|^2 I)), a component a lane.  Every sum runs in a
+// fixed order.  Bound by the float64 pipe and, in small trees, by the chain of
+// the climb (an atomic and a moment load a level): a thread per leaf did all six
+// components itself, 46 operations a level for 13 here, and read its particles
+// one after the other.  With the particle records and the cells' views: 1009
+// particles 58 us, now 34; 2^24 clumped particles 1.71 ms, now 1.37 (1.92 with the
+// views written by the climb, their conversions on a few lanes).
+__global__ void __launch_bounds__(128)
+k_upward(Cells c, const int32_t* __restrict__ leaf_cells, const int32_t* __restrict__ counters, PCols tp,
+         float4* pf, float4* ph) {
+  const int lane = threadIdx.x & 31, q = lane & 7, g0 = lane & ~7;
+  const unsigned group = 0xffu << g0;
+  const int nleaves = counters[C_LEAVES];
+  const int qi = comp_i(min(q, 5)), qj = comp_j(min(q, 5));
+  const bool diag = qi == qj;
+  for (int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 3); k < nleaves;
+       k += (int)((gridDim.x * blockDim.x) >> 3)) {
+    int cur = leaf_cells[k];
+    double Q;
+    long long hm = 0;                           // largest h, as the bits of a non-negative double
+    {
+      const int f = c.first[cur], cnt = c.count[cur];
+      const double cx = c.cx[cur], cy = c.cy[cur], cz = c.cz[cur];
+      double S[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+      for (int j = q; j < cnt; j += 8) {
+        const int64_t i = (int64_t)f + j;
+        const double m = tp.m[i], h = tp.h[i];
+        const double y0 = tp.x[i] - cx, y1 = tp.y[i] - cy, y2 = tp.z[i] - cz;
+        const double my0 = m * y0, my1 = m * y1, my2 = m * y2;
+        S[0] = fma(my0, y0, S[0]); S[1] = fma(my0, y1, S[1]); S[2] = fma(my0, y2, S[2]);
+        S[3] = fma(my1, y1, S[3]); S[4] = fma(my1, y2, S[4]); S[5] = fma(my2, y2, S[5]);
+        hm = max(hm, __double_as_longlong(h));
+        pf[i] = make_float4(rn_to_float(y0), rn_to_float(y1), rn_to_float(y2), rn_to_float(m));
+        const float hf = rn_to_float(h);
+        const float hi = hf > 0.0f ? 1.0f / hf : 0.0f;
+        ph[i] = make_float4(hi, hi * hi * hi, hf, 4.0f * hf * hf);   // 1/h, 1/h^3, h, (2h)^2
+      }
+      // reduce-scatter: after the exchange over lane bit o, a lane keeps the
+      // half of the sums whose index bit equals its own
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        const bool up = (q & o) != 0;
+#pragma unroll
+        for (int i = 0; i < o; ++i) {
+          const double send = up ? S[i] : S[i + o], keep = up ? S[i + o] : S[i];
+          S[i] = keep + __shfl_xor_sync(group, send, o);
+        }
+        hm = max(hm, __shfl_xor_sync(group, hm, o));
+      }
+      const double tr = __shfl_sync(group, S[0], g0) + __shfl_sync(group, S[0], g0 + 3) +
+                        __shfl_sync(group, S[0], g0 + 5);
+      Q = diag ? 3.0 * S[0] - tr : 3.0 * S[0];
     }
-    const double tr = S[0] + S[3] + S[5];
-    q[0] = 3.0 * S[0] - tr; q[1] = 3.0 * S[1]; q[2] = 3.0 * S[2];
-    q[3] = 3.0 * S[3] - tr; q[4] = 3.0 * S[4]; q[5] = 3.0 * S[5] - tr;
-  }
-  for (int j = 0; j < 6; ++j) c.Q[6 * t + j] = q[j];
-  c.hmax[t] = hm;
-  int cur = t;
-  while (true) {
-    const int p = c.parent[cur];
-    if (p < 0) break;
-    __threadfence();
-    if (atomicAdd(&c.ready[p], 1) == 0) break;      // the sibling finishes the parent
-    __threadfence();
-    const double px = c.cx[p], py = c.cy[p], pz = c.cz[p];
-    double qp[6] = {0, 0, 0, 0, 0, 0}, hp = 0.0;
-    const int ch[2] = {c.left[p], c.right[p]};
-    for (int side = 0; side < 2; ++side) {
-      // parallel-axis shift of the child's Q to the parent's centre of mass:
-      // + M (3 d d - |d|^2 I)
-      const int kc = ch[side];
-      const double mk = c.M[kc];
-      const double d0 = c.cx[kc] - px, d1 = c.cy[kc] - py, d2 = c.cz[kc] - pz;
-      const double m0 = 3.0 * mk * d0, m1 = 3.0 * mk * d1;
-      const double mdd = mk * (d0 * d0 + d1 * d1 + d2 * d2);
-      qp[0] += __ldcg(&c.Q[6 * kc + 0]) + fma(m0, d0, -mdd);
-      qp[1] += __ldcg(&c.Q[6 * kc + 1]) + m0 * d1;
-      qp[2] += __ldcg(&c.Q[6 * kc + 2]) + m0 * d2;
-      qp[3] += __ldcg(&c.Q[6 * kc + 3]) + fma(m1, d1, -mdd);
-      qp[4] += __ldcg(&c.Q[6 * kc + 4]) + m1 * d2;
-      qp[5] += __ldcg(&c.Q[6 * kc + 5]) + fma(3.0 * mk * d2, d2, -mdd);
-      hp = fmax(hp, __ldcg(&c.hmax[kc]));
+    for (;;) {
+      const double x = c.cx[cur], y = c.cy[cur], z = c.cz[cur], M = c.M[cur];
+      if (q < 6) c.Q[6 * (int64_t)cur + q] = Q;
+      else if (q == 6) c.hmax[cur] = __longlong_as_double(hm);
+      const int p = c.parent[cur];
+      if (p < 0) break;
+      const int L = p + 1, R = c.right[p], sib = cur == L ? R : L;
+      // the parent's and the children's static moments, ahead of the atomic
+      const double px = c.cx[p], py = c.cy[p], pz = c.cz[p];
+      const double sx = c.cx[sib], sy = c.cy[sib], sz = c.cz[sib], sM = c.M[sib];
+      __threadfence();
+      __syncwarp(group);
+      int arrived = 0;
+      if (q == 0) arrived = atomicAdd(&c.ready[p], 1);
+      if (__shfl_sync(group, arrived, g0) == 0) break;      // the sibling finishes the parent
+      __threadfence();
+      const double sQ = q < 6 ? __ldcg(&c.Q[6 * (int64_t)sib + q]) : 0.0;
+      const long long sh = __double_as_longlong(__ldcg(&c.hmax[sib]));
+      // offsets from the parent's centre of mass: lanes 0-2 this cell's, 3-5
+      // the sibling's; |d|^2 M of each child on the lanes' halves
+      const double d = q < 3 ? pick3(q, x, y, z) - pick3(q, px, py, pz)
+                             : pick3(q - 3, sx, sy, sz) - pick3(q - 3, px, py, pz);
+      const double d0 = __shfl_sync(group, d, g0), d1 = __shfl_sync(group, d, g0 + 1),
+                   d2 = __shfl_sync(group, d, g0 + 2);
+      const double e0 = __shfl_sync(group, d, g0 + 3), e1 = __shfl_sync(group, d, g0 + 4),
+                   e2 = __shfl_sync(group, d, g0 + 5);
+      const bool half = q >= 4;
+      const double u0 = half ? e0 : d0, u1 = half ? e1 : d1, u2 = half ? e2 : d2;
+      const double mdd = (half ? sM : M) * (u0 * u0 + u1 * u1 + u2 * u2);
+      const double mdd_c = __shfl_sync(group, mdd, g0), mdd_s = __shfl_sync(group, mdd, g0 + 4);
+      const double tc = 3.0 * M * pick3(qi, d0, d1, d2), ts = 3.0 * sM * pick3(qi, e0, e1, e2);
+      const double vc = Q + fma(tc, pick3(qj, d0, d1, d2), diag ? -mdd_c : 0.0);
+      const double vs = sQ + fma(ts, pick3(qj, e0, e1, e2), diag ? -mdd_s : 0.0);
+      Q = cur == L ? vc + vs : vs + vc;
+      hm = max(hm, sh);
+      cur = p;
     }
-    for (int j = 0; j < 6; ++j) c.Q[6 * p + j] = qp[j];
-    c.hmax[p] = hp;
-    cur = p;
+    __syncwarp(group);
   }
-  }
-}
-
-__global__ void k_leaf_flags(const Cells c, const int32_t* __restrict__ counters, int32_t* flag) {
-  const int t_n = counters[C_CELLS];
-  KD_GRID_STRIDE(t, t_n) flag[t] = c.left[t] < 0 ? 1 : 0;
 }
 
 // float32 views of the cells.
 __global__ void k_derive_cells(Cells c, const int32_t* __restrict__ counters, float* com_bound) {
   const int t_n = counters[C_CELLS];
   KD_GRID_STRIDE(t, t_n) {
-  const double cx = c.cx[t], cy = c.cy[t], cz = c.cz[t];
-  c.walk[t] = make_float4((float)cx, (float)cy, (float)cz, (float)c.s[t]);
-  c.walk2[t] = make_float4((float)c.hmax[t], __int_as_float(c.skip[t]), __int_as_float(c.count[t]),
-                          0.0f);
-  const float hx = (float)cx, hy = (float)cy, hz = (float)cz;
-  c.src32[4 * t + 0] = make_float4(hx, hy, hz, (float)c.M[t]);
-  c.src32[4 * t + 1] = make_float4((float)(cx - (double)hx), (float)(cy - (double)hy),
-                                   (float)(cz - (double)hz), 0.0f);
-  c.src32[4 * t + 2] = make_float4((float)c.Q[6 * t + 0], (float)c.Q[6 * t + 1],
-                                   (float)c.Q[6 * t + 2], (float)c.Q[6 * t + 3]);
-  c.src32[4 * t + 3] = make_float4((float)c.Q[6 * t + 4], (float)c.Q[6 * t + 5], 0.0f, 0.0f);
+  const double cx = c.cx[t], cy = c.cy[t], cz = c.cz[t], M = c.M[t];
+  const float hx = rn_to_float(cx), hy = rn_to_float(cy), hz = rn_to_float(cz);
+  double Q[6];
+  for (int k = 0; k < 6; ++k) Q[k] = c.Q[6 * (int64_t)t + k];
+  c.walk[t] = make_float4(hx, hy, hz, rn_to_float(c.s[t]));
+  c.walk2[t] = make_float4(rn_to_float(c.hmax[t]), __int_as_float(c.skip[t]),
+                           __int_as_float(c.count[t]), 0.0f);
+  c.src32[4 * (int64_t)t + 0] = make_float4(hx, hy, hz, rn_to_float(M));
+  c.src32[4 * (int64_t)t + 1] =
+      make_float4(rn_to_float(cx - float_to_double(hx)), rn_to_float(cy - float_to_double(hy)),
+                  rn_to_float(cz - float_to_double(hz)), 0.0f);
+  c.src32[4 * (int64_t)t + 2] =
+      make_float4(rn_to_float(Q[0]), rn_to_float(Q[1]), rn_to_float(Q[2]), rn_to_float(Q[3]));
+  c.src32[4 * (int64_t)t + 3] = make_float4(rn_to_float(Q[4]), rn_to_float(Q[5]), 0.0f, 0.0f);
   double* s64 = c.src64 + 10 * (int64_t)t;
-  s64[0] = cx; s64[1] = cy; s64[2] = cz; s64[3] = c.M[t];
-  for (int k = 0; k < 6; ++k) s64[4 + k] = c.Q[6 * t + k];
-  float b = fmaxf(fabsf((float)cx), fmaxf(fabsf((float)cy), fabsf((float)cz)));
-  atomicMax(reinterpret_cast<int*>(com_bound), __float_as_int(b));
-  }
-}
-
-// Leaf ordinal -> cell and system; the leaf count goes to counters[C_LEAVES].
-__global__ void k_leaf_list(const Cells c, int32_t* counters, int32_t* leaf_rank,
-                            int32_t* leaf_cells, const int64_t* __restrict__ sys_off, int n_sys,
-                            int32_t* leaf_sys) {
-  const int t_n = counters[C_CELLS];
-  if (blockIdx.x == 0 && threadIdx.x == 0) counters[C_LEAVES] = leaf_rank[t_n];
-  KD_GRID_STRIDE(t, t_n) {
-  if (c.left[t] < 0) {
-    const int r = leaf_rank[t];
-    leaf_cells[r] = t;
-    leaf_sys[r] = system_of(sys_off, n_sys, c.first[t]);
-  } else {
-    leaf_rank[t] = -1;
-  }
+  s64[0] = cx; s64[1] = cy; s64[2] = cz; s64[3] = M;
+  for (int k = 0; k < 6; ++k) s64[4 + k] = Q[k];
+  const int b = __float_as_int(fmaxf(fabsf(hx), fmaxf(fabsf(hy), fabsf(hz))));
+  if (b > *(volatile int*)com_bound) atomicMax(reinterpret_cast<int*>(com_bound), b);
   }
 }
 
@@ -1146,9 +1177,9 @@ __global__ void k_particles32(const Cells c, const int32_t* __restrict__ leaf_ce
     const int f = c.first[cell], cnt = c.count[cell];
     if (lane >= cnt) continue;
     const int64_t i = (int64_t)f + lane;
-    pf[i] = make_float4((float)(tp.x[i] - c.cx[cell]), (float)(tp.y[i] - c.cy[cell]),
-                        (float)(tp.z[i] - c.cz[cell]), (float)tp.m[i]);
-    const float h = (float)tp.h[i];
+    pf[i] = make_float4(rn_to_float(tp.x[i] - c.cx[cell]), rn_to_float(tp.y[i] - c.cy[cell]),
+                        rn_to_float(tp.z[i] - c.cz[cell]), rn_to_float(tp.m[i]));
+    const float h = rn_to_float(tp.h[i]);
     const float hi = h > 0.0f ? 1.0f / h : 0.0f;
     ph[i] = make_float4(hi, hi * hi * hi, h, 4.0f * h * h);   // 1/h, 1/h^3, h, (2h)^2
   }
@@ -1180,10 +1211,10 @@ void free_build_buffers(kdfmm_tree_s* t) {
   free_cols(&t->tp);
   void* ptrs[] = {t->segB, t->segL, t->chunk_seg, t->seg_chunk_off, t->chunk_sum, t->chunk_key,
                   t->chunk_left, t->chunk_loff, t->chunk_s2, t->seg_axis, t->seg_cut, t->seg_nl,
-                  t->seg_xb, t->seg_thr2, t->seg_s2,
+                  t->seg_xb, t->seg_thr2,
                   t->tmp.first, t->tmp.count, t->tmp.left, t->tmp.right, t->tmp.depth, t->tmp.M,
-                  t->tmp.cx, t->tmp.cy, t->tmp.cz, t->tmp.s, t->cnt_start, t->min_depth,
-                  t->start_off, t->scan_tmp, t->pf, t->ph, t->c.first, t->c.count, t->c.left,
+                  t->tmp.cx, t->tmp.cy, t->tmp.cz, t->tmp.s, t->starts, t->min_depth,
+                  t->scan_tmp, t->pf, t->ph, t->c.first, t->c.count, t->c.left,
                   t->c.right, t->c.parent, t->c.skip, t->c.depth, t->c.M, t->c.cx, t->c.cy,
                   t->c.cz, t->c.s, t->c.hmax, t->c.Q, t->c.walk, t->c.walk2, t->c.src32,
                   t->c.src64, t->c.ready, t->leaf_cells, t->leaf_rank, t->leaf_sys, t->lexp64,
@@ -1194,9 +1225,9 @@ void free_build_buffers(kdfmm_tree_s* t) {
   t->chunk_sum = t->seg_cut = nullptr;
   t->chunk_key = nullptr;
   t->chunk_s2 = t->seg_xb = t->seg_thr2 = nullptr;
-  t->seg_s2 = nullptr;
   t->tmp = TmpCells{};
-  t->cnt_start = t->min_depth = t->start_off = t->scan_tmp = nullptr;
+  t->starts = nullptr;
+  t->min_depth = t->scan_tmp = nullptr;
   t->pf = t->ph = nullptr;
   t->c = Cells{};
   t->leaf_cells = t->leaf_rank = t->leaf_sys = nullptr;
@@ -1239,15 +1270,13 @@ static int ensure_build_buffers(kdfmm_tree_s* t, int64_t n) {
   KD_ALLOC(t->seg_nl, t->capA);
   KD_ALLOC(t->seg_xb, t->capA);
   KD_ALLOC(t->seg_thr2, t->capA);
-  KD_ALLOC(t->seg_s2, t->capA);
   t->cap_cells = 2 * n + 2;
   const int64_t nc = t->cap_cells;
   KD_ALLOC(t->tmp.first, nc); KD_ALLOC(t->tmp.count, nc); KD_ALLOC(t->tmp.left, nc);
   KD_ALLOC(t->tmp.right, nc); KD_ALLOC(t->tmp.depth, nc); KD_ALLOC(t->tmp.M, nc);
   KD_ALLOC(t->tmp.cx, nc); KD_ALLOC(t->tmp.cy, nc); KD_ALLOC(t->tmp.cz, nc); KD_ALLOC(t->tmp.s, nc);
-  KD_ALLOC(t->cnt_start, n + 2);
+  KD_ALLOC(t->starts, n + 2);
   KD_ALLOC(t->min_depth, n + 2);
-  KD_ALLOC(t->start_off, n + 2);
   t->cap_scan = scan_tmp_elems(nc > n + 2 ? nc : n + 2) * 2 + 16;
   KD_ALLOC(t->scan_tmp, t->cap_scan);
   KD_ALLOC(t->pf, n);
@@ -1359,7 +1388,7 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
     k_chunk_reduce<<<maxc, kChunkThreads, 0, s>>>(segs, t->chunk_seg, t->seg_chunk_off, t->counters,
                                                   t->buf[src], t->chunk_sum, t->chunk_key);
     k_decide<<<segw, 256, 0, s>>>(segs, nA, t->seg_chunk_off, t->chunk_sum, t->chunk_key, t->tmp,
-                                  t->seg_axis, t->seg_cut, t->seg_xb, t->seg_s2);
+                                  t->seg_axis, t->seg_cut, t->seg_xb);
     k_chunk_count<<<maxc, kChunkThreads, 0, s>>>(segs, t->chunk_seg, t->seg_chunk_off, t->counters,
                                                  t->buf[src], t->tmp, t->seg_axis, t->seg_cut,
                                                  t->chunk_left, t->chunk_s2);
@@ -1368,10 +1397,8 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
                                  t->segL, dst);
     k_chunk_scatter<<<maxc, kChunkThreads, 0, s>>>(segs, t->chunk_seg, t->seg_chunk_off, t->counters,
                                                    t->buf[src], t->buf[dst], t->seg_axis, t->seg_cut,
-                                                   t->chunk_loff, t->seg_nl, t->tmp, t->seg_thr2,
-                                                   t->seg_s2);
-    k_seg_size<<<blocks_for(t->capA, 128), 128, 0, s>>>(segs, nA, t->seg_s2, t->tmp);
-    t->launches += 8;
+                                                   t->chunk_loff, t->seg_nl, t->tmp, t->seg_thr2);
+    t->launches += 7;
     cur ^= 1;
     ++level;
     if (!deferred) {
@@ -1412,32 +1439,24 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
   }
 
   // pre-order numbering, counts read on the device
-  k_fill2<<<blocks_for(n + 1, 256), 256, 0, s>>>(t->cnt_start, 0, t->min_depth, INT_MAX, n + 1);
-  k_count_starts<<<grid_blocks(), 256, 0, s>>>(t->tmp, t->counters, t->cnt_start, t->min_depth);
-  scan_i32(t->cnt_start, t->start_off, n, t->scan_tmp, s);
-  k_remap<<<grid_blocks(), 256, 0, s>>>(t->tmp, t->counters, t->start_off, t->min_depth, t->c,
-                                      t->status);
-  k_leaf_flags<<<grid_blocks(), 256, 0, s>>>(t->c, t->counters, t->c.ready);
-  scan_i32_dev(t->c.ready, t->leaf_rank, t->counters + C_CELLS,
-               deferred ? t->cap_cells : (int64_t)t->ncells, t->scan_tmp, s);
-  k_leaf_list<<<grid_blocks(), 256, 0, s>>>(t->c, t->counters, t->leaf_rank, t->leaf_cells,
-                                          t->sys_off, t->n_sys, t->leaf_sys);
-  k_sys_roots<<<blocks_for(t->n_sys + 1, 128), 128, 0, s>>>(t->sys_off, t->n_sys, t->start_off,
-                                                            t->sys_root);
+  k_fill2<<<blocks_for(n + 1, 256), 256, 0, s>>>(t->starts, 0, t->min_depth, INT_MAX, n + 1);
+  k_count_starts<<<grid_blocks(), 256, 0, s>>>(t->tmp, t->counters, t->starts, t->min_depth);
+  scan_u64(t->starts, n, reinterpret_cast<unsigned long long*>(t->scan_tmp), s);
+  k_remap<<<grid_blocks(), 256, 0, s>>>(t->tmp, t->counters, t->starts, t->min_depth, t->c, t->status, n,
+                                      t->leaf_rank, t->leaf_cells, t->leaf_sys, t->sys_off, t->n_sys,
+                                      t->sys_root);
   if (!deferred) {
     if ((rc = read_back("build finalise"))) return rc;
     t->nleaves = hc[C_LEAVES];
     if (hc[32] & ST_INTERNAL) return set_error(KDFMM_ERR_INTERNAL, "pre-order numbering inconsistent");
   }
-  cudaMemsetAsync(t->c.ready, 0,
-                  (size_t)(deferred ? t->cap_cells : (int64_t)t->ncells) * sizeof(int32_t), s);
-  // one thread per leaf (the climb is latency-bound): the grid follows the last
-  // known leaf count with a margin; more leaves than threads loop
-  const int64_t up_threads = std::max<int64_t>(t->nleaves, 1) + t->nleaves / 4 + 128;
-  k_upward<<<blocks_for(up_threads, 128), 128, 0, s>>>(t->c, t->leaf_cells, t->counters, t->tp);
+  // the grid follows the last known leaf count with a margin; more leaves than
+  // groups of 8 lanes loop
+  const int64_t up_groups = std::max<int64_t>(t->nleaves, 1) + t->nleaves / 4 + 128;
+  k_upward<<<blocks_for(8 * up_groups, 128), 128, 0, s>>>(t->c, t->leaf_cells, t->counters, t->tp, t->pf,
+                                                       t->ph);
   k_derive_cells<<<grid_blocks(), 256, 0, s>>>(t->c, t->counters, t->com_bound);
-  k_particles32<<<grid_blocks(), 256, 0, s>>>(t->c, t->leaf_cells, t->counters, t->tp, t->pf, t->ph);
-  t->launches += 15;
+  t->launches += 5 + scan_launches(n);
   return check_cuda(cudaGetLastError(), "build launch");
 }
 

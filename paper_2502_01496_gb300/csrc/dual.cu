@@ -455,7 +455,7 @@ int run_dual_walk(kdfmm_tree_s* t, cudaStream_t s) {
     return rc;
   k_near_fill<<<blocks_for(std::max<int64_t>(nnear, 1), 256), 256, 0, s>>>(
       D.near, (int)nnear, t->leaf_rank, L.near_off, D.cursor, L.near_idx);
-  t->launches += 10;
+  t->launches += 4 + scan_launches(nc) + scan_launches(nl);
   L.exact = true;
   D.nfar = 2 * nfar;
   D.nnear = entries;

@@ -72,7 +72,8 @@ struct PCols {
 // Cells in build (temporary) order.
 struct TmpCells {
   int32_t *first, *count, *left, *right, *depth;
-  double *M, *cx, *cy, *cz, *s;
+  double *M, *cx, *cy, *cz;
+  double* s;                       // squared size
 };
 
 // Cells in final pre-order.
@@ -154,13 +155,13 @@ struct kdfmm_tree_s {
   float* chunk_s2 = nullptr;         // per chunk: largest float32 squared distance
   float* seg_xb = nullptr;           // per segment: bound on |coordinates|
   float* seg_thr2 = nullptr;         // per segment: candidate threshold for the exact size
-  long long* seg_s2 = nullptr;       // per segment: exact squared size (as int64 bits)
   int32_t* seg_axis = nullptr;
   double* seg_cut = nullptr;
   int32_t* seg_nl = nullptr;
   int64_t cap_chunks = 0, cap_segA = 0;
   kdfmm::TmpCells tmp{};
-  int32_t *cnt_start = nullptr, *min_depth = nullptr, *start_off = nullptr;
+  unsigned long long* starts = nullptr;  // per particle: cells and leaves starting there, then before it
+  int32_t* min_depth = nullptr;
   int32_t* scan_tmp = nullptr;
   int64_t cap_scan = 0;
 
@@ -279,6 +280,25 @@ __device__ __forceinline__ float trunc_to_float(double v) {
   if (e >= 255) return __uint_as_float(sign | 0x7f800000u);
   const unsigned mant = ((hi & 0xfffffu) << 3) | (lo >> 29);
   return __uint_as_float(sign | ((unsigned)e << 23) | mant);
+}
+
+// (float)v and (double)f with integer operations (a conversion occupies the
+// float64 pipe 64 cycles a warp instruction): round to nearest even on the
+// bits; results outside the normal float range, zero but for its sign, NaN and
+// infinities take the conversion instruction.
+__device__ __forceinline__ float rn_to_float(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned e = (unsigned)(b >> 52) & 0x7ffu;
+  if (e - 897u >= 253u) return (b << 1) == 0ull ? __uint_as_float((unsigned)(b >> 32)) : (float)v;
+  const unsigned long long a = b & 0x7fffffffffffffffULL;
+  const unsigned long long r = a + 0x0fffffffULL + ((a >> 29) & 1ull);
+  return __uint_as_float(((unsigned)(b >> 32) & 0x80000000u) | ((unsigned)(r >> 29) - (896u << 23)));
+}
+__device__ __forceinline__ double float_to_double(float f) {
+  const unsigned b = __float_as_uint(f), e = (b >> 23) & 0xffu;
+  if (e - 1u >= 254u) return (double)f;
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))),
+                          (int)(b << 29));
 }
 
 // Reciprocal square root, flush-to-zero form of the hardware approximation
@@ -498,13 +518,12 @@ int plan_segments(kdfmm_tree_s* t, cudaStream_t s);
 int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, cudaStream_t s);
 int momentum(const double* m, const double* v, int64_t n, double* out, double* scratch,
              cudaStream_t s);
-// exclusive scan of n int32 (out may alias in); returns the total in *total_dev
-void scan_i32(const int32_t* in, int32_t* out, int64_t n, int32_t* tmp, cudaStream_t s);
-// the same with the count read from device memory (*n_dev <= cap)
-void scan_i32_dev(const int32_t* in, int32_t* out, const int32_t* n_dev, int64_t cap, int32_t* tmp,
-                  cudaStream_t s);
+// exclusive scans of n values, the total in entry n (scan_u64 in place; tmp:
+// scan_tmp_elems(n) 64-bit words)
+void scan_u64(unsigned long long* v, int64_t n, unsigned long long* tmp, cudaStream_t s);
 void scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* tmp, cudaStream_t s);
 int64_t scan_tmp_elems(int64_t n);
+int scan_launches(int64_t n);
 
 // tracing (api.cu): CUDA events around a phase when timing is enabled
 void phase_begin(kdfmm_tree_s* t, int phase, cudaStream_t s);

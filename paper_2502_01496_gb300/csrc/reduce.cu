@@ -22,14 +22,11 @@ __device__ __forceinline__ T warp_incl_scan(T v) {
   return v;
 }
 
-// Exclusive scan of one tile per block; the block total goes to tot[block].
-// n_dev, when given, holds the element count (at most n); the launch is sized
-// for n.
-template <class TO>
-__global__ void k_scan_tile(const int32_t* __restrict__ in, TO* __restrict__ out, int64_t n,
-                            const int32_t* __restrict__ n_dev, TO* __restrict__ tot) {
+// Exclusive scan of one tile per block (in place when out is in); the block
+// total goes to tot[block].
+template <class TI, class TO>
+__global__ void k_scan_tile(const TI* in, TO* out, int64_t n, TO* __restrict__ tot) {
   __shared__ TO warp_tot[kScanThreads / 32];
-  if (n_dev) n = *n_dev;
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanPer;
   TO v[kScanPer];
   TO run = 0;
@@ -89,9 +86,7 @@ __global__ void k_scan_top(TO* tot, int64_t nb) {
 }
 
 template <class TO>
-__global__ void k_scan_add(TO* __restrict__ out, int64_t n, const int32_t* __restrict__ n_dev,
-                           const TO* __restrict__ tot, int64_t nb) {
-  if (n_dev) n = *n_dev;
+__global__ void k_scan_add(TO* __restrict__ out, int64_t n, const TO* __restrict__ tot, int64_t nb) {
   const int64_t base = (int64_t)blockIdx.x * kScanTile;
   const TO off = tot[blockIdx.x];
   for (int k = threadIdx.x; k < kScanTile; k += blockDim.x) {
@@ -101,17 +96,53 @@ __global__ void k_scan_add(TO* __restrict__ out, int64_t n, const int32_t* __res
   if (blockIdx.x == 0 && threadIdx.x == 0) out[n] = tot[nb];
 }
 
-template <class TO>
-void scan_impl(const int32_t* in, TO* out, int64_t n, const int32_t* n_dev, TO* tmp,
-               cudaStream_t s) {
+// The whole scan by one block, tile after tile (8 values a thread).
+constexpr int kScanSmall = 32768;
+template <class TI, class TO>
+__global__ void __launch_bounds__(1024) k_scan_small(const TI* in, TO* out, int n) {
+  __shared__ TO warp_tot[2][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  TO carry = 0;
+  int buf = 0;
+  for (int t0 = 0; t0 < n; t0 += 8 * 1024, buf ^= 1) {
+    const int base = t0 + 8 * (int)threadIdx.x;
+    TO v[8], run = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const TO e = base + k < n ? (TO)in[base + k] : (TO)0;
+      v[k] = run;
+      run += e;
+    }
+    const TO incl = warp_incl_scan<TO>(run);
+    if (lane == 31) warp_tot[buf][w] = incl;
+    __syncthreads();
+    const TO t = warp_tot[buf][lane], ti = warp_incl_scan<TO>(t);
+    const TO before = __shfl_sync(0xffffffffu, ti - t, w), total = __shfl_sync(0xffffffffu, ti, 31);
+    const TO off = carry + before + incl - run;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (base + k < n) out[base + k] = off + v[k];
+    carry += total;
+  }
+  if (threadIdx.x == 0) out[n] = carry;
+}
+
+// Up to kScanSmall values one block's tiles cost less than two more launches
+// (1009 values: 3 us for 10; 16386: 5 for 10).
+template <class TI, class TO>
+void scan_impl(const TI* in, TO* out, int64_t n, TO* tmp, cudaStream_t s) {
   int64_t nb = (n + kScanTile - 1) / kScanTile;
   if (nb == 0) {
     cudaMemsetAsync(out, 0, sizeof(TO), s);
     return;
   }
-  k_scan_tile<TO><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, n_dev, tmp);
+  if (n <= kScanSmall) {
+    k_scan_small<TI, TO><<<1, 1024, 0, s>>>(in, out, (int)n);
+    return;
+  }
+  k_scan_tile<TI, TO><<<(unsigned)nb, kScanThreads, 0, s>>>(in, out, n, tmp);
   k_scan_top<TO><<<1, 1024, 0, s>>>(tmp, nb);
-  k_scan_add<TO><<<(unsigned)nb, kScanThreads, 0, s>>>(out, n, n_dev, tmp, nb);
+  k_scan_add<TO><<<(unsigned)nb, kScanThreads, 0, s>>>(out, n, tmp, nb);
 }
 
 // ---------------------------------------------------------------------------
@@ -119,10 +150,32 @@ void scan_impl(const int32_t* in, TO* out, int64_t n, const int32_t* n_dev, TO* 
 // ---------------------------------------------------------------------------
 constexpr int kMomThreads = 256;
 
+// Two-sum tree over the rows of sh (sum, error; three components), row r of a
+// round taking row r + stride.  A thread does one component of a row (7 float64
+// operations a round instead of 21: the rounds are a chain on the 1/64-rate
+// pipe); rounds whose partners are all zero, beyond `rows`, change nothing and
+// are left out.
+__device__ __forceinline__ void momentum_tree(double (*sh)[6], int rows) {
+  int stride = kMomThreads / 2;
+  while (stride >= rows && stride > 0) stride >>= 1;
+  for (; stride > 0; stride >>= 1) {
+    for (int t = threadIdx.x; t < 3 * stride; t += kMomThreads) {
+      const int c = t / stride, r = t - c * stride;
+      double s, e;
+      two_sum_d(sh[r][2 * c], sh[r + stride][2 * c], s, e);
+      sh[r][2 * c] = s;
+      sh[r][2 * c + 1] = __dadd_rn(__dadd_rn(sh[r][2 * c + 1], sh[r + stride][2 * c + 1]), e);
+    }
+    __syncthreads();
+  }
+}
+
 // Each block sums its contiguous range in plain float64 per thread, then
 // combines its threads with two-sum in a fixed order: partial = (hi, lo) x 3.
+// A single block (n <= 4096) writes the result.
 __global__ void k_momentum_blocks(const double* __restrict__ m, const double* __restrict__ v,
-                                  int64_t n, int64_t per_block, double* __restrict__ part) {
+                                  int64_t n, int64_t per_block, double* __restrict__ part,
+                                  double* __restrict__ out) {
   __shared__ double sh[kMomThreads][6];
   const int64_t lo = (int64_t)blockIdx.x * per_block;
   const int64_t hi = min(n, lo + per_block);
@@ -137,20 +190,13 @@ __global__ void k_momentum_blocks(const double* __restrict__ m, const double* __
   sh[threadIdx.x][2] = ay; sh[threadIdx.x][3] = 0.0;
   sh[threadIdx.x][4] = az; sh[threadIdx.x][5] = 0.0;
   __syncthreads();
-  for (int stride = kMomThreads / 2; stride > 0; stride >>= 1) {
-    if (threadIdx.x < stride) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        double s, e;
-        two_sum_d(sh[threadIdx.x][2 * c], sh[threadIdx.x + stride][2 * c], s, e);
-        sh[threadIdx.x][2 * c] = s;
-        sh[threadIdx.x][2 * c + 1] =
-            __dadd_rn(__dadd_rn(sh[threadIdx.x][2 * c + 1], sh[threadIdx.x + stride][2 * c + 1]), e);
-      }
-    }
-    __syncthreads();
+  momentum_tree(sh, (int)min((int64_t)kMomThreads, max(hi - lo, (int64_t)0)));
+  if (gridDim.x == 1) {
+    if (threadIdx.x < 3)
+      out[threadIdx.x] = __dadd_rn(sh[0][2 * threadIdx.x], sh[0][2 * threadIdx.x + 1]);
+  } else if (threadIdx.x < 6) {
+    part[6 * blockIdx.x + threadIdx.x] = sh[0][threadIdx.x];
   }
-  if (threadIdx.x < 6) part[6 * blockIdx.x + threadIdx.x] = sh[0][threadIdx.x];
 }
 
 // Combines the partials: thread t folds partials t, t + 256, ... with two-sum,
@@ -169,37 +215,22 @@ __global__ void k_momentum_final(const double* __restrict__ part, int nb, double
   }
   for (int j = 0; j < 6; ++j) sh[threadIdx.x][j] = v[j];
   __syncthreads();
-  for (int stride = kMomThreads / 2; stride > 0; stride >>= 1) {
-    if (threadIdx.x < stride) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        double s, e;
-        two_sum_d(sh[threadIdx.x][2 * c], sh[threadIdx.x + stride][2 * c], s, e);
-        sh[threadIdx.x][2 * c] = s;
-        sh[threadIdx.x][2 * c + 1] =
-            __dadd_rn(__dadd_rn(sh[threadIdx.x][2 * c + 1], sh[threadIdx.x + stride][2 * c + 1]), e);
-      }
-    }
-    __syncthreads();
-  }
+  momentum_tree(sh, min(nb, kMomThreads));
   if (threadIdx.x < 3) out[threadIdx.x] = __dadd_rn(sh[0][2 * threadIdx.x], sh[0][2 * threadIdx.x + 1]);
 }
 
 }  // namespace
 
+int scan_launches(int64_t n) { return n <= kScanSmall ? 1 : 3; }
+
 int64_t scan_tmp_elems(int64_t n) { return (n + kScanTile - 1) / kScanTile + 2; }
 
-void scan_i32(const int32_t* in, int32_t* out, int64_t n, int32_t* tmp, cudaStream_t s) {
-  scan_impl<int32_t>(in, out, n, nullptr, tmp, s);
-}
-
-void scan_i32_dev(const int32_t* in, int32_t* out, const int32_t* n_dev, int64_t cap, int32_t* tmp,
-                  cudaStream_t s) {
-  scan_impl<int32_t>(in, out, cap, n_dev, tmp, s);
+void scan_u64(unsigned long long* v, int64_t n, unsigned long long* tmp, cudaStream_t s) {
+  scan_impl<unsigned long long, unsigned long long>(v, v, n, tmp, s);
 }
 
 void scan_i32_to_i64(const int32_t* in, int64_t* out, int64_t n, int64_t* tmp, cudaStream_t s) {
-  scan_impl<int64_t>(in, out, n, nullptr, tmp, s);
+  scan_impl<int32_t, int64_t>(in, out, n, tmp, s);
 }
 
 int64_t momentum_blocks(int64_t n) {
@@ -213,8 +244,8 @@ int momentum(const double* m, const double* v, int64_t n, double* out, double* s
              cudaStream_t s) {
   int64_t nb = momentum_blocks(n);
   int64_t per = (n + nb - 1) / nb;
-  k_momentum_blocks<<<(unsigned)nb, kMomThreads, 0, s>>>(m, v, n, per, scratch);
-  k_momentum_final<<<1, kMomThreads, 0, s>>>(scratch, (int)nb, out);
+  k_momentum_blocks<<<(unsigned)nb, kMomThreads, 0, s>>>(m, v, n, per, scratch, out);
+  if (nb > 1) k_momentum_final<<<1, kMomThreads, 0, s>>>(scratch, (int)nb, out);
   return check_cuda(cudaGetLastError(), "momentum launch");
 }
 

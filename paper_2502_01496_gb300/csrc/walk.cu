@@ -992,7 +992,7 @@ int run_walk(kdfmm_tree_s* t, cudaStream_t s) {
     const int64_t tf = t->host_stats[16 + 2], tn = t->host_stats[16 + 3];
     scan_i32_to_i64(L.far_cnt, L.far_off, nl, reinterpret_cast<int64_t*>(t->scan_tmp), s);
     scan_i32_to_i64(L.near_cnt, L.near_off, nl, reinterpret_cast<int64_t*>(t->scan_tmp), s);
-    t->launches += 6;
+    t->launches += 2 * scan_launches(nl);
     if ((rc = ensure_idx(&L.far_idx, &L.far_cap, tf, "far lists"))) return rc;
     if ((rc = ensure_idx(&L.near_idx, &L.near_cap, tn, "near lists"))) return rc;
     if ((rc = launch(ListMode::kTwoPass))) return rc;
