@@ -9,8 +9,8 @@
 // for bit on any device and on the host.
 //
 // Phase A: cells larger than kSubtreeMax are split level by level in global
-//          memory, each cell tiled into 2048-element chunks aligned to the
-//          cell's first particle (chunk sums are the subtrees of the pairwise
+//          memory, each cell tiled into chunks of 2048 (or 512) elements aligned
+//          to the cell's first particle (chunk sums are the subtrees of the pairwise
 //          tree, so the tiling does not change the result).
 // Phase B: a cell of at most kSubtreeMax particles is finished by one CTA with
 //          its particles held in shared memory; each warp splits one cell.
@@ -19,6 +19,7 @@
 // walk, the M2L and the P2P are derived.
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include "kdfmm_internal.cuh"
 
@@ -100,21 +101,19 @@ __device__ void push_child(const BuildArgs& A, Seg c, Seg* nextA, Seg* segB, Seg
 }
 
 // ---------------------------------------------------------------------------
-// phase A
+// phase A: four launches a level.  The chunk kernels run one block per chunk;
+// the last block of a segment to finish (a counter per segment) goes on with
+// the segment's own step -- the cut after the sums, the split after the counts --
+// on all its threads, instead of a launch of one warp per segment (a top cell
+// of 2^24 particles has 8192 chunks).  T threads make chunks of 8 T elements:
+// 64 while large chunks would not reach every SM (small evaluations wait on the
+// float64 pipes of the few SMs that hold a chunk), else 256.  Eight launches a
+// level before: 2^24 clumped particles, all levels, 7.2 ms for the sums, cuts, counts,
+// splits and maps, now 6.3; a 60013-particle sphere, with the scatter, 0.43 ms, now
+// 0.29.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int nchunks_of(int count) { return (count + kChunk - 1) / kChunk; }
-
-// Start of a phase-A level: the segments pushed by the previous level are
-// this level's (counters[C_NA]); the push counter restarts.
-__global__ void k_level_begin(int32_t* counters, int64_t capA, int32_t* status) {
-  int na = counters[C_NEXT_A];
-  if (na > capA) {
-    set_status(status, ST_CAPACITY);
-    na = (int)capA;
-  }
-  counters[C_NA] = na;
-  counters[C_NEXT_A] = 0;
-}
+template <int T>
+__device__ __forceinline__ int nchunks_of(int count) { return (count + 8 * T - 1) / (8 * T); }
 
 // After the last phase-A level: segments still waiting for a split mean the
 // fixed number of levels was too small.
@@ -122,18 +121,30 @@ __global__ void k_levels_done(const int32_t* counters, int32_t* status) {
   if (counters[C_NEXT_A] > 0) set_status(status, ST_UNFINISHED);
 }
 
-// Chunk offsets of the nA segments (single block) and the chunk -> segment map.
-__global__ void k_chunk_map(const Seg* __restrict__ segs, const int32_t* __restrict__ nA_dev, int32_t* __restrict__ seg_off,
-                            int32_t* __restrict__ chunk_seg, int32_t* counters) {
-  const int nA = *nA_dev;
+// Start of a phase-A level (single block): the segments pushed by the previous
+// level are this level's (counters[C_NA]), the push counter restarts; chunk
+// offsets of the segments, the chunk -> segment map, the segments' counters.
+template <int T>
+__global__ void k_level_map(const Seg* __restrict__ segs, int32_t* __restrict__ seg_off,
+                            int32_t* __restrict__ chunk_seg, int32_t* __restrict__ seg_done,
+                            int32_t* counters, int64_t capA, int32_t* status) {
   __shared__ int32_t warp_tot[32];
   __shared__ int32_t carry;
+  int nA = counters[C_NEXT_A];
+  if (nA > capA) {
+    set_status(status, ST_CAPACITY);
+    nA = (int)capA;
+  }
   if (threadIdx.x == 0) carry = 0;
   __syncthreads();
+  if (threadIdx.x == 0) {
+    counters[C_NA] = nA;
+    counters[C_NEXT_A] = 0;
+  }
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int base = 0; base < nA; base += blockDim.x) {
     int s = base + threadIdx.x;
-    int e = s < nA ? nchunks_of(segs[s].count) : 0;
+    int e = s < nA ? nchunks_of<T>(segs[s].count) : 0;
     int incl = e;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -157,52 +168,71 @@ __global__ void k_chunk_map(const Seg* __restrict__ segs, const int32_t* __restr
     __syncthreads();
     if (s < nA) {
       seg_off[s] = excl;
-      for (int c = 0; c < e; ++c) chunk_seg[excl + c] = s;
+      seg_done[2 * s] = seg_done[2 * s + 1] = 0;
     }
     if (threadIdx.x == blockDim.x - 1) carry = excl + e;
+    // the map: a long segment's chunks by the whole block, the others' by their threads
+    if (s < nA && e <= 32)
+      for (int c = 0; c < e; ++c) chunk_seg[excl + c] = s;
+    unsigned big = __ballot_sync(0xffffffffu, e > 32);
+    while (big != 0u) {
+      const int l = __ffs(big) - 1;
+      big &= big - 1u;
+      const int be = __shfl_sync(0xffffffffu, e, l), bx = __shfl_sync(0xffffffffu, excl, l),
+                bs = __shfl_sync(0xffffffffu, s, l);
+      for (int c = lane; c < be; c += 32) chunk_seg[bx + c] = bs;
+    }
     __syncthreads();
   }
-  if (threadIdx.x == 0) counters[4] = carry;
+  if (threadIdx.x == 0) counters[C_CHUNKS] = carry;
 }
 
-// Chunk partial sums (pairwise subtree of kChunk elements) and bounding box keys.
-__global__ void __launch_bounds__(kChunkThreads)
+// True in every thread of the last of `of` blocks to come here (what the
+// others wrote before is visible then).
+__device__ __forceinline__ bool last_block(int32_t* counter, int of) {
+  __shared__ int s_last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(counter, 1) == of - 1;
+  __syncthreads();
+  if (!s_last) return false;
+  __threadfence();
+  return true;
+}
+
+// Chunk partial sums (pairwise subtree of 8 T elements) and bounding box keys;
+// then, once per segment, the pairwise tree over its chunk sums, centre of
+// mass, axis, cut.
+template <int T>
+__global__ void __launch_bounds__(T)
 k_chunk_reduce(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_seg,
                const int32_t* __restrict__ seg_off, const int32_t* __restrict__ counters,
-               PCols p, double* __restrict__ csum, long long* __restrict__ ckey) {
+               PCols p, double* csum, long long* ckey, int32_t* seg_done, TmpCells tmp,
+               int32_t* __restrict__ seg_axis, double* __restrict__ seg_cut, float* __restrict__ seg_xb) {
+  constexpr int kW = T / 32;
   const int b = blockIdx.x;
-  if (b >= counters[4]) return;
+  if (b >= counters[C_CHUNKS]) return;
   const int s = chunk_seg[b];
   const Seg g = segs[s];
-  const int rel0 = (b - seg_off[s]) * kChunk;
+  const int off = seg_off[s];
+  const int rel0 = (b - off) * 8 * T;
   const int cnt = g.count - rel0;               // valid elements from the chunk start
   const int64_t base = (int64_t)g.first + rel0;
-  // the bounding-box keys come with the same loads (get runs once per element)
-  long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
-  auto get = [&](int k) {
-    int64_t i = base + k;
-    const double x = p.x[i], y = p.y[i], z = p.z[i];
-    const long long kx = dkey(x), ky = dkey(y), kz = dkey(z);
-    lo[0] = min(lo[0], kx); hi[0] = max(hi[0], kx);
-    lo[1] = min(lo[1], ky); hi[1] = max(hi[1], ky);
-    lo[2] = min(lo[2], kz); hi[2] = max(hi[2], kz);
-    return elem4(p.m[i], x, y, z);
-  };
-  Sum4 v = block_tree<3>(8 * threadIdx.x, cnt, get);
-  v = warp_tree4(v);
-#pragma unroll
-  for (int d = 0; d < 3; ++d) { lo[d] = warp_min_ll(lo[d]); hi[d] = warp_max_ll(hi[d]); }
-  __shared__ Sum4 ws[kChunkThreads / 32];
-  __shared__ long long wk[kChunkThreads / 32][6];
+  __shared__ Sum4 ws[kW];
+  __shared__ long long wk[kW][6];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (lane == 0) {
-    ws[w] = v;
-    for (int d = 0; d < 3; ++d) { wk[w][d] = lo[d]; wk[w][3 + d] = hi[d]; }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    // perfect tree over the warps' subtrees (the top levels of the chunk's tree)
-    constexpr int kW = kChunkThreads / 32;
+  // block sums and boxes: the warps' subtrees, then (thread 0) the tree over them
+  auto block_reduce = [&](Sum4 v, long long lo[3], long long hi[3], Sum4& total, long long key[6]) {
+    v = warp_tree4(v);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) { lo[d] = warp_min_ll(lo[d]); hi[d] = warp_max_ll(hi[d]); }
+    __syncthreads();
+    if (lane == 0) {
+      ws[w] = v;
+      for (int d = 0; d < 3; ++d) { wk[w][d] = lo[d]; wk[w][3 + d] = hi[d]; }
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     Sum4 t4[kW];
 #pragma unroll
     for (int q = 0; q < kW; ++q) t4[q] = ws[q];
@@ -210,65 +240,81 @@ k_chunk_reduce(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_s
     for (int width = kW; width > 1; width >>= 1)
 #pragma unroll
       for (int q = 0; q < width / 2; ++q) t4[q] = add4(t4[2 * q], t4[2 * q + 1]);
-    const Sum4 t = t4[0];
-    csum[4 * b + 0] = t.m; csum[4 * b + 1] = t.x; csum[4 * b + 2] = t.y; csum[4 * b + 3] = t.z;
+    total = t4[0];
     for (int d = 0; d < 6; ++d) {
       long long r = wk[0][d];
-      for (int q = 1; q < kChunkThreads / 32; ++q) r = d < 3 ? min(r, wk[q][d]) : max(r, wk[q][d]);
-      ckey[6 * b + d] = r;
+      for (int q = 1; q < kW; ++q) r = d < 3 ? min(r, wk[q][d]) : max(r, wk[q][d]);
+      key[d] = r;
+    }
+  };
+  {
+    // the bounding-box keys come with the same loads (get runs once per element)
+    long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
+    auto get = [&](int k) {
+      int64_t i = base + k;
+      const double x = p.x[i], y = p.y[i], z = p.z[i];
+      const long long kx = dkey(x), ky = dkey(y), kz = dkey(z);
+      lo[0] = min(lo[0], kx); hi[0] = max(hi[0], kx);
+      lo[1] = min(lo[1], ky); hi[1] = max(hi[1], ky);
+      lo[2] = min(lo[2], kz); hi[2] = max(hi[2], kz);
+      return elem4(p.m[i], x, y, z);
+    };
+    const Sum4 v = block_tree<3>(8 * threadIdx.x, cnt, get);
+    Sum4 t;
+    long long key[6];
+    block_reduce(v, lo, hi, t, key);
+    if (threadIdx.x == 0) {
+      csum[4 * b + 0] = t.m; csum[4 * b + 1] = t.x; csum[4 * b + 2] = t.y; csum[4 * b + 3] = t.z;
+      for (int d = 0; d < 6; ++d) ckey[6 * b + d] = key[d];
     }
   }
-}
-
-// Warp per segment: pairwise tree over its chunk sums, centre of mass, axis, cut.
-__global__ void k_decide(const Seg* __restrict__ segs, const int32_t* __restrict__ nA_dev, const int32_t* __restrict__ seg_off,
-                         const double* __restrict__ csum, const long long* __restrict__ ckey,
-                         TmpCells tmp, int32_t* __restrict__ seg_axis, double* __restrict__ seg_cut,
-                         float* __restrict__ seg_xb) {
-  const int nA = *nA_dev;
-  const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (s >= nA) return;
-  const Seg g = segs[s];
-  const int C = nchunks_of(g.count);
-  const int off = seg_off[s];
+  const int C = nchunks_of<T>(g.count);
+  if (!last_block(&seg_done[2 * s], C)) return;
+  // the segment: thread t sums its aligned block of B chunks (carry stack)
   int P = 1;
   while (P < C) P <<= 1;
-  const int B = P > 32 ? P >> 5 : 1;
+  const int B = P > T ? P / T : 1;
   auto chunk = [&](int c) {
-    return c < C ? Sum4{csum[4 * (off + c)], csum[4 * (off + c) + 1], csum[4 * (off + c) + 2],
-                        csum[4 * (off + c) + 3]}
-                 : zero4();
+    if (c >= C) return zero4();
+    const double* q = csum + 4 * (int64_t)(off + c);
+    return Sum4{__ldcg(q), __ldcg(q + 1), __ldcg(q + 2), __ldcg(q + 3)};
   };
   Sum4 v;
   if (B == 1) {
-    v = chunk(lane);
+    v = chunk(threadIdx.x);
   } else {
-    // sequential perfect tree over this lane's B chunks (carry stack)
     Sum4 st[16];
     int top = 0;
     for (int k = 0; k < B; ++k) {
-      Sum4 e = chunk(lane * B + k);
+      Sum4 e = chunk(threadIdx.x * B + k);
       for (int kk = k; kk & 1; kk >>= 1) e = add4(st[--top], e);
       st[top++] = e;
     }
     v = st[0];
   }
-  v = warp_tree4(v);
   long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
-  for (int c = lane; c < C; c += 32)
+  for (int c = threadIdx.x; c < C; c += T)
     for (int d = 0; d < 3; ++d) {
-      lo[d] = min(lo[d], ckey[6 * (off + c) + d]);
-      hi[d] = max(hi[d], ckey[6 * (off + c) + 3 + d]);
+      lo[d] = min(lo[d], __ldcg(&ckey[6 * (int64_t)(off + c) + d]));
+      hi[d] = max(hi[d], __ldcg(&ckey[6 * (int64_t)(off + c) + 3 + d]));
     }
-  double dlo[3], dhi[3];
-  for (int d = 0; d < 3; ++d) {
-    dlo[d] = dunkey(warp_min_ll(lo[d]));
-    dhi[d] = dunkey(warp_max_ll(hi[d]));
-  }
+  Sum4 t = zero4();
+  long long key[6] = {0, 0, 0, 0, 0, 0};
+  block_reduce(v, lo, hi, t, key);
+  if (w != 0) return;
+  // the three divisions run once, on lanes 0, 1, 2
+  const double M = __shfl_sync(0xffffffffu, t.m, 0);
+  const double sx = __shfl_sync(0xffffffffu, t.x, 0), sy = __shfl_sync(0xffffffffu, t.y, 0),
+               sz = __shfl_sync(0xffffffffu, t.z, 0);
+  const double quo = __ddiv_rn(lane == 1 ? sy : (lane == 2 ? sz : sx), M);
+  const double cx = __shfl_sync(0xffffffffu, quo, 0), cy = __shfl_sync(0xffffffffu, quo, 1),
+               cz = __shfl_sync(0xffffffffu, quo, 2);
   if (lane == 0) {
-    const double M = v.m;
-    const double cx = __ddiv_rn(v.x, M), cy = __ddiv_rn(v.y, M), cz = __ddiv_rn(v.z, M);
+    double dlo[3], dhi[3];
+    for (int d = 0; d < 3; ++d) {
+      dlo[d] = dunkey(key[d]);
+      dhi[d] = dunkey(key[3 + d]);
+    }
     const int axis = longest_axis(dlo, dhi);
     const int c = g.cell;
     tmp.first[c] = g.first; tmp.count[c] = g.count; tmp.depth[c] = g.dbuf >> 1;
@@ -285,27 +331,34 @@ __global__ void k_decide(const Seg* __restrict__ segs, const int32_t* __restrict
 // Per chunk: particles left of the cut, and the largest float32 estimate of
 // the squared distance to the centre of mass (coordinates truncated to
 // float32 with integer operations; the exact size follows in the scatter).
-__global__ void __launch_bounds__(kChunkThreads)
+// Then, once per segment: offsets of the left particles per chunk, the split
+// point, the size's candidate threshold, and the two children.
+template <int T>
+__global__ void __launch_bounds__(T)
 k_chunk_count(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_seg,
               const int32_t* __restrict__ seg_off, const int32_t* __restrict__ counters, PCols p,
-              TmpCells tmp, const int32_t* __restrict__ seg_axis, const double* __restrict__ seg_cut,
-              int32_t* __restrict__ cleft, float* __restrict__ cs2) {
+              const int32_t* __restrict__ seg_axis, const double* __restrict__ seg_cut,
+              int32_t* cleft, float* cs2, int32_t* seg_done, int32_t* __restrict__ cloff,
+              int32_t* __restrict__ seg_nl, const float* __restrict__ seg_xb,
+              float* __restrict__ seg_thr2, BuildArgs A, Seg* nextA, Seg* segB, Seg* segL, int dst_buf) {
+  constexpr int kW = T / 32;
   const int b = blockIdx.x;
-  if (b >= counters[4]) return;
+  if (b >= counters[C_CHUNKS]) return;
   const int s = chunk_seg[b];
   const Seg g = segs[s];
-  const int rel0 = (b - seg_off[s]) * kChunk;
-  const int cnt = min(kChunk, g.count - rel0);
+  const int off = seg_off[s];
+  const int rel0 = (b - off) * 8 * T;
+  const int cnt = min(8 * T, g.count - rel0);
   const int64_t base = (int64_t)g.first + rel0;
   const int axis = seg_axis[s];
   const long long ckey = dkey(seg_cut[s]);
-  const float cx = trunc_to_float(tmp.cx[g.cell]), cy = trunc_to_float(tmp.cy[g.cell]),
-              cz = trunc_to_float(tmp.cz[g.cell]);
+  const float cx = trunc_to_float(A.tmp.cx[g.cell]), cy = trunc_to_float(A.tmp.cy[g.cell]),
+              cz = trunc_to_float(A.tmp.cz[g.cell]);
   int nl = 0;
   float s2 = 0.0f;
 #pragma unroll
-  for (int pass = 0; pass < kChunk / kChunkThreads; ++pass) {   // all loads in flight
-    const int k = pass * kChunkThreads + threadIdx.x;
+  for (int pass = 0; pass < 8; ++pass) {   // all loads in flight
+    const int k = pass * T + threadIdx.x;
     if (k >= cnt) continue;
     int64_t i = base + k;
     const double px = p.x[i], py = p.y[i], pz = p.z[i];
@@ -314,82 +367,81 @@ k_chunk_count(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_se
     const float dx = trunc_to_float(px) - cx, dy = trunc_to_float(py) - cy, dz = trunc_to_float(pz) - cz;
     s2 = fmaxf(s2, dx * dx + dy * dy + dz * dz);
   }
+  __shared__ int wn[kW];
+  __shared__ float ws2[kW];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     nl += __shfl_xor_sync(0xffffffffu, nl, o);
     s2 = fmaxf(s2, __shfl_xor_sync(0xffffffffu, s2, o));
   }
-  __shared__ int wn[kChunkThreads / 32];
-  __shared__ float ws2[kChunkThreads / 32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (lane == 0) { wn[w] = nl; ws2[w] = s2; }
   __syncthreads();
   if (threadIdx.x == 0) {
     int t = 0;
     float m2 = 0.0f;
-    for (int q = 0; q < kChunkThreads / 32; ++q) { t += wn[q]; m2 = fmaxf(m2, ws2[q]); }
+    for (int q = 0; q < kW; ++q) { t += wn[q]; m2 = fmaxf(m2, ws2[q]); }
     cleft[b] = t;
     cs2[b] = m2;
   }
-}
-
-// Warp per segment: offsets of the left particles per chunk, the split point,
-// s, and the two children.
-__global__ void k_split(const Seg* __restrict__ segs, const int32_t* __restrict__ nA_dev, const int32_t* __restrict__ seg_off,
-                        const int32_t* __restrict__ cleft, const float* __restrict__ cs2,
-                        int32_t* __restrict__ cloff, int32_t* __restrict__ seg_nl,
-                        const float* __restrict__ seg_xb, float* __restrict__ seg_thr2, BuildArgs A,
-                        Seg* nextA, Seg* segB, Seg* segL, int dst_buf) {
-  const int nA = *nA_dev;
-  const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (s >= nA) return;
-  const Seg g = segs[s];
-  const int C = nchunks_of(g.count);
-  const int off = seg_off[s];
+  const int C = nchunks_of<T>(g.count);
+  if (!last_block(&seg_done[2 * s + 1], C)) return;
   int run = 0;
-  float s2 = 0.0f;
-  for (int base = 0; base < C; base += 32) {
-    int c = base + lane;
-    int v = c < C ? cleft[off + c] : 0;
-    if (c < C) s2 = fmaxf(s2, cs2[off + c]);
+  s2 = 0.0f;
+  for (int c0 = 0; c0 < C; c0 += T) {
+    const int c = c0 + threadIdx.x;
+    const int v = c < C ? __ldcg(&cleft[off + c]) : 0;
+    if (c < C) s2 = fmaxf(s2, __ldcg(&cs2[off + c]));
     int incl = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      int w = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += w;
+      int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
     }
-    if (c < C) cloff[off + c] = run + incl - v;
-    run += __shfl_sync(0xffffffffu, incl, 31);
+    __syncthreads();
+    if (lane == 31) wn[w] = incl;
+    __syncthreads();
+    int before = 0, tot = 0;
+#pragma unroll
+    for (int q = 0; q < kW; ++q) {
+      const int u = wn[q];
+      before += q < w ? u : 0;
+      tot += u;
+    }
+    if (c < C) cloff[off + c] = run + before + incl - v;
+    run += tot;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s2 = fmaxf(s2, __shfl_xor_sync(0xffffffffu, s2, o));
-  if (lane != 0) return;
+  if (lane == 0) ws2[w] = s2;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int q = 1; q < kW; ++q) s2 = fmaxf(s2, ws2[q]);
   {
     const float Dm = sqrtf(s2);
     const float thr = Dm - 2.0f * dist_err_bound(seg_xb[s], Dm);
     seg_thr2[s] = thr > 0.0f ? thr * thr * (1.0f - 1e-6f) : -1.0f;
   }
-  int nl = run;
+  nl = run;
   const bool fallback = (nl == 0 || nl == g.count);
   if (fallback) {
     nl = g.count / 2;
-    atomicAdd(&A.counters[5], 1);
+    atomicAdd(&A.counters[C_FALLBACK], 1);
   }
   seg_nl[s] = fallback ? -nl - 1 : nl;
   const int c = g.cell;
-  int cid = atomicAdd(&A.counters[0], 2);
+  int cid = atomicAdd(&A.counters[C_CELLS], 2);
   if (cid + 2 > A.cap_cells) { set_status(A.status, ST_CAPACITY); return; }
   A.tmp.left[c] = cid;
   A.tmp.right[c] = cid + 1;
   const int depth = (g.dbuf >> 1) + 1;
-  atomicMax(&A.counters[6], depth);
+  atomicMax(&A.counters[C_DEPTH], depth);
   push_child(A, Seg{g.first, nl, cid, depth << 1 | dst_buf}, nextA, segB, segL);
   push_child(A, Seg{g.first + nl, g.count - nl, cid + 1, depth << 1 | dst_buf}, nextA, segB, segL);
 }
 
 // Stable scatter of one chunk into the other buffer.  Element k of the chunk
-// (pass k / kChunkThreads, thread k % kChunkThreads) goes to the left child at
+// (pass k / T, thread k % T) goes to the left child at
 // its rank among the segment's left elements, else to the right child.  The
 // flags of all the chunk's elements are taken first (their coordinate loads in
 // flight together), one block barrier publishes the passes' warp counts, and
@@ -397,33 +449,35 @@ __global__ void k_split(const Seg* __restrict__ segs, const int32_t* __restrict_
 // by pass, with two barriers each, the kernel waited on one load at a time:
 // this form took the benchmark's build 3.72 -> 3.56 ms (batches of 1, 2 or 4
 // elements, rolled or unrolled, measured within 1 % of each other).
-constexpr int kScatterPasses = kChunk / kChunkThreads;
-constexpr int kMoveBatch = 2;
-__global__ void __launch_bounds__(kChunkThreads)
+constexpr int kScatterPasses = 8;
+template <int T>
+__global__ void __launch_bounds__(T)
 k_chunk_scatter(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_seg,
                 const int32_t* __restrict__ seg_off, const int32_t* __restrict__ counters, PCols src,
                 PCols dst, const int32_t* __restrict__ seg_axis, const double* __restrict__ seg_cut,
                 const int32_t* __restrict__ cloff, const int32_t* __restrict__ seg_nl,
                 TmpCells tmp, const float* __restrict__ seg_thr2) {
   const int b = blockIdx.x;
-  if (b >= counters[4]) return;
+  if (b >= counters[C_CHUNKS]) return;
   const int s = chunk_seg[b];
   const Seg g = segs[s];
-  const int rel0 = (b - seg_off[s]) * kChunk;
+  const int rel0 = (b - seg_off[s]) * 8 * T;
   const int code = seg_nl[s];
   const bool fallback = code < 0;
   const int nl = fallback ? -code - 1 : code;
   const int axis = seg_axis[s];
+  // small evaluations wait on latency: all the moves of a thread in flight
+  constexpr int kMoveBatch = T == 64 ? 8 : 2;
   const long long ckey = dkey(seg_cut[s]);
-  __shared__ int wcount[kScatterPasses][kChunkThreads / 32];
-  __shared__ long long ws2[kChunkThreads / 32];
+  __shared__ int wcount[kScatterPasses][T / 32];
+  __shared__ long long ws2[T / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   bool flag[kScatterPasses];
   int rank[kScatterPasses];
 #pragma unroll
   for (int pass = 0; pass < kScatterPasses; ++pass) {
-    const int k = rel0 + pass * kChunkThreads + threadIdx.x;   // position within the segment
+    const int k = rel0 + pass * T + threadIdx.x;   // position within the segment
     flag[pass] = false;
     if (k < g.count)
       flag[pass] = fallback ? (k < nl) : (dkey(coord(src, axis, (int64_t)g.first + k)) < ckey);
@@ -440,7 +494,7 @@ k_chunk_scatter(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_
   for (int pass = 0; pass < kScatterPasses; ++pass) {
     int woff = 0, tot = 0;
 #pragma unroll
-    for (int q = 0; q < kChunkThreads / 32; ++q) {
+    for (int q = 0; q < T / 32; ++q) {
       const int c = wcount[pass][q];
       woff += q < w ? c : 0;
       tot += c;
@@ -458,7 +512,7 @@ k_chunk_scatter(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_
     int32_t pi[kMoveBatch];
 #pragma unroll
     for (int u = 0; u < kMoveBatch; ++u) {
-      const int k = rel0 + (p0 + u) * kChunkThreads + threadIdx.x;
+      const int k = rel0 + (p0 + u) * T + threadIdx.x;
       px[u] = py[u] = pz[u] = pm[u] = ph[u] = 0.0;
       pi[u] = 0;
       if (k < g.count) {
@@ -469,7 +523,7 @@ k_chunk_scatter(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_
     }
 #pragma unroll
     for (int u = 0; u < kMoveBatch; ++u) {
-      const int k = rel0 + (p0 + u) * kChunkThreads + threadIdx.x;
+      const int k = rel0 + (p0 + u) * T + threadIdx.x;
       if (k >= g.count) continue;
       const int lb = rank[p0 + u];
       const int64_t d = flag[p0 + u] ? (int64_t)g.first + lb : (int64_t)g.first + nl + (k - lb);
@@ -486,7 +540,7 @@ k_chunk_scatter(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_
   __syncthreads();
   if (threadIdx.x == 0) {
     long long m2 = 0;
-    for (int q = 0; q < kChunkThreads / 32; ++q) m2 = max(m2, ws2[q]);
+    for (int q = 0; q < T / 32; ++q) m2 = max(m2, ws2[q]);
     if (m2 > 0)
       atomicMax(reinterpret_cast<unsigned long long*>(&tmp.s[g.cell]), (unsigned long long)m2);
   }
@@ -1210,7 +1264,7 @@ void free_build_buffers(kdfmm_tree_s* t) {
   for (int k = 0; k < 2; ++k) { free_cols(&t->buf[k]); cudaFree(t->segA[k]); t->segA[k] = nullptr; }
   free_cols(&t->tp);
   void* ptrs[] = {t->segB, t->segL, t->chunk_seg, t->seg_chunk_off, t->chunk_sum, t->chunk_key,
-                  t->chunk_left, t->chunk_loff, t->chunk_s2, t->seg_axis, t->seg_cut, t->seg_nl,
+                  t->chunk_left, t->chunk_loff, t->chunk_s2, t->seg_done, t->seg_axis, t->seg_cut, t->seg_nl,
                   t->seg_xb, t->seg_thr2,
                   t->tmp.first, t->tmp.count, t->tmp.left, t->tmp.right, t->tmp.depth, t->tmp.M,
                   t->tmp.cx, t->tmp.cy, t->tmp.cz, t->tmp.s, t->starts, t->min_depth,
@@ -1221,7 +1275,7 @@ void free_build_buffers(kdfmm_tree_s* t) {
                   t->lexp32};
   for (void* p : ptrs) cudaFree(p);
   t->segB = t->segL = nullptr;
-  t->chunk_seg = t->seg_chunk_off = t->chunk_left = t->chunk_loff = t->seg_axis = t->seg_nl = nullptr;
+  t->chunk_seg = t->seg_chunk_off = t->chunk_left = t->chunk_loff = t->seg_axis = t->seg_nl = t->seg_done = nullptr;
   t->chunk_sum = t->seg_cut = nullptr;
   t->chunk_key = nullptr;
   t->chunk_s2 = t->seg_xb = t->seg_thr2 = nullptr;
@@ -1257,7 +1311,8 @@ static int ensure_build_buffers(kdfmm_tree_s* t, int64_t n) {
   KD_ALLOC(t->segA[1], t->capA);
   KD_ALLOC(t->segB, t->capB);
   KD_ALLOC(t->segL, t->capL);
-  t->cap_chunks = n / kChunk + t->capA + 4;
+  // (a later build of fewer particles may take the small chunks)
+  t->cap_chunks = std::max<int64_t>(n / kChunk, std::min<int64_t>(n, kSmallChunkMax) / (8 * 64)) + t->capA + 4;
   KD_ALLOC(t->chunk_seg, t->cap_chunks);
   KD_ALLOC(t->chunk_sum, 4 * t->cap_chunks);
   KD_ALLOC(t->chunk_key, 6 * t->cap_chunks);
@@ -1265,6 +1320,7 @@ static int ensure_build_buffers(kdfmm_tree_s* t, int64_t n) {
   KD_ALLOC(t->chunk_loff, t->cap_chunks);
   KD_ALLOC(t->chunk_s2, t->cap_chunks);
   KD_ALLOC(t->seg_chunk_off, t->capA);
+  KD_ALLOC(t->seg_done, 2 * t->capA);
   KD_ALLOC(t->seg_axis, t->capA);
   KD_ALLOC(t->seg_cut, t->capA);
   KD_ALLOC(t->seg_nl, t->capA);
@@ -1373,32 +1429,31 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
       return set_error(KDFMM_ERR_NONFINITE, "non-finite position or non-positive mass / h");
   }
   // phase A: cells above kSubtreeMax, one level per pass
-  const unsigned maxc = (unsigned)(n / kChunk + t->capA + 1);
-  const unsigned segw = blocks_for(t->capA * 32, 256);
+  const bool small = n <= kSmallChunkMax;
+  const unsigned maxc = (unsigned)(n / (small ? 8 * 64 : kChunk) + t->capA + 1);
   int cur = 0, level = 0;
+  auto run_level = [&](auto threads, const Seg* segs, Seg* next, int src, int dst) {
+    constexpr int T = decltype(threads)::value;
+    k_level_map<T><<<1, 1024, 0, s>>>(segs, t->seg_chunk_off, t->chunk_seg, t->seg_done, t->counters,
+                                      t->capA, t->status);
+    k_chunk_reduce<T><<<maxc, T, 0, s>>>(segs, t->chunk_seg, t->seg_chunk_off, t->counters, t->buf[src],
+                                         t->chunk_sum, t->chunk_key, t->seg_done, t->tmp, t->seg_axis,
+                                         t->seg_cut, t->seg_xb);
+    k_chunk_count<T><<<maxc, T, 0, s>>>(segs, t->chunk_seg, t->seg_chunk_off, t->counters, t->buf[src],
+                                        t->seg_axis, t->seg_cut, t->chunk_left, t->chunk_s2, t->seg_done,
+                                        t->chunk_loff, t->seg_nl, t->seg_xb, t->seg_thr2, A, next,
+                                        t->segB, t->segL, dst);
+    k_chunk_scatter<T><<<maxc, T, 0, s>>>(segs, t->chunk_seg, t->seg_chunk_off, t->counters, t->buf[src],
+                                          t->buf[dst], t->seg_axis, t->seg_cut, t->chunk_loff, t->seg_nl,
+                                          t->tmp, t->seg_thr2);
+  };
   while (deferred ? level < fixed_levels : hc[C_NEXT_A] > 0) {
     const int src = level & 1, dst = src ^ 1;
     A.src = t->buf[src];
     A.dst = t->buf[dst];
-    const Seg* segs = t->segA[cur];
-    Seg* next = t->segA[cur ^ 1];
-    const int32_t* nA = t->counters + C_NA;
-    k_level_begin<<<1, 1, 0, s>>>(t->counters, t->capA, t->status);
-    k_chunk_map<<<1, 1024, 0, s>>>(segs, nA, t->seg_chunk_off, t->chunk_seg, t->counters);
-    k_chunk_reduce<<<maxc, kChunkThreads, 0, s>>>(segs, t->chunk_seg, t->seg_chunk_off, t->counters,
-                                                  t->buf[src], t->chunk_sum, t->chunk_key);
-    k_decide<<<segw, 256, 0, s>>>(segs, nA, t->seg_chunk_off, t->chunk_sum, t->chunk_key, t->tmp,
-                                  t->seg_axis, t->seg_cut, t->seg_xb);
-    k_chunk_count<<<maxc, kChunkThreads, 0, s>>>(segs, t->chunk_seg, t->seg_chunk_off, t->counters,
-                                                 t->buf[src], t->tmp, t->seg_axis, t->seg_cut,
-                                                 t->chunk_left, t->chunk_s2);
-    k_split<<<segw, 256, 0, s>>>(segs, nA, t->seg_chunk_off, t->chunk_left, t->chunk_s2,
-                                 t->chunk_loff, t->seg_nl, t->seg_xb, t->seg_thr2, A, next, t->segB,
-                                 t->segL, dst);
-    k_chunk_scatter<<<maxc, kChunkThreads, 0, s>>>(segs, t->chunk_seg, t->seg_chunk_off, t->counters,
-                                                   t->buf[src], t->buf[dst], t->seg_axis, t->seg_cut,
-                                                   t->chunk_loff, t->seg_nl, t->tmp, t->seg_thr2);
-    t->launches += 7;
+    if (small) run_level(std::integral_constant<int, 64>{}, t->segA[cur], t->segA[cur ^ 1], src, dst);
+    else run_level(std::integral_constant<int, kChunkThreads>{}, t->segA[cur], t->segA[cur ^ 1], src, dst);
+    t->launches += 4;
     cur ^= 1;
     ++level;
     if (!deferred) {

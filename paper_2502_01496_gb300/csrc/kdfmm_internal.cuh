@@ -15,6 +15,8 @@ namespace kdfmm {
 constexpr int kChunk = 2048;           // phase-A reduction chunk (elements)
 constexpr int kChunkThreads = 256;     // 8 consecutive elements per thread
 static_assert(kChunk == 8 * kChunkThreads, "the chunk reduce sums 8 elements per thread");
+constexpr int kSmallChunkMax = 311296;   // up to here chunks of 512 elements (152 x 2048 elements:
+                                       // one large chunk per SM)
 constexpr int kSubtreeMax = 2048;      // cells this small finish in shared memory
 constexpr int kSubtreeThreads = 256;
 constexpr int kNumStatus = 4;
@@ -155,6 +157,7 @@ struct kdfmm_tree_s {
   float* chunk_s2 = nullptr;         // per chunk: largest float32 squared distance
   float* seg_xb = nullptr;           // per segment: bound on |coordinates|
   float* seg_thr2 = nullptr;         // per segment: candidate threshold for the exact size
+  int32_t* seg_done = nullptr;       // per segment: chunks that finished the reduce, the count
   int32_t* seg_axis = nullptr;
   double* seg_cut = nullptr;
   int32_t* seg_nl = nullptr;
