@@ -186,22 +186,22 @@ struct VjpArgs {
   double* msrc;                         // P2P source-side part of m_bar (N, atomics)
   double* cbar;                         // per leaf: 20 expansion cotangents
   double* cell_bar;                     // per cell: M_bar, com_bar (3), Q_bar (6)
-  // the evaluation's split of long near lists (segment items after the
-  // leaves; their target-side partial sums are added in segment order)
-  const int32_t* counters;
-  const int32_t *seg_first, *seg_leaf;
+  // near lists and transposed near lists are cut into pieces of `entries`:
+  // piece 0 is the leaf's own work item, the others extra items after the leaves
+  // (seg_leaf: their leaf; seg_first: a leaf's first extra item); the targets'
+  // partial sums of the extra items (seg_part) are added in piece order
+  int entries;
+  int32_t *seg_first, *seg_leaf;
   double* seg_part;
   int64_t seg_cap;
-  int seg_entries;
   // transposed near lists: leaf ordinal r is a source of the target leaves
-  // tidx[toff[r] ...) (ordinals), tcnt[r] of them; cut into pieces of
-  // kSrcEntries, piece 0 the leaf's own work item, the others extra items
+  // tidx[toff[r] ...) (ordinals), tcnt[r] of them
   int32_t *tcnt, *tcur, *tidx;
   int64_t* toff;
   int64_t tcap;                         // entries of tidx
-  int32_t *tseg_leaf, *tseg_first;      // per extra item: its leaf; per leaf: its first extra item
+  int32_t *tseg_leaf, *tseg_first;
   int64_t tseg_cap;
-  unsigned long long* tctr;             // [0] entries reserved, [1] extra items
+  unsigned long long* tctr;             // [0] entries reserved, [1] extra source items, [2] extra target items
 };
 
 // A coordinate as x0 + x1 + x2 on the grids 2^(k-22), 2^(k-45) and 2^(k-68) of
@@ -720,23 +720,33 @@ __global__ void __launch_bounds__(kM2LWarps * 32) k_vjp_m2l64(VjpArgs V) {
 // took four float64 atomics per (target leaf, source) and butterflies over
 // the leaf's targets per pair (47 ms of the 2^20 Plummer sphere's adjoint).
 // ---------------------------------------------------------------------------
-constexpr int kSrcEntries = 128;        // target leaves per source work item
+// Extra items of the near lists (any order: a leaf's are contiguous).
+__global__ void k_near_plan(VjpArgs V) {
+  KD_GRID_STRIDE(k, V.nleaves) {
+    const int x = extra_segments(min((int64_t)V.near_cnt[k], V.cap_near), V.entries);
+    const int64_t first = x > 0 ? (int64_t)atomicAdd(&V.tctr[2], (unsigned long long)x) : 0;
+    V.seg_first[k] = (int32_t)first;
+    for (int q = 0; q < x; ++q)
+      if (first + q < V.seg_cap) V.seg_leaf[first + q] = k;
+  }
+}
 
-// The entries of a work item: a leaf's first near segment, or an extra one.
+// The entries of a target item.
+__device__ __forceinline__ int near_items(const VjpArgs& V) {
+  return V.nleaves + (int)min((int64_t)V.tctr[2], V.seg_cap);
+}
 __device__ __forceinline__ int near_item(const VjpArgs& V, int item, int* k, int64_t* e0) {
   const bool seg = item >= V.nleaves;
   const int g = item - V.nleaves;
   *k = seg ? V.seg_leaf[g] : item;
-  if (*k < 0) return 0;
-  const int64_t sidx = seg ? (int64_t)(g - V.seg_first[*k] + 1) : 0;
-  *e0 = V.near_off[*k] + sidx * V.seg_entries;
-  return (int)(min(min((int64_t)V.near_cnt[*k], V.cap_near), (sidx + 1) * V.seg_entries) -
-               sidx * V.seg_entries);
+  const int64_t piece = seg ? (int64_t)(g - V.seg_first[*k] + 1) : 0;
+  *e0 = V.near_off[*k] + piece * V.entries;
+  return (int)(min(min((int64_t)V.near_cnt[*k], V.cap_near), (piece + 1) * V.entries) - piece * V.entries);
 }
 
 __global__ void k_tr_count(VjpArgs V) {
   const int lane = threadIdx.x & 31;
-  const int nitems = V.nleaves + (int)min((int64_t)V.counters[C_SEGS], V.seg_cap);
+  const int nitems = near_items(V);
   for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
        item += (int)((gridDim.x * blockDim.x) >> 5)) {
     int k;
@@ -753,7 +763,7 @@ __global__ void k_tr_plan(VjpArgs V) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r - lane >= V.nleaves) return;
   const int cnt = r < V.nleaves ? V.tcnt[r] : 0;
-  const int extra = cnt > kSrcEntries ? (cnt - 1) / kSrcEntries : 0;
+  const int extra = extra_segments(cnt, V.entries);
   long long ic = cnt;
   int ie = extra;
 #pragma unroll
@@ -779,7 +789,7 @@ __global__ void k_tr_plan(VjpArgs V) {
 
 __global__ void k_tr_fill(VjpArgs V) {
   const int lane = threadIdx.x & 31;
-  const int nitems = V.nleaves + (int)min((int64_t)V.counters[C_SEGS], V.seg_cap);
+  const int nitems = near_items(V);
   for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
        item += (int)((gridDim.x * blockDim.x) >> 5)) {
     int k;
@@ -859,10 +869,48 @@ __device__ __forceinline__ void pair_fg32(float r2, float eps2, float hinv_i, fl
   g = 0.5f * gs;
 }
 
-// The leaves of a batch of up to 32 list entries, one per lane, in shared memory.
-struct LeafBatch {
-  int first[32], count[32];
+// A chunk of list entries in shared memory: up to 32 leaves whose particles fit
+// in kVjpStage records.
+constexpr int kVjpStage = 128;
+struct LeafChunk {
+  float4 p0[kVjpStage], p1[kVjpStage], p2[kVjpStage];
+  int beg[33];                          // staged start of each leaf
+  int first[32];
 };
+// Stages the records of the leading leaves of the entries' cells (cell: this
+// lane's, or -1) that fit; returns their number.  The loads of a batch of rounds
+// are issued before any is used (L2 gathers: latency-bound).
+template <class Put>
+__device__ __forceinline__ int stage_chunk(const VjpArgs& V, LeafChunk& B, int lane, int cell, Put put) {
+  const unsigned full = 0xffffffffu;
+  int cnt = 0;
+  __syncwarp();
+  if (cell >= 0) {
+    cnt = V.c.count[cell];
+    B.first[lane] = V.c.first[cell];
+  }
+  int incl = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int w = __shfl_up_sync(full, incl, o);
+    if (lane >= o) incl += w;
+  }
+  B.beg[lane] = incl - cnt;
+  const int L = __popc(__ballot_sync(full, cell >= 0 && incl <= kVjpStage));
+  if (lane == L - 1) B.beg[L] = incl;
+  __syncwarp();
+  const int total = B.beg[L];
+#pragma unroll 2
+  for (int i = lane; i < total; i += 32) {
+    int l = 0;
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1)
+      if (l + step < L && B.beg[l + step] <= i) l += step;
+    put(i, B.first[l] + i - B.beg[l]);
+  }
+  __syncwarp();
+  return L;
+}
 
 constexpr int kVjpWarps = 4;
 
@@ -877,11 +925,11 @@ constexpr int kVjpWarps = 4;
 // when one kernel walked the pairs by target.
 template <int SOFT>
 __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target32(VjpArgs V) {
-  __shared__ LeafBatch s_batch[kVjpWarps];
+  __shared__ LeafChunk s_chunk[kVjpWarps];
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  LeafBatch& B = s_batch[threadIdx.x >> 5];
-  const int nitems = V.nleaves + (int)min((int64_t)V.counters[C_SEGS], V.seg_cap);
+  LeafChunk& B = s_chunk[threadIdx.x >> 5];
+  const int nitems = near_items(V);
   for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
        item += (int)((gridDim.x * blockDim.x) >> 5)) {
     const bool seg = item >= V.nleaves;
@@ -889,7 +937,6 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target32(VjpArgs V) {
     int k;
     int64_t e0 = 0;
     const int nn = near_item(V, item, &k, &e0);
-    if (k < 0) continue;
     const int a = V.leaf_cells[k];
     const int fa = V.c.first[a], nt = V.c.count[a];
     const int K = 32 / nt, t = lane % nt, sl = lane / nt;
@@ -902,21 +949,21 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target32(VjpArgs V) {
     float eps2 = (float)(eps * eps);
     asm("" : "+f"(eps2));
     float gxh = 0.f, gxl = 0.f, gyh = 0.f, gyl = 0.f, gzh = 0.f, gzl = 0.f;
-    for (int eb = 0; eb < nn; eb += 32) {
-      __syncwarp();
-      if (eb + lane < nn) {
-        const int bc = V.near_idx[e0 + eb + lane];
-        B.first[lane] = V.c.first[bc];
-        B.count[lane] = V.c.count[bc];
-      }
-      __syncwarp();
-      const int m = min(32, nn - eb);
-      for (int q = 0; act && q < m; ++q) {
-        const int fb = B.first[q], nb = B.count[q];
-        for (int j = sl; j < nb; j += K) {
-          const int pj = fb + j;
-          const float4 s0 = V.q0[pj], s1 = V.q1[pj], s2 = V.q2[pj];
-          if (pj == pi) continue;
+    for (int eb = 0; eb < nn;) {
+      const int L = stage_chunk(V, B, lane, eb + lane < nn ? V.near_idx[e0 + eb + lane] : -1,
+                                [&](int at, int pj) {
+                                  B.p0[at] = V.q0[pj];
+                                  B.p1[at] = V.q1[pj];
+                                  float4 s = V.q2[pj];
+                                  s.w = __int_as_float(pj);
+                                  B.p2[at] = s;
+                                });
+      const int total = B.beg[L];
+      if (act) {
+#pragma unroll 2
+        for (int j = sl; j < total; j += K) {
+          const float4 s0 = B.p0[j], s1 = B.p1[j], s2 = B.p2[j];
+          if (__float_as_int(s2.w) == pi) continue;
           const float d0 = grid_diff(o0.x, o1.x, o2.x, s0.x, s1.x, s2.x),
                       d1 = grid_diff(o0.y, o1.y, o2.y, s0.y, s1.y, s2.y),
                       d2 = grid_diff(o0.z, o1.z, o2.z, s0.z, s1.z, s2.z);
@@ -933,6 +980,7 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target32(VjpArgs V) {
           df_add(gzh, gzl, __fmul_rn(s0.w, jz));
         }
       }
+      eb += L;
     }
     double gx = (double)gxh + (double)gxl, gy = (double)gyh + (double)gyl,
            gz = (double)gzh + (double)gzl;
@@ -962,10 +1010,11 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target32(VjpArgs V) {
 // low) float32 pair; one float64 atomic per source and item at the end.
 template <int SOFT>
 __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source32(VjpArgs V) {
-  __shared__ LeafBatch s_batch[kVjpWarps];
+  __shared__ float2 s_b[kVjpWarps][kVjpStage];
+  __shared__ LeafChunk s_chunk[kVjpWarps];
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  LeafBatch& B = s_batch[threadIdx.x >> 5];
+  LeafChunk& B = s_chunk[threadIdx.x >> 5];
   const int nitems = V.nleaves + (int)min((int64_t)V.tctr[1], V.tseg_cap);
   for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
        item += (int)((gridDim.x * blockDim.x) >> 5)) {
@@ -983,30 +1032,31 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source32(VjpArgs V) {
     float eps2 = (float)(eps * eps);
     asm("" : "+f"(eps2));
     float sh[4] = {0.f, 0.f, 0.f, 0.f}, slo[4] = {0.f, 0.f, 0.f, 0.f};
-    const int64_t e0 = V.toff[r] + (int64_t)piece * kSrcEntries;
-    const int nn = min(V.tcnt[r] - piece * kSrcEntries, kSrcEntries);
-    for (int eb = 0; eb < nn; eb += 32) {
-      __syncwarp();
-      if (eb + lane < nn) {
-        const int bc = V.leaf_cells[V.tidx[e0 + eb + lane]];
-        B.first[lane] = V.c.first[bc];
-        B.count[lane] = V.c.count[bc];
-      }
-      __syncwarp();
-      const int m = min(32, nn - eb);
-      if (!act) continue;
-      for (int q = sl; q < m; q += K) {
-        const int fb = B.first[q], nb = B.count[q];
+    const int64_t e0 = V.toff[r] + (int64_t)piece * V.entries;
+    const int nn = min(V.tcnt[r] - piece * V.entries, V.entries);
+    for (int eb = 0; eb < nn;) {
+      const int L = stage_chunk(V, B, lane, eb + lane < nn ? V.leaf_cells[V.tidx[e0 + eb + lane]] : -1,
+                                [&](int at, int pi) {
+                                  float4 s = V.q0[pi];
+                                  const float2 b = V.q3[pi];
+                                  s.w = __int_as_float(pi);
+                                  B.p0[at] = s;
+                                  B.p1[at] = V.q1[pi];
+                                  B.p2[at] = V.q2[pi];
+                                  s_b[threadIdx.x >> 5][at] = b;
+                                });
+      for (int q = sl; act && q < L; q += K) {
+        const int fb = B.beg[q], nb = B.beg[q + 1] - fb;
         float h1[4], h2[4], h3[4], acc[4];
         for (int i0 = 0; i0 < nb; i0 += 4) {
           float s[4][4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            const int pi = fb + i0 + u;
+            const int at = fb + i0 + u;
             s[u][0] = s[u][1] = s[u][2] = s[u][3] = 0.0f;
-            if (i0 + u < nb && pi != pj) {
-              const float4 t0 = V.q0[pi], t1 = V.q1[pi], t2 = V.q2[pi];
-              const float2 t3 = V.q3[pi];
+            if (i0 + u < nb && __float_as_int(B.p0[at].w) != pj) {
+              const float4 t0 = B.p0[at], t1 = B.p1[at], t2 = B.p2[at];
+              const float2 t3 = s_b[threadIdx.x >> 5][at];
               const float3 b = make_float3(t2.w, t3.x, t3.y);
               const float d0 = grid_diff(t0.x, t1.x, t2.x, o0.x, o1.x, o2.x),
                           d1 = grid_diff(t0.y, t1.y, t2.y, o0.y, o1.y, o2.y),
@@ -1056,6 +1106,7 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source32(VjpArgs V) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) df_add(sh[c], slo[c], acc[c]);
       }
+      eb += L;
     }
     double g[4];
 #pragma unroll
@@ -1112,7 +1163,7 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target64(VjpArgs V) {
   constexpr bool M4 = SOFT == KDFMM_SOFT_M4;
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int nitems = V.nleaves + (int)min((int64_t)V.counters[C_SEGS], V.seg_cap);
+  const int nitems = near_items(V);
   for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
        item += (int)((gridDim.x * blockDim.x) >> 5)) {
     const bool seg = item >= V.nleaves;
@@ -1120,7 +1171,6 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target64(VjpArgs V) {
     int k;
     int64_t e0 = 0;
     const int nn = near_item(V, item, &k, &e0);
-    if (k < 0) continue;
     const int a = V.leaf_cells[k];
     const int fa = V.c.first[a], nt = V.c.count[a];
     const int K = 32 / nt, t = lane % nt, sl = lane / nt;
@@ -1205,8 +1255,8 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source64(VjpArgs V) {
     const double hinv_j = M4 ? V.hinv[pj] : 0.0;
     const double eps = V.sys_eps[V.leaf_sys[r]], eps2 = M4 ? 0.0 : eps * eps;
     double g[4] = {0.0, 0.0, 0.0, 0.0};
-    const int64_t e0 = V.toff[r] + (int64_t)piece * kSrcEntries;
-    const int nn = min(V.tcnt[r] - piece * kSrcEntries, kSrcEntries);
+    const int64_t e0 = V.toff[r] + (int64_t)piece * V.entries;
+    const int nn = min(V.tcnt[r] - piece * V.entries, V.entries);
     for (int e = 0; act && e < nn; ++e) {
       const int bc = V.leaf_cells[V.tidx[e0 + e]];
       const int fb = V.c.first[bc], nb = V.c.count[bc];
@@ -1263,16 +1313,15 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source64(VjpArgs V) {
 // warp of its first extra segment), lane per target, in segment order.
 __global__ void k_vjp_seg_combine(VjpArgs V) {
   const int lane = threadIdx.x & 31;
-  const int nseg = (int)min((int64_t)V.counters[C_SEGS], V.seg_cap);
+  const int nseg = (int)min((int64_t)V.tctr[2], V.seg_cap);
   for (int g = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); g < nseg;
        g += (int)((gridDim.x * blockDim.x) >> 5)) {
     const int k = V.seg_leaf[g];
-    if (k < 0) continue;
     const int f = V.seg_first[k];
     if (g != f) continue;
     const int a = V.leaf_cells[k];
     if (lane >= V.c.count[a]) continue;
-    const int x = extra_segments(min((int64_t)V.near_cnt[k], V.cap_near), V.seg_entries);
+    const int x = extra_segments(min((int64_t)V.near_cnt[k], V.cap_near), V.entries);
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
     for (int q = 0; q < x; ++q) {
       const double* P = V.seg_part + (int64_t)(f + q) * 128 + 4 * lane;
@@ -1377,14 +1426,12 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
   V.far_off = t->L.far_off; V.near_off = t->L.near_off;
   V.cap_far = t->L.exact ? INT64_MAX : t->L.cap_far;
   V.cap_near = t->L.exact ? INT64_MAX : t->L.cap_near;
-  V.counters = t->counters;
-  V.seg_first = t->L.seg_first;
-  V.seg_leaf = t->L.seg_leaf;
-  V.seg_part = t->L.seg_part;
-  V.seg_cap = t->L.seg_cap;
-  V.seg_entries = t->L.seg_entries;
+  // pieces short enough for a dozen warps on each of the SMs' four schedulers,
+  // between 8 and 256 leaves
+  V.entries = 256;
+  while (V.entries > 8 && nnear / V.entries < (int64_t)sm_count() * 48) V.entries >>= 1;
   V.tcap = nnear;
-  V.tseg_cap = nnear / kSrcEntries + 1;
+  V.seg_cap = V.tseg_cap = nnear / V.entries + 1;
   // scratch, in two parts: what starts at zero first (one memset), then the
   // rest; every array on a 16-byte boundary
   size_t at = 0, zeroed = 0;
@@ -1395,11 +1442,13 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
   };
   const size_t o_cell = take((size_t)nc * 10 * 8), o_xsrc = take((size_t)n * 3 * 8),
                o_msrc = take((size_t)n * 8), o_mbar = take((size_t)n * 8),
-               o_tcnt = take((size_t)nl * 4), o_tcur = take((size_t)nl * 4), o_tctr = take(16);
+               o_tcnt = take((size_t)nl * 4), o_tcur = take((size_t)nl * 4), o_tctr = take(32);
   zeroed = at;
   const size_t o_xbar = take((size_t)n * 3 * 8), o_cbar = take((size_t)nl * 20 * 8),
                o_toff = take((size_t)nl * 8), o_tfirst = take((size_t)nl * 4),
-               o_tidx = take((size_t)nnear * 4), o_tseg = take((size_t)V.tseg_cap * 4);
+               o_tidx = take((size_t)nnear * 4), o_tseg = take((size_t)V.tseg_cap * 4),
+               o_nfirst = take((size_t)nl * 4), o_nseg = take((size_t)V.seg_cap * 4),
+               o_npart = take((size_t)V.seg_cap * 128 * 8);
   const size_t o_q = V.mixed ? take((size_t)n * 56) : take((size_t)n * 32);
   // a call that is being captured takes its scratch from the stream's pool (a
   // graph must not refer to memory that the handle may replace)
@@ -1424,6 +1473,9 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
   V.tseg_first = (int32_t*)(buf + o_tfirst);
   V.tidx = (int32_t*)(buf + o_tidx);
   V.tseg_leaf = (int32_t*)(buf + o_tseg);
+  V.seg_first = (int32_t*)(buf + o_nfirst);
+  V.seg_leaf = (int32_t*)(buf + o_nseg);
+  V.seg_part = (double*)(buf + o_npart);
   V.q0 = (float4*)(buf + o_q);
   V.q1 = V.q0 + n;
   V.q2 = V.q1 + n;
@@ -1433,6 +1485,7 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
   cudaMemsetAsync(buf, 0, zeroed, s);
   const bool m4 = t->p.soft_kind == KDFMM_SOFT_M4;
   const unsigned gw = blocks_for((int64_t)nl * 32, 128);
+  const unsigned gi = blocks_for((nl + V.seg_cap) * 32, 128);    // a warp per item that there may be
   k_vjp_l2p<<<gw, kL2PWarps * 32, 0, s>>>(a_bar, V, m4);
   const bool std_exp = t->p.expansion == KDFMM_EXPANSION_STANDARD;
   if (V.mixed) {
@@ -1442,30 +1495,31 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
     if (std_exp) k_vjp_m2l64<true><<<gw, kM2LWarps * 32, 0, s>>>(V);
     else k_vjp_m2l64<false><<<gw, kM2LWarps * 32, 0, s>>>(V);
   }
+  k_near_plan<<<std::min<unsigned>(blocks_for(nl, 128), grid_blocks()), 128, 0, s>>>(V);
   k_tr_count<<<grid_blocks(), 256, 0, s>>>(V);
   k_tr_plan<<<blocks_for(nl, 128), 128, 0, s>>>(V);
   k_tr_fill<<<grid_blocks(), 256, 0, s>>>(V);
   if (V.mixed) {
     if (m4) {
-      k_vjp_target32<KDFMM_SOFT_M4><<<gw, kVjpWarps * 32, 0, s>>>(V);
-      k_vjp_source32<KDFMM_SOFT_M4><<<gw, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_target32<KDFMM_SOFT_M4><<<gi, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_source32<KDFMM_SOFT_M4><<<gi, kVjpWarps * 32, 0, s>>>(V);
     } else {
-      k_vjp_target32<KDFMM_SOFT_PLUMMER><<<gw, kVjpWarps * 32, 0, s>>>(V);
-      k_vjp_source32<KDFMM_SOFT_PLUMMER><<<gw, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_target32<KDFMM_SOFT_PLUMMER><<<gi, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_source32<KDFMM_SOFT_PLUMMER><<<gi, kVjpWarps * 32, 0, s>>>(V);
     }
   } else {
     if (m4) {
-      k_vjp_target64<KDFMM_SOFT_M4><<<gw, kVjpWarps * 32, 0, s>>>(V);
-      k_vjp_source64<KDFMM_SOFT_M4><<<gw, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_target64<KDFMM_SOFT_M4><<<gi, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_source64<KDFMM_SOFT_M4><<<gi, kVjpWarps * 32, 0, s>>>(V);
     } else {
-      k_vjp_target64<KDFMM_SOFT_PLUMMER><<<gw, kVjpWarps * 32, 0, s>>>(V);
-      k_vjp_source64<KDFMM_SOFT_PLUMMER><<<gw, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_target64<KDFMM_SOFT_PLUMMER><<<gi, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_source64<KDFMM_SOFT_PLUMMER><<<gi, kVjpWarps * 32, 0, s>>>(V);
     }
   }
   k_vjp_seg_combine<<<grid_blocks(2), 256, 0, s>>>(V);
   k_vjp_moments<<<blocks_for(nl, 128), 128, 0, s>>>(V);
   k_scatter_bar<<<blocks_for(n, 256), 256, 0, s>>>(V, x_bar, m_bar);
-  t->launches += 10;
+  t->launches += 11;
   rc = check_cuda(cudaGetLastError(), "adjoint launch");
   if (pooled) cudaFreeAsync(buf, s);
   return rc;
