@@ -42,8 +42,6 @@ template <class T>
 __device__ __forceinline__ T rsqrt_t(T v);
 template <>
 __device__ __forceinline__ float rsqrt_t<float>(float v) { return rsqrtf(v); }
-template <>
-__device__ __forceinline__ double rsqrt_t<double>(double v) { return rsqrt(v); }
 
 // Error-free transforms (float32): a * b = p + e exactly (FMA), and the
 // float-float monopole of a far cell: C0 = -M / R and C1 = M R / R^3 as
@@ -267,8 +265,21 @@ __global__ void __launch_bounds__(128) k_m2l_mixed(M2LArgs A) {
   }
 }
 
+// FP64 mode.  Bound by the float64 pipe (1/64 rate), so written for few
+// operations, about 130 a pair where the generic coefficients took 260:
+// the potential is harmonic, so C2 and C3 are traceless and 16 sums (C0; C1;
+// C2 xx xy xz yy yz; C3 xxx xxy xxz xyy xyz yyy yyz) give all 20 coefficients;
+// with h_n = g0^(2n+1) (g_n up to its integer factor), v = s3 R / 3 + t4 u,
+// w = s2 R / 2 + t3 u and p = s2 R + t3 u,
+//   C2_ab = R_a w_b + R_b w_a + t2 Q_ab + s1 d_ab,
+//   C3_abc = R_b R_c v_a + R_a R_c v_b + R_a R_b v_c
+//          + t3 (R_a Q_bc + R_b Q_ac + R_c Q_ab) + d_ab p_c + d_ac p_b + d_bc p_a,
+// each product added to its sum directly.  The lanes' sums are scattered over
+// lanes 0..15 (16 float64 additions a leaf instead of a butterfly's 100).
+// Binary of 2 x 2^20, 6.7e7 pairs: 33 ms, now 16.0; 32770 at theta 0.3 0.65, now 0.30.
 template <bool STD>
-__global__ void __launch_bounds__(256) k_m2l_fp64(M2LArgs A) {
+__global__ void __launch_bounds__(128) k_m2l_fp64(M2LArgs A) {
+  const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int nleaves = A.nsinks > 0 ? A.nsinks : min(A.counters[C_LEAVES], A.max_leaves);
   for (int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); k < nleaves;
@@ -276,30 +287,97 @@ __global__ void __launch_bounds__(256) k_m2l_fp64(M2LArgs A) {
   const int a = A.nsinks > 0 ? k : A.leaf_cells[k];
   const double* sa = A.src64 + 10 * (int64_t)a;
   const double ax = sa[0], ay = sa[1], az = sa[2];
-  double acc[20];
+  // acc: C0, C1 x y z, C2 xx xy xz yy yz, C3 xxx/3 xxy xxz xyy xyz yyy/3 yyz
+  double acc[16];
 #pragma unroll
-  for (int j = 0; j < 20; ++j) acc[j] = 0.0;
+  for (int j = 0; j < 16; ++j) acc[j] = 0.0;
   const int64_t off = A.far_off[k], nf = min((int64_t)A.far_cnt[k], A.cap_far);
   for (int64_t e = lane; e < nf; e += 32) {
     const int b = A.far_idx[off + e];
     const double* sb = A.src64 + 10 * (int64_t)b;
-    double C[20];
-    m2l_coeffs<double, STD>(ax - sb[0], ay - sb[1], az - sb[2], sb[3], sb + 4, C);
-#pragma unroll
-    for (int j = 0; j < 20; ++j) acc[j] += C[j];
+    const double x = ax - sb[0], y = ay - sb[1], z = az - sb[2], M = sb[3];
+    const double xx_ = sb[4], xy_ = sb[5], xz_ = sb[6], yy_ = sb[7], yz_ = sb[8], zz_ = sb[9];
+    const double h0 = rsqrt64(fma(z, z, fma(y, y, x * x)));
+    const double i2 = h0 * h0, h1 = h0 * i2, h2 = h1 * i2, h3 = h2 * i2;
+    const double ux = fma(xz_, z, fma(xy_, y, xx_ * x)), uy = fma(yz_, z, fma(yy_, y, xy_ * x)),
+                 uz = fma(zz_, z, fma(yz_, y, xz_ * x));
+    const double q = 0.5 * fma(uz, z, fma(uy, y, ux * x));
+    // s_n = -M g_n - g_(n+2) q / 6 and t_n = -g_n / 3 in terms of h_n (q halved)
+    const double M1 = M * h1;
+    acc[0] -= fma(q, h2, M * h0);
+    const double s1 = fma(5.0 * q, h3, M1), t2 = -h2;
+    acc[1] = fma(s1, x, fma(t2, ux, acc[1]));
+    acc[2] = fma(s1, y, fma(t2, uy, acc[2]));
+    acc[3] = fma(s1, z, fma(t2, uz, acc[3]));
+    const double M3 = -3.0 * (M * h2);
+    if (STD) {
+      const double s2 = M3, s3 = 15.0 * (M * h3);
+      const double wx = s2 * x, wy = s2 * y;
+      acc[4] += fma(wx, x, M1);
+      acc[5] = fma(wx, y, acc[5]);
+      acc[6] = fma(wx, z, acc[6]);
+      acc[7] += fma(wy, y, M1);
+      acc[8] = fma(wy, z, acc[8]);
+      const double vx = s3 * (x * x), vy = s3 * (y * y), xy = s3 * (x * y), s2z = s2 * z;
+      acc[9] = fma(vx, x * (1.0 / 3.0), acc[9] + wx);
+      acc[10] = fma(vx, y, acc[10] + wy);
+      acc[11] = fma(vx, z, acc[11] + s2z);
+      acc[12] = fma(vy, x, acc[12] + wx);
+      acc[13] = fma(xy, z, acc[13]);
+      acc[14] = fma(vy, y * (1.0 / 3.0), acc[14] + wy);
+      acc[15] = fma(vy, z, acc[15] + s2z);
+    } else {
+      const double h4 = h3 * i2, h5 = h4 * i2;
+      const double s2 = fma(-35.0 * q, h4, M3);
+      const double s3 = fma(105.0 * q, h5, 5.0 * (M * h3));          // a third of s3
+      const double t3 = 5.0 * h3, t4 = -35.0 * h4;
+      // p = s2 R + t3 u, w = p - s2 R / 2
+      const double tx = t3 * ux, ty = t3 * uy, tz = t3 * uz;
+      const double px = fma(s2, x, tx), py = fma(s2, y, ty), pz = fma(s2, z, tz);
+      const double hs = 0.5 * s2;
+      const double wx = fma(hs, x, tx), wy = fma(hs, y, ty), wz = fma(hs, z, tz);
+      const double x2 = x + x, y2 = y + y;
+      acc[4] = fma(x2, wx, fma(t2, xx_, acc[4] + s1));
+      acc[5] = fma(x, wy, fma(y, wx, fma(t2, xy_, acc[5])));
+      acc[6] = fma(x, wz, fma(z, wx, fma(t2, xz_, acc[6])));
+      acc[7] = fma(y2, wy, fma(t2, yy_, acc[7] + s1));
+      acc[8] = fma(y, wz, fma(z, wy, fma(t2, yz_, acc[8])));
+      const double vx = fma(s3, x, t4 * ux), vy = fma(s3, y, t4 * uy), vz = fma(s3, z, t4 * uz);
+      const double rx = t3 * x, ry = t3 * y, rz = t3 * z;
+      const double xx = x * x, xy = x * y, xz = x * z, yy = y * y, yz = y * z;
+      const double vx2 = vx + vx, vy2 = vy + vy, rx2 = rx + rx, ry2 = ry + ry;
+      acc[9] = fma(vx, xx, fma(rx, xx_, acc[9] + px));
+      acc[10] = fma(vx2, xy, fma(rx2, xy_, fma(vy, xx, fma(ry, xx_, acc[10] + py))));
+      acc[11] = fma(vx2, xz, fma(rx2, xz_, fma(vz, xx, fma(rz, xx_, acc[11] + pz))));
+      acc[12] = fma(vy2, xy, fma(ry2, xy_, fma(vx, yy, fma(rx, yy_, acc[12] + px))));
+      acc[13] = fma(vx, yz, fma(vy, xz, fma(vz, xy, fma(rx, yz_, fma(ry, xz_, fma(rz, xy_, acc[13]))))));
+      acc[14] = fma(vy, yy, fma(ry, yy_, acc[14] + py));
+      acc[15] = fma(vy2, yz, fma(ry2, yz_, fma(vz, yy, fma(rz, yy_, acc[15] + pz))));
+    }
   }
+  // reduce-scatter over the lane bits 3..0 (lane l keeps sum l & 15), then the
+  // two halves of the warp
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
+  for (int o = 8; o > 0; o >>= 1) {
+    const bool up = (lane & o) != 0;
 #pragma unroll
-    for (int j = 0; j < 20; ++j) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], o);
+    for (int i = 0; i < o; ++i) {
+      const double send = up ? acc[i] : acc[i + o], keep = up ? acc[i + o] : acc[i];
+      acc[i] = keep + __shfl_xor_sync(full, send, o);
+    }
   }
-  double* out = A.lexp64 + 20 * (int64_t)k;
-  if (lane < 20) {
-    double v = acc[0];
+  double v = acc[0] + __shfl_xor_sync(full, acc[0], 16);
+  const int own = lane & 15;
+  if (own == 9 || own == 14) v *= 3.0;
+  // coefficient j from the sums: itself, or minus two others (traces vanish)
+  constexpr int kOne[20] = {0, 1, 2, 3, 4, 5, 6, 7, 8, 4, 9, 10, 11, 12, 13, 9, 14, 15, 10, 11};
+  constexpr int kTwo[20] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, 7, -1, -1, -1, -1, -1, 12, -1, -1, 14, 15};
+  int one = 0, two = -1;
 #pragma unroll
-    for (int j = 1; j < 20; ++j) v = lane == j ? acc[j] : v;
-    out[lane] = v;
-  }
+  for (int j = 0; j < 20; ++j)
+    if (lane == j) { one = kOne[j]; two = kTwo[j]; }
+  const double c1 = __shfl_sync(full, v, one), c2 = __shfl_sync(full, v, two < 0 ? 0 : two);
+  if (lane < 20) A.lexp64[20 * (int64_t)k + lane] = two < 0 ? c1 : -(c1 + c2);
   }
 }
 
@@ -320,15 +398,14 @@ int run_m2l(kdfmm_tree_s* t, cudaStream_t s) {
   A.src64 = t->c.src64;
   A.lexp32 = t->lexp32;
   A.lexp64 = t->lexp64;
-  const unsigned g = blocks_for((int64_t)std::max(t->grid_leaves, 1) * 32, 256);
   const unsigned gm = blocks_for((int64_t)std::max(t->grid_leaves, 1) * 32, 128);
   const bool std_exp = t->p.expansion == KDFMM_EXPANSION_STANDARD;
   if (t->p.precision == KDFMM_MIXED) {
     if (std_exp) k_m2l_mixed<true><<<gm, 128, 0, s>>>(A);
     else k_m2l_mixed<false><<<gm, 128, 0, s>>>(A);
   } else {
-    if (std_exp) k_m2l_fp64<true><<<g, 256, 0, s>>>(A);
-    else k_m2l_fp64<false><<<g, 256, 0, s>>>(A);
+    if (std_exp) k_m2l_fp64<true><<<gm, 128, 0, s>>>(A);
+    else k_m2l_fp64<false><<<gm, 128, 0, s>>>(A);
   }
   t->launches += 1;
   return check_cuda(cudaGetLastError(), "m2l launch");
@@ -352,15 +429,14 @@ int run_m2l_cells(kdfmm_tree_s* t, const int32_t* far_cnt, const int64_t* far_of
   A.src64 = t->c.src64;
   A.lexp32 = out32;
   A.lexp64 = out64;
-  const unsigned g = blocks_for((int64_t)std::max(t->ncells, 1) * 32, 256);
   const unsigned gm = blocks_for((int64_t)std::max(t->ncells, 1) * 32, 128);
   const bool std_exp = t->p.expansion == KDFMM_EXPANSION_STANDARD;
   if (t->p.precision == KDFMM_MIXED) {
     if (std_exp) k_m2l_mixed<true><<<gm, 128, 0, s>>>(A);
     else k_m2l_mixed<false><<<gm, 128, 0, s>>>(A);
   } else {
-    if (std_exp) k_m2l_fp64<true><<<g, 256, 0, s>>>(A);
-    else k_m2l_fp64<false><<<g, 256, 0, s>>>(A);
+    if (std_exp) k_m2l_fp64<true><<<gm, 128, 0, s>>>(A);
+    else k_m2l_fp64<false><<<gm, 128, 0, s>>>(A);
   }
   t->launches += 1;
   return check_cuda(cudaGetLastError(), "m2l (cells) launch");

@@ -447,32 +447,27 @@ __global__ void __launch_bounds__(kP2PWarps * 32, 6) k_p2p_mixed(P2PArgs A) {
   }
 }
 
-constexpr int kStage64 = 128;      // staged sources per warp and chunk (float64 path)
+constexpr int kStage64 = 256;      // staged sources per warp and chunk (float64 path)
 constexpr int kP2P64Warps = 4;
 
-// Force over distance and potential of the symmetrised M4 pair (Eq. 13) in
-// float64; hinv and h3inv = 1/h and 1/h^3 of each side.  Branches of q >= 1 as
-// in m4_side (t = 0 outside the support).
-__device__ __forceinline__ void m4pair64(double r2, double hinv_i, double h3inv_i, double hinv_j,
-                                         double& f, double& p) {
-  const double inv = rsqrt64(r2);
-  const double r = r2 * inv, inv3 = inv * inv * inv;
-  f = p = 0.0;
-#pragma unroll
-  for (int side = 0; side < 2; ++side) {
-    const double hinv = side ? hinv_j : hinv_i, q = r * hinv;
-    if (q < 1.0) {
-      const double q2 = q * q, h3inv = side ? hinv * hinv * hinv : h3inv_i;
-      f = fma(fma(q2, fma(0.5, q, -1.2), 4.0 / 3.0), h3inv, f);
-      p = fma(fma(q2, fma(q2, fma(-0.1, q, 0.3), -2.0 / 3.0), 1.4), hinv, p);
-    } else {
-      const double t = fmax(2.0 - q, 0.0), t2 = t * t, t4 = t2 * t2;
-      f = fma(fma(-t4, fma(t, fma(t, 1.0 / 6.0, -0.8), 1.0), 1.0), inv3, f);
-      p = fma(fma(-t4 * t, fma(t, -1.0 / 30.0, 0.1), 1.0), inv, p);
-    }
-  }
-  f *= 0.5;
-  p *= 0.5;
+// One side of the symmetrised M4 pair in float64, added to f (force over
+// distance) and p (potential): the polynomials of m4_side, for q < 1 in v = q and
+// else in v = 2 - q (0 outside the support), as one evaluation
+//   f += (A + w (B + v (C + v D))) h^-3 or r^-3,   w = q^2 or t^4,
+// whose constants are selected (integer instructions): 13 float64 operations,
+// where a warp whose lanes take both branches runs 20.
+__device__ __forceinline__ void m4_side64(double r, double inv, double inv3, double hinv, double h3inv,
+                                          double& f, double& p) {
+  const double q = r * hinv;
+  const bool in = __double2hiint(q) < 0x3ff00000;            // q < 1 (q >= 0)
+  const double t = 2.0 - q;
+  const double tp = __double2hiint(t) < 0 ? 0.0 : t;
+  const double v = in ? q : tp, v2 = v * v, v4 = v2 * v2, w = in ? v2 : v4;
+  const double f1 = fma(v, fma(v, in ? 0.0 : -1.0 / 6.0, in ? 0.5 : 0.8), in ? -1.2 : -1.0);
+  f = fma(fma(w, f1, in ? 4.0 / 3.0 : 1.0), in ? h3inv : inv3, f);
+  const double p1 = fma(v, fma(v, fma(v, in ? -0.1 : 0.0, in ? 0.3 : 1.0 / 30.0), in ? 0.0 : -0.1),
+                        in ? -2.0 / 3.0 : 0.0);
+  p = fma(fma(w, p1, in ? 1.4 : 1.0), in ? hinv : inv, p);
 }
 
 // Float64 mode: lanes = (target, source slice) as K = 32 / n_t slices;
@@ -485,8 +480,8 @@ __device__ __forceinline__ void m4pair64(double r2, double hinv_i, double h3inv_
 // ones: a 1/r^2 pair takes 17 of them (3 differences, 3 for r^2, 4 for 1/r
 // (rsqrt64), 4 for m/r and m/r^3, 3 for the force), the tests of the kernel
 // supports are float32.  With the library's rsqrt, float64 tests and divisions
-// per kernel pair it was ~45 (M4 binary of 2 x 2^20: 133 ms, now 98; Plummer
-// sphere of 4096: 1.42 ms in long segments, now 0.29).
+// per kernel pair it was ~45 (M4 binary of 2 x 2^20: 133 ms, now 91; Plummer
+// sphere of 4096: 1.42 ms in long segments, now 0.3).
 template <int SOFT>
 __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
   constexpr bool M4 = SOFT == KDFMM_SOFT_M4;
@@ -536,38 +531,50 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
       sh2[at] = A.ph[src].w;
     }
   };
-  // the lane's slice of the staged sources but `skip`.  M4, 32 sources of the
+  // the lane's slice of the staged sources but `skip`.  M4, 128 sources of the
   // slice at a time: every pair as 1/r^2 except those that may lie inside
   // either support, which are marked and follow with the kernel (a warp
   // branching per pair ran the kernel path for all its lanes whenever one
-  // needed it)
+  // needed it; the longer the stretch, the more alike the lanes' marks)
   auto sum_staged = [&](int total, int skip) {
-    for (int j0 = sl; j0 < total; j0 += 32 * K) {
-      uint32_t in = 0u;
-      for (int b = 0; b < 32; ++b) {
-        const int j = j0 + b * K;
-        if (j >= total) break;
-        if (j == skip) continue;
-        const double rx = xi - sx[j], ry = yi - sy[j], rz = zi - sz[j];
-        const double r2 = fma(rz, rz, fma(ry, ry, fma(rx, rx, soft2)));
-        if (M4 && maybe_inside(r2, h2i, sh2[j])) {
-          in |= 1u << b;
-          continue;
+    for (int j0 = sl; j0 < total; j0 += 128 * K) {
+      uint32_t in[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        for (int b = 0; b < 32; ++b) {
+          const int j = j0 + (32 * w + b) * K;
+          if (j >= total) break;
+          if (j == skip) continue;
+          const double rx = xi - sx[j], ry = yi - sy[j], rz = zi - sz[j];
+          const double r2 = fma(rz, rz, fma(ry, ry, fma(rx, rx, soft2)));
+          if (M4 && maybe_inside(r2, h2i, sh2[j])) {
+            in[w] |= 1u << b;
+            continue;
+          }
+          const double inv = rsqrt64(r2);
+          const double minv = sm[j] * inv, f = minv * (inv * inv);
+          fx = fma(-f, rx, fx); fy = fma(-f, ry, fy); fz = fma(-f, rz, fz);
+          fp -= minv;
         }
-        const double inv = rsqrt64(r2);
-        const double minv = sm[j] * inv, f = minv * (inv * inv);
-        fx = fma(-f, rx, fx); fy = fma(-f, ry, fy); fz = fma(-f, rz, fz);
-        fp -= minv;
       }
-      while (M4 && in != 0u) {
-        const int j = j0 + (__ffs(in) - 1) * K;
-        in &= in - 1u;
-        const double rx = xi - sx[j], ry = yi - sy[j], rz = zi - sz[j];
-        double f, p;
-        m4pair64(fma(rz, rz, fma(ry, ry, fma(rx, rx, soft2))), hinv_i, h3inv_i, shinv[j], f, p);
-        f *= sm[j];
-        fx = fma(-f, rx, fx); fy = fma(-f, ry, fy); fz = fma(-f, rz, fz);
-        fp = fma(-sm[j], p, fp);
+      if (!M4) continue;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        uint32_t msk = in[w];
+        while (msk != 0u) {
+          const int j = j0 + (32 * w + __ffs(msk) - 1) * K;
+          msk &= msk - 1u;
+          const double rx = xi - sx[j], ry = yi - sy[j], rz = zi - sz[j];
+          const double r2 = fma(rz, rz, fma(ry, ry, fma(rx, rx, soft2)));
+          const double inv = rsqrt64(r2), r = r2 * inv, inv3 = inv * inv * inv;
+          const double hj = shinv[j], mh = 0.5 * sm[j];
+          double f = 0.0, p = 0.0;
+          m4_side64(r, inv, inv3, hinv_i, h3inv_i, f, p);
+          m4_side64(r, inv, inv3, hj, hj * hj * hj, f, p);
+          f *= mh;
+          fx = fma(-f, rx, fx); fy = fma(-f, ry, fy); fz = fma(-f, rz, fz);
+          fp = fma(-mh, p, fp);
+        }
       }
     }
   };
