@@ -161,6 +161,9 @@ static int set_systems(kdfmm_tree_s* t, const int64_t* off, int32_t n_sys, const
     same = ht[i] == (theta ? theta[i] : p->theta) && he[i] == (eps ? eps[i] : p->eps) &&
            hn[i] == (nleaf ? nleaf[i] : p->n_leaf);
   if (same) return KDFMM_OK;
+  int64_t mx = 0;
+  for (int32_t i = 0; i < n_sys; ++i) mx = std::max(mx, off[i + 1] - off[i]);
+  t->max_sys = mx;
   int32_t mn = KDFMM_MAX_LEAF;
   for (int32_t i = 0; i <= n_sys; ++i) ho[i] = off[i];
   for (int32_t i = 0; i < n_sys; ++i) {
@@ -217,13 +220,14 @@ static int build_common(kdfmm_tree_s* t, const double* x, const double* m, const
   // and read the counters once; a tree that needed more levels is rebuilt
   // with the host following the counters.
   bool done = false;
-  if (t->levels_used > 0 && t->cap_n >= n) {
-    if ((rc = build_tree(t, x, m, h, s, t->levels_used + 1))) return rc;
+  // Systems that fit in shared memory need no phase A, which is known before.
+  const bool small = t->max_sys <= kSubtreeMax;
+  if (small || (t->levels_used >= 0 && t->cap_n >= n)) {
+    if ((rc = build_tree(t, x, m, h, s, small ? 0 : t->levels_used + 1))) return rc;
     int32_t* hc = t->host_counters;
-    cudaMemcpyAsync(hc, t->counters, 32 * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(&hc[32], t->status, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(hc, t->counters, C_BUILD_END * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
     if ((rc = check_cuda(cudaStreamSynchronize(s), "build"))) return rc;
-    const int32_t st = hc[32];
+    const int32_t st = hc[C_STATUS];
     if (st & ST_NONFINITE)
       return set_error(KDFMM_ERR_NONFINITE, "non-finite position or non-positive mass / h");
     if (st & ST_INTERNAL) return set_error(KDFMM_ERR_INTERNAL, "pre-order numbering inconsistent");
@@ -235,7 +239,7 @@ static int build_common(kdfmm_tree_s* t, const double* x, const double* m, const
       done = true;
     }
   }
-  if (!done && (rc = build_tree(t, x, m, h, s, 0))) return rc;
+  if (!done && (rc = build_tree(t, x, m, h, s, -1))) return rc;
   phase_end(t, KDFMM_PHASE_BUILD, s);
   t->grid_leaves = t->nleaves;
   if (t->cap_n != old_cap || t->L.far_cnt == nullptr)
@@ -314,7 +318,7 @@ static void graph_capture(kdfmm_tree_s* t, const double* x, const double* m, con
     cudaGetLastError();
     return;
   }
-  t->graph_levels = t->levels_used + 2;
+  t->graph_levels = std::max(t->levels_used, 0) + 2;
   t->graph_leaves = (int32_t)std::min<int64_t>(t->n, (int64_t)t->nleaves + t->nleaves / 4 + 64);
   if (t->L.arena ? ensure_arena(t, t->graph_leaves, 1.25) : ensure_slots(t, t->graph_leaves)) return;
   if (ensure_segments(t, segments_bound(t) + segments_bound(t) / 4)) return;
@@ -352,11 +356,10 @@ static int graph_replay(kdfmm_tree_s* t, cudaStream_t s) {
   if (rc) return rc;
   t->launches += t->graph_launches;
   int32_t* hc = t->host_counters;
-  cudaMemcpyAsync(hc, t->counters, 32 * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-  cudaMemcpyAsync(&hc[32], t->status, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-  cudaMemcpyAsync(t->host_stats + 16, t->L.near_np, 4 * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
+  cudaMemcpyAsync(hc, t->counters, C_END * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
   if ((rc = check_cuda(cudaStreamSynchronize(s), "graph replay"))) return rc;
-  const int32_t st = hc[32];
+  memcpy(t->host_stats + 16, hc + C_STATS, 4 * sizeof(int64_t));
+  const int32_t st = hc[C_STATUS];
   t->built = t->evaluated = t->lists_frozen = false;
   if (st & ST_NONFINITE)
     return set_error(KDFMM_ERR_NONFINITE, "non-finite position or non-positive mass / h");
@@ -397,10 +400,12 @@ int kdfmm_tree_create(kdfmm_tree* out) {
   kdfmm_tree_s* t = new (std::nothrow) kdfmm_tree_s();
   if (!t) return set_error(KDFMM_ERR_OOM, "handle allocation");
   int rc = check_cuda(cudaGetDevice(&t->device), "cudaGetDevice");
-  if (!rc) rc = check_cuda(cudaMalloc(&t->counters, 32 * sizeof(int32_t)), "counters");
-  if (!rc) rc = check_cuda(cudaMalloc(&t->status, sizeof(int32_t)), "status");
-  if (!rc) rc = check_cuda(cudaMalloc(&t->com_bound, sizeof(float)), "bound");
-  if (!rc) rc = check_cuda(cudaMalloc(&t->L.near_np, 4 * sizeof(int64_t)), "stats");
+  if (!rc) rc = check_cuda(cudaMalloc(&t->counters, C_END * sizeof(int32_t)), "counters");
+  if (!rc) {
+    t->status = t->counters + C_STATUS;
+    t->com_bound = reinterpret_cast<float*>(t->counters + C_BOUND);
+    t->L.near_np = reinterpret_cast<int64_t*>(t->counters + C_STATS);
+  }
   if (!rc) rc = check_cuda(cudaHostAlloc(&t->host_stats, 64 * sizeof(int64_t), 0), "host stats");
   if (!rc) rc = check_cuda(cudaHostAlloc(&t->host_counters, 64 * sizeof(int32_t), 0), "host counters");
   if (rc) {
@@ -419,9 +424,9 @@ void kdfmm_tree_destroy(kdfmm_tree t) {
   cudaSetDevice(t->device);
   cudaDeviceSynchronize();
   free_build_buffers(t);
-  cudaFree(t->counters); cudaFree(t->status); cudaFree(t->com_bound);
+  cudaFree(t->counters);
   cudaFree(t->L.far_cnt); cudaFree(t->L.near_cnt); cudaFree(t->L.far_off); cudaFree(t->L.near_off);
-  cudaFree(t->L.far_idx); cudaFree(t->L.near_idx); cudaFree(t->L.near_np);
+  cudaFree(t->L.far_idx); cudaFree(t->L.near_idx);
   cudaFree(t->L.heavy); cudaFree(t->L.seg_first); cudaFree(t->L.seg_leaf); cudaFree(t->L.seg_part);
   cudaFree(t->L.temp);
   cudaFree(t->mom_partial);
@@ -555,6 +560,7 @@ int kdfmm_total_momentum(const double* m, const double* v, int64_t n, double* ou
     return set_error(KDFMM_ERR_INVALID_ARG, "m, v and out must be device pointers");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int64_t nb = momentum_blocks(n);
+  if (nb == 1) return momentum(m, v, n, out, nullptr, s);     // one block: no partial sums
   double* scratch = nullptr;
   int rc = check_cuda(cudaMallocAsync(&scratch, (size_t)nb * 6 * sizeof(double), s), "momentum scratch");
   if (rc) return rc;

@@ -1386,10 +1386,10 @@ static int subtree_setup(kdfmm_tree_s* t, size_t smem) {
   return KDFMM_OK;
 }
 
-// Builds the tree (or forest).  fixed_levels <= 0: the host follows the
+// Builds the tree (or forest).  fixed_levels < 0: the host follows the
 // device counters (a synchronisation after the first step, each phase-A
 // level, the subtrees and the numbering) and records the number of phase-A
-// levels in t->levels_used.  fixed_levels > 0: the same launches with no
+// levels in t->levels_used.  fixed_levels >= 0: the same launches with no
 // synchronisation -- exactly that many phase-A levels, every launch sized
 // from capacities and reading its count on the device -- so the sequence can
 // be captured in a CUDA graph; a phase A that needed more levels, or any
@@ -1397,13 +1397,11 @@ static int subtree_setup(kdfmm_tree_s* t, size_t smem) {
 int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* h, cudaStream_t s,
                int fixed_levels) {
   const int64_t n = t->n;
-  const bool deferred = fixed_levels > 0;
+  const bool deferred = fixed_levels >= 0;
   int rc = ensure_build_buffers(t, n);
   if (rc) return rc;
   const kdfmm_params& P = t->p;
-  cudaMemsetAsync(t->counters, 0, 32 * sizeof(int32_t), s);
-  cudaMemsetAsync(t->status, 0, sizeof(int32_t), s);
-  cudaMemsetAsync(t->com_bound, 0, sizeof(float), s);
+  cudaMemsetAsync(t->counters, 0, C_BUILD_END * sizeof(int32_t), s);
   BuildArgs A{};
   A.tmp = t->tmp;
   A.counters = t->counters;
@@ -1419,13 +1417,12 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
 
   int32_t* hc = t->host_counters;
   auto read_back = [&](const char* what) {
-    cudaMemcpyAsync(hc, t->counters, 32 * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(&hc[32], t->status, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(hc, t->counters, C_BUILD_END * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
     return check_cuda(cudaStreamSynchronize(s), what);
   };
   if (!deferred) {
     if ((rc = read_back("build init"))) return rc;
-    if (hc[32] & ST_NONFINITE)
+    if (hc[C_STATUS] & ST_NONFINITE)
       return set_error(KDFMM_ERR_NONFINITE, "non-finite position or non-positive mass / h");
   }
   // phase A: cells above kSubtreeMax, one level per pass
@@ -1458,13 +1455,15 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
     ++level;
     if (!deferred) {
       if ((rc = read_back("build level"))) return rc;
-      if (hc[32] & ST_CAPACITY) return set_error(KDFMM_ERR_CAPACITY, "segment lists overflow");
+      if (hc[C_STATUS] & ST_CAPACITY) return set_error(KDFMM_ERR_CAPACITY, "segment lists overflow");
       if (level > 200) return set_error(KDFMM_ERR_INTERNAL, "phase A did not terminate");
     }
   }
   if (deferred) {
-    k_levels_done<<<1, 1, 0, s>>>(t->counters, t->status);
-    t->launches += 1;
+    if (fixed_levels > 0) {             // (none: no system needs phase A)
+      k_levels_done<<<1, 1, 0, s>>>(t->counters, t->status);
+      t->launches += 1;
+    }
   } else {
     t->levels_used = level;
   }
@@ -1485,9 +1484,9 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
   t->launches += 2;
   if (!deferred) {
     if ((rc = read_back("build subtrees"))) return rc;
-    if (hc[32] & ST_NONFINITE)
+    if (hc[C_STATUS] & ST_NONFINITE)
       return set_error(KDFMM_ERR_NONFINITE, "non-finite position or non-positive mass / h");
-    if (hc[32] & ST_CAPACITY) return set_error(KDFMM_ERR_CAPACITY, "build capacity exceeded");
+    if (hc[C_STATUS] & ST_CAPACITY) return set_error(KDFMM_ERR_CAPACITY, "build capacity exceeded");
     t->ncells = hc[C_CELLS];
     t->nfallback = hc[C_FALLBACK];
     t->depth = hc[C_DEPTH];
@@ -1503,7 +1502,7 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
   if (!deferred) {
     if ((rc = read_back("build finalise"))) return rc;
     t->nleaves = hc[C_LEAVES];
-    if (hc[32] & ST_INTERNAL) return set_error(KDFMM_ERR_INTERNAL, "pre-order numbering inconsistent");
+    if (hc[C_STATUS] & ST_INTERNAL) return set_error(KDFMM_ERR_INTERNAL, "pre-order numbering inconsistent");
   }
   // the grid follows the last known leaf count with a margin; more leaves than
   // groups of 8 lanes loop

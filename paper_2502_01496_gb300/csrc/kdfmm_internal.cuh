@@ -31,8 +31,10 @@ enum : int {
   ST_LISTS = 32,        // the leaves or an interaction list outgrew a fixed capacity
 };
 
-// Slots of the handle's device counter block (32 int32).  Kernels read the
-// sizes they work on from here, so a launch needs no host-side count.
+// Slots of the handle's device counter block (int32).  Kernels read the sizes
+// they work on from here, so a launch needs no host-side count.  The build
+// clears and the host reads back [0, C_BUILD_END) with one call each, a walk
+// [C_MAXFAR, C_END); the last eight hold the walk's four 64-bit statistics.
 enum : int {
   C_CELLS = 0,      // cells allocated
   C_NEXT_A = 1,     // segments pushed for the next phase-A level
@@ -41,13 +43,18 @@ enum : int {
   C_CHUNKS = 4,     // chunks of the current phase-A level
   C_FALLBACK = 5,   // degenerate cuts
   C_DEPTH = 6,      // deepest level
-  C_MAXFAR = 8,     // longest far list of the last walk
-  C_MAXNEAR = 9,    // longest near list of the last walk
   C_NA = 10,        // segments of the current phase-A level
   C_LEAVES = 11,    // leaves
   C_WORK = 12,      // dynamic work counter of the persistent subtree kernel
-  C_HEAVY = 13,     // leaves whose walk outgrew the per-thread budget (queued)
-  C_SEGS = 14,      // extra P2P segments of leaves with long near lists
+  C_STATUS = 16,    // status word (ST_ bits)
+  C_BOUND = 17,     // max |com component| over the cells (float)
+  C_BUILD_END = 18,
+  C_SEGS = 19,      // extra P2P segments of leaves with long near lists
+  C_MAXFAR = 21,    // longest far list of the last walk
+  C_MAXNEAR = 22,   // longest near list of the last walk
+  C_HEAVY = 23,     // leaves whose walk outgrew the per-thread budget (queued)
+  C_STATS = 24,     // (four int64) P2P interactions, float64 decisions, far and near entries
+  C_END = 32,
 };
 
 // Streaming multiprocessors of the current device (queried once per device).
@@ -106,7 +113,7 @@ struct Lists {
   int32_t* temp;                   // arena walk: per-thread scratch
   int64_t temp_cap;                // its entries
   int32_t arena_grid;              // blocks of the arena walk
-  int64_t* near_np;                // device statistics of the walk (4)
+  int64_t* near_np;                // in the counter block: statistics of the walk (4)
   int32_t* heavy;                  // leaves queued for the block-wide walk (nleaves)
   // near lists longer than seg_entries are split: segment 0 stays with the
   // leaf, the others are work items of their own whose partial sums
@@ -134,7 +141,8 @@ struct kdfmm_tree_s {
   int64_t n = 0, cap_n = 0;
   int32_t ncells = 0, nleaves = 0, depth = 0, nfallback = 0;
   int32_t grid_leaves = 0;         // leaves the launches of an evaluation are sized for
-  int32_t levels_used = 0;         // phase-A levels of the last host-followed build
+  int32_t levels_used = -1;        // phase-A levels of the last host-followed build (-1: none yet)
+  int64_t max_sys = 0;             // particles of the largest system
   int32_t subtree_grid = 0;        // persistent grid of the subtree kernel
   size_t subtree_smem = 0;
   int64_t cap_cells = 0;
@@ -146,8 +154,8 @@ struct kdfmm_tree_s {
   kdfmm::Seg* segA[2]{};
   kdfmm::Seg *segB = nullptr, *segL = nullptr;
   int64_t capA = 0, capB = 0, capL = 0;
-  int32_t* counters = nullptr;     // device: [0] cells, [1] nextA, [2] nB, [3] nL, [4] chunks, [5] nfallback, [6] depth, [7] nexact
-  int32_t* status = nullptr;       // device status word
+  int32_t* counters = nullptr;     // device counter block (C_END int32)
+  int32_t* status = nullptr;       // in it: the status word
   int32_t* chunk_seg = nullptr;
   int32_t* seg_chunk_off = nullptr;
   double* chunk_sum = nullptr;     // 4 per chunk
@@ -175,7 +183,7 @@ struct kdfmm_tree_s {
   kdfmm::Cells c{};
   int32_t* leaf_cells = nullptr;   // pre-order ids of the leaves
   int32_t* leaf_rank = nullptr;    // cell -> leaf ordinal (-1 for super-cells)
-  float* com_bound = nullptr;      // device: max |com component| over cells
+  float* com_bound = nullptr;      // in the counter block: max |com component| over cells
   kdfmm::Lists L{};
   double* lexp64 = nullptr;        // 20 per leaf
   float* lexp32 = nullptr;         // 24 per leaf (20 coefficients + 4 low parts)

@@ -879,9 +879,7 @@ static void walk_launch(kdfmm_tree_s* t, WalkArgs W, ListMode mode, int64_t cf, 
   W.temp = L.temp;
   W.heavy_scratch = arena ? L.temp_cap / grid_blocks(2) : 0;
   W.slot_leaves = slot_leaves;
-  cudaMemsetAsync(L.near_np, 0, 4 * sizeof(int64_t), s);
-  cudaMemsetAsync(t->counters + C_MAXFAR, 0, 2 * sizeof(int32_t), s);
-  cudaMemsetAsync(t->counters + C_HEAVY, 0, sizeof(int32_t), s);
+  cudaMemsetAsync(t->counters + C_MAXFAR, 0, (C_END - C_MAXFAR) * sizeof(int32_t), s);
   if (arena) {
     // one round (no more leaves than threads): the walk is latency-bound and
     // its lanes run free; several rounds fill the GPU and the synchronous loop
@@ -972,10 +970,11 @@ int run_walk(kdfmm_tree_s* t, cudaStream_t s) {
   int rc;
   auto launch = [&](ListMode mode) {
     walk_launch(t, W, mode, cf, cn, nl, s);
-    cudaMemcpyAsync(hc + C_MAXFAR, t->counters + C_MAXFAR, 2 * sizeof(int32_t),
+    cudaMemcpyAsync(hc + C_MAXFAR, t->counters + C_MAXFAR, (C_END - C_MAXFAR) * sizeof(int32_t),
                     cudaMemcpyDeviceToHost, s);
-    cudaMemcpyAsync(t->host_stats + 16, L.near_np, 4 * sizeof(int64_t), cudaMemcpyDeviceToHost, s);
-    return check_cuda(cudaStreamSynchronize(s), "walk");
+    const int err = check_cuda(cudaStreamSynchronize(s), "walk");
+    memcpy(t->host_stats + 16, hc + C_STATS, 4 * sizeof(int64_t));
+    return err;
   };
   auto done = [&](ListMode mode) {
     L.arena = mode == ListMode::kArena;
