@@ -13,9 +13,9 @@
 // One warp per target leaf.  A leaf of n_t <= 32 targets uses K = 32 / n_t
 // source slices: lane = target + n_t * slice, slice k takes sources k, k+K, ...
 // of every near leaf, and the slices are combined at the end.  A near list
-// longer than a segment (256 leaves; fewer in small float64 evaluations) (a large leaf in the sparse outskirts of a
-// centrally condensed system can have most of the system in it) is split
-// into segments: the leaf's warp takes the first, the others
+// longer than a segment (256 leaves; fewer in small float64 systems) is split
+// (a large leaf in the sparse outskirts of a centrally condensed system can have
+// most of the system in it): the leaf's warp takes the first segment, the others
 // are separate work items, and their partial sums are added afterwards in
 // segment order, so the result does not depend on scheduling.
 //
@@ -58,15 +58,37 @@ struct P2PArgs {
   const double* sys_eps;     // Plummer softening length of each system
   double* a;
   double* phi;
-  // near lists longer than seg_entries: segment 0 is the leaf's own work
+  // near lists longer than leaf_segment(): segment 0 is the leaf's own work
   // item, the others (counters[C_SEGS], at most seg_cap) are items after the
   // leaves, whose partial sums seg_part k_seg_combine adds in segment order
   const int32_t* seg_first;
   const int32_t* seg_leaf;
   double* seg_part;
   int64_t seg_cap;
-  int seg_entries;
+  const int64_t* sys_off;    // float64: first particle of each system; mixed: null
 };
+
+// Near entries per segment, by the particles of the leaf's own system alone: an
+// eager evaluation, a replayed graph and a batch that holds the system split
+// alike.  Float64 evaluations of few particles take short segments: their leaves
+// are too few warps for the GPU's 608 float64 pipes (4096 particles: 367 leaves
+// with ~108 near leaves each).  Mixed evaluations keep 256: a shorter segment
+// would move the chunks of 256 sources whose float32 sums are folded at once.
+constexpr int kSegSteps = 3;
+__host__ __device__ __forceinline__ int64_t seg_below(int step) {      // particles, exclusive
+  return step == 0 ? 8192 : (step == 1 ? 65536 : 262144);
+}
+__host__ __device__ __forceinline__ int seg_length(int step) {
+  return step == 0 ? 8 : (step == 1 ? 32 : (step == 2 ? 64 : kSegEntries));
+}
+__host__ __device__ __forceinline__ int seg_step(int64_t n) {
+  int step = 0;
+  while (step < kSegSteps && n >= seg_below(step)) ++step;
+  return step;
+}
+__device__ __forceinline__ int leaf_segment(const int64_t* __restrict__ sys_off, int sys) {
+  return sys_off == nullptr ? kSegEntries : seg_length(seg_step(sys_off[sys + 1] - sys_off[sys]));
+}
 
 // M4 cubic spline, q = r/h < 2: F(q)/q^3 and P(q) (qi = 1/q).
 __device__ __forceinline__ float m4_fq3(float q, float qi) {
@@ -270,8 +292,9 @@ __global__ void __launch_bounds__(kP2PWarps * 32, 6) k_p2p_mixed(P2PArgs A) {
   const unsigned full = 0xffffffffu, lt = (1u << lane) - 1u;
   const int64_t nall = min((int64_t)A.near_cnt[k], A.cap_near);
   const int64_t sidx = seg ? (int64_t)(g - A.seg_first[k] + 1) : 0;
-  const int64_t e1 = A.near_off[k] + min(nall, (sidx + 1) * A.seg_entries);
-  for (int64_t e = A.near_off[k] + sidx * A.seg_entries; e < e1;) {
+  const int seglen = leaf_segment(A.sys_off, A.leaf_sys[k]);
+  const int64_t e1 = A.near_off[k] + min(nall, (sidx + 1) * seglen);
+  for (int64_t e = A.near_off[k] + sidx * seglen; e < e1;) {
     // up to 32 candidate leaves, one per lane
     const int64_t my = e + lane;
     int cnt = 0, first = 0;
@@ -586,8 +609,9 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
   }
   const int64_t nall = min((int64_t)A.near_cnt[k], A.cap_near);
   const int64_t sidx = seg ? (int64_t)(g - A.seg_first[k] + 1) : 0;
-  const int64_t e1 = A.near_off[k] + min(nall, (sidx + 1) * A.seg_entries);
-  for (int64_t e = A.near_off[k] + sidx * A.seg_entries; e < e1;) {
+  const int seglen = leaf_segment(A.sys_off, A.leaf_sys[k]);
+  const int64_t e1 = A.near_off[k] + min(nall, (sidx + 1) * seglen);
+  for (int64_t e = A.near_off[k] + sidx * seglen; e < e1;) {
     const int64_t my = e + lane;
     int cnt = 0, first = 0;
     if (my < e1) {
@@ -651,11 +675,11 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
 // their entries below seg_cap are marked -1, which every consumer skips.
 __global__ void k_seg_plan(const int32_t* __restrict__ near_cnt, int64_t cap_near,
                            int max_leaves, int32_t* counters, int32_t* seg_first,
-                           int32_t* seg_leaf, int64_t seg_cap, int seg_entries,
-                           int32_t* status) {
+                           int32_t* seg_leaf, int64_t seg_cap, const int64_t* __restrict__ sys_off,
+                           const int32_t* __restrict__ leaf_sys, int32_t* status) {
   const int nleaves = min(counters[C_LEAVES], max_leaves);
   KD_GRID_STRIDE(k, nleaves) {
-    const int x = extra_segments(min((int64_t)near_cnt[k], cap_near), seg_entries);
+    const int x = extra_segments(min((int64_t)near_cnt[k], cap_near), leaf_segment(sys_off, leaf_sys[k]));
     int first = -1;
     if (x > 0) {
       const int base = atomicAdd(&counters[C_SEGS], x);
@@ -684,7 +708,8 @@ __global__ void k_seg_combine(P2PArgs A) {
     if (g != f) continue;
     const int a = A.leaf_cells[k];
     if (lane >= A.ccount[a]) continue;
-    const int x = extra_segments(min((int64_t)A.near_cnt[k], A.cap_near), A.seg_entries);
+    const int x = extra_segments(min((int64_t)A.near_cnt[k], A.cap_near),
+                                 leaf_segment(A.sys_off, A.leaf_sys[k]));
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
     for (int q = 0; q < x; ++q) {
       const double* P = A.seg_part + (int64_t)(f + q) * 128 + 4 * lane;
@@ -730,30 +755,31 @@ int ensure_segments(kdfmm_tree_s* t, int64_t need) {
   return KDFMM_OK;
 }
 
-// Near entries per segment: by the particle count alone, so that an eager
-// evaluation and a replayed graph split alike.  Float64 evaluations of few
-// particles take short segments: their leaves are too few warps for the GPU's
-// 608 float64 pipes (4096 particles: 367 leaves with ~108 near leaves each).
-// Mixed evaluations keep 256: a shorter segment would move the chunks of 256
-// sources whose float32 sums are folded at once.
-static int segment_entries(const kdfmm_tree_s* t) {
-  if (t->p.precision != KDFMM_FP64) return kSegEntries;
-  return t->n < 65536 ? 32 : (t->n < 262144 ? 64 : kSegEntries);
-}
-
+// At most so many extra segments: of each length class the entries of its
+// systems (no more than all, no more than their particles squared) over the length.
 int64_t segments_bound(const kdfmm_tree_s* t) {
   const Lists& L = t->L;
   const int64_t entries = L.exact ? L.near_cap : t->host_stats[KDFMM_STAT_NNEAR];
-  return entries / segment_entries(t) + 64;
+  if (t->p.precision != KDFMM_FP64) return entries / kSegEntries + 64;
+  if (t->n_sys == 1) return entries / seg_length(seg_step(t->n)) + 64;
+  double own[kSegSteps + 1] = {};
+  for (int k = 0; k < t->n_sys; ++k) {
+    const int64_t n = t->host_sys_off[k + 1] - t->host_sys_off[k];
+    own[seg_step(n)] += (double)n * (double)n;
+  }
+  int64_t bound = 64;
+  for (int q = 0; q <= kSegSteps; ++q)
+    bound += (int64_t)std::min((double)entries, own[q]) / seg_length(q);
+  return bound;
 }
 
 int plan_segments(kdfmm_tree_s* t, cudaStream_t s) {
   const int gl = std::max(t->grid_leaves, 1);
-  t->L.seg_entries = segment_entries(t);
   cudaMemsetAsync(t->counters + C_SEGS, 0, sizeof(int32_t), s);
   k_seg_plan<<<std::min<unsigned>(blocks_for(gl, 256), grid_blocks()), 256, 0, s>>>(
       t->L.near_cnt, t->L.exact ? INT64_MAX : t->L.cap_near, gl, t->counters, t->L.seg_first,
-      t->L.seg_leaf, t->L.seg_cap, t->L.seg_entries, t->status);
+      t->L.seg_leaf, t->L.seg_cap, t->p.precision == KDFMM_FP64 ? t->sys_off : nullptr, t->leaf_sys,
+      t->status);
   t->launches += 1;
   return check_cuda(cudaGetLastError(), "segment plan");
 }
@@ -788,7 +814,7 @@ int run_p2p(kdfmm_tree_s* t, double* a, double* phi, cudaStream_t s) {
   A.seg_cap = t->L.seg_cap;
   int rc = plan_segments(t, s);
   if (rc) return rc;
-  A.seg_entries = t->L.seg_entries;
+  A.sys_off = t->p.precision == KDFMM_FP64 ? t->sys_off : nullptr;
   const int gl = std::max(t->grid_leaves, 1);
   const bool m4 = t->p.soft_kind == KDFMM_SOFT_M4;
   if (t->p.precision == KDFMM_MIXED) {
