@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
           fp -= minv;
         }
       }
-      if (!M4) continue;
+      if constexpr (M4) {
 #pragma unroll
       for (int w = 0; w < 4; ++w) {
         uint32_t msk = in[w];
@@ -598,6 +598,7 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
           fx = fma(-f, rx, fx); fy = fma(-f, ry, fy); fz = fma(-f, rz, fz);
           fp = fma(-mh, p, fp);
         }
+      }
       }
     }
   };
@@ -711,9 +712,12 @@ __global__ void k_seg_combine(P2PArgs A) {
     const int x = extra_segments(min((int64_t)A.near_cnt[k], A.cap_near),
                                  leaf_segment(A.sys_off, A.leaf_sys[k]));
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    // (a heavy leaf has hundreds of segments: eight pieces' loads in flight)
+#pragma unroll 8
     for (int q = 0; q < x; ++q) {
-      const double* P = A.seg_part + (int64_t)(f + q) * 128 + 4 * lane;
-      s0 += P[0]; s1 += P[1]; s2 += P[2]; s3 += P[3];
+      const double2* P = reinterpret_cast<const double2*>(A.seg_part + (int64_t)(f + q) * 128 + 4 * lane);
+      const double2 p01 = P[0], p23 = P[1];
+      s0 += p01.x; s1 += p01.y; s2 += p23.x; s3 += p23.y;
     }
     const int64_t ci = A.tp.idx[A.cfirst[a] + lane];
     A.a[3 * ci + 0] += s0;

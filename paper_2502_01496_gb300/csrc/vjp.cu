@@ -181,7 +181,6 @@ struct VjpArgs {
   float4 *q0, *q1, *q2;
   float2* q3;
   double* xbar;                         // tree order (N x 3)
-  double* mbar;                         // tree order (N)
   double* xsrc;                         // P2P source-side part of x_bar (N x 3, atomics)
   double* msrc;                         // P2P source-side part of m_bar (N, atomics)
   double* cbar;                         // per leaf: 20 expansion cotangents
@@ -1309,8 +1308,9 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source64(VjpArgs V) {
   }
 }
 
-// Adds the extra segments' target-side sums to x_bar, warp per leaf (the
-// warp of its first extra segment), lane per target, in segment order.
+// Adds the extra items' target-side sums to x_bar, in piece order, warp per leaf
+// (the warp of its first extra item), lane per target; eight pieces' loads in
+// flight.
 __global__ void k_vjp_seg_combine(VjpArgs V) {
   const int lane = threadIdx.x & 31;
   const int nseg = (int)min((int64_t)V.tctr[2], V.seg_cap);
@@ -1323,9 +1323,12 @@ __global__ void k_vjp_seg_combine(VjpArgs V) {
     if (lane >= V.c.count[a]) continue;
     const int x = extra_segments(min((int64_t)V.near_cnt[k], V.cap_near), V.entries);
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+#pragma unroll 8
     for (int q = 0; q < x; ++q) {
       const double* P = V.seg_part + (int64_t)(f + q) * 128 + 4 * lane;
-      s0 += P[0]; s1 += P[1]; s2 += P[2];
+      const double2 p01 = *reinterpret_cast<const double2*>(P);
+      const double p2 = P[2];
+      s0 += p01.x; s1 += p01.y; s2 += p2;
     }
     const int64_t pi = (int64_t)V.c.first[a] + lane;
     V.xbar[3 * pi] += s0;
@@ -1341,51 +1344,55 @@ __global__ void k_vjp_seg_combine(VjpArgs V) {
 //   m_bar_i += M_bar' + x.S_bar + y^T G y / 2,   x_bar_i += m_i (S_bar + G y).
 // As polynomials in x: a0 + a1.x + x^T (G/2) x and m_i (a1 + G x), with
 // a1 = S_bar - G com, a0 = M_bar' + com^T G com / 2; summed over ancestors.
-__global__ void k_vjp_moments(VjpArgs V) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= V.nleaves) return;
-  const int leaf = V.leaf_cells[k];
-  double a0 = 0.0, a1[3] = {0.0, 0.0, 0.0}, G[6] = {0, 0, 0, 0, 0, 0};   // G: xx xy xz yy yz zz
-  for (int c = leaf; c >= 0; c = V.c.parent[c]) {
-    const double* cb = V.cell_bar + 10 * (int64_t)c;
-    const double M = V.c.M[c];
+// Each cell's polynomial once, in place of its cotangents (every leaf formed all
+// its ancestors' before: four divisions a level and leaf).
+__global__ void k_vjp_cell_poly(VjpArgs V) {
+  KD_GRID_STRIDE(c, V.ncells) {
+    double* cb = V.cell_bar + 10 * (int64_t)c;
+    const double inv = 1.0 / V.c.M[c];
     const double com[3] = {V.c.cx[c], V.c.cy[c], V.c.cz[c]};
-    const double Sb[3] = {cb[1] / M, cb[2] / M, cb[3] / M};
-    const double Mb = cb[0] - (cb[1] * com[0] + cb[2] * com[1] + cb[3] * com[2]) / M;
+    const double Sb[3] = {cb[1] * inv, cb[2] * inv, cb[3] * inv};
+    const double Mb = cb[0] - (Sb[0] * com[0] + Sb[1] * com[1] + Sb[2] * com[2]);
     const double q0 = cb[4], q1 = cb[5], q2 = cb[6], q3 = cb[7], q4 = cb[8], q5 = cb[9];
     const double g[6] = {4 * q0 - 2 * q3 - 2 * q5, 3 * q1, 3 * q2, 4 * q3 - 2 * q0 - 2 * q5, 3 * q4,
                          4 * q5 - 2 * q0 - 2 * q3};
     const double Gc[3] = {g[0] * com[0] + g[1] * com[1] + g[2] * com[2],
                           g[1] * com[0] + g[3] * com[1] + g[4] * com[2],
                           g[2] * com[0] + g[4] * com[1] + g[5] * com[2]};
-    a0 += Mb + 0.5 * (com[0] * Gc[0] + com[1] * Gc[1] + com[2] * Gc[2]);
-    for (int d = 0; d < 3; ++d) a1[d] += Sb[d] - Gc[d];
-    for (int d = 0; d < 6; ++d) G[d] += g[d];
-  }
-  const int f = V.c.first[leaf], cnt = V.c.count[leaf];
-  for (int j = 0; j < cnt; ++j) {
-    const int64_t p = (int64_t)f + j;
-    const double x[3] = {V.tp.x[p], V.tp.y[p], V.tp.z[p]};
-    const double Gx[3] = {G[0] * x[0] + G[1] * x[1] + G[2] * x[2],
-                          G[1] * x[0] + G[3] * x[1] + G[4] * x[2],
-                          G[2] * x[0] + G[4] * x[1] + G[5] * x[2]};
-    const double mi = V.tp.m[p];
-    V.mbar[p] += a0 + a1[0] * x[0] + a1[1] * x[1] + a1[2] * x[2] +
-                 0.5 * (x[0] * Gx[0] + x[1] * Gx[1] + x[2] * Gx[2]);
-    V.xbar[3 * p] += mi * (a1[0] + Gx[0]);
-    V.xbar[3 * p + 1] += mi * (a1[1] + Gx[1]);
-    V.xbar[3 * p + 2] += mi * (a1[2] + Gx[2]);
+    cb[0] = Mb + 0.5 * (com[0] * Gc[0] + com[1] * Gc[1] + com[2] * Gc[2]);
+    for (int d = 0; d < 3; ++d) cb[1 + d] = Sb[d] - Gc[d];
+    for (int d = 0; d < 6; ++d) cb[4 + d] = g[d];
   }
 }
 
-__global__ void k_scatter_bar(VjpArgs V, double* __restrict__ x_bar, double* __restrict__ m_bar) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= V.n) return;
-  const int64_t i = V.tp.idx[p];
-  x_bar[3 * i] = V.xbar[3 * p] + V.xsrc[3 * p];
-  x_bar[3 * i + 1] = V.xbar[3 * p + 1] + V.xsrc[3 * p + 1];
-  x_bar[3 * i + 2] = V.xbar[3 * p + 2] + V.xsrc[3 * p + 2];
-  m_bar[i] = V.mbar[p] + V.msrc[p];
+// Half a warp per leaf: lanes 0..9 sum a coefficient each over the leaf and its
+// ancestors, then every lane takes particles, adds the parts of x_bar and m_bar
+// and writes them in the caller's order.
+__global__ void __launch_bounds__(128) k_vjp_moments(VjpArgs V, double* __restrict__ x_bar,
+                                                     double* __restrict__ m_bar) {
+  const int lane = threadIdx.x & 31, l = lane & 15, g0 = lane & 16;
+  const unsigned half = 0xffffu << g0;
+  const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+  if (k >= V.nleaves) return;
+  const int leaf = V.leaf_cells[k];
+  double s = 0.0;
+  for (int c = leaf; c >= 0; c = V.c.parent[c])
+    if (l < 10) s += V.cell_bar[10 * (int64_t)c + l];
+  double w[10];
+#pragma unroll
+  for (int j = 0; j < 10; ++j) w[j] = __shfl_sync(half, s, g0 + j);
+  const double *a1 = w + 1, *G = w + 4;
+  const int f = V.c.first[leaf], cnt = V.c.count[leaf];
+  for (int j = l; j < cnt; j += 16) {
+    const int64_t p = (int64_t)f + j, i = V.tp.idx[p];
+    const double x = V.tp.x[p], y = V.tp.y[p], z = V.tp.z[p], m = V.tp.m[p];
+    const double gx = G[0] * x + G[1] * y + G[2] * z, gy = G[1] * x + G[3] * y + G[4] * z,
+                 gz = G[2] * x + G[4] * y + G[5] * z;
+    m_bar[i] = V.msrc[p] + (w[0] + a1[0] * x + a1[1] * y + a1[2] * z + 0.5 * (x * gx + y * gy + z * gz));
+    x_bar[3 * i] = V.xbar[3 * p] + V.xsrc[3 * p] + m * (a1[0] + gx);
+    x_bar[3 * i + 1] = V.xbar[3 * p + 1] + V.xsrc[3 * p + 1] + m * (a1[1] + gy);
+    x_bar[3 * i + 2] = V.xbar[3 * p + 2] + V.xsrc[3 * p + 2] + m * (a1[2] + gz);
+  }
 }
 
 }  // namespace
@@ -1441,7 +1448,7 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
     return was;
   };
   const size_t o_cell = take((size_t)nc * 10 * 8), o_xsrc = take((size_t)n * 3 * 8),
-               o_msrc = take((size_t)n * 8), o_mbar = take((size_t)n * 8),
+               o_msrc = take((size_t)n * 8),
                o_tcnt = take((size_t)nl * 4), o_tcur = take((size_t)nl * 4), o_tctr = take(32);
   zeroed = at;
   const size_t o_xbar = take((size_t)n * 3 * 8), o_cbar = take((size_t)nl * 20 * 8),
@@ -1463,7 +1470,6 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
   V.cell_bar = (double*)(buf + o_cell);
   V.xsrc = (double*)(buf + o_xsrc);
   V.msrc = (double*)(buf + o_msrc);
-  V.mbar = (double*)(buf + o_mbar);
   V.tcnt = (int32_t*)(buf + o_tcnt);
   V.tcur = (int32_t*)(buf + o_tcur);
   V.tctr = (unsigned long long*)(buf + o_tctr);
@@ -1517,8 +1523,8 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
     }
   }
   k_vjp_seg_combine<<<grid_blocks(2), 256, 0, s>>>(V);
-  k_vjp_moments<<<blocks_for(nl, 128), 128, 0, s>>>(V);
-  k_scatter_bar<<<blocks_for(n, 256), 256, 0, s>>>(V, x_bar, m_bar);
+  k_vjp_cell_poly<<<std::min<unsigned>(blocks_for(nc, 128), grid_blocks()), 128, 0, s>>>(V);
+  k_vjp_moments<<<blocks_for((int64_t)nl * 16, 128), 128, 0, s>>>(V, x_bar, m_bar);
   t->launches += 11;
   rc = check_cuda(cudaGetLastError(), "adjoint launch");
   if (pooled) cudaFreeAsync(buf, s);
