@@ -34,7 +34,8 @@ inline unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + thre
 
 constexpr int kLevelsPerSync = 8;
 
-enum { DQ_OUT = 0, DQ_FAR = 1, DQ_NEAR = 2, DQ_OVER = 3, DQ_IN = 4 };
+// DQ_IN: pairs of the level; DQ_DONE: blocks that finished it
+enum { DQ_OUT = 0, DQ_FAR = 1, DQ_NEAR = 2, DQ_OVER = 3, DQ_IN = 4, DQ_DONE = 5 };
 
 struct DualArgs {
   Cells c;
@@ -103,25 +104,21 @@ __device__ __forceinline__ int64_t warp_reserve(int32_t* ctr, int slot, int n, i
   return (int64_t)base + incl - n;
 }
 
-// One level of the pair recursion: thread per pair, warp-aggregated queue
-// pushes, grid-stride over the ctr[DQ_IN] pairs of the level.
-__global__ void k_dual_level(DualArgs D) {
+// One level of the pair recursion over the n_in pairs of `in`: thread per pair
+// (whole warps, this warp's from `first` on), warp-aggregated queue pushes.
+__device__ __forceinline__ void dual_pairs(const DualArgs& D, const int2* in, int2* out, int n_in,
+                                           int first, int stride) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  // after an overflow the level's results are discarded (the walk is redone
-  // with larger queues); the count never exceeds the queue's entries
-  if (D.ctr[DQ_OVER]) return;
-  const int n_in = (int)min((int64_t)D.ctr[DQ_IN], D.cap_out);
   const Cells& c = D.c;
   const float bound = *D.com_bound;
-  const int stride = gridDim.x * blockDim.x;
-  for (int base = blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n_in; base += stride) {
+  for (int base = first; base < n_in; base += stride) {
     const int p = base + lane;
     int n_out = 0, n_far = 0, n_near = 0;
     int2 o0 = make_int2(0, 0), o1 = o0, o2 = o0, fp = o0, np = o0;
     unsigned long long pairs = 0;
     if (p < n_in) {
-      const int A = D.in[p].x, B = D.in[p].y;
+      const int A = in[p].x, B = in[p].y;
       const bool leafA = c.left[A] < 0, leafB = c.left[B] < 0;
       if (A == B) {
         if (leafA) {
@@ -163,9 +160,9 @@ __global__ void k_dual_level(DualArgs D) {
     const int64_t pf = warp_reserve(D.ctr, DQ_FAR, n_far, D.cap_far);
     const int64_t pn = warp_reserve(D.ctr, DQ_NEAR, n_near, D.cap_near);
     if (po >= 0 && n_out > 0) {
-      D.out[po] = o0;
-      D.out[po + 1] = o1;
-      if (n_out == 3) D.out[po + 2] = o2;
+      out[po] = o0;
+      out[po + 1] = o1;
+      if (n_out == 3) out[po + 2] = o2;
     }
     if (pf >= 0 && n_far) D.far[pf] = fp;
     if (pn >= 0 && n_near) D.near[pn] = np;
@@ -175,10 +172,50 @@ __global__ void k_dual_level(DualArgs D) {
   }
 }
 
-// Makes the last level's output the next level's input.
-__global__ void k_dual_advance(int32_t* ctr) {
-  ctr[DQ_IN] = ctr[DQ_OUT];
-  ctr[DQ_OUT] = 0;
+// The first `levels` levels by one block -- a few hundred pairs at most each,
+// which a launch of their own took 8 us each -- and the roots as the next
+// level's input.  An even number: the queues' roles are those at the start.
+constexpr int kSeedLevels = 8;
+__global__ void __launch_bounds__(1024) k_dual_seed(DualArgs D, int levels) {
+  volatile int32_t* ctr = D.ctr;
+  for (int l = 0; l < levels; ++l) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      ctr[DQ_IN] = ctr[DQ_OUT];
+      ctr[DQ_OUT] = 0;
+    }
+    __syncthreads();
+    if (!ctr[DQ_OVER])                  // (after an overflow the walk is redone with larger queues)
+      dual_pairs(D, l & 1 ? D.out : D.in, l & 1 ? const_cast<int2*>(D.in) : D.out, ctr[DQ_IN],
+                 (int)(threadIdx.x & ~31), (int)blockDim.x);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    ctr[DQ_IN] = ctr[DQ_OUT];
+    ctr[DQ_OUT] = 0;
+  }
+}
+
+// One level, grid-stride over its ctr[DQ_IN] pairs; the last block to finish
+// makes its output the next level's input.
+__global__ void k_dual_level(DualArgs D) {
+  __shared__ int s_last;
+  // after an overflow the level's results are discarded (the walk is redone
+  // with larger queues); the count never exceeds the queue's entries
+  const int n_in = D.ctr[DQ_OVER] ? 0 : (int)min((int64_t)D.ctr[DQ_IN], D.cap_out);
+  dual_pairs(D, D.in, D.out, n_in, (int)(blockIdx.x * blockDim.x + (threadIdx.x & ~31)),
+             (int)(gridDim.x * blockDim.x));
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicAdd(&D.ctr[DQ_DONE], 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (s_last && threadIdx.x == 0) {
+    __threadfence();
+    volatile int32_t* ctr = D.ctr;
+    ctr[DQ_IN] = ctr[DQ_OUT];
+    ctr[DQ_OUT] = 0;
+    ctr[DQ_DONE] = 0;
+  }
 }
 
 __global__ void k_dual_roots(const int32_t* __restrict__ sys_root, int n_sys, int2* q) {
@@ -285,8 +322,9 @@ __device__ __forceinline__ void recentre_add(const double C[20], const double d[
 struct L2LArgs {
   Cells c;
   const int32_t* leaf_rank;
-  int ncells;
-  int level;
+  const int32_t* by_depth;   // cells ordered by depth
+  const int32_t* depth_off;  // first of each depth in it
+  int l0, l1;                // levels l0 .. l1 - 1
   bool mixed;
   const float* cell32;
   const double* cell64;
@@ -295,11 +333,37 @@ struct L2LArgs {
   double* leaf64;
 };
 
-// The cells of one tree level (all systems): total = own + parent's total
-// re-centred; leaves also write their expansion in the evaluation's format.
+// Cells by depth: counts, (host-sized) offsets, fill.  Taking the cells of a
+// level from all cells by their depth left every warp with a few active lanes
+// at every level, each running the full float64 re-centring.
+__global__ void k_depth_count(Cells c, int ncells, int32_t* cnt) {
+  KD_GRID_STRIDE(i, ncells) atomicAdd(&cnt[c.depth[i]], 1);
+}
+__global__ void k_depth_off(const int32_t* __restrict__ cnt, int levels, int32_t* off, int32_t* cursor) {
+  int run = 0;
+  for (int l = 0; l < levels; ++l) {
+    off[l] = cursor[l] = run;
+    run += cnt[l];
+  }
+  off[levels] = run;
+}
+__global__ void k_depth_fill(Cells c, int ncells, int32_t* cursor, int32_t* by_depth) {
+  KD_GRID_STRIDE(i, ncells) by_depth[atomicAdd(&cursor[c.depth[i]], 1)] = i;
+}
+
+// The cells of tree levels l0 .. l1 - 1 (all systems), one level after the other
+// (several levels: one block): total = own + parent's total re-centred; leaves
+// also write their expansion in the evaluation's format.
 __global__ void k_l2l_level(L2LArgs A) {
-  KD_GRID_STRIDE(cell, A.ncells) {
-    if (A.c.depth[cell] != A.level) continue;
+  for (int level = A.l0; level < A.l1; ++level) {
+  if (level > A.l0) {
+    __threadfence();
+    __syncthreads();
+  }
+  const int n0 = A.depth_off[level], n1 = A.depth_off[level + 1];
+  for (int at = n0 + (int)(blockIdx.x * blockDim.x + threadIdx.x); at < n1;
+       at += (int)(gridDim.x * blockDim.x)) {
+    const int cell = A.by_depth[at];
     double acc[20];
     if (A.mixed) {
       const float* f = A.cell32 + 24 * (int64_t)cell;
@@ -317,7 +381,7 @@ __global__ void k_l2l_level(L2LArgs A) {
       double P[20];
       const double* tp = A.tot + 20 * (int64_t)p;
 #pragma unroll
-      for (int j = 0; j < 20; ++j) P[j] = tp[j];
+      for (int j = 0; j < 20; ++j) P[j] = __ldcg(tp + j);
       const double d[3] = {A.c.cx[cell] - A.c.cx[p], A.c.cy[cell] - A.c.cy[p],
                            A.c.cz[cell] - A.c.cz[p]};
       recentre_add(P, d, acc);
@@ -338,6 +402,7 @@ __global__ void k_l2l_level(L2LArgs A) {
 #pragma unroll
       for (int j = 0; j < 20; ++j) out[j] = acc[j];
     }
+  }
   }
 }
 
@@ -361,7 +426,7 @@ void free_dual(kdfmm_tree_s* t) {
   auto& D = t->dual;
   cudaFree(D.q[0]); cudaFree(D.q[1]); cudaFree(D.far); cudaFree(D.near); cudaFree(D.ctr);
   cudaFree(D.far_cnt); cudaFree(D.far_off); cudaFree(D.far_idx); cudaFree(D.cursor);
-  cudaFree(D.lcell32); cudaFree(D.lcell64); cudaFree(D.ltot);
+  cudaFree(D.lcell32); cudaFree(D.lcell64); cudaFree(D.ltot); cudaFree(D.depth_tab);
   D = kdfmm_tree_s::Dual{};
 }
 
@@ -414,19 +479,22 @@ int run_dual_walk(kdfmm_tree_s* t, cudaStream_t s) {
     // counts on the device, the host looks at the queue between batches
     int cur = 0;
     bool over = false;
+    A.in = D.q[0];
+    A.out = D.q[1];
+    k_dual_seed<<<1, 1024, 0, s>>>(A, t->n_sys <= 4 ? kSeedLevels : 0);
+    t->launches += 1;
     for (;;) {
       for (int l = 0; l < kLevelsPerSync; ++l) {
         A.in = D.q[cur];
         A.out = D.q[cur ^ 1];
-        k_dual_advance<<<1, 1, 0, s>>>(D.ctr);
         k_dual_level<<<grid_blocks(), 256, 0, s>>>(A);
-        t->launches += 2;
+        t->launches += 1;
         cur ^= 1;
       }
       cudaMemcpyAsync(hc + 40, D.ctr, 5 * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
       if ((rc = check_cuda(cudaStreamSynchronize(s), "dual walk levels"))) return rc;
       if (hc[40 + DQ_OVER]) { over = true; break; }
-      if (hc[40 + DQ_OUT] == 0) break;
+      if (hc[40 + DQ_IN] == 0) break;
     }
     if (!over) {
       nfar = hc[40 + DQ_FAR];
@@ -481,19 +549,45 @@ int run_dual_local(kdfmm_tree_s* t, cudaStream_t s) {
   L2LArgs A{};
   A.c = t->c;
   A.leaf_rank = t->leaf_rank;
-  A.ncells = t->ncells;
   A.mixed = mixed;
   A.cell32 = D.lcell32;
   A.cell64 = D.lcell64;
   A.tot = D.ltot;
   A.leaf32 = t->lexp32;
   A.leaf64 = t->lexp64;
-  const unsigned grid = std::min<unsigned>(blocks_for(std::max(t->ncells, 1), 128), grid_blocks());
-  for (int level = 0; level <= t->depth; ++level) {
-    A.level = level;
-    k_l2l_level<<<grid, 128, 0, s>>>(A);
+  // scratch (free between the lists and the next walk): D.cursor holds the
+  // cells by depth, D.far_cnt stays; the counters are in t->min_depth
+  const int levels = t->depth + 1;
+  int32_t* cnt = t->min_depth;
+  int32_t *off = cnt + levels, *cursor = off + levels + 1;
+  if (3 * (int64_t)levels + 1 > t->cap_n + 2) {             // fewer particles than that: own room
+    int64_t have_d = D.depth_cap;
+    if ((rc = grow(&D.depth_tab, &have_d, 3 * (int64_t)levels + 1, "levels"))) return rc;
+    D.depth_cap = have_d;
+    cnt = D.depth_tab;
+    off = cnt + levels;
+    cursor = off + levels + 1;
   }
-  t->launches += t->depth + 1;
+  cudaMemsetAsync(cnt, 0, (size_t)levels * sizeof(int32_t), s);
+  k_depth_count<<<grid_blocks(2), 256, 0, s>>>(t->c, t->ncells, cnt);
+  k_depth_off<<<1, 1, 0, s>>>(cnt, levels, off, cursor);
+  k_depth_fill<<<grid_blocks(2), 256, 0, s>>>(t->c, t->ncells, cursor, D.cursor);
+  A.by_depth = D.cursor;
+  A.depth_off = off;
+  // the top levels of up to 2^8 cells a system by one block, then a launch a level
+  const int top = t->n_sys <= 4 ? std::min(levels, 9) : 0;
+  if (top > 0) {
+    A.l0 = 0;
+    A.l1 = top;
+    k_l2l_level<<<1, 256, 0, s>>>(A);
+  }
+  const unsigned grid = std::min<unsigned>(blocks_for(std::max(t->ncells, 1), 64), grid_blocks());
+  for (int level = top; level < levels; ++level) {
+    A.l0 = level;
+    A.l1 = level + 1;
+    k_l2l_level<<<grid, 64, 0, s>>>(A);
+  }
+  t->launches += levels - top + (top > 0) + 3;
   return check_cuda(cudaGetLastError(), "l2l launch");
 }
 

@@ -219,7 +219,9 @@ struct kdfmm_tree_s {
     int64_t* far_off = nullptr;          // per cell + 1
     int32_t* far_idx = nullptr;
     int64_t far_idx_cap = 0, cells_cap = 0;
-    int32_t* cursor = nullptr;           // per cell (fill cursors)
+    int32_t* cursor = nullptr;           // per cell (fill cursors, then the cells by depth)
+    int32_t* depth_tab = nullptr;        // per level: counts, offsets, cursors
+    int64_t depth_cap = 0;
     float* lcell32 = nullptr;            // 24 per cell
     double* lcell64 = nullptr;           // 20 per cell
     double* ltot = nullptr;              // 20 per cell: own + ancestors' expansions, at its com
