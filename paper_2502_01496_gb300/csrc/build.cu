@@ -63,7 +63,7 @@ __global__ void k_init(const double* __restrict__ x, const double* __restrict__ 
   bool ok = isfinite(xi) && isfinite(yi) && isfinite(zi) && isfinite(mi) && isfinite(hi) &&
             mi > 0.0 && (soft_kind == KDFMM_SOFT_M4 ? hi > 0.0 : hi >= 0.0);
   if (!ok) set_status(status, ST_NONFINITE);
-  b.x[i] = xi; b.y[i] = yi; b.z[i] = zi; b.m[i] = mi; b.h[i] = hi;
+  b.x[i] = xi; b.y[i] = yi; b.z[i] = zi; b.m[i] = mi;      // (h joins at the leaves)
   b.idx[i] = (int32_t)i;
 }
 
@@ -218,29 +218,39 @@ k_chunk_reduce(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_s
   const int rel0 = (b - off) * 8 * T;
   const int cnt = g.count - rel0;               // valid elements from the chunk start
   const int64_t base = (int64_t)g.first + rel0;
-  __shared__ Sum4 ws[kW];
+  __shared__ double ws[kW][4];
   __shared__ long long wk[kW][6];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  // block sums and boxes: the warps' subtrees, then (thread 0) the tree over them
-  auto block_reduce = [&](Sum4 v, long long lo[3], long long hi[3], Sum4& total, long long key[6]) {
-    v = warp_tree4(v);
+  // block sums and boxes: the perfect tree over the lanes as a reduce-scatter
+  // (two components, then one: 6 float64 additions a warp instead of 20, same
+  // bits: the pairs are those of the butterfly), then the tree over the warps.
+  // lane 0 .. 3 of warp 0 end with components m, y, x, z of the total, thread 0
+  // with the keys.
+  auto block_reduce = [&](const Sum4& v, long long lo[3], long long hi[3], double& total, long long key[6]) {
+    const unsigned full = 0xffffffffu;
+    const bool odd = lane & 1, second = lane & 2;
+    const double a0 = (odd ? v.y : v.m) + __shfl_xor_sync(full, odd ? v.m : v.y, 1);
+    const double a1 = (odd ? v.z : v.x) + __shfl_xor_sync(full, odd ? v.x : v.z, 1);
+    double s = (second ? a1 : a0) + __shfl_xor_sync(full, second ? a0 : a1, 2);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) s = __dadd_rn(s, __shfl_xor_sync(full, s, o));
 #pragma unroll
     for (int d = 0; d < 3; ++d) { lo[d] = warp_min_ll(lo[d]); hi[d] = warp_max_ll(hi[d]); }
     __syncthreads();
-    if (lane == 0) {
-      ws[w] = v;
+    if (lane < 4) ws[w][lane] = s;
+    if (lane == 0)
       for (int d = 0; d < 3; ++d) { wk[w][d] = lo[d]; wk[w][3 + d] = hi[d]; }
-    }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    Sum4 t4[kW];
+    if (threadIdx.x >= 4) return;
+    double t4[kW];
 #pragma unroll
-    for (int q = 0; q < kW; ++q) t4[q] = ws[q];
+    for (int q = 0; q < kW; ++q) t4[q] = ws[q][lane];
 #pragma unroll
     for (int width = kW; width > 1; width >>= 1)
 #pragma unroll
-      for (int q = 0; q < width / 2; ++q) t4[q] = add4(t4[2 * q], t4[2 * q + 1]);
+      for (int q = 0; q < width / 2; ++q) t4[q] = __dadd_rn(t4[2 * q], t4[2 * q + 1]);
     total = t4[0];
+    if (threadIdx.x != 0) return;
     for (int d = 0; d < 6; ++d) {
       long long r = wk[0][d];
       for (int q = 1; q < kW; ++q) r = d < 3 ? min(r, wk[q][d]) : max(r, wk[q][d]);
@@ -260,13 +270,12 @@ k_chunk_reduce(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_s
       return elem4(p.m[i], x, y, z);
     };
     const Sum4 v = block_tree<3>(8 * threadIdx.x, cnt, get);
-    Sum4 t;
+    double t;
     long long key[6];
     block_reduce(v, lo, hi, t, key);
-    if (threadIdx.x == 0) {
-      csum[4 * b + 0] = t.m; csum[4 * b + 1] = t.x; csum[4 * b + 2] = t.y; csum[4 * b + 3] = t.z;
-      for (int d = 0; d < 6; ++d) ckey[6 * b + d] = key[d];
-    }
+    if (threadIdx.x < 4) csum[4 * (int64_t)b + ((lane & 1) << 1 | lane >> 1)] = t;
+    if (threadIdx.x == 0)
+      for (int d = 0; d < 6; ++d) ckey[6 * (int64_t)b + d] = key[d];
   }
   const int C = nchunks_of<T>(g.count);
   if (!last_block(&seg_done[2 * s], C)) return;
@@ -298,14 +307,14 @@ k_chunk_reduce(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_s
       lo[d] = min(lo[d], __ldcg(&ckey[6 * (int64_t)(off + c) + d]));
       hi[d] = max(hi[d], __ldcg(&ckey[6 * (int64_t)(off + c) + 3 + d]));
     }
-  Sum4 t = zero4();
+  double t = 0.0;
   long long key[6] = {0, 0, 0, 0, 0, 0};
   block_reduce(v, lo, hi, t, key);
   if (w != 0) return;
   // the three divisions run once, on lanes 0, 1, 2
-  const double M = __shfl_sync(0xffffffffu, t.m, 0);
-  const double sx = __shfl_sync(0xffffffffu, t.x, 0), sy = __shfl_sync(0xffffffffu, t.y, 0),
-               sz = __shfl_sync(0xffffffffu, t.z, 0);
+  const double M = __shfl_sync(0xffffffffu, t, 0);
+  const double sx = __shfl_sync(0xffffffffu, t, 2), sy = __shfl_sync(0xffffffffu, t, 1),
+               sz = __shfl_sync(0xffffffffu, t, 3);
   const double quo = __ddiv_rn(lane == 1 ? sy : (lane == 2 ? sz : sx), M);
   const double cx = __shfl_sync(0xffffffffu, quo, 0), cy = __shfl_sync(0xffffffffu, quo, 1),
                cz = __shfl_sync(0xffffffffu, quo, 2);
@@ -328,19 +337,16 @@ k_chunk_reduce(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_s
   }
 }
 
-// Per chunk: particles left of the cut, and the largest float32 estimate of
-// the squared distance to the centre of mass (coordinates truncated to
-// float32 with integer operations; the exact size follows in the scatter).
-// Then, once per segment: offsets of the left particles per chunk, the split
-// point, the size's candidate threshold, and the two children.
+// Per chunk: particles left of the cut (one coordinate read).  Then, once per
+// segment: offsets of the left particles per chunk, the split point and the two
+// children.
 template <int T>
 __global__ void __launch_bounds__(T)
 k_chunk_count(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_seg,
               const int32_t* __restrict__ seg_off, const int32_t* __restrict__ counters, PCols p,
               const int32_t* __restrict__ seg_axis, const double* __restrict__ seg_cut,
-              int32_t* cleft, float* cs2, int32_t* seg_done, int32_t* __restrict__ cloff,
-              int32_t* __restrict__ seg_nl, const float* __restrict__ seg_xb,
-              float* __restrict__ seg_thr2, BuildArgs A, Seg* nextA, Seg* segB, Seg* segL, int dst_buf) {
+              int32_t* cleft, int32_t* seg_done, int32_t* __restrict__ cloff,
+              int32_t* __restrict__ seg_nl, BuildArgs A, Seg* nextA, Seg* segB, Seg* segL, int dst_buf) {
   constexpr int kW = T / 32;
   const int b = blockIdx.x;
   if (b >= counters[C_CHUNKS]) return;
@@ -351,47 +357,30 @@ k_chunk_count(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_se
   const int cnt = min(8 * T, g.count - rel0);
   const int64_t base = (int64_t)g.first + rel0;
   const int axis = seg_axis[s];
+  const double* const x = axis == 0 ? p.x : (axis == 1 ? p.y : p.z);
   const long long ckey = dkey(seg_cut[s]);
-  const float cx = trunc_to_float(A.tmp.cx[g.cell]), cy = trunc_to_float(A.tmp.cy[g.cell]),
-              cz = trunc_to_float(A.tmp.cz[g.cell]);
   int nl = 0;
-  float s2 = 0.0f;
 #pragma unroll
   for (int pass = 0; pass < 8; ++pass) {   // all loads in flight
     const int k = pass * T + threadIdx.x;
-    if (k >= cnt) continue;
-    int64_t i = base + k;
-    const double px = p.x[i], py = p.y[i], pz = p.z[i];
-    const double a = axis == 0 ? px : (axis == 1 ? py : pz);
-    nl += dkey(a) < ckey;
-    const float dx = trunc_to_float(px) - cx, dy = trunc_to_float(py) - cy, dz = trunc_to_float(pz) - cz;
-    s2 = fmaxf(s2, dx * dx + dy * dy + dz * dz);
+    if (k < cnt) nl += dkey(x[base + k]) < ckey;
   }
   __shared__ int wn[kW];
-  __shared__ float ws2[kW];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    nl += __shfl_xor_sync(0xffffffffu, nl, o);
-    s2 = fmaxf(s2, __shfl_xor_sync(0xffffffffu, s2, o));
-  }
-  if (lane == 0) { wn[w] = nl; ws2[w] = s2; }
+  nl = __reduce_add_sync(0xffffffffu, nl);
+  if (lane == 0) wn[w] = nl;
   __syncthreads();
   if (threadIdx.x == 0) {
     int t = 0;
-    float m2 = 0.0f;
-    for (int q = 0; q < kW; ++q) { t += wn[q]; m2 = fmaxf(m2, ws2[q]); }
+    for (int q = 0; q < kW; ++q) t += wn[q];
     cleft[b] = t;
-    cs2[b] = m2;
   }
   const int C = nchunks_of<T>(g.count);
   if (!last_block(&seg_done[2 * s + 1], C)) return;
   int run = 0;
-  s2 = 0.0f;
   for (int c0 = 0; c0 < C; c0 += T) {
     const int c = c0 + threadIdx.x;
     const int v = c < C ? __ldcg(&cleft[off + c]) : 0;
-    if (c < C) s2 = fmaxf(s2, __ldcg(&cs2[off + c]));
     int incl = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -411,17 +400,7 @@ k_chunk_count(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_se
     if (c < C) cloff[off + c] = run + before + incl - v;
     run += tot;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s2 = fmaxf(s2, __shfl_xor_sync(0xffffffffu, s2, o));
-  if (lane == 0) ws2[w] = s2;
-  __syncthreads();
   if (threadIdx.x != 0) return;
-  for (int q = 1; q < kW; ++q) s2 = fmaxf(s2, ws2[q]);
-  {
-    const float Dm = sqrtf(s2);
-    const float thr = Dm - 2.0f * dist_err_bound(seg_xb[s], Dm);
-    seg_thr2[s] = thr > 0.0f ? thr * thr * (1.0f - 1e-6f) : -1.0f;
-  }
   nl = run;
   const bool fallback = (nl == 0 || nl == g.count);
   if (fallback) {
@@ -456,7 +435,7 @@ k_chunk_scatter(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_
                 const int32_t* __restrict__ seg_off, const int32_t* __restrict__ counters, PCols src,
                 PCols dst, const int32_t* __restrict__ seg_axis, const double* __restrict__ seg_cut,
                 const int32_t* __restrict__ cloff, const int32_t* __restrict__ seg_nl,
-                TmpCells tmp, const float* __restrict__ seg_thr2) {
+                TmpCells tmp, const float* __restrict__ seg_xb) {
   const int b = blockIdx.x;
   if (b >= counters[C_CHUNKS]) return;
   const int s = chunk_seg[b];
@@ -471,6 +450,7 @@ k_chunk_scatter(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_
   const long long ckey = dkey(seg_cut[s]);
   __shared__ int wcount[kScatterPasses][T / 32];
   __shared__ long long ws2[T / 32];
+  __shared__ int wd2[T / 32];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const unsigned lt = (1u << lane) - 1u;
   bool flag[kScatterPasses];
@@ -504,36 +484,55 @@ k_chunk_scatter(const Seg* __restrict__ segs, const int32_t* __restrict__ chunk_
   }
   const double cx = tmp.cx[g.cell], cy = tmp.cy[g.cell], cz = tmp.cz[g.cell];
   const float cxf = trunc_to_float(cx), cyf = trunc_to_float(cy), czf = trunc_to_float(cz);
-  const float thr2 = seg_thr2[s];
-  long long s2 = 0;
-#pragma unroll 1
+  float d2[kScatterPasses], dmax = 0.0f;       // float32 squared distances to the centre of mass
+#pragma unroll
   for (int p0 = 0; p0 < kScatterPasses; p0 += kMoveBatch) {
-    double px[kMoveBatch], py[kMoveBatch], pz[kMoveBatch], pm[kMoveBatch], ph[kMoveBatch];
+    double px[kMoveBatch], py[kMoveBatch], pz[kMoveBatch], pm[kMoveBatch];
     int32_t pi[kMoveBatch];
 #pragma unroll
     for (int u = 0; u < kMoveBatch; ++u) {
       const int k = rel0 + (p0 + u) * T + threadIdx.x;
-      px[u] = py[u] = pz[u] = pm[u] = ph[u] = 0.0;
+      px[u] = py[u] = pz[u] = pm[u] = 0.0;
       pi[u] = 0;
       if (k < g.count) {
         const int64_t i = (int64_t)g.first + k;
         px[u] = src.x[i]; py[u] = src.y[i]; pz[u] = src.z[i];
-        pm[u] = src.m[i]; ph[u] = src.h[i]; pi[u] = src.idx[i];
+        pm[u] = src.m[i]; pi[u] = src.idx[i];
       }
     }
 #pragma unroll
     for (int u = 0; u < kMoveBatch; ++u) {
       const int k = rel0 + (p0 + u) * T + threadIdx.x;
+      d2[p0 + u] = -2.0f;
       if (k >= g.count) continue;
       const int lb = rank[p0 + u];
       const int64_t d = flag[p0 + u] ? (int64_t)g.first + lb : (int64_t)g.first + nl + (k - lb);
       dst.x[d] = px[u]; dst.y[d] = py[u]; dst.z[d] = pz[u];
-      dst.m[d] = pm[u]; dst.h[d] = ph[u]; dst.idx[d] = pi[u];
+      dst.m[d] = pm[u]; dst.idx[d] = pi[u];
       const float ex = trunc_to_float(px[u]) - cxf, ey = trunc_to_float(py[u]) - cyf,
                   ez = trunc_to_float(pz[u]) - czf;
-      if (ex * ex + ey * ey + ez * ez >= thr2)
-        s2 = max(s2, __double_as_longlong(dist2_rn(px[u], py[u], pz[u], cx, cy, cz)));
+      d2[p0 + u] = ex * ex + ey * ey + ez * ez;
+      dmax = fmaxf(dmax, d2[p0 + u]);
     }
+  }
+  // the chunk's largest exact distance, from the elements whose float32 distance
+  // is within its error of the chunk's largest (the segment's largest is the
+  // largest of its chunks')
+  const int dm = __reduce_max_sync(0xffffffffu, __float_as_int(dmax));
+  if (lane == 0) wd2[w] = dm;
+  __syncthreads();
+  int db = 0;
+#pragma unroll
+  for (int q = 0; q < T / 32; ++q) db = max(db, wd2[q]);
+  const float Dm = sqrtf(__int_as_float(db));
+  const float thr = Dm - 2.0f * dist_err_bound(seg_xb[s], Dm);
+  const float thr2 = thr > 0.0f ? thr * thr * (1.0f - 1e-6f) : -1.0f;
+  long long s2 = 0;
+#pragma unroll
+  for (int pass = 0; pass < kScatterPasses; ++pass) {
+    if (!(d2[pass] >= thr2)) continue;
+    const int64_t i = (int64_t)g.first + rel0 + pass * T + threadIdx.x;
+    s2 = max(s2, __double_as_longlong(dist2_rn(src.x[i], src.y[i], src.z[i], cx, cy, cz)));
   }
   s2 = warp_max_ll(s2);
   if (lane == 0) ws2[w] = s2;
@@ -554,6 +553,8 @@ struct SubArgs {
   PCols buf0, buf1, out;
   const Seg* segB;
   int qcap;
+  const double* h;                     // caller's smoothing lengths, or NULL: the systems' softening
+  const double* sys_eps;
 };
 
 // All cells of a tree level are processed together, in batches of up to
@@ -644,7 +645,8 @@ k_subtree(SubArgs S) {
   const Seg g = S.segB[s_seg];
   const PCols in = (g.dbuf & 1) ? S.buf1 : S.buf0;
   const int n = g.count, gfirst = g.first;
-  const int n_leaf = nleaf_at(A, gfirst);
+  const int sys = system_of(A.sys_off, A.n_sys, gfirst);
+  const int n_leaf = A.sys_nleaf[sys];
   for (int k = tid; k < n; k += kSubtreeThreads) {
     L.x[k] = in.x[gfirst + k]; L.y[k] = in.y[gfirst + k]; L.z[k] = in.z[gfirst + k];
     L.m[k] = in.m[gfirst + k];
@@ -971,8 +973,9 @@ k_subtree(SubArgs S) {
     const int src = L.fin[k];
     const int64_t p = (int64_t)gfirst + k;
     S.out.x[p] = L.x[src]; S.out.y[p] = L.y[src]; S.out.z[p] = L.z[src]; S.out.m[p] = L.m[src];
-    S.out.h[p] = in.h[gfirst + src];
-    S.out.idx[p] = in.idx[gfirst + src];
+    const int32_t i = in.idx[gfirst + src];
+    S.out.h[p] = S.h ? S.h[i] : S.sys_eps[sys];
+    S.out.idx[p] = i;
   }
   }
 }
@@ -1006,7 +1009,8 @@ __global__ void k_leaf_segs(SubArgs S, const Seg* __restrict__ segL) {
     const int64_t i = (int64_t)g.first + k;
     s2 = max(s2, __double_as_longlong(dist2_rn(in.x[i], in.y[i], in.z[i], cx, cy, cz)));
     S.out.x[i] = in.x[i]; S.out.y[i] = in.y[i]; S.out.z[i] = in.z[i];
-    S.out.m[i] = in.m[i]; S.out.h[i] = in.h[i]; S.out.idx[i] = in.idx[i];
+    S.out.m[i] = in.m[i]; S.out.idx[i] = in.idx[i];
+    S.out.h[i] = S.h ? S.h[in.idx[i]] : S.sys_eps[system_of(S.A.sys_off, S.A.n_sys, g.first)];
   }
   TmpCells t = S.A.tmp;
   const int c = g.cell;
@@ -1246,12 +1250,12 @@ inline unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + thre
 // ---------------------------------------------------------------------------
 // host orchestration
 // ---------------------------------------------------------------------------
-static int alloc_cols(PCols* c, int64_t n) {
+static int alloc_cols(PCols* c, int64_t n, bool with_h) {
   if (cudaMalloc(&c->x, n * sizeof(double)) != cudaSuccess) return -1;
   if (cudaMalloc(&c->y, n * sizeof(double)) != cudaSuccess) return -1;
   if (cudaMalloc(&c->z, n * sizeof(double)) != cudaSuccess) return -1;
   if (cudaMalloc(&c->m, n * sizeof(double)) != cudaSuccess) return -1;
-  if (cudaMalloc(&c->h, n * sizeof(double)) != cudaSuccess) return -1;
+  if (with_h && cudaMalloc(&c->h, n * sizeof(double)) != cudaSuccess) return -1;
   if (cudaMalloc(&c->idx, n * sizeof(int32_t)) != cudaSuccess) return -1;
   return 0;
 }
@@ -1264,8 +1268,8 @@ void free_build_buffers(kdfmm_tree_s* t) {
   for (int k = 0; k < 2; ++k) { free_cols(&t->buf[k]); cudaFree(t->segA[k]); t->segA[k] = nullptr; }
   free_cols(&t->tp);
   void* ptrs[] = {t->segB, t->segL, t->chunk_seg, t->seg_chunk_off, t->chunk_sum, t->chunk_key,
-                  t->chunk_left, t->chunk_loff, t->chunk_s2, t->seg_done, t->seg_axis, t->seg_cut, t->seg_nl,
-                  t->seg_xb, t->seg_thr2,
+                  t->chunk_left, t->chunk_loff, t->seg_done, t->seg_axis, t->seg_cut, t->seg_nl,
+                  t->seg_xb,
                   t->tmp.first, t->tmp.count, t->tmp.left, t->tmp.right, t->tmp.depth, t->tmp.M,
                   t->tmp.cx, t->tmp.cy, t->tmp.cz, t->tmp.s, t->starts, t->min_depth,
                   t->scan_tmp, t->pf, t->ph, t->c.first, t->c.count, t->c.left,
@@ -1278,7 +1282,7 @@ void free_build_buffers(kdfmm_tree_s* t) {
   t->chunk_seg = t->seg_chunk_off = t->chunk_left = t->chunk_loff = t->seg_axis = t->seg_nl = t->seg_done = nullptr;
   t->chunk_sum = t->seg_cut = nullptr;
   t->chunk_key = nullptr;
-  t->chunk_s2 = t->seg_xb = t->seg_thr2 = nullptr;
+  t->seg_xb = nullptr;
   t->tmp = TmpCells{};
   t->starts = nullptr;
   t->min_depth = t->scan_tmp = nullptr;
@@ -1302,8 +1306,8 @@ static int ensure_build_buffers(kdfmm_tree_s* t, int64_t n) {
   free_build_buffers(t);
   cudaGetLastError();
   for (int k = 0; k < 2; ++k)
-    if (alloc_cols(&t->buf[k], n)) return set_error(KDFMM_ERR_OOM, "particle buffers");
-  if (alloc_cols(&t->tp, n)) return set_error(KDFMM_ERR_OOM, "tree-order particles");
+    if (alloc_cols(&t->buf[k], n, false)) return set_error(KDFMM_ERR_OOM, "particle buffers");
+  if (alloc_cols(&t->tp, n, true)) return set_error(KDFMM_ERR_OOM, "tree-order particles");
   t->capA = n / kSubtreeMax + 4;
   t->capB = n / 2 + 4;
   t->capL = n / 4 + 64;
@@ -1318,14 +1322,12 @@ static int ensure_build_buffers(kdfmm_tree_s* t, int64_t n) {
   KD_ALLOC(t->chunk_key, 6 * t->cap_chunks);
   KD_ALLOC(t->chunk_left, t->cap_chunks);
   KD_ALLOC(t->chunk_loff, t->cap_chunks);
-  KD_ALLOC(t->chunk_s2, t->cap_chunks);
   KD_ALLOC(t->seg_chunk_off, t->capA);
   KD_ALLOC(t->seg_done, 2 * t->capA);
   KD_ALLOC(t->seg_axis, t->capA);
   KD_ALLOC(t->seg_cut, t->capA);
   KD_ALLOC(t->seg_nl, t->capA);
   KD_ALLOC(t->seg_xb, t->capA);
-  KD_ALLOC(t->seg_thr2, t->capA);
   t->cap_cells = 2 * n + 2;
   const int64_t nc = t->cap_cells;
   KD_ALLOC(t->tmp.first, nc); KD_ALLOC(t->tmp.count, nc); KD_ALLOC(t->tmp.left, nc);
@@ -1437,12 +1439,11 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
                                          t->chunk_sum, t->chunk_key, t->seg_done, t->tmp, t->seg_axis,
                                          t->seg_cut, t->seg_xb);
     k_chunk_count<T><<<maxc, T, 0, s>>>(segs, t->chunk_seg, t->seg_chunk_off, t->counters, t->buf[src],
-                                        t->seg_axis, t->seg_cut, t->chunk_left, t->chunk_s2, t->seg_done,
-                                        t->chunk_loff, t->seg_nl, t->seg_xb, t->seg_thr2, A, next,
-                                        t->segB, t->segL, dst);
+                                        t->seg_axis, t->seg_cut, t->chunk_left, t->seg_done,
+                                        t->chunk_loff, t->seg_nl, A, next, t->segB, t->segL, dst);
     k_chunk_scatter<T><<<maxc, T, 0, s>>>(segs, t->chunk_seg, t->seg_chunk_off, t->counters, t->buf[src],
                                           t->buf[dst], t->seg_axis, t->seg_cut, t->chunk_loff, t->seg_nl,
-                                          t->tmp, t->seg_thr2);
+                                          t->tmp, t->seg_xb);
   };
   while (deferred ? level < fixed_levels : hc[C_NEXT_A] > 0) {
     const int src = level & 1, dst = src ^ 1;
@@ -1475,6 +1476,8 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
   S.buf1 = t->buf[1];
   S.out = t->tp;
   S.segB = t->segB;
+  S.h = P.soft_kind == KDFMM_SOFT_M4 ? h : nullptr;
+  S.sys_eps = t->sys_eps;
   S.qcap = subtree_qcap(t->min_nleaf);
   const size_t smem = subtree_smem_for(S.qcap);
   if ((rc = subtree_setup(t, smem))) return rc;

@@ -72,7 +72,7 @@ struct Seg {
   int32_t dbuf;    // depth << 1 | buffer holding the particles
 };
 
-// Particle columns, float64, in one tree order.
+// Particle columns, float64, in one tree order (h: the final order only).
 struct PCols {
   double *x, *y, *z, *m, *h;
   int32_t* idx;    // caller index
@@ -161,9 +161,7 @@ struct kdfmm_tree_s {
   long long* chunk_key = nullptr;  // 6 per chunk: min xyz, max xyz
   int32_t* chunk_left = nullptr;
   int32_t* chunk_loff = nullptr;
-  float* chunk_s2 = nullptr;         // per chunk: largest float32 squared distance
   float* seg_xb = nullptr;           // per segment: bound on |coordinates|
-  float* seg_thr2 = nullptr;         // per segment: candidate threshold for the exact size
   int32_t* seg_done = nullptr;       // per segment: chunks that finished the reduce, the count
   int32_t* seg_axis = nullptr;
   double* seg_cut = nullptr;
