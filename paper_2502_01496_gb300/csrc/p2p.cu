@@ -470,7 +470,8 @@ __global__ void __launch_bounds__(kP2PWarps * 32, 6) k_p2p_mixed(P2PArgs A) {
   }
 }
 
-constexpr int kStage64 = 256;      // staged sources per warp and chunk (float64 path)
+constexpr int kStage64 = 192;      // staged sources per warp and chunk (float64 path; at most 256)
+constexpr int kQueue64 = 512;      // kernel pairs queued per warp
 constexpr int kP2P64Warps = 4;
 
 // One side of the symmetrised M4 pair in float64, added to f (force over
@@ -514,6 +515,10 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
   __shared__ float s_h2[M4 ? kP2P64Warps : 1][M4 ? kStage64 : 1];
   __shared__ uint8_t s_leaf[kP2P64Warps][kStage64];
   __shared__ int s_tbeg[kP2P64Warps][32], s_tfirst[kP2P64Warps][32];
+  constexpr int kW4 = M4 ? kP2P64Warps : 1;
+  __shared__ uint16_t s_queue[kW4][M4 ? kQueue64 : 1];    // kernel pairs: owner lane << 8 | source
+  __shared__ double s_term[kW4][4][M4 ? 32 : 1];
+  __shared__ unsigned s_own[kW4][M4 ? 32 : 1];            // a lane's entries of the batch
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned full = 0xffffffffu;
   const int nleaves = min(A.counters[C_LEAVES], A.max_leaves);
@@ -554,26 +559,60 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
       sh2[at] = A.ph[src].w;
     }
   };
-  // the lane's slice of the staged sources but `skip`.  M4, 128 sources of the
-  // slice at a time: every pair as 1/r^2 except those that may lie inside
-  // either support, which are marked and follow with the kernel (a warp
-  // branching per pair ran the kernel path for all its lanes whenever one
-  // needed it; the longer the stretch, the more alike the lanes' marks)
+  // the lane's slice of the staged sources but `skip`: pairs outside both
+  // supports as 1/r^2.  M4: those that may lie inside are queued by source
+  // (ballots), and the warp takes 32 of them at a time, whatever lanes they
+  // belong to: the pair's target comes by shuffle, its terms go back through
+  // shared memory, each lane adding its own in queue order.  Left to their own
+  // lanes the kernel pairs (a twentieth of all) kept a warp busy for as long as
+  // its unluckiest lane and took 40 % of the kernel.
+  auto kernel_pairs = [&](int nq) {
+    __syncwarp();
+    for (int i0 = 0; i0 < nq; i0 += 32) {
+      const bool v = i0 + lane < nq;
+      const int e = v ? s_queue[warp][i0 + lane] : 0, o = e >> 8, j = e & 255;
+      const double tx = __shfl_sync(full, xi, o), ty = __shfl_sync(full, yi, o),
+                   tz = __shfl_sync(full, zi, o);
+      const double hi = __shfl_sync(full, hinv_i, o), h3i = __shfl_sync(full, h3inv_i, o);
+      s_own[warp][lane] = 0u;
+      const unsigned mine = __match_any_sync(full, v ? o : 32);
+      __syncwarp();
+      if (v) {
+        if ((mine & ((1u << lane) - 1u)) == 0u) s_own[warp][o] = mine;
+        const double rx = tx - sx[j], ry = ty - sy[j], rz = tz - sz[j];
+        const double r2 = fma(rz, rz, fma(ry, ry, fma(rx, rx, soft2)));
+        const double inv = rsqrt64(r2), r = r2 * inv, inv3 = inv * inv * inv;
+        const double hj = shinv[j], mh = 0.5 * sm[j];
+        double f = 0.0, p = 0.0;
+        m4_side64(r, inv, inv3, hi, h3i, f, p);
+        m4_side64(r, inv, inv3, hj, hj * hj * hj, f, p);
+        f *= mh;
+        s_term[warp][0][lane] = f * rx;
+        s_term[warp][1][lane] = f * ry;
+        s_term[warp][2][lane] = f * rz;
+        s_term[warp][3][lane] = mh * p;
+      }
+      __syncwarp();
+      for (unsigned m = s_own[warp][lane]; m != 0u; m &= m - 1u) {
+        const int k2 = __ffs(m) - 1;
+        fx -= s_term[warp][0][k2];
+        fy -= s_term[warp][1][k2];
+        fz -= s_term[warp][2][k2];
+        fp -= s_term[warp][3][k2];
+      }
+      __syncwarp();
+    }
+  };
   auto sum_staged = [&](int total, int skip) {
-    for (int j0 = sl; j0 < total; j0 += 128 * K) {
-      uint32_t in[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        for (int b = 0; b < 32; ++b) {
-          const int j = j0 + (32 * w + b) * K;
-          if (j >= total) break;
-          if (j == skip) continue;
-          const double rx = xi - sx[j], ry = yi - sy[j], rz = zi - sz[j];
-          const double r2 = fma(rz, rz, fma(ry, ry, fma(rx, rx, soft2)));
-          if (M4 && maybe_inside(r2, h2i, sh2[j])) {
-            in[w] |= 1u << b;
-            continue;
-          }
+    int nq = 0;
+    for (int j0 = 0; j0 < total; j0 += K) {
+      const int j = j0 + sl;
+      bool in = false;
+      if (act && j < total && j != skip) {
+        const double rx = xi - sx[j], ry = yi - sy[j], rz = zi - sz[j];
+        const double r2 = fma(rz, rz, fma(ry, ry, fma(rx, rx, soft2)));
+        in = M4 && maybe_inside(r2, h2i, sh2[j]);
+        if (!in) {
           const double inv = rsqrt64(r2);
           const double minv = sm[j] * inv, f = minv * (inv * inv);
           fx = fma(-f, rx, fx); fy = fma(-f, ry, fy); fz = fma(-f, rz, fz);
@@ -581,31 +620,25 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
         }
       }
       if constexpr (M4) {
-#pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        uint32_t msk = in[w];
-        while (msk != 0u) {
-          const int j = j0 + (32 * w + __ffs(msk) - 1) * K;
-          msk &= msk - 1u;
-          const double rx = xi - sx[j], ry = yi - sy[j], rz = zi - sz[j];
-          const double r2 = fma(rz, rz, fma(ry, ry, fma(rx, rx, soft2)));
-          const double inv = rsqrt64(r2), r = r2 * inv, inv3 = inv * inv * inv;
-          const double hj = shinv[j], mh = 0.5 * sm[j];
-          double f = 0.0, p = 0.0;
-          m4_side64(r, inv, inv3, hinv_i, h3inv_i, f, p);
-          m4_side64(r, inv, inv3, hj, hj * hj * hj, f, p);
-          f *= mh;
-          fx = fma(-f, rx, fx); fy = fma(-f, ry, fy); fz = fma(-f, rz, fz);
-          fp = fma(-mh, p, fp);
+        const unsigned marks = __ballot_sync(full, in);
+        if (marks != 0u) {
+          if (in) s_queue[warp][nq + __popc(marks & ((1u << lane) - 1u))] = (uint16_t)(lane << 8 | j);
+          nq += __popc(marks);
+          if (nq > kQueue64 - 32) {
+            kernel_pairs(nq);
+            nq = 0;
+          }
         }
       }
-      }
+    }
+    if constexpr (M4) {
+      if (nq > 0) kernel_pairs(nq);
     }
   };
   if (!seg) {
     if (lane < nt) stage(lane, (int64_t)fa + lane);
     __syncwarp();
-    if (act) sum_staged(nt, t);
+    sum_staged(nt, t);
     __syncwarp();
   }
   const int64_t nall = min((int64_t)A.near_cnt[k], A.cap_near);
@@ -642,7 +675,7 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
       stage(idx, (int64_t)tf[l] + idx - tb[l]);
     }
     __syncwarp();
-    if (act) sum_staged(total, -1);
+    sum_staged(total, -1);
     __syncwarp();
     e += L;
   }
