@@ -807,13 +807,15 @@ static int arena_grid_for(int leaves) {
                                                      (int64_t)per_sm * sms));
 }
 
-// Lanes per leaf of the slot-mode walk: as many as one round of resident
-// threads allows (32 up to 6080 leaves on 152 SMs), one beyond 48640 leaves, where
-// the thread walk has the GPU's threads busy by itself.
+// Lanes per leaf of the slot-mode walk: 32 while that is at most two rounds of
+// resident threads (12160 leaves on 152 SMs), else as many as one round allows,
+// one beyond 48640 leaves, where the thread walk has the GPU's threads busy by
+// itself.
 static int split_lanes(int leaves) {
-  const int64_t threads = (int64_t)sm_count() * 10 * 128;
-  for (int k = 32; k >= 4; k >>= 1)
-    if ((int64_t)std::max(leaves, 1) * k <= threads) return k;
+  const int64_t threads = (int64_t)sm_count() * 10 * 128, n = std::max(leaves, 1);
+  if (32 * n <= 2 * threads) return 32;
+  for (int k = 8; k >= 4; k >>= 1)
+    if (k * n <= threads) return k;
   return 1;
 }
 
@@ -898,7 +900,6 @@ static void walk_launch(kdfmm_tree_s* t, WalkArgs W, ListMode mode, int64_t cf, 
     const unsigned grid = blocks_for((int64_t)std::max(slot_leaves, 1) * lanes, 128);
     switch (lanes) {
       case 32: k_walk_split<32><<<grid, 128, 0, s>>>(W); break;
-      case 16: k_walk_split<16><<<grid, 128, 0, s>>>(W); break;
       case 8: k_walk_split<8><<<grid, 128, 0, s>>>(W); break;
       case 4: k_walk_split<4><<<grid, 128, 0, s>>>(W); break;
       default: k_walk<<<grid, 128, 0, s>>>(W);

@@ -15,10 +15,9 @@ def _lists(f):
 
 
 # leaves of one particle: as many leaves as particles.  On a GPU of 152 SMs 32
-# lanes serve a leaf up to 6080 leaves, 16 to 12160, 8 to 24320, 4 to 48640, one
-# beyond; theta = 0 with 20000 leaves overflows a lane's scratch of 512 entries
+# lanes serve a leaf up to 12160 leaves, 8 to 24320, 4 to 48640, one beyond; theta = 0 with 20000 leaves overflows a lane's scratch of 512 entries
 @pytest.mark.parametrize("n,theta", [(1, 0.5), (2, 0.5), (31, 0.5), (33, 0.0), (700, 0.4), (6080, 0.7),
-                                     (6081, 0.7), (12161, 0.8), (24321, 0.9), (48641, 1.0), (20000, 0.0)])
+                                     (6081, 0.7), (12160, 0.8), (12161, 0.8), (24321, 0.9), (48641, 1.0), (20000, 0.0)])
 def test_split_walk_equals_thread_walk(n, theta, monkeypatch):
     import torch
     from paper_2502_01496_gb300 import native
