@@ -254,8 +254,9 @@ __global__ void __launch_bounds__(kP2PWarps * 32, 6) k_p2p_mixed(P2PArgs A) {
   constexpr int R = M4 ? kStageRounds / 2 : kStageRounds;
   __shared__ float4 s_pos[kP2PWarps][kStageCap];
   __shared__ float4 s_ker[M4 ? kP2PWarps : 1][M4 ? kStageCap : 1];
-  __shared__ int s_tbeg[kP2PWarps][32], s_tfirst[kP2PWarps][32];   // chunk's leaves: staged start, first
-  __shared__ float4 s_toff[kP2PWarps][32];                          // and offset to the target com
+  __shared__ int s_tbeg[kP2PWarps][32];                    // chunk's leaves: first particle - staged start
+  __shared__ float4 s_toff[kP2PWarps][32];                 // and offset to the target com
+  __shared__ unsigned s_bits[kP2PWarps][kStageCap / 32];   // staged starts
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nleaves = min(A.counters[C_LEAVES], A.max_leaves);
   const int nitems = nleaves + (int)min((int64_t)A.counters[C_SEGS], A.seg_cap);
@@ -267,7 +268,6 @@ __global__ void __launch_bounds__(kP2PWarps * 32, 6) k_p2p_mixed(P2PArgs A) {
   float4* sp = s_pos[warp];
   float4* sk = s_ker[M4 ? warp : 0];
   int* tb = s_tbeg[warp];
-  int* tf = s_tfirst[warp];
   float4* toff = s_toff[warp];
   const int a = A.leaf_cells[k];
   const int fa = A.cfirst[a], nt = A.ccount[a];
@@ -317,33 +317,39 @@ __global__ void __launch_bounds__(kP2PWarps * 32, 6) k_p2p_mixed(P2PArgs A) {
       if (lane >= o) incl += w;
     }
     const int L = __popc(__ballot_sync(full, my < e1 && incl <= kStageCap));
-    // stage the chunk's sources with flat indexing: lane r*32 + lane of a
-    // batch of R rounds takes staged index idx, finds its leaf by
-    // binary search over the leaves' starts, and every load of the batch is
-    // issued before any is used (the loads are L2 gathers: latency-bound)
-    if (lane < L) {
-      tb[lane] = incl - cnt;
-      tf[lane] = first;
-      toff[lane] = make_float4(dx, dy, dz, 0.0f);
+    // stage the chunk's sources with flat indexing: a lane takes staged index
+    // idx = 32 round + lane; the leaf of idx is the number of leaves that start
+    // at or before it, counted on a bitmap of the starts (one word a round, so a
+    // population count; a binary search over the starts took a sixth of the
+    // kernel on Plummer spheres).  Every load of a batch of R rounds is issued
+    // before any is used (the loads are L2 gathers: latency-bound)
+    const bool has = lane < L && cnt > 0;
+    const unsigned leaves = __ballot_sync(full, has);
+    if (lane < kStageCap / 32) s_bits[warp][lane] = 0u;
+    __syncwarp();
+    if (has) {
+      const int slot = __popc(leaves & lt), beg = incl - cnt;
+      tb[slot] = first - beg;             // particle = tb + staged index
+      toff[slot] = make_float4(dx, dy, dz, 0.0f);
+      atomicOr(&s_bits[warp][beg >> 5], 1u << (beg & 31));
     }
     __syncwarp();
     const int total = __shfl_sync(full, incl, L - 1);
-    int nN = 0, nK = 0;
+    int nN = 0, nK = 0, before = -1;      // leaves that start before the round, minus one
     for (int r0 = 0; r0 < total; r0 += 32 * R) {
       float4 pv[R], hv[R];
       int lv[R];
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         const int idx = r0 + 32 * r + lane;
-        int l = 0;
-#pragma unroll
-        for (int step = 16; step > 0; step >>= 1)
-          if (l + step < L && tb[l + step] <= idx) l += step;
+        const unsigned starts = r0 + 32 * r < total ? s_bits[warp][(r0 >> 5) + r] : 0u;
+        const int l = before + __popc(starts & (lt << 1 | 1u));
+        before += __popc(starts);
         lv[r] = l;
         pv[r] = make_float4(0.f, 0.f, 0.f, 0.f);
         hv[r] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (idx < total) {
-          const int src = tf[l] + idx - tb[l];
+          const int src = tb[l] + idx;
           pv[r] = A.pf[src];
           if (M4) hv[r] = A.ph[src];
         }
