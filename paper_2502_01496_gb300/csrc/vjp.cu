@@ -879,8 +879,8 @@ struct LeafChunk {
 // Stages the records of the leading leaves of the entries' cells (cell: this
 // lane's, or -1) that fit; returns their number.  The loads of a batch of rounds
 // are issued before any is used (L2 gathers: latency-bound).
-template <class Put>
-__device__ __forceinline__ int stage_chunk(const VjpArgs& V, LeafChunk& B, int lane, int cell, Put put) {
+template <class Chunk, class Put>
+__device__ __forceinline__ int stage_chunk(const VjpArgs& V, Chunk& B, int lane, int cell, Put put) {
   const unsigned full = 0xffffffffu;
   int cnt = 0;
   __syncwarp();
@@ -1127,183 +1127,223 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source32(VjpArgs V) {
   }
 }
 
-// Float64 f and g of the M4 pair, r2 > 0 or = 0 (finite: the q < 1 form).
-__device__ __forceinline__ void m4_fg64(double r2, double hinv_i, double hinv_j, double& f, double& g) {
-  const double inv = rsqrt64(fmax(r2, 1e-290));
-  const double r = r2 * inv;
-  const double inv2 = inv * inv, inv3 = inv2 * inv, inv5 = inv3 * inv2;
-  const double hs[2] = {hinv_i, hinv_j};
+// One side of the symmetrised M4 pair in float64, added to f and g: the branches
+// of q < 1 (v = q) and q >= 1 (v = 2 - q, 0 outside the support) as one
+// evaluation with selected constants.
+__device__ __forceinline__ void m4_fg64(double r, double inv3, double inv5, double hinv, double& f,
+                                        double& g) {
+  const double q = r * hinv, q2 = q * q, h2inv = hinv * hinv, h3inv = h2inv * hinv;
+  const bool in = __double2hiint(q) < 0x3ff00000;            // q < 1 (q >= 0)
+  const double t = 2.0 - q;
+  const double v = in ? q : (__double2hiint(t) < 0 ? 0.0 : t), v2 = v * v;
+  const double p1 = fma(v, fma(v, in ? 0.0 : -1.0 / 6.0, in ? 0.5 : 0.8), in ? -1.2 : -1.0);
+  const double F = fma(in ? v2 : v2 * v2, p1, in ? 4.0 / 3.0 : 1.0);
+  const double G = in ? fma(1.5, q, -2.4) : fma(-3.0, F, v2 * v * (q2 * q));
+  f = fma(F, in ? h3inv : inv3, f);
+  g = fma(G, in ? h3inv * h2inv : inv5, g);
+}
+__device__ __forceinline__ void m4_pair_fg64(double r2, double hinv_i, double hinv_j, double& f, double& g) {
+  const double inv = rsqrt64(r2), inv2 = inv * inv, inv3 = inv2 * inv, inv5 = inv3 * inv2, r = r2 * inv;
   f = g = 0.0;
-#pragma unroll
-  for (int side = 0; side < 2; ++side) {
-    const double hinv = hs[side], q = r * hinv;
-    if (q < 1.0) {
-      const double h2inv = hinv * hinv, h3inv = h2inv * hinv;
-      f += (4.0 / 3.0 + q * q * (-1.2 + 0.5 * q)) * h3inv;
-      g += (-2.4 + 1.5 * q) * (h3inv * h2inv);
-    } else {
-      const double t = fmax(2.0 - q, 0.0);
-      const double t3 = t * t * t;
-      const double F = 1.0 - t3 * t * (1.0 + t * (-0.8 + t * (1.0 / 6.0)));
-      f += F * inv3;
-      g += (t3 * (q * q * q) - 3.0 * F) * inv5;
-    }
-  }
+  m4_fg64(r, inv3, inv5, hinv_i, f, g);
+  m4_fg64(r, inv3, inv5, hinv_j, f, g);
   f *= 0.5;
   g *= 0.5;
 }
 
-// FP64 mode, target side (as k_vjp_target32, in float64).  x_bar_i gets
-// -(a_bar_i sum m f + sum m g (d.a_bar_i) d).  M4: pairs outside both supports
-// first (f = r^-3, g = -3 r^-5), those that may be inside are marked and
-// follow with the kernel, so that a warp does not run both paths per pair.
-template <int SOFT>
-__global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target64(VjpArgs V) {
+// A chunk of list entries in float64: positions, w (the target side: m in w0;
+// the source side: a_bar), 1/h, (2h)^2, particle; the pairs inside a support
+// queued for the warp as in the evaluation's P2P.
+struct Chunk64 {
+  double x[kVjpStage], y[kVjpStage], z[kVjpStage], w0[kVjpStage], w1[kVjpStage], w2[kVjpStage],
+      hinv[kVjpStage];
+  float h2[kVjpStage];
+  int id[kVjpStage];
+  int beg[33], first[32];
+  double term[4][32];
+  unsigned own[32];
+  uint16_t queue[512];
+};
+
+// FP64 mode, one kernel for both sides (SOURCE: the source side), warp per own
+// leaf and piece, lanes = (own particle, slice).  With d = x_i - x_j (i the
+// target), f and g of the pair: the target side sums m_j f and m_j g (d.b_i) d,
+// the source side f b_i + g (d.b_i) d and -f d.b_i.  Pairs outside both supports
+// first (f = r^-3, g = -3 r^-5); those that may be inside follow 32 at a time
+// from a queue, whatever lanes they belong to.  Bound by the float64 pipe (28
+// operations a pair outside the supports, some 60 inside).
+template <int SOFT, bool SOURCE>
+__global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_pairs64(VjpArgs V) {
   constexpr bool M4 = SOFT == KDFMM_SOFT_M4;
+  __shared__ Chunk64 s_chunk[kVjpWarps];
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const int nitems = near_items(V);
+  const unsigned lt = (1u << lane) - 1u;
+  Chunk64& B = s_chunk[threadIdx.x >> 5];
+  const int nitems = SOURCE ? V.nleaves + (int)min((int64_t)V.tctr[1], V.tseg_cap) : near_items(V);
   for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
        item += (int)((gridDim.x * blockDim.x) >> 5)) {
     const bool seg = item >= V.nleaves;
     const int gi = item - V.nleaves;
-    int k;
+    int k, nn;
     int64_t e0 = 0;
-    const int nn = near_item(V, item, &k, &e0);
+    if (SOURCE) {
+      k = seg ? V.tseg_leaf[gi] : item;
+      const int piece = seg ? gi - V.tseg_first[k] + 1 : 0;
+      e0 = V.toff[k] + (int64_t)piece * V.entries;
+      nn = min(V.tcnt[k] - piece * V.entries, V.entries);
+    } else {
+      nn = near_item(V, item, &k, &e0);
+    }
     const int a = V.leaf_cells[k];
     const int fa = V.c.first[a], nt = V.c.count[a];
     const int K = 32 / nt, t = lane % nt, sl = lane / nt;
     const bool act = sl < K;
-    const int64_t pi = (int64_t)fa + t;
-    const double xi = V.tp.x[pi], yi = V.tp.y[pi], zi = V.tp.z[pi];
-    const double b0 = V.ab[3 * pi], b1 = V.ab[3 * pi + 1], b2 = V.ab[3 * pi + 2];
-    const float h2i = M4 ? V.ph[pi].w : 0.0f;
-    const double hinv_i = M4 ? V.hinv[pi] : 0.0;
-    const double eps = V.sys_eps[V.leaf_sys[k]], eps2 = M4 ? 0.0 : eps * eps;
-    double sf = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
-    for (int e = 0; act && e < nn; ++e) {
-      const int bc = V.near_idx[e0 + e];
-      const int fb = V.c.first[bc], nb = V.c.count[bc];
-      unsigned in = 0u;
-      for (int j = sl; j < nb; j += K) {
-        const int64_t pj = (int64_t)fb + j;
-        if (pj == pi) continue;
-        const double d0 = xi - V.tp.x[pj], d1 = yi - V.tp.y[pj], d2 = zi - V.tp.z[pj];
-        const double r2 = fma(d2, d2, fma(d1, d1, fma(d0, d0, eps2)));
-        if (M4 && maybe_inside(r2, h2i, V.ph[pj].w)) { in |= 1u << j; continue; }
-        const double inv = rsqrt64(r2), inv2 = inv * inv;
-        const double mf = V.tp.m[pj] * (inv2 * inv);
-        const double db = d0 * b0 + d1 * b1 + d2 * b2;
-        const double u = -3.0 * (mf * inv2) * db;
-        sf += mf;
-        gx = fma(u, d0, gx); gy = fma(u, d1, gy); gz = fma(u, d2, gz);
+    const int64_t own = (int64_t)fa + t;
+    const double xo = V.tp.x[own], yo = V.tp.y[own], zo = V.tp.z[own];
+    const double b0 = SOURCE ? 0.0 : V.ab[3 * own], b1 = SOURCE ? 0.0 : V.ab[3 * own + 1],
+                 b2 = SOURCE ? 0.0 : V.ab[3 * own + 2];
+    const float h2o = M4 ? V.ph[own].w : 0.0f;
+    const double hinv_o = M4 ? V.hinv[own] : 0.0;
+    const double eps = V.sys_eps[V.leaf_sys[k]];
+    const double soft2 = M4 ? 1e-290 : eps * eps;    // (M4: 1/r finite for coincident particles)
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;   // vector sum and scalar sum
+    // a pair's terms: f, g, own or partner's b, d, partner's mass
+    auto terms = [&](double f, double g, double c0, double c1, double c2, double d0, double d1, double d2,
+                     double m, double out[4]) {
+      const double db = d0 * c0 + d1 * c1 + d2 * c2;
+      if (SOURCE) {
+        const double u = g * db;
+        out[0] = fma(f, c0, u * d0);
+        out[1] = fma(f, c1, u * d1);
+        out[2] = fma(f, c2, u * d2);
+        out[3] = -f * db;
+      } else {
+        const double u = m * g * db;
+        out[0] = u * d0;
+        out[1] = u * d1;
+        out[2] = u * d2;
+        out[3] = m * f;
       }
-      while (M4 && in != 0u) {
-        const int j = __ffs(in) - 1;
-        in &= in - 1u;
-        const int64_t pj = (int64_t)fb + j;
-        const double d0 = xi - V.tp.x[pj], d1 = yi - V.tp.y[pj], d2 = zi - V.tp.z[pj];
-        double f, g;
-        m4_fg64(d0 * d0 + d1 * d1 + d2 * d2, hinv_i, V.hinv[pj], f, g);
-        const double mj = V.tp.m[pj];
-        const double u = mj * g * (d0 * b0 + d1 * b1 + d2 * b2);
-        sf = fma(mj, f, sf);
-        gx = fma(u, d0, gx); gy = fma(u, d1, gy); gz = fma(u, d2, gz);
+    };
+    auto kernel_pairs = [&](int nq) {
+      __syncwarp();
+      for (int i0 = 0; i0 < nq; i0 += 32) {
+        const bool v = i0 + lane < nq;
+        const int e = v ? B.queue[i0 + lane] : 0, o = e >> 8, j = e & 255;
+        const double ox = __shfl_sync(full, xo, o), oy = __shfl_sync(full, yo, o),
+                     oz = __shfl_sync(full, zo, o), oh = __shfl_sync(full, hinv_o, o);
+        double c0 = 0.0, c1 = 0.0, c2 = 0.0;
+        if (!SOURCE) {
+          c0 = __shfl_sync(full, b0, o);
+          c1 = __shfl_sync(full, b1, o);
+          c2 = __shfl_sync(full, b2, o);
+        }
+        B.own[lane] = 0u;
+        const unsigned mine = __match_any_sync(full, v ? o : 32);
+        __syncwarp();
+        if (v) {
+          if ((mine & lt) == 0u) B.own[o] = mine;
+          if (SOURCE) { c0 = B.w0[j]; c1 = B.w1[j]; c2 = B.w2[j]; }
+          const double d0 = SOURCE ? B.x[j] - ox : ox - B.x[j], d1 = SOURCE ? B.y[j] - oy : oy - B.y[j],
+                       d2 = SOURCE ? B.z[j] - oz : oz - B.z[j];
+          double f, g, out[4];
+          m4_pair_fg64(fma(d2, d2, fma(d1, d1, fma(d0, d0, soft2))), oh, B.hinv[j], f, g);
+          terms(f, g, c0, c1, c2, d0, d1, d2, B.w0[j], out);
+          for (int q = 0; q < 4; ++q) B.term[q][lane] = out[q];
+        }
+        __syncwarp();
+        for (unsigned m = B.own[lane]; m != 0u; m &= m - 1u) {
+          const int q = __ffs(m) - 1;
+          s0 += B.term[0][q]; s1 += B.term[1][q]; s2 += B.term[2][q]; s3 += B.term[3][q];
+        }
+        __syncwarp();
       }
+    };
+    for (int eb = 0; eb < nn;) {
+      int cell = -1;
+      if (eb + lane < nn)
+        cell = SOURCE ? V.leaf_cells[V.tidx[e0 + eb + lane]] : V.near_idx[e0 + eb + lane];
+      const int L = stage_chunk(V, B, lane, cell, [&](int at, int p) {
+        B.x[at] = V.tp.x[p]; B.y[at] = V.tp.y[p]; B.z[at] = V.tp.z[p];
+        if (SOURCE) {
+          B.w0[at] = V.ab[3 * (int64_t)p];
+          B.w1[at] = V.ab[3 * (int64_t)p + 1];
+          B.w2[at] = V.ab[3 * (int64_t)p + 2];
+        } else {
+          B.w0[at] = V.tp.m[p];
+        }
+        if (M4) { B.hinv[at] = V.hinv[p]; B.h2[at] = V.ph[p].w; }
+        B.id[at] = p;
+      });
+      const int total = B.beg[L];
+      int nq = 0;
+      for (int j0 = 0; j0 < total; j0 += K) {
+        const int j = j0 + sl;
+        bool in = false;
+        if (act && j < total && B.id[j] != (int)own) {
+          const double d0 = SOURCE ? B.x[j] - xo : xo - B.x[j], d1 = SOURCE ? B.y[j] - yo : yo - B.y[j],
+                       d2 = SOURCE ? B.z[j] - zo : zo - B.z[j];
+          const double r2 = fma(d2, d2, fma(d1, d1, fma(d0, d0, soft2)));
+          in = M4 && maybe_inside(r2, h2o, B.h2[j]);
+          if (!in) {
+            const double inv = rsqrt64(r2), inv2 = inv * inv;
+            if (SOURCE) {
+              const double c0 = B.w0[j], c1 = B.w1[j], c2 = B.w2[j], f = inv2 * inv;
+              const double fdb = f * (d0 * c0 + d1 * c1 + d2 * c2), u = -3.0 * inv2 * fdb;
+              s0 = fma(f, c0, fma(u, d0, s0));
+              s1 = fma(f, c1, fma(u, d1, s1));
+              s2 = fma(f, c2, fma(u, d2, s2));
+              s3 -= fdb;
+            } else {
+              const double mf = B.w0[j] * (inv2 * inv);
+              const double u = -3.0 * (mf * inv2) * (d0 * b0 + d1 * b1 + d2 * b2);
+              s3 += mf;
+              s0 = fma(u, d0, s0); s1 = fma(u, d1, s1); s2 = fma(u, d2, s2);
+            }
+          }
+        }
+        if constexpr (M4) {
+          const unsigned marks = __ballot_sync(full, in);
+          if (marks != 0u) {
+            if (in) B.queue[nq + __popc(marks & lt)] = (uint16_t)(lane << 8 | j);
+            nq += __popc(marks);
+            if (nq > 512 - 32) {
+              kernel_pairs(nq);
+              nq = 0;
+            }
+          }
+        }
+      }
+      if constexpr (M4) {
+        if (nq > 0) kernel_pairs(nq);
+      }
+      eb += L;
     }
-    gx = -fma(sf, b0, gx); gy = -fma(sf, b1, gy); gz = -fma(sf, b2, gz);
+    if (!SOURCE) {                     // x_bar_i: -(b_i sum m f + sum m g (d.b_i) d)
+      s0 = -fma(s3, b0, s0); s1 = -fma(s3, b1, s1); s2 = -fma(s3, b2, s2);
+    }
     for (int s = 1; s < K; ++s) {
       const int src = t + s * nt;
-      const double ox = __shfl_sync(full, gx, src), oy = __shfl_sync(full, gy, src),
-                   oz = __shfl_sync(full, gz, src);
-      if (sl == 0) { gx += ox; gy += oy; gz += oz; }
+      const double q0 = __shfl_sync(full, s0, src), q1 = __shfl_sync(full, s1, src),
+                   q2 = __shfl_sync(full, s2, src), q3 = __shfl_sync(full, s3, src);
+      if (sl == 0) { s0 += q0; s1 += q1; s2 += q2; s3 += q3; }
     }
     if (act && sl == 0) {
-      if (seg) {
+      if (SOURCE) {
+        const double mj = V.tp.m[own];
+        atomicAdd(&V.xsrc[3 * own], mj * s0);
+        atomicAdd(&V.xsrc[3 * own + 1], mj * s1);
+        atomicAdd(&V.xsrc[3 * own + 2], mj * s2);
+        atomicAdd(&V.msrc[own], s3);
+      } else if (seg) {
         double* P = V.seg_part + (int64_t)gi * 128 + 4 * t;
-        P[0] = gx; P[1] = gy; P[2] = gz;
+        P[0] = s0; P[1] = s1; P[2] = s2;
       } else {
-        V.xbar[3 * pi] += gx;
-        V.xbar[3 * pi + 1] += gy;
-        V.xbar[3 * pi + 2] += gz;
+        V.xbar[3 * own] += s0;
+        V.xbar[3 * own + 1] += s1;
+        V.xbar[3 * own + 2] += s2;
       }
-    }
-  }
-}
-
-// FP64 mode, source side (as k_vjp_source32, in float64):
-// x_bar_j += m_j sum_i (f a_bar_i + g (d.a_bar_i) d), m_bar_j -= sum_i f d.a_bar_i.
-template <int SOFT>
-__global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source64(VjpArgs V) {
-  constexpr bool M4 = SOFT == KDFMM_SOFT_M4;
-  const unsigned full = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const int nitems = V.nleaves + (int)min((int64_t)V.tctr[1], V.tseg_cap);
-  for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
-       item += (int)((gridDim.x * blockDim.x) >> 5)) {
-    const bool seg = item >= V.nleaves;
-    const int r = seg ? V.tseg_leaf[item - V.nleaves] : item;
-    const int piece = seg ? item - V.nleaves - V.tseg_first[r] + 1 : 0;
-    const int a = V.leaf_cells[r];
-    const int fa = V.c.first[a], ns = V.c.count[a];
-    const int K = 32 / ns, js = lane % ns, sl = lane / ns;
-    const bool act = sl < K;
-    const int64_t pj = (int64_t)fa + js;
-    const double xj = V.tp.x[pj], yj = V.tp.y[pj], zj = V.tp.z[pj];
-    const float h2j = M4 ? V.ph[pj].w : 0.0f;
-    const double hinv_j = M4 ? V.hinv[pj] : 0.0;
-    const double eps = V.sys_eps[V.leaf_sys[r]], eps2 = M4 ? 0.0 : eps * eps;
-    double g[4] = {0.0, 0.0, 0.0, 0.0};
-    const int64_t e0 = V.toff[r] + (int64_t)piece * V.entries;
-    const int nn = min(V.tcnt[r] - piece * V.entries, V.entries);
-    for (int e = 0; act && e < nn; ++e) {
-      const int bc = V.leaf_cells[V.tidx[e0 + e]];
-      const int fb = V.c.first[bc], nb = V.c.count[bc];
-      unsigned in = 0u;
-      for (int i = sl; i < nb; i += K) {
-        const int64_t pi = (int64_t)fb + i;
-        if (pi == pj) continue;
-        const double d0 = V.tp.x[pi] - xj, d1 = V.tp.y[pi] - yj, d2 = V.tp.z[pi] - zj;
-        const double r2 = fma(d2, d2, fma(d1, d1, fma(d0, d0, eps2)));
-        if (M4 && maybe_inside(r2, h2j, V.ph[pi].w)) { in |= 1u << i; continue; }
-        const double b0 = V.ab[3 * pi], b1 = V.ab[3 * pi + 1], b2 = V.ab[3 * pi + 2];
-        const double inv = rsqrt64(r2), inv2 = inv * inv, f = inv2 * inv;
-        const double fdb = f * (d0 * b0 + d1 * b1 + d2 * b2);
-        const double u = -3.0 * inv2 * fdb;
-        g[0] = fma(f, b0, fma(u, d0, g[0]));
-        g[1] = fma(f, b1, fma(u, d1, g[1]));
-        g[2] = fma(f, b2, fma(u, d2, g[2]));
-        g[3] -= fdb;
-      }
-      while (M4 && in != 0u) {
-        const int i = __ffs(in) - 1;
-        in &= in - 1u;
-        const int64_t pi = (int64_t)fb + i;
-        const double d0 = V.tp.x[pi] - xj, d1 = V.tp.y[pi] - yj, d2 = V.tp.z[pi] - zj;
-        const double b0 = V.ab[3 * pi], b1 = V.ab[3 * pi + 1], b2 = V.ab[3 * pi + 2];
-        double f, gg;
-        m4_fg64(d0 * d0 + d1 * d1 + d2 * d2, V.hinv[pi], hinv_j, f, gg);
-        const double db = d0 * b0 + d1 * b1 + d2 * b2, u = gg * db;
-        g[0] = fma(f, b0, fma(u, d0, g[0]));
-        g[1] = fma(f, b1, fma(u, d1, g[1]));
-        g[2] = fma(f, b2, fma(u, d2, g[2]));
-        g[3] = fma(-f, db, g[3]);
-      }
-    }
-    for (int s = 1; s < K; ++s) {
-      const int src = js + s * ns;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const double o = __shfl_sync(full, g[c], src);
-        if (sl == 0) g[c] += o;
-      }
-    }
-    if (act && sl == 0) {
-      const double mj = V.tp.m[pj];
-      atomicAdd(&V.xsrc[3 * pj], mj * g[0]);
-      atomicAdd(&V.xsrc[3 * pj + 1], mj * g[1]);
-      atomicAdd(&V.xsrc[3 * pj + 2], mj * g[2]);
-      atomicAdd(&V.msrc[pj], g[3]);
     }
   }
 }
@@ -1515,11 +1555,11 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
     }
   } else {
     if (m4) {
-      k_vjp_target64<KDFMM_SOFT_M4><<<gi, kVjpWarps * 32, 0, s>>>(V);
-      k_vjp_source64<KDFMM_SOFT_M4><<<gi, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_pairs64<KDFMM_SOFT_M4, false><<<gi, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_pairs64<KDFMM_SOFT_M4, true><<<gi, kVjpWarps * 32, 0, s>>>(V);
     } else {
-      k_vjp_target64<KDFMM_SOFT_PLUMMER><<<gi, kVjpWarps * 32, 0, s>>>(V);
-      k_vjp_source64<KDFMM_SOFT_PLUMMER><<<gi, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_pairs64<KDFMM_SOFT_PLUMMER, false><<<gi, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_pairs64<KDFMM_SOFT_PLUMMER, true><<<gi, kVjpWarps * 32, 0, s>>>(V);
     }
   }
   k_vjp_seg_combine<<<grid_blocks(2), 256, 0, s>>>(V);
