@@ -222,15 +222,14 @@ __global__ void __launch_bounds__(128, 10) k_walk(WalkArgs W) {
   atomicAdd(&W.stats[3], (unsigned long long)nn);
 }
 
-// Slot mode with few leaves: K lanes of a warp share a leaf's walk.  The tree
-// below its first log2 K levels is K runs of pre-order cells; lane s of a leaf
-// descends to run s (deciding the cells on its way: a closed or leaf cell is
-// emitted by the first lane below it) and walks that run alone, into its own
-// scratch of kSplitCap entries (far from the front, near from the back).  The
-// lanes' lists in lane order are the leaf's lists in ascending id; the warp
+// Slot mode with 12160 to 48640 leaves: K lanes of a warp (8 or 4) share a leaf's
+// walk.  The tree below its first log2 K levels is K runs of pre-order cells;
+// lane s of a leaf descends to run s (deciding the cells on its way: a closed or
+// leaf cell is emitted by the first lane below it) and walks that run alone, into
+// its own scratch of kSplitCap entries (far from the front, near from the back).
+// The lanes' lists in lane order are the leaf's lists in ascending id; the warp
 // moves them to the leaf's slot.  One thread per leaf leaves the GPU waiting on
-// single chains of dependent record loads (about 350 ns a step): 7040 leaves of
-// a 60013-particle Plummer sphere took 1.41 ms on chains of up to 4096 steps.
+// single chains of dependent record loads (about 350 ns a step).
 // A lane that passes W.budget visited cells or fills its scratch hands the leaf
 // to k_walk_heavy.
 constexpr int kSplitCap = 512;
@@ -380,6 +379,152 @@ __global__ void __launch_bounds__(128, 10) k_walk_split(WalkArgs W) {
         dst[e] = temp0[at];
       }
     }
+  }
+}
+
+// Slot mode with at most kMapLeaves leaves: a warp per leaf.  Undecided cells lie
+// on a stack in shared memory; each round the lanes take up to 64 off its top,
+// decide them, and push the children of the opened ones.  The order of the
+// decisions is free: a far or near cell sets its bit in a map over its system's
+// cells, and the set bits in ascending order are the leaf's lists.  No scratch.
+// The thread walk is a chain of dependent record loads (about 350 ns a step, up to
+// 10000 steps for a leaf in the outskirts: 1.41 ms for the 7040 leaves of a
+// 60013-particle Plummer sphere); 32 lanes that each walked a 32nd of the tree
+// took 0.59 ms (the lane near the leaf has most of its cells), this takes 0.31.
+// Bound by issue slots (0.56 of them) and the records' latency; 16 blocks of two
+// warps an SM with 64 registers, where 20 (spilled records, less L1) took 0.47 ms
+// and 32 cells a round 0.35.  With 262146 particles (23000 leaves) the maps' zero
+// words and the fewer warps make 8 lanes a leaf the faster (1.88 ms a call
+// against 1.99).
+// A leaf that passes W.budget rounds, or outgrows the stack, goes to k_walk_heavy.
+constexpr int kMapLeaves = 12160;
+constexpr int kMapWarps = 2, kMapStack = 1024, kMapTake = 2;
+__global__ void __launch_bounds__(32 * kMapWarps, 16) k_walk_map(WalkArgs W, int words) {
+  extern __shared__ unsigned s_dyn[];
+  const unsigned full = 0xffffffffu;
+  const int nleaves = W.counters[C_LEAVES];
+  if (nleaves > W.slot_leaves && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(W.status, ST_LISTS);
+  const int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  const int lane = threadIdx.x & 31;
+  if (k >= nleaves || k >= W.slot_leaves) return;
+  const unsigned lt = (1u << lane) - 1u;
+  unsigned* const map_f = s_dyn + (threadIdx.x >> 5) * (2 * words + kMapStack / 2);
+  unsigned* const map_n = map_f + words;
+  uint16_t* const stack = reinterpret_cast<uint16_t*>(map_n + words);
+  const int a = W.leaf_cells[k];
+  const float4 wa = W.walk[a];
+  const float ha = W.walk2[a].x;
+  const double ax = W.cx[a], ay = W.cy[a], az = W.cz[a], sa = W.s[a], ha64 = W.hmax[a];
+  const int sys = W.leaf_sys[k];
+  const double theta = W.sys_theta[sys];
+  const float bound = *W.com_bound;
+  float thf = (float)theta, rkf = (float)W.r_kern;
+  int always = theta == 0.0;
+  asm("" : "+f"(thf), "+f"(rkf), "+r"(always));           // opaque: see walk_leaf
+  const int i0 = W.sys_root[sys], cells = W.sys_root[sys + 1] - i0;
+  const int used = (cells + 31) >> 5;
+  bool ok = used <= words && cells <= 65536;              // (at most two cells a leaf: always)
+  int nex = 0, top = ok ? 1 : 0, rounds = 0;
+  long long np = 0;
+  if (ok) {
+    for (int w = lane; w < used; w += 32) map_f[w] = map_n[w] = 0u;
+    if (lane == 0) stack[0] = 0;
+  }
+  __syncwarp();
+  while (top > 0) {
+    if (++rounds > W.budget || top > kMapStack - 64 * kMapTake) {
+      ok = false;
+      break;
+    }
+    const int take = min(top, 32 * kMapTake);
+    int c[kMapTake];
+    float4 wb[kMapTake], w2[kMapTake];
+    int right[kMapTake];
+#pragma unroll
+    for (int u = 0; u < kMapTake; ++u) {
+      const int q = 32 * u + lane;
+      c[u] = q < take ? (int)stack[top - 1 - q] : -1;
+      if (c[u] < 0) continue;
+      const int i = i0 + c[u];
+      wb[u] = W.walk[i];
+      w2[u] = W.walk2[i];
+      right[u] = c[u] + 1 < cells ? __float_as_int(W.walk2[i + 1].y) : 0;   // (the left child's next)
+    }
+    top -= take;
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < kMapTake; ++u) {
+      if (32 * u >= take) break;
+      bool push = false;
+      if (c[u] >= 0) {
+        const int i = i0 + c[u];
+        int o = always ? 1 : open_filter(wa, ha, wb[u], w2[u].x, thf, rkf, bound);
+        if (o < 0) {
+          o = open_exact(ax, ay, az, sa, ha64, W.cx[i], W.cy[i], W.cz[i], W.s[i], W.hmax[i], theta,
+                         W.r_kern);
+          ++nex;
+        }
+        push = o && __float_as_int(w2[u].y) != i + 1;
+        if (!push) {
+          atomicOr((o ? map_n : map_f) + (c[u] >> 5), 1u << (c[u] & 31));
+          if (o) np += __float_as_int(w2[u].z);
+        }
+      }
+      const unsigned m = __ballot_sync(full, push);
+      if (push) {
+        const int at = top + 2 * __popc(m & lt);
+        stack[at] = (uint16_t)(right[u] - i0);
+        stack[at + 1] = (uint16_t)(c[u] + 1);
+      }
+      top += 2 * __popc(m);
+    }
+    __syncwarp();
+  }
+  if (lane == 0) {
+    W.far_off[k] = (int64_t)k * W.cap_far;
+    W.near_off[k] = (int64_t)k * W.cap_near;
+  }
+  if (!ok) {
+    if (lane == 0) W.heavy[atomicAdd(W.heavy_n, 1)] = k;
+    return;
+  }
+  // the maps' bits in ascending order: 32 words at a time, a lane writes its word's
+  // cells (word by word for all lanes took a third of the kernel's instructions)
+  int tot[2];
+  for (int kind = 0; kind < 2; ++kind) {
+    const unsigned* map = kind ? map_n : map_f;
+    const int64_t cap = kind ? W.cap_near : W.cap_far;
+    int32_t* const dst = kind ? W.near_idx + k * cap : W.far_idx + k * cap;
+    int n = 0;
+    for (int w0 = 0; w0 < used; w0 += 32) {
+      const unsigned word = w0 + lane < used ? map[w0 + lane] : 0u;
+      if (__ballot_sync(full, word != 0u) == 0u) continue;
+      int pre = __popc(word);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(full, pre, o);
+        if (lane >= o) pre += v;
+      }
+      const int all = __shfl_sync(full, pre, 31);
+      pre -= __popc(word);
+      int e = n + pre;
+      for (unsigned bits = word; bits != 0u; bits &= bits - 1u, ++e)
+        if (e < cap) dst[e] = i0 + 32 * (w0 + lane) + __ffs(bits) - 1;
+      n += all;
+    }
+    tot[kind] = n;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    np += __shfl_xor_sync(full, np, o);
+    nex += __shfl_xor_sync(full, nex, o);
+  }
+  if (lane == 0) {
+    W.far_cnt[k] = tot[0];
+    W.near_cnt[k] = tot[1];
+    walk_stats(W, k, tot[0], tot[1], np, nex);
+    atomicAdd(&W.stats[2], (unsigned long long)tot[0]);
+    atomicAdd(&W.stats[3], (unsigned long long)tot[1]);
   }
 }
 
@@ -807,23 +952,22 @@ static int arena_grid_for(int leaves) {
                                                      (int64_t)per_sm * sms));
 }
 
-// Lanes per leaf of the slot-mode walk: 32 while that is at most two rounds of
-// resident threads (12160 leaves on 152 SMs), else as many as one round allows,
-// one beyond 48640 leaves, where the thread walk has the GPU's threads busy by
-// itself.
+// Lanes per leaf of the slot-mode walk: 32 (k_walk_map) up to kMapLeaves, else as
+// many as one round of resident threads allows, one beyond 48640 leaves on 152
+// SMs, where the thread walk has the GPU's threads busy by itself.
 static int split_lanes(int leaves) {
   const int64_t threads = (int64_t)sm_count() * 10 * 128, n = std::max(leaves, 1);
-  if (32 * n <= 2 * threads) return 32;
+  if (n <= kMapLeaves) return 32;
   for (int k = 8; k >= 4; k >>= 1)
     if (k * n <= threads) return k;
   return 1;
 }
 
-// Scratch of the slot-mode walk over `leaves` leaves; without it (no memory)
-// the walk takes one thread per leaf.
+// Scratch of the slot-mode walk over `leaves` leaves (8 or 4 lanes a leaf);
+// without it (no memory) the walk takes one thread per leaf.
 static int64_t split_scratch(int leaves) {
   const int k = split_lanes(leaves);
-  return k == 1 ? 0 : ((int64_t)std::max(leaves, 1) * k + 127) / 128 * 128 * kSplitCap;
+  return k == 1 || k == 32 ? 0 : ((int64_t)std::max(leaves, 1) * k + 127) / 128 * 128 * kSplitCap;
 }
 static void ensure_split(kdfmm_tree_s* t, int leaves) {
   Lists& L = t->L;
@@ -899,7 +1043,12 @@ static void walk_launch(kdfmm_tree_s* t, WalkArgs W, ListMode mode, int64_t cf, 
                           ? split_lanes(slot_leaves) : 1;
     const unsigned grid = blocks_for((int64_t)std::max(slot_leaves, 1) * lanes, 128);
     switch (lanes) {
-      case 32: k_walk_split<32><<<grid, 128, 0, s>>>(W); break;
+      case 32: {
+        const int n = std::max(slot_leaves, 1), words = (2 * n + 31) / 32;
+        k_walk_map<<<blocks_for(n, kMapWarps), 32 * kMapWarps,
+                     kMapWarps * (2 * words + kMapStack / 2) * sizeof(unsigned), s>>>(W, words);
+        break;
+      }
       case 8: k_walk_split<8><<<grid, 128, 0, s>>>(W); break;
       case 4: k_walk_split<4><<<grid, 128, 0, s>>>(W); break;
       default: k_walk<<<grid, 128, 0, s>>>(W);

@@ -1,4 +1,4 @@
-"""The slot-mode walk with several lanes per leaf against the thread walk: the
+"""The slot-mode walk with several lanes or a warp per leaf against the thread walk: the
 leaf counts where the number of lanes changes, trees smaller than the lanes'
 runs, scratch overflow, forests."""
 import numpy as np
@@ -14,9 +14,10 @@ def _lists(f):
     return [ex.far_off, ex.far_idx, ex.near_off, ex.near_idx], [st[k] for k in ("nfar", "nnear", "np2p", "nexact")]
 
 
-# leaves of one particle: as many leaves as particles.  On a GPU of 152 SMs 32
-# lanes serve a leaf up to 12160 leaves, 8 to 24320, 4 to 48640, one beyond; theta = 0 with 20000 leaves overflows a lane's scratch of 512 entries
-@pytest.mark.parametrize("n,theta", [(1, 0.5), (2, 0.5), (31, 0.5), (33, 0.0), (700, 0.4), (6080, 0.7),
+# leaves of one particle: as many leaves as particles.  A warp serves a leaf up to
+# 12160 leaves, 8 lanes to 24320 (on 152 SMs), 4 to 48640, one beyond; theta = 0
+# opens every cell and, with 20000 leaves, overflows a lane's scratch of 512 entries
+@pytest.mark.parametrize("n,theta", [(1, 0.5), (2, 0.5), (31, 0.5), (33, 0.0), (4000, 0.0), (700, 0.4), (6080, 0.7),
                                      (6081, 0.7), (12160, 0.8), (12161, 0.8), (24321, 0.9), (48641, 1.0), (20000, 0.0)])
 def test_split_walk_equals_thread_walk(n, theta, monkeypatch):
     import torch
