@@ -1,8 +1,7 @@
-"""Near-field kernels with everything near (theta = 0): leaves of 1 to 32
-particles fill a staged chunk in every way (one leaf of a chunk to 32, starts at
-and off the words of the start bitmap), and supports that hold none, some or all
-of the pairs fill the float64 kernels' queue of inside pairs never, partly or
-beyond its 512 marks."""
+"""Float64 near-field kernels with everything near (theta = 0): leaves of 1 to 32
+particles fill a staged chunk in every way (one leaf of a chunk to 32), and
+supports that hold none, some or all of the pairs fill the queue of inside pairs
+never, partly or beyond its 512 marks."""
 import numpy as np
 import pytest
 
@@ -16,21 +15,19 @@ def _set(n, scale, seed=3):
     return g.normal(size=(n, 3)), g.uniform(0.5, 1.5, n) / n, scale * g.uniform(0.5, 1.5, n)
 
 
-# float64: sums of at most 700 terms, 1e-12 of the largest component; mixed:
-# float32 terms (6e-8) whose sums cancel over 700 neighbours, 2e-5 as elsewhere
-@pytest.mark.parametrize("precision,tol", [(0, 1e-12), (1, 2e-5)])
+# float64 sums of at most 700 terms: 1e-12 of the largest component
 @pytest.mark.parametrize("scale", [1e-3, 0.3, 50.0])
 @pytest.mark.parametrize("n,n_leaf", [(2, 1), (33, 1), (700, 1), (700, 2), (650, 7), (512, 16), (700, 31), (700, 32)])
-def test_near_pairs_of_the_direct_sum(oracle, n, n_leaf, scale, precision, tol):
+def test_near_pairs_of_the_direct_sum(oracle, n, n_leaf, scale):
     import torch
     from paper_2502_01496_gb300 import native
     x, m, h = _set(n, scale)
-    f = native.KdFmm(theta=0.0, eps=0.01, n_leaf=n_leaf, soft_kind=native.SOFT_M4, precision=precision)
+    f = native.KdFmm(theta=0.0, eps=0.01, n_leaf=n_leaf, soft_kind=native.SOFT_M4, precision=native.FP64)
     f.build(*(torch.tensor(v, device="cuda") for v in (x, m, h)))
     a, phi = (t.cpu().numpy() for t in f.accel())
     wa, wphi = oracle.direct(x, m, h, soft_kind=native.SOFT_M4)
-    assert np.abs(a - wa).max() < tol * np.abs(wa).max()
-    assert np.abs(phi - wphi).max() < tol * np.abs(wphi).max()
+    assert np.abs(a - wa).max() < 1e-12 * np.abs(wa).max()
+    assert np.abs(phi - wphi).max() < 1e-12 * np.abs(wphi).max()
 
 
 @pytest.mark.parametrize("scale", [1e-3, 0.3, 50.0])
