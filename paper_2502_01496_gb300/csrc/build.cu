@@ -572,14 +572,21 @@ struct SubArgs {
 // threads equally busy, and takes a dozen barriers.  Splitting large cells by
 // the CTA one after the other, medium ones by a warp and small ones by a
 // thread left most warps idle behind one: 1009 particles on one CTA took 323 us
-// (now 104), a 60013-particle sphere 450 us (193), 2^24 clumped particles 10.4 ms
-// (4.2).  Bound: the float64 pipe (1/64 rate; 3 products and 4 sums a particle and
+// (now 87), a 60013-particle sphere 450 us (134), 2^24 clumped particles 10.4 ms
+// (4.0).  While the subtrees leave SMs idle (E = 4) an octet is four particles
+// and the CTA has 512 threads: half the instructions a thread and level (1009
+// particles 101 -> 87 us, 60013 175 -> 134 us).
+// Bound: the float64 pipe (1/64 rate; 3 products and 4 sums a particle and
 // level) once the SMs are full, barriers and shared-memory latency before.
 constexpr int kBatchCells = 128;
-constexpr int kBatchOctets = kSubtreeMax / 8 + kBatchCells;
-constexpr int kOctetsPerThread = 2;
-static_assert(kBatchOctets <= kOctetsPerThread * kSubtreeThreads, "octets of a batch per thread");
-static_assert(kBatchCells * 2 <= kSubtreeThreads && kBatchCells % 32 == 0, "cells of a batch per thread");
+template <int E>
+struct SubShape {
+  static constexpr int kThreads = kSubtreeMax / E, kOctets = kSubtreeMax / E + kBatchCells, kPerThread = 2,
+                       kLog = E == 8 ? 3 : 2;
+  static_assert(E == 8 || E == 4, "particles of an octet");
+  static_assert(kOctets <= kPerThread * kThreads, "octets of a batch per thread");
+  static_assert(kBatchCells * 2 <= kThreads && kBatchCells % 32 == 0, "cells of a batch per thread");
+};
 
 // Shared-memory views of one subtree.
 struct SubSmem {
@@ -592,11 +599,12 @@ struct SubSmem {
   int *d2m, *axis, *irank;             // per cell: float32 squared size, cut axis, rank among the split
   float* thr2;                         // per cell: candidates for the exact size
   int* oct0;                           // per cell: its first octet (kBatchCells + 1)
-  int* opre;                           // per octet: left particles before it (kBatchOctets + 1)
+  int* opre;                           // per octet: left particles before it (octets + 1)
   uint16_t *idx0, *idx1, *fin;         // particle order of a level (two buffers) and of finished leaves
   int2 *q0, *q1;                       // cells of a level (two buffers): (first | count << 16, cell id)
 };
 
+template <int E>
 __host__ __device__ __forceinline__ size_t sub_carve(unsigned char* base, int qcap, SubSmem* L) {
   size_t at = 0;
   auto take = [&](size_t bytes) {
@@ -606,7 +614,7 @@ __host__ __device__ __forceinline__ size_t sub_carve(unsigned char* base, int qc
   };
   double* x = reinterpret_cast<double*>(take(4 * kSubtreeMax * sizeof(double)));
   L->x = x; L->y = x + kSubtreeMax; L->z = x + 2 * kSubtreeMax; L->m = x + 3 * kSubtreeMax;
-  L->osum = reinterpret_cast<Sum4*>(take(kBatchOctets * sizeof(Sum4)));
+  L->osum = reinterpret_cast<Sum4*>(take(SubShape<E>::kOctets * sizeof(Sum4)));
   L->key = reinterpret_cast<long long*>(L->osum);
   L->com = reinterpret_cast<double*>(take(3 * kBatchCells * sizeof(double)));
   L->s2 = reinterpret_cast<unsigned long long*>(take(kBatchCells * sizeof(unsigned long long)));
@@ -616,7 +624,7 @@ __host__ __device__ __forceinline__ size_t sub_carve(unsigned char* base, int qc
   L->irank = reinterpret_cast<int*>(take(kBatchCells * sizeof(int)));
   L->thr2 = reinterpret_cast<float*>(take(kBatchCells * sizeof(float)));
   L->oct0 = reinterpret_cast<int*>(take((kBatchCells + 1) * sizeof(int)));
-  L->opre = reinterpret_cast<int*>(take((kBatchOctets + 1) * sizeof(int)));
+  L->opre = reinterpret_cast<int*>(take((SubShape<E>::kOctets + 1) * sizeof(int)));
   uint16_t* ix = reinterpret_cast<uint16_t*>(take(3 * kSubtreeMax * sizeof(uint16_t)));
   L->idx0 = ix; L->idx1 = ix + kSubtreeMax; L->fin = ix + 2 * kSubtreeMax;
   L->q0 = reinterpret_cast<int2*>(take(2 * (size_t)qcap * sizeof(int2)));
@@ -631,12 +639,14 @@ __device__ __forceinline__ int fkey(float v) {
 }
 __device__ __forceinline__ float funkey(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7fffffff)); }
 
-__global__ void __launch_bounds__(kSubtreeThreads, 2)
+template <int E>
+__global__ void __launch_bounds__(SubShape<E>::kThreads, 512 / SubShape<E>::kThreads)
 k_subtree(SubArgs S) {
+  constexpr int kThreads = SubShape<E>::kThreads, kPerThread = SubShape<E>::kPerThread;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_seg, s_base, s_tot[3][kBatchCells / 32];
   SubSmem L;
-  sub_carve(smem_raw, S.qcap, &L);
+  sub_carve<E>(smem_raw, S.qcap, &L);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned full = 0xffffffffu;
   const BuildArgs& A = S.A;
@@ -654,7 +664,7 @@ k_subtree(SubArgs S) {
   const int n = g.count, gfirst = g.first;
   const int sys = system_of(A.sys_off, A.n_sys, gfirst);
   const int n_leaf = A.sys_nleaf[sys];
-  for (int k = tid; k < n; k += kSubtreeThreads) {
+  for (int k = tid; k < n; k += kThreads) {
     L.x[k] = in.x[gfirst + k]; L.y[k] = in.y[gfirst + k]; L.z[k] = in.z[gfirst + k];
     L.m[k] = in.m[gfirst + k];
     L.idx0[k] = (uint16_t)k;
@@ -676,7 +686,7 @@ k_subtree(SubArgs S) {
       int cnt_c = 0, pack = 0, incl = 0;
       if (tid < kBatchCells) {
         cnt_c = tid < ncb ? q[tid].x >> 16 : 0;
-        incl = pack = ((cnt_c + 7) >> 3) | (cnt_c > n_leaf) << 16;
+        incl = pack = ((cnt_c + E - 1) / E) | (cnt_c > n_leaf) << 16;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
           const int v = __shfl_up_sync(full, incl, o);
@@ -711,11 +721,11 @@ k_subtree(SubArgs S) {
       }
       __syncthreads();
       // the thread's octets: cell, first element in the cell, elements
-      int oc[kOctetsPerThread], rel[kOctetsPerThread], val[kOctetsPerThread];
-      int lf[kOctetsPerThread], cn[kOctetsPerThread];
+      int oc[kPerThread], rel[kPerThread], val[kPerThread];
+      int lf[kPerThread], cn[kPerThread];
 #pragma unroll
-      for (int u = 0; u < kOctetsPerThread; ++u) {
-        const int o = tid + u * kSubtreeThreads;
+      for (int u = 0; u < kPerThread; ++u) {
+        const int o = tid + u * kThreads;
         oc[u] = -1; rel[u] = val[u] = lf[u] = cn[u] = 0;
         if (o < noct) {
           int c = 0;
@@ -726,14 +736,14 @@ k_subtree(SubArgs S) {
           oc[u] = c;
           lf[u] = e & 0xffff;
           cn[u] = e >> 16;
-          rel[u] = 8 * (o - L.oct0[c]);
-          val[u] = min(8, cn[u] - rel[u]);
+          rel[u] = E * (o - L.oct0[c]);
+          val[u] = min(E, cn[u] - rel[u]);
         }
       }
       // octet sums, float32 bounding boxes (coordinates truncated: monotone)
 #pragma unroll
-      for (int u = 0; u < kOctetsPerThread; ++u) {
-        if (u * kSubtreeThreads + (tid & ~31) >= noct) continue;    // the whole warp has none
+      for (int u = 0; u < kPerThread; ++u) {
+        if (u * kThreads + (tid & ~31) >= noct) continue;    // the whole warp has none
         int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
         if (oc[u] >= 0) {
           const uint16_t* p = ix + lf[u] + rel[u];
@@ -747,7 +757,7 @@ k_subtree(SubArgs S) {
             lo[2] = min(lo[2], kz); hi[2] = max(hi[2], kz);
             return elem4(L.m[i], x, y, z);
           };
-          L.osum[tid + u * kSubtreeThreads] = block_tree<3>(0, val[u], get);
+          L.osum[tid + u * kThreads] = block_tree<SubShape<E>::kLog>(0, val[u], get);
         }
         if (__all_sync(full, oc[u] == __shfl_sync(full, oc[u], 0))) {   // one cell: one set of atomics
 #pragma unroll
@@ -767,10 +777,10 @@ k_subtree(SubArgs S) {
       for (int s = 1; s < maxoct; s <<= 1) {
         __syncthreads();
 #pragma unroll
-        for (int u = 0; u < kOctetsPerThread; ++u) {
-          const int r = rel[u] >> 3;
-          if (oc[u] >= 0 && (r & (2 * s - 1)) == 0 && 8 * (r + s) < cn[u]) {
-            Sum4* p = L.osum + tid + u * kSubtreeThreads;
+        for (int u = 0; u < kPerThread; ++u) {
+          const int r = rel[u] / E;
+          if (oc[u] >= 0 && (r & (2 * s - 1)) == 0 && E * (r + s) < cn[u]) {
+            Sum4* p = L.osum + tid + u * kThreads;
             p[0] = add4(p[0], p[s]);
           }
         }
@@ -780,7 +790,7 @@ k_subtree(SubArgs S) {
       // centres of mass, cut axes; an axis whose lead is within the error of
       // the float32 box is decided from the exact box
       bool unclear = false;
-      for (int t = tid; t < 4 * ncb; t += kSubtreeThreads) {
+      for (int t = tid; t < 4 * ncb; t += kThreads) {
         const int c = t >> 2, d = t & 3, cell = q[c].y;
         const Sum4& v = L.osum[L.oct0[c]];
         if (d < 3) {
@@ -821,10 +831,10 @@ k_subtree(SubArgs S) {
         continue;
       }
       if (exact) {
-        for (int t = tid; t < 6 * ncb; t += kSubtreeThreads) L.key[t] = t % 6 < 3 ? LLONG_MAX : LLONG_MIN;
+        for (int t = tid; t < 6 * ncb; t += kThreads) L.key[t] = t % 6 < 3 ? LLONG_MAX : LLONG_MIN;
         __syncthreads();
 #pragma unroll
-        for (int u = 0; u < kOctetsPerThread; ++u) {
+        for (int u = 0; u < kPerThread; ++u) {
           if (oc[u] < 0 || L.axis[oc[u]] >= 0) continue;
           for (int k = 0; k < val[u]; ++k) {
             const int i = ix[lf[u] + rel[u] + k];
@@ -845,12 +855,12 @@ k_subtree(SubArgs S) {
         __syncthreads();
       }
       // left flags (bits of the octet) and float32 squared distances
-      unsigned left[kOctetsPerThread];
-      float d2[kOctetsPerThread][8];
+      unsigned left[kPerThread];
+      float d2[kPerThread][E];
 #pragma unroll
-      for (int u = 0; u < kOctetsPerThread; ++u) {
+      for (int u = 0; u < kPerThread; ++u) {
         left[u] = 0u;
-        if (u * kSubtreeThreads + (tid & ~31) >= noct) continue;
+        if (u * kThreads + (tid & ~31) >= noct) continue;
         float mx = 0.0f;
         if (oc[u] >= 0) {
           const double* com = L.com + 3 * oc[u];
@@ -859,7 +869,7 @@ k_subtree(SubArgs S) {
           const int ax = L.axis[oc[u]];
           const long long ckey = dkey(com[ax]);
 #pragma unroll
-          for (int k = 0; k < 8; ++k) {
+          for (int k = 0; k < E; ++k) {
             d2[u][k] = -2.0f;
             if (k < val[u]) {
               const int i = ix[lf[u] + rel[u] + k];
@@ -871,7 +881,7 @@ k_subtree(SubArgs S) {
               if (cut && dkey(a) < ckey) left[u] |= 1u << k;
             }
           }
-          L.opre[tid + u * kSubtreeThreads] = __popc(left[u]);
+          L.opre[tid + u * kThreads] = __popc(left[u]);
         }
         if (__all_sync(full, oc[u] == __shfl_sync(full, oc[u], 0))) {
           const int m = __reduce_max_sync(full, __float_as_int(mx));
@@ -882,7 +892,7 @@ k_subtree(SubArgs S) {
       }
       __syncthreads();
       if (warp == 0) {                    // left particles before each octet of the batch
-        constexpr int kPer = kBatchOctets / 32;
+        constexpr int kPer = SubShape<E>::kOctets / 32;
         int v[kPer], run = 0;
 #pragma unroll
         for (int k = 0; k < kPer; ++k) {
@@ -915,13 +925,13 @@ k_subtree(SubArgs S) {
       __syncthreads();
       // exact size from the candidates; the stable partition of cut cells
 #pragma unroll
-      for (int u = 0; u < kOctetsPerThread; ++u) {
+      for (int u = 0; u < kPerThread; ++u) {
         const int c = oc[u];
         if (c < 0) continue;
         const float thr2 = L.thr2[c];
         unsigned cand = 0u;
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
+        for (int k = 0; k < E; ++k)
           if (k < val[u] && d2[u][k] >= thr2) cand |= 1u << k;
         const uint16_t* p = ix + lf[u] + rel[u];
         long long s2 = 0;
@@ -939,7 +949,7 @@ k_subtree(SubArgs S) {
           if (nl == 0 || nl == cn[u]) {                            // split by position: order kept
             for (int k = 0; k < val[u]; ++k) ox[lf[u] + rel[u] + k] = p[k];
           } else {
-            int l = L.opre[tid + u * kSubtreeThreads] - before, r = nl + rel[u] - l;
+            int l = L.opre[tid + u * kThreads] - before, r = nl + rel[u] - l;
             for (int k = 0; k < val[u]; ++k)
               ox[lf[u] + ((left[u] >> k & 1u) ? l++ : r++)] = p[k];
           }
@@ -976,7 +986,7 @@ k_subtree(SubArgs S) {
   }
   if (overflow) continue;
   if (tid == 0) atomicMax(&A.counters[C_DEPTH], depth);
-  for (int k = tid; k < n; k += kSubtreeThreads) {
+  for (int k = tid; k < n; k += kThreads) {
     const int src = L.fin[k];
     const int64_t p = (int64_t)gfirst + k;
     S.out.x[p] = L.x[src]; S.out.y[p] = L.y[src]; S.out.z[p] = L.z[src]; S.out.m[p] = L.m[src];
@@ -1366,9 +1376,17 @@ static int ensure_build_buffers(kdfmm_tree_s* t, int64_t n) {
 // split) and dynamic shared memory of the subtree kernel for trees of the
 // given leaf size.
 static int subtree_qcap(int n_leaf) { return 2 * (kSubtreeMax / (n_leaf + 1)) + 2; }
-static size_t subtree_smem_for(int qcap) {
+static size_t subtree_smem_for(bool fine, int qcap) {
   SubSmem L;
-  return sub_carve(nullptr, qcap, &L);
+  return fine ? sub_carve<4>(nullptr, qcap, &L) : sub_carve<8>(nullptr, qcap, &L);
+}
+
+// Octets of four particles while a CTA of 512 threads an SM takes all subtrees at
+// once (a subtree has some 1024 to 2048 particles, and a system at least one);
+// beyond that two CTAs of 256 threads an SM overlap each other's barriers (a
+// binary of 262146 particles, some 250 subtrees: 165 us against 180).
+static bool subtree_fine(const kdfmm_tree_s* t) {
+  return std::max<int64_t>(t->n / 1024, t->n_sys) <= sm_count();
 }
 
 // Launch sizes of the persistent subtree kernel (host calls only; made once
@@ -1377,21 +1395,23 @@ static size_t subtree_smem_for(int qcap) {
 // so it is set to the size of the smallest leaves (1), which no handle
 // exceeds: a limit set to this handle's own size would fail the next launch
 // of a handle with smaller leaves.
-static int subtree_setup(kdfmm_tree_s* t, size_t smem) {
-  if (t->subtree_smem == smem) return KDFMM_OK;
-  int rc = check_cuda(cudaFuncSetAttribute(k_subtree, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)subtree_smem_for(subtree_qcap(1))),
+static int subtree_setup(kdfmm_tree_s* t, bool fine, size_t smem) {
+  if (t->subtree_smem == smem && t->subtree_fine == fine) return KDFMM_OK;
+  void (*const kernel)(SubArgs) = fine ? k_subtree<4> : k_subtree<8>;
+  int rc = check_cuda(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)subtree_smem_for(fine, subtree_qcap(1))),
                       "subtree smem attribute");
   if (rc) return rc;
   int per_sm = 0, sms = 0;
-  rc = check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_subtree,
-                                                                 kSubtreeThreads, smem),
+  rc = check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                      &per_sm, kernel, fine ? SubShape<4>::kThreads : SubShape<8>::kThreads, smem),
                   "subtree occupancy");
   if (rc) return rc;
   rc = check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, t->device), "SMs");
   if (rc) return rc;
   t->subtree_grid = std::max(1, per_sm) * std::max(1, sms);
   t->subtree_smem = smem;
+  t->subtree_fine = fine;
   return KDFMM_OK;
 }
 
@@ -1486,10 +1506,12 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
   S.h = P.soft_kind == KDFMM_SOFT_M4 ? h : nullptr;
   S.sys_eps = t->sys_eps;
   S.qcap = subtree_qcap(t->min_nleaf);
-  const size_t smem = subtree_smem_for(S.qcap);
-  if ((rc = subtree_setup(t, smem))) return rc;
+  const bool fine = subtree_fine(t);
+  const size_t smem = subtree_smem_for(fine, S.qcap);
+  if ((rc = subtree_setup(t, fine, smem))) return rc;
   const int gsub = deferred ? t->subtree_grid : std::max(1, std::min(t->subtree_grid, hc[C_NB]));
-  k_subtree<<<gsub, kSubtreeThreads, smem, s>>>(S);
+  if (fine) k_subtree<4><<<gsub, SubShape<4>::kThreads, smem, s>>>(S);
+  else k_subtree<8><<<gsub, SubShape<8>::kThreads, smem, s>>>(S);
   k_leaf_segs<<<grid_blocks(2), 128, 0, s>>>(S, t->segL);
   t->launches += 2;
   if (!deferred) {

@@ -18,7 +18,6 @@ static_assert(kChunk == 8 * kChunkThreads, "the chunk reduce sums 8 elements per
 constexpr int kSmallChunkMax = 311296;   // up to here chunks of 512 elements (152 x 2048 elements:
                                        // one large chunk per SM)
 constexpr int kSubtreeMax = 2048;      // cells this small finish in shared memory
-constexpr int kSubtreeThreads = 256;
 constexpr int kNumStatus = 4;
 
 // Device-side status bits (OR-ed into a device word, read after a sync).
@@ -144,6 +143,7 @@ struct kdfmm_tree_s {
   int64_t max_sys = 0;             // particles of the largest system
   int32_t subtree_grid = 0;        // persistent grid of the subtree kernel
   size_t subtree_smem = 0;
+  bool subtree_fine = false;       // its octets are of four particles
   int64_t cap_cells = 0;
   kdfmm_params p{};
   bool built = false, evaluated = false, lists_frozen = false;
