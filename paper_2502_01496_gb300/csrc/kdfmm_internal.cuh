@@ -33,7 +33,7 @@ enum : int {
 // Slots of the handle's device counter block (int32).  Kernels read the sizes
 // they work on from here, so a launch needs no host-side count.  The build
 // clears and the host reads back [0, C_BUILD_END) with one call each, a walk
-// [C_MAXFAR, C_END); the last eight hold the walk's four 64-bit statistics.
+// [C_LONG, C_END); the last eight hold the walk's four 64-bit statistics.
 enum : int {
   C_CELLS = 0,      // cells allocated
   C_NEXT_A = 1,     // segments pushed for the next phase-A level
@@ -49,6 +49,7 @@ enum : int {
   C_BOUND = 17,     // max |com component| over the cells (float)
   C_BUILD_END = 18,
   C_SEGS = 19,      // extra P2P segments of leaves with long near lists
+  C_LONG = 20,      // leaves whose map walk is long
   C_MAXFAR = 21,    // longest far list of the last walk
   C_MAXNEAR = 22,   // longest near list of the last walk
   C_HEAVY = 23,     // leaves whose walk outgrew the per-thread budget (queued)

@@ -56,6 +56,8 @@ struct WalkArgs {
   int budget;                      // cells one thread visits before handing its leaf on
   int32_t* heavy;                  // queue of the leaves handed on
   int32_t* heavy_n;                // its length (counters[C_HEAVY])
+  int32_t* long_n;                 // long map walks (counters[C_LONG])
+  int sms;
 };
 
 __device__ __forceinline__ bool open_exact(double ax, double ay, double az, double sa, double ha,
@@ -396,8 +398,13 @@ __global__ void __launch_bounds__(128, 10) k_walk_split(WalkArgs W) {
 // and 32 cells a round 0.35.  With 262146 particles (23000 leaves) the maps' zero
 // words and the fewer warps make 8 lanes a leaf the faster (1.88 ms a call
 // against 1.99).
-// A leaf that passes W.budget rounds, or outgrows the stack, goes to k_walk_heavy.
-constexpr int kMapLeaves = 12160;
+// A leaf that passes W.budget rounds, or outgrows the stack, goes to k_walk_heavy;
+// so do the first leaves to reach kMapLong rounds, one for each of its blocks: they
+// would end the walk alone (60013 particles: 310 -> 118 us + 38 us of k_walk_heavy;
+// at 64 rounds 136 + 40).
+// With all of them handed over a small theta, where most leaves are long, lost by it
+// (theta = 0.2: 1.55 -> 1.86 ms a call).
+constexpr int kMapLeaves = 12160, kMapLong = 40, kMapHandOver = 2;
 constexpr int kMapWarps = 2, kMapStack = 1024, kMapTake = 2;
 __global__ void __launch_bounds__(32 * kMapWarps, 16) k_walk_map(WalkArgs W, int words) {
   extern __shared__ unsigned s_dyn[];
@@ -432,7 +439,14 @@ __global__ void __launch_bounds__(32 * kMapWarps, 16) k_walk_map(WalkArgs W, int
   }
   __syncwarp();
   while (top > 0) {
-    if (++rounds > W.budget || top > kMapStack - 64 * kMapTake) {
+    ++rounds;
+    bool leave = rounds > W.budget || top > kMapStack - 64 * kMapTake;
+    if (rounds == kMapLong) {
+      int before = 0;
+      if (lane == 0) before = atomicAdd(W.long_n, 1);
+      leave = leave || __shfl_sync(full, before, 0) < (int)(kMapHandOver * W.sms);
+    }
+    if (leave) {
       ok = false;
       break;
     }
@@ -1004,6 +1018,8 @@ static WalkArgs walk_args(kdfmm_tree_s* t) {
   W.budget = walk_budget(t);
   W.heavy = L.heavy;
   W.heavy_n = t->counters + C_HEAVY;
+  W.long_n = t->counters + C_LONG;
+  W.sms = sm_count();
   return W;
 }
 
@@ -1025,7 +1041,7 @@ static void walk_launch(kdfmm_tree_s* t, WalkArgs W, ListMode mode, int64_t cf, 
   W.temp = L.temp;
   W.heavy_scratch = arena ? L.temp_cap / grid_blocks(2) : 0;
   W.slot_leaves = slot_leaves;
-  cudaMemsetAsync(t->counters + C_MAXFAR, 0, (C_END - C_MAXFAR) * sizeof(int32_t), s);
+  cudaMemsetAsync(t->counters + C_LONG, 0, (C_END - C_LONG) * sizeof(int32_t), s);
   if (arena) {
     // one round (no more leaves than threads): the walk is latency-bound and
     // its lanes run free; several rounds fill the GPU and the synchronous loop
