@@ -183,7 +183,9 @@ int kdfmm_tree_moments(kdfmm_tree t, const double* x, const double* m, const dou
  * fixed slots per leaf or, when a few lists are far longer than the rest (a
  * centrally condensed system), in room reserved per leaf by a one-pass walk
  * whose threads each use a scratch of 4096 int32 entries (at most ~3.2 GB;
- * when that cannot be allocated, in two passes: count, then fill).
+ * when that cannot be allocated, in two passes: count, then fill).  The slot
+ * walk of some 10^4 to 5 10^4 leaves keeps a scratch of at most 0.4 GB, and
+ * works without it where it cannot be allocated.
  * Synchronises `stream` once (list sizes), again when the lists outgrew their
  * buffers and the walk is repeated. */
 int kdfmm_fmm_accel(kdfmm_tree t, double* a, double* phi, void* stream);

@@ -13,7 +13,7 @@
 //          to the cell's first particle (chunk sums are the subtrees of the pairwise
 //          tree, so the tiling does not change the result).
 // Phase B: a cell of at most kSubtreeMax particles is finished by one CTA with
-//          its particles held in shared memory; each warp splits one cell.
+//          its particles held in shared memory, all cells of a level together.
 // Then the cells are renumbered in pre-order from their particle ranges, the
 // quadrupoles and h_max are accumulated bottom-up, and float32 views for the
 // walk, the M2L and the P2P are derived.

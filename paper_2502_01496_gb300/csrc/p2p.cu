@@ -510,8 +510,8 @@ __device__ __forceinline__ void m4_side64(double r, double inv, double inv3, dou
 // ones: a 1/r^2 pair takes 17 of them (3 differences, 3 for r^2, 4 for 1/r
 // (rsqrt64), 4 for m/r and m/r^3, 3 for the force), the tests of the kernel
 // supports are float32.  With the library's rsqrt, float64 tests and divisions
-// per kernel pair it was ~45 (M4 binary of 2 x 2^20: 133 ms, now 91; Plummer
-// sphere of 4096: 1.42 ms in long segments, now 0.3).
+// per kernel pair it was ~45 (M4 binary of 2 x 2^20: 133 ms, now 74; Plummer
+// sphere of 4096: 1.42 ms in long segments, now 0.23).
 template <int SOFT>
 __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
   constexpr bool M4 = SOFT == KDFMM_SOFT_M4;
