@@ -406,6 +406,9 @@ __global__ void k_l2l_level(L2LArgs A) {
   }
 }
 
+// Room for `need` entries in *p, of which *have are there: each buffer carries the
+// capacity it was allocated with (none after a failure), since a handle may be
+// rebuilt with any number of particles.
 template <class T>
 int grow(T** p, int64_t* have, int64_t need, const char* what) {
   if (*have >= need) return KDFMM_OK;
@@ -437,27 +440,20 @@ int run_dual_walk(kdfmm_tree_s* t, cudaStream_t s) {
   int rc;
   if (!D.ctr && (rc = check_cuda(cudaMalloc(&D.ctr, 8 * sizeof(int32_t)), "dual counters")))
     return rc;
-  // the three per-cell arrays always share one capacity
-  int64_t cap = D.cells_cap;
-  if ((rc = grow(&D.far_cnt, &cap, (int64_t)nc + 2, "dual far counts"))) return rc;
-  cap = D.cells_cap;
-  if ((rc = grow(&D.cursor, &cap, (int64_t)nc + 2, "dual cursors"))) return rc;
-  cap = D.cells_cap;
-  if ((rc = grow(&D.far_off, &cap, (int64_t)nc + 2, "dual far offsets"))) return rc;
-  D.cells_cap = cap;
-  int64_t qc = std::max<int64_t>(D.q_cap, 4 * (int64_t)nc + 1024);
+  if ((rc = grow(&D.far_cnt, &D.far_cnt_cap, (int64_t)nc + 2, "dual far counts"))) return rc;
+  if ((rc = grow(&D.cursor, &D.cursor_cap, (int64_t)nc + 2, "dual cursors"))) return rc;
+  if ((rc = grow(&D.far_off, &D.far_off_cap, (int64_t)nc + 2, "dual far offsets"))) return rc;
+  int64_t qc = std::max<int64_t>(std::min(D.q_cap[0], D.q_cap[1]), 4 * (int64_t)nc + 1024);
   int64_t fc = std::max<int64_t>(D.far_cap, 8 * (int64_t)nc + 1024);
   int64_t ncap = std::max<int64_t>(D.near_cap, 8 * (int64_t)nl + 1024);
   int32_t* hc = t->host_counters;
   int64_t nfar = 0, nnear = 0;
   for (int attempt = 0;; ++attempt) {
     if (attempt > 8) return set_error(KDFMM_ERR_CAPACITY, "dual walk kept outgrowing its queues");
-    int64_t h0 = D.q_cap, h1 = D.q_cap, h2 = D.far_cap, h3 = D.near_cap;
-    if ((rc = grow(&D.q[0], &h0, qc, "pair queue"))) return rc;
-    if ((rc = grow(&D.q[1], &h1, qc, "pair queue"))) return rc;
-    if ((rc = grow(&D.far, &h2, fc, "far pairs"))) return rc;
-    if ((rc = grow(&D.near, &h3, ncap, "near pairs"))) return rc;
-    D.q_cap = qc; D.far_cap = fc; D.near_cap = ncap;
+    if ((rc = grow(&D.q[0], &D.q_cap[0], qc, "pair queue"))) return rc;
+    if ((rc = grow(&D.q[1], &D.q_cap[1], qc, "pair queue"))) return rc;
+    if ((rc = grow(&D.far, &D.far_cap, fc, "far pairs"))) return rc;
+    if ((rc = grow(&D.near, &D.near_cap, ncap, "near pairs"))) return rc;
     cudaMemsetAsync(D.ctr, 0, 8 * sizeof(int32_t), s);
     cudaMemsetAsync(L.near_np, 0, 4 * sizeof(int64_t), s);
     cudaMemcpyAsync(D.ctr + DQ_OUT, &t->n_sys, sizeof(int32_t), cudaMemcpyHostToDevice, s);
@@ -536,14 +532,9 @@ int run_dual_local(kdfmm_tree_s* t, cudaStream_t s) {
   auto& D = t->dual;
   const bool mixed = t->p.precision == KDFMM_MIXED;
   int rc;
-  int64_t have = 0;
-  if (mixed) {
-    have = D.lcell32 ? t->cap_cells * 24 : 0;
-    if ((rc = grow(&D.lcell32, &have, t->cap_cells * 24, "cell expansions"))) return rc;
-  } else {
-    have = D.lcell64 ? t->cap_cells * 20 : 0;
-    if ((rc = grow(&D.lcell64, &have, t->cap_cells * 20, "cell expansions"))) return rc;
-  }
+  if (mixed) rc = grow(&D.lcell32, &D.lcell32_cap, t->cap_cells * 24, "cell expansions");
+  else rc = grow(&D.lcell64, &D.lcell64_cap, t->cap_cells * 20, "cell expansions");
+  if (rc) return rc;
   if ((rc = run_m2l_cells(t, D.far_cnt, D.far_off, D.far_idx, D.lcell32, D.lcell64, s))) return rc;
   if ((rc = grow(&D.ltot, &D.ltot_cap, t->cap_cells * 20, "cell expansion totals"))) return rc;
   L2LArgs A{};
@@ -561,9 +552,7 @@ int run_dual_local(kdfmm_tree_s* t, cudaStream_t s) {
   int32_t* cnt = t->min_depth;
   int32_t *off = cnt + levels, *cursor = off + levels + 1;
   if (3 * (int64_t)levels + 1 > t->cap_n + 2) {             // fewer particles than that: own room
-    int64_t have_d = D.depth_cap;
-    if ((rc = grow(&D.depth_tab, &have_d, 3 * (int64_t)levels + 1, "levels"))) return rc;
-    D.depth_cap = have_d;
+    if ((rc = grow(&D.depth_tab, &D.depth_cap, 3 * (int64_t)levels + 1, "levels"))) return rc;
     cnt = D.depth_tab;
     off = cnt + levels;
     cursor = off + levels + 1;

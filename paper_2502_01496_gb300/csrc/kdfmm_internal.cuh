@@ -211,20 +211,20 @@ struct kdfmm_tree_s {
   // pair lists, per-cell far lists and per-cell local expansions
   struct Dual {
     int2 *q[2] = {nullptr, nullptr}, *far = nullptr, *near = nullptr;
-    int64_t q_cap = 0, far_cap = 0, near_cap = 0;
+    int64_t q_cap[2] = {0, 0}, far_cap = 0, near_cap = 0;   // entries allocated
     int32_t* ctr = nullptr;              // device: [0] queue out, [1] far pairs, [2] near pairs, [3] overflow
     int64_t* np2p = nullptr;             // device: particle pairs of the near list
     int32_t* far_cnt = nullptr;          // per cell
     int64_t* far_off = nullptr;          // per cell + 1
     int32_t* far_idx = nullptr;
-    int64_t far_idx_cap = 0, cells_cap = 0;
+    int64_t far_cnt_cap = 0, far_off_cap = 0, far_idx_cap = 0, cursor_cap = 0;
     int32_t* cursor = nullptr;           // per cell (fill cursors, then the cells by depth)
     int32_t* depth_tab = nullptr;        // per level: counts, offsets, cursors
     int64_t depth_cap = 0;
     float* lcell32 = nullptr;            // 24 per cell
     double* lcell64 = nullptr;           // 20 per cell
     double* ltot = nullptr;              // 20 per cell: own + ancestors' expansions, at its com
-    int64_t ltot_cap = 0;
+    int64_t lcell32_cap = 0, lcell64_cap = 0, ltot_cap = 0;
     int64_t nfar = 0, nnear = 0;         // entries (both directions)
   } dual;
 
