@@ -1049,9 +1049,17 @@ typedef unsigned long long Starts;
 __device__ __forceinline__ int cells_before(const Starts* off, int64_t p) { return (int)(unsigned)off[p]; }
 __device__ __forceinline__ int leaves_before(const Starts* off, int64_t p) { return (int)(off[p] >> 32); }
 
-__global__ void k_fill2(Starts* a, Starts va, int32_t* b, int32_t vb, int64_t n) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) { a[i] = va; b[i] = vb; }
+// Clears the scan's words.  A build that did not come to its end (too few
+// phase-A levels, a full list, refused input) leaves cells whose links are those
+// of an earlier tree: its cell count becomes 0 here, so that the numbering finds
+// no cells, counts no leaves, and neither the kernels after it nor the walk, M2L
+// and P2P of a captured evaluation touch that tree.  The status word tells the
+// host.
+__global__ void k_number_init(Starts* starts, int32_t* min_depth, int64_t n, int32_t* counters,
+                              const int32_t* __restrict__ status) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0 && (*status & (ST_UNFINISHED | ST_CAPACITY | ST_NONFINITE))) counters[C_CELLS] = 0;
+  if (i < n) { starts[i] = 0; min_depth[i] = INT_MAX; }
 }
 
 __global__ void k_count_starts(TmpCells tmp, const int32_t* __restrict__ counters, Starts* cnt,
@@ -1422,7 +1430,8 @@ static int subtree_setup(kdfmm_tree_s* t, bool fine, size_t smem) {
 // synchronisation -- exactly that many phase-A levels, every launch sized
 // from capacities and reading its count on the device -- so the sequence can
 // be captured in a CUDA graph; a phase A that needed more levels, or any
-// capacity overflow, is left in the status word for the caller to check.
+// capacity overflow, is left in the status word for the caller to check (the
+// tree then has no cells: k_number_init).
 int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* h, cudaStream_t s,
                int fixed_levels) {
   const int64_t n = t->n;
@@ -1525,7 +1534,7 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
   }
 
   // pre-order numbering, counts read on the device
-  k_fill2<<<blocks_for(n + 1, 256), 256, 0, s>>>(t->starts, 0, t->min_depth, INT_MAX, n + 1);
+  k_number_init<<<blocks_for(n + 1, 256), 256, 0, s>>>(t->starts, t->min_depth, n + 1, t->counters, t->status);
   k_count_starts<<<grid_blocks(), 256, 0, s>>>(t->tmp, t->counters, t->starts, t->min_depth);
   scan_u64(t->starts, n, reinterpret_cast<unsigned long long*>(t->scan_tmp), s);
   k_remap<<<grid_blocks(), 256, 0, s>>>(t->tmp, t->counters, t->starts, t->min_depth, t->c, t->status, n,
