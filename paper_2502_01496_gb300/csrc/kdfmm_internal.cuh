@@ -344,12 +344,19 @@ __device__ __forceinline__ double rsqrt64(double v) {
   return fma(y, fma(0.5, e, c), y);
 }
 
-// Whether a pair may lie inside either smoothing kernel's support: float32
-// test with a margin, h2 = (2 h)^2 of each side (true where the squared
-// distance leaves the float range; the kernel's formulas hold outside too).
+// Whether a pair may lie inside either smoothing kernel's support: float32 test
+// with a margin, h2 = (2 h)^2 of each side.  True for every pair whose squared
+// distance leaves the normal float range, coincident ones among them: below it
+// r2f is 0, which is not above any h2, and an h2 that is subnormal or 0 in
+// float32 (h < 6e-20) is below the least r2f that is left.  The kernel's formulas
+// hold outside the supports too (far_sqrt).
 __device__ __forceinline__ bool maybe_inside(double r2, float h2i, float h2j) {
   const float r2f = trunc_to_float(r2);
-  return !(r2f >= fmaxf(h2i, h2j) * 1.000001f && r2f < __int_as_float(0x7f800000));
+  return !(r2f > fmaxf(h2i, h2j) * 1.000001f && r2f < __int_as_float(0x7f800000));
+}
+// The distance from r2 and its reciprocal root: 0 and infinity are themselves.
+__device__ __forceinline__ double far_sqrt(double r2, double inv) {
+  return r2 > 0.0 && r2 < __longlong_as_double(0x7ff0000000000000LL) ? r2 * inv : r2;
 }
 
 // Bound on |d_float32 - d| for a distance d whose coordinates and centre lie

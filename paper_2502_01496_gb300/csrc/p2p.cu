@@ -551,9 +551,7 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
   const double h3inv_i = hinv_i * hinv_i * hinv_i;
   const float h2i = M4 ? A.ph[it].w : 0.0f;
   const double eps = A.sys_eps[A.leaf_sys[k]];
-  // added to r^2: the softening, or (M4) what keeps 1/r finite for coincident
-  // particles, whose force is 0 and whose potential the q < 1 form's
-  const double soft2 = M4 ? 1e-290 : eps * eps;
+  const double soft2 = M4 ? 0.0 : eps * eps;      // added to r^2
   double fx = 0.0, fy = 0.0, fz = 0.0, fp = 0.0;
   auto stage = [&](int at, int64_t src) {
     sx[at] = A.tp.x[src];
@@ -587,12 +585,12 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
         if ((mine & ((1u << lane) - 1u)) == 0u) s_own[warp][o] = mine;
         const double rx = tx - sx[j], ry = ty - sy[j], rz = tz - sz[j];
         const double r2 = fma(rz, rz, fma(ry, ry, fma(rx, rx, soft2)));
-        const double inv = rsqrt64(r2), r = r2 * inv, inv3 = inv * inv * inv;
+        const double inv = rsqrt64(r2), r = far_sqrt(r2, inv), inv3 = inv * inv * inv;
         const double hj = shinv[j], mh = 0.5 * sm[j];
         double f = 0.0, p = 0.0;
         m4_side64(r, inv, inv3, hi, h3i, f, p);
         m4_side64(r, inv, inv3, hj, hj * hj * hj, f, p);
-        f *= mh;
+        f = r2 > 0.0 ? f * mh : 0.0;               // coincident: no force, whatever h^-3 is
         s_term[warp][0][lane] = f * rx;
         s_term[warp][1][lane] = f * ry;
         s_term[warp][2][lane] = f * rz;

@@ -1132,18 +1132,19 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source32(VjpArgs V) {
 // evaluation with selected constants.
 __device__ __forceinline__ void m4_fg64(double r, double inv3, double inv5, double hinv, double& f,
                                         double& g) {
-  const double q = r * hinv, q2 = q * q, h2inv = hinv * hinv, h3inv = h2inv * hinv;
+  const double q = r * hinv, h2inv = hinv * hinv, h3inv = h2inv * hinv;
   const bool in = __double2hiint(q) < 0x3ff00000;            // q < 1 (q >= 0)
   const double t = 2.0 - q;
-  const double v = in ? q : (__double2hiint(t) < 0 ? 0.0 : t), v2 = v * v;
+  const bool outside = __double2hiint(t) < 0;                // its q^3 may overflow
+  const double v = in ? q : (outside ? 0.0 : t), v2 = v * v, qs = outside ? 0.0 : q;
   const double p1 = fma(v, fma(v, in ? 0.0 : -1.0 / 6.0, in ? 0.5 : 0.8), in ? -1.2 : -1.0);
   const double F = fma(in ? v2 : v2 * v2, p1, in ? 4.0 / 3.0 : 1.0);
-  const double G = in ? fma(1.5, q, -2.4) : fma(-3.0, F, v2 * v * (q2 * q));
+  const double G = in ? fma(1.5, q, -2.4) : fma(-3.0, F, v2 * v * (qs * qs * qs));
   f = fma(F, in ? h3inv : inv3, f);
   g = fma(G, in ? h3inv * h2inv : inv5, g);
 }
 __device__ __forceinline__ void m4_pair_fg64(double r2, double hinv_i, double hinv_j, double& f, double& g) {
-  const double inv = rsqrt64(r2), inv2 = inv * inv, inv3 = inv2 * inv, inv5 = inv3 * inv2, r = r2 * inv;
+  const double inv = rsqrt64(r2), inv2 = inv * inv, inv3 = inv2 * inv, inv5 = inv3 * inv2, r = far_sqrt(r2, inv);
   f = g = 0.0;
   m4_fg64(r, inv3, inv5, hinv_i, f, g);
   m4_fg64(r, inv3, inv5, hinv_j, f, g);
@@ -1206,7 +1207,7 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_pairs64(VjpArgs V) {
     const float h2o = M4 ? V.ph[own].w : 0.0f;
     const double hinv_o = M4 ? V.hinv[own] : 0.0;
     const double eps = V.sys_eps[V.leaf_sys[k]];
-    const double soft2 = M4 ? 1e-290 : eps * eps;    // (M4: 1/r finite for coincident particles)
+    const double soft2 = M4 ? 0.0 : eps * eps;       // added to r^2
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;   // vector sum and scalar sum
     // a pair's terms: f, g, own or partner's b, d, partner's mass
     auto terms = [&](double f, double g, double c0, double c1, double c2, double d0, double d1, double d2,
