@@ -203,7 +203,7 @@ int kdfmm_fmm_accel(kdfmm_tree t, double* a, double* phi, void* stream);
  * (as its evaluation does) from float64 differences, with float64 sums.  Cell
  * cotangents and the P2P source-side terms are summed with float64 atomics,
  * so the last bits may vary run to run.  Its scratch (at most 112 bytes per
- * particle, 184 per leaf, 80 per cell, 8 per near-list entry, 16 MB) stays with the
+ * particle, 192 per leaf, 80 per cell, 8 per near-list entry, 16 MB) stays with the
  * handle; a call on a capturing stream takes it with cudaMallocAsync.  Errors:
  * KDFMM_ERR_INVALID_ARG before any evaluation or for non-device pointers,
  * KDFMM_ERR_CUDA on allocation or launch failure. */

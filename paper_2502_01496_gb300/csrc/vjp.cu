@@ -200,18 +200,43 @@ struct VjpArgs {
   int64_t tcap;                         // entries of tidx
   int32_t *tseg_leaf, *tseg_first;
   int64_t tseg_cap;
-  unsigned long long* tctr;             // [0] entries reserved, [1] extra source items, [2] extra target items
+  // [0] entries reserved, [1] extra source items, [2] extra target items, [3] and
+  // [4] target and source items with close pairs (mixed mode), listed in close_t, close_s
+  unsigned long long* tctr;
+  int32_t *close_t, *close_s;
 };
 
 // A coordinate as x0 + x1 + x2 on the grids 2^(k-22), 2^(k-45) and 2^(k-68) of
 // its system (|x| <= 2^k): the difference of two coordinates is then three
-// exact float32 subtractions, and grid_diff their sum rounded to float32 -- the
-// float64 difference rounded to float32 -- without the float64 pipe (1/64 rate).
+// exact float32 subtractions, and grid_diff their sum rounded to float32, without
+// the float64 pipe (1/64 rate).  A coordinate below 2^(k-16) may have bits under
+// the last grid: the difference is off by less than 2^(k-68), so pairs closer
+// than 2^(k-36) take the float64 difference, and for the others that is 2^-32 of
+// their distance at most, against the 2^-25 of float32's rounding.  An item that
+// meets such a pair (close_pairs) is left to the float64-difference form of its
+// kernel: the branch within the loop cost the 2^20 Plummer sphere's call 5 % by
+// the registers it took.
+__device__ __forceinline__ int grid_exponent(double bound) {
+  return max(((__double2hiint(bound) >> 20) & 0x7ff) - 1022, -900);           // bound < 2^k
+}
+// Bound on the |coordinates| of a leaf's system.
+__device__ __forceinline__ double system_bound(const VjpArgs& V, int leaf) {
+  const int root = V.sys_root[V.leaf_sys[leaf]];
+  return fmax(fabs(V.c.cx[root]), fmax(fabs(V.c.cy[root]), fabs(V.c.cz[root]))) + V.c.s[root];
+}
+// Whether an item whose smallest r^2 is `lowest` has a pair closer than that: its
+// r^2 is below 2^(2 (k - 36)), but no less than the smallest normal number (the
+// grids' own underflow is 2^-149).  Always from 2^100 on, where a coordinate may
+// leave float32.
+__device__ __forceinline__ bool close_pairs(float lowest, double bound) {
+  const int e = 2 * (grid_exponent(bound) - 36);
+  return e > 127 || lowest < __int_as_float((max(e, -126) + 127) << 23);
+}
 struct GridScale {
   double c0, c1, c2;                    // adding and subtracting rounds to the grid
 };
 __device__ __forceinline__ GridScale grid_scale(double bound) {
-  const int k = max(((__double2hiint(bound) >> 20) & 0x7ff) - 1022, -900);   // bound < 2^k
+  const int k = grid_exponent(bound);
   GridScale g;
   g.c0 = __hiloint2double((min(k + 30, 1023) + 1023) << 20 | 0x80000, 0);     // 1.5 * 2^(k+30)
   g.c1 = __hiloint2double((k + 7 + 1023) << 20 | 0x80000, 0);
@@ -273,9 +298,7 @@ __global__ void __launch_bounds__(kL2PWarps * 32) k_vjp_l2p(const double* __rest
     const double x = V.tp.x[p] - V.c.cx[a], y = V.tp.y[p] - V.c.cy[a], z = V.tp.z[p] - V.c.cz[a];
     const double b0 = abar[3 * i], b1 = abar[3 * i + 1], b2 = abar[3 * i + 2];
     if (V.mixed) {
-      const int root = V.sys_root[V.leaf_sys[k]];
-      const GridScale g = grid_scale(
-          fmax(fabs(V.c.cx[root]), fmax(fabs(V.c.cy[root]), fabs(V.c.cz[root]))) + V.c.s[root]);
+      const GridScale g = grid_scale(system_bound(V, k));
       float4 u0, u1, u2;
       split_grid(V.tp.x[p], g, u0.x, u1.x, u2.x);
       split_grid(V.tp.y[p], g, u0.y, u1.y, u2.y);
@@ -821,6 +844,14 @@ __global__ void k_tr_fill(VjpArgs V) {
 __device__ __forceinline__ float dot_rn(float a0, float b0, float a1, float b1, float a2, float b2) {
   return __fmaf_rn(a2, b2, __fmaf_rn(a0, b0, __fmul_rn(a1, b1)));
 }
+// Differences of a pair that its system's grids are too coarse for: float64,
+// rounded to float32.
+__device__ __forceinline__ void exact_diff(const VjpArgs& V, int i, int j, float& d0, float& d1,
+                                           float& d2) {
+  d0 = (float)(V.tp.x[i] - V.tp.x[j]);
+  d1 = (float)(V.tp.y[i] - V.tp.y[j]);
+  d2 = (float)(V.tp.z[i] - V.tp.z[j]);
+}
 // One component of J b = -f b - g d (d.b).
 __device__ __forceinline__ float jb_term(float f, float b, float g, float d, float db) {
   return __fmaf_rn(-f, b, -__fmul_rn(__fmul_rn(g, d), db));
@@ -922,15 +953,15 @@ constexpr int kVjpWarps = 4;
 // longer than the rest of the pair).  2^20 Plummer sphere, 1.17e9 pairs: 4.7 ms
 // here and 5.7 ms on the source side, against 47.3 ms for the two together
 // when one kernel walked the pairs by target.
-template <int SOFT>
-__global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target32(VjpArgs V) {
-  __shared__ LeafChunk s_chunk[kVjpWarps];
+// EXACT: the items of close_t, with float64 differences.
+template <int SOFT, bool EXACT>
+__device__ __forceinline__ void target32_items(const VjpArgs& V, LeafChunk& B) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  LeafChunk& B = s_chunk[threadIdx.x >> 5];
-  const int nitems = near_items(V);
-  for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
-       item += (int)((gridDim.x * blockDim.x) >> 5)) {
+  const int nwork = EXACT ? (int)V.tctr[3] : near_items(V);
+  for (int at0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); at0 < nwork;
+       at0 += (int)((gridDim.x * blockDim.x) >> 5)) {
+    const int item = EXACT ? V.close_t[at0] : at0;
     const bool seg = item >= V.nleaves;
     const int gi = item - V.nleaves;
     int k;
@@ -947,6 +978,7 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target32(VjpArgs V) {
     const double eps = V.sys_eps[V.leaf_sys[k]];
     float eps2 = (float)(eps * eps);
     asm("" : "+f"(eps2));
+    float lowest = __int_as_float(0x7f800000);
     float gxh = 0.f, gxl = 0.f, gyh = 0.f, gyl = 0.f, gzh = 0.f, gzl = 0.f;
     for (int eb = 0; eb < nn;) {
       const int L = stage_chunk(V, B, lane, eb + lane < nn ? V.near_idx[e0 + eb + lane] : -1,
@@ -963,10 +995,16 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target32(VjpArgs V) {
         for (int j = sl; j < total; j += K) {
           const float4 s0 = B.p0[j], s1 = B.p1[j], s2 = B.p2[j];
           if (__float_as_int(s2.w) == pi) continue;
-          const float d0 = grid_diff(o0.x, o1.x, o2.x, s0.x, s1.x, s2.x),
-                      d1 = grid_diff(o0.y, o1.y, o2.y, s0.y, s1.y, s2.y),
-                      d2 = grid_diff(o0.z, o1.z, o2.z, s0.z, s1.z, s2.z);
+          float d0, d1, d2;
+          if constexpr (EXACT) {
+            exact_diff(V, pi, __float_as_int(s2.w), d0, d1, d2);
+          } else {
+            d0 = grid_diff(o0.x, o1.x, o2.x, s0.x, s1.x, s2.x);
+            d1 = grid_diff(o0.y, o1.y, o2.y, s0.y, s1.y, s2.y);
+            d2 = grid_diff(o0.z, o1.z, o2.z, s0.z, s1.z, s2.z);
+          }
           const float r2 = dot_rn(d0, d0, d1, d1, d2, d2);
+          if constexpr (!EXACT) lowest = fminf(lowest, r2);
           float f, g;
           pair_fg32<SOFT>(r2, eps2, o1.w, s1.w, f, g);
           const float db = dot_rn(d0, b.x, d1, b.y, d2, b.z);
@@ -980,6 +1018,10 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target32(VjpArgs V) {
         }
       }
       eb += L;
+    }
+    if (!EXACT && __any_sync(full, close_pairs(lowest, system_bound(V, k)))) {
+      if (lane == 0) V.close_t[atomicAdd(&V.tctr[3], 1ull)] = item;
+      continue;
     }
     double gx = (double)gxh + (double)gxl, gy = (double)gyh + (double)gyl,
            gz = (double)gzh + (double)gzl;
@@ -1007,16 +1049,15 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_target32(VjpArgs V) {
 // leaf.  A leaf's terms are summed over its targets in float32 as a perfect
 // binary tree (four at a time, then a carry stack), then added to a (high,
 // low) float32 pair; one float64 atomic per source and item at the end.
-template <int SOFT>
-__global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source32(VjpArgs V) {
-  __shared__ float2 s_b[kVjpWarps][kVjpStage];
-  __shared__ LeafChunk s_chunk[kVjpWarps];
+// EXACT: the items of close_s, with float64 differences.
+template <int SOFT, bool EXACT>
+__device__ __forceinline__ void source32_items(const VjpArgs& V, LeafChunk& B, float2* sb) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  LeafChunk& B = s_chunk[threadIdx.x >> 5];
-  const int nitems = V.nleaves + (int)min((int64_t)V.tctr[1], V.tseg_cap);
-  for (int item = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); item < nitems;
-       item += (int)((gridDim.x * blockDim.x) >> 5)) {
+  const int nwork = EXACT ? (int)V.tctr[4] : V.nleaves + (int)min((int64_t)V.tctr[1], V.tseg_cap);
+  for (int at0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); at0 < nwork;
+       at0 += (int)((gridDim.x * blockDim.x) >> 5)) {
+    const int item = EXACT ? V.close_s[at0] : at0;
     const bool seg = item >= V.nleaves;
     const int r = seg ? V.tseg_leaf[item - V.nleaves] : item;
     const int piece = seg ? item - V.nleaves - V.tseg_first[r] + 1 : 0;
@@ -1030,6 +1071,7 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source32(VjpArgs V) {
     const double eps = V.sys_eps[V.leaf_sys[r]];
     float eps2 = (float)(eps * eps);
     asm("" : "+f"(eps2));
+    float lowest = __int_as_float(0x7f800000);
     float sh[4] = {0.f, 0.f, 0.f, 0.f}, slo[4] = {0.f, 0.f, 0.f, 0.f};
     const int64_t e0 = V.toff[r] + (int64_t)piece * V.entries;
     const int nn = min(V.tcnt[r] - piece * V.entries, V.entries);
@@ -1042,7 +1084,7 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source32(VjpArgs V) {
                                   B.p0[at] = s;
                                   B.p1[at] = V.q1[pi];
                                   B.p2[at] = V.q2[pi];
-                                  s_b[threadIdx.x >> 5][at] = b;
+                                  sb[at] = b;
                                 });
       for (int q = sl; act && q < L; q += K) {
         const int fb = B.beg[q], nb = B.beg[q + 1] - fb;
@@ -1055,12 +1097,18 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source32(VjpArgs V) {
             s[u][0] = s[u][1] = s[u][2] = s[u][3] = 0.0f;
             if (i0 + u < nb && __float_as_int(B.p0[at].w) != pj) {
               const float4 t0 = B.p0[at], t1 = B.p1[at], t2 = B.p2[at];
-              const float2 t3 = s_b[threadIdx.x >> 5][at];
+              const float2 t3 = sb[at];
               const float3 b = make_float3(t2.w, t3.x, t3.y);
-              const float d0 = grid_diff(t0.x, t1.x, t2.x, o0.x, o1.x, o2.x),
-                          d1 = grid_diff(t0.y, t1.y, t2.y, o0.y, o1.y, o2.y),
-                          d2 = grid_diff(t0.z, t1.z, t2.z, o0.z, o1.z, o2.z);
+              float d0, d1, d2;
+              if constexpr (EXACT) {
+                exact_diff(V, __float_as_int(t0.w), pj, d0, d1, d2);
+              } else {
+                d0 = grid_diff(t0.x, t1.x, t2.x, o0.x, o1.x, o2.x);
+                d1 = grid_diff(t0.y, t1.y, t2.y, o0.y, o1.y, o2.y);
+                d2 = grid_diff(t0.z, t1.z, t2.z, o0.z, o1.z, o2.z);
+              }
               const float r2 = dot_rn(d0, d0, d1, d1, d2, d2);
+              if constexpr (!EXACT) lowest = fminf(lowest, r2);
               float f, g;
               pair_fg32<SOFT>(r2, eps2, t1.w, o1.w, f, g);
               const float db = dot_rn(d0, b.x, d1, b.y, d2, b.z);
@@ -1107,6 +1155,10 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source32(VjpArgs V) {
       }
       eb += L;
     }
+    if (!EXACT && __any_sync(full, close_pairs(lowest, system_bound(V, r)))) {
+      if (lane == 0) V.close_s[atomicAdd(&V.tctr[4], 1ull)] = item;
+      continue;
+    }
     double g[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) g[c] = (double)sh[c] + (double)slo[c];
@@ -1125,6 +1177,27 @@ __global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_source32(VjpArgs V) {
       atomicAdd(&V.msrc[pj], g[3]);
     }
   }
+}
+
+template <int SOFT>
+__global__ void __launch_bounds__(kVjpWarps * 32, SOFT == KDFMM_SOFT_M4 ? 7 : 8) k_vjp_target32(VjpArgs V) {
+  __shared__ LeafChunk s_chunk[kVjpWarps];
+  target32_items<SOFT, false>(V, s_chunk[threadIdx.x >> 5]);
+}
+template <int SOFT>
+__global__ void __launch_bounds__(kVjpWarps * 32, SOFT == KDFMM_SOFT_M4 ? 5 : 6) k_vjp_source32(VjpArgs V) {
+  __shared__ LeafChunk s_chunk[kVjpWarps];
+  __shared__ float2 s_b[kVjpWarps][kVjpStage];
+  source32_items<SOFT, false>(V, s_chunk[threadIdx.x >> 5], s_b[threadIdx.x >> 5]);
+}
+// The items that both left (none, as a rule).
+template <int SOFT>
+__global__ void __launch_bounds__(kVjpWarps * 32) k_vjp_close32(VjpArgs V) {
+  __shared__ LeafChunk s_chunk[kVjpWarps];
+  __shared__ float2 s_b[kVjpWarps][kVjpStage];
+  target32_items<SOFT, true>(V, s_chunk[threadIdx.x >> 5]);
+  __syncwarp();
+  source32_items<SOFT, true>(V, s_chunk[threadIdx.x >> 5], s_b[threadIdx.x >> 5]);
 }
 
 // One side of the symmetrised M4 pair in float64, added to f and g: the branches
@@ -1490,13 +1563,14 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
   };
   const size_t o_cell = take((size_t)nc * 10 * 8), o_xsrc = take((size_t)n * 3 * 8),
                o_msrc = take((size_t)n * 8),
-               o_tcnt = take((size_t)nl * 4), o_tcur = take((size_t)nl * 4), o_tctr = take(32);
+               o_tcnt = take((size_t)nl * 4), o_tcur = take((size_t)nl * 4), o_tctr = take(64);
   zeroed = at;
   const size_t o_xbar = take((size_t)n * 3 * 8), o_cbar = take((size_t)nl * 20 * 8),
                o_toff = take((size_t)nl * 8), o_tfirst = take((size_t)nl * 4),
                o_tidx = take((size_t)nnear * 4), o_tseg = take((size_t)V.tseg_cap * 4),
                o_nfirst = take((size_t)nl * 4), o_nseg = take((size_t)V.seg_cap * 4),
                o_npart = take((size_t)V.seg_cap * 128 * 8);
+  const size_t o_close = V.mixed ? take((size_t)(2 * nl + V.seg_cap + V.tseg_cap) * 4) : 0;
   const size_t o_q = V.mixed ? take((size_t)n * 56) : take((size_t)n * 32);
   // a call that is being captured takes its scratch from the stream's pool (a
   // graph must not refer to memory that the handle may replace)
@@ -1523,6 +1597,8 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
   V.seg_first = (int32_t*)(buf + o_nfirst);
   V.seg_leaf = (int32_t*)(buf + o_nseg);
   V.seg_part = (double*)(buf + o_npart);
+  V.close_t = (int32_t*)(buf + o_close);
+  V.close_s = V.close_t + nl + V.seg_cap;
   V.q0 = (float4*)(buf + o_q);
   V.q1 = V.q0 + n;
   V.q2 = V.q1 + n;
@@ -1533,6 +1609,7 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
   const bool m4 = t->p.soft_kind == KDFMM_SOFT_M4;
   const unsigned gw = blocks_for((int64_t)nl * 32, 128);
   const unsigned gi = blocks_for((nl + V.seg_cap) * 32, 128);    // a warp per item that there may be
+  const unsigned gclose = std::min<unsigned>(gi, grid_blocks(5));   // (resident blocks: found work in a loop)
   k_vjp_l2p<<<gw, kL2PWarps * 32, 0, s>>>(a_bar, V, m4);
   const bool std_exp = t->p.expansion == KDFMM_EXPANSION_STANDARD;
   if (V.mixed) {
@@ -1550,10 +1627,13 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
     if (m4) {
       k_vjp_target32<KDFMM_SOFT_M4><<<gi, kVjpWarps * 32, 0, s>>>(V);
       k_vjp_source32<KDFMM_SOFT_M4><<<gi, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_close32<KDFMM_SOFT_M4><<<gclose, kVjpWarps * 32, 0, s>>>(V);
     } else {
       k_vjp_target32<KDFMM_SOFT_PLUMMER><<<gi, kVjpWarps * 32, 0, s>>>(V);
       k_vjp_source32<KDFMM_SOFT_PLUMMER><<<gi, kVjpWarps * 32, 0, s>>>(V);
+      k_vjp_close32<KDFMM_SOFT_PLUMMER><<<gclose, kVjpWarps * 32, 0, s>>>(V);
     }
+    t->launches += 1;
   } else {
     if (m4) {
       k_vjp_pairs64<KDFMM_SOFT_M4, false><<<gi, kVjpWarps * 32, 0, s>>>(V);
