@@ -3,7 +3,7 @@
 // and smoothing lengths held fixed).  The paper has no adjoint; this is the
 // derivative of the evaluation of Sec. 2 (Eqs. 3, 6, 7, 8, 13).  FP64 mode
 // runs every step in float64; mixed mode runs the M2L and P2P reverses with
-// float32 terms (as its forward does) and float64 sums.
+// float32 terms (as its forward does) and sums of float64 or wider.
 //
 // a_i = sum_{j in near(leaf i), j != i} m_j K(x_i - x_j)            (P2P)
 //     + L(C_alpha, x_i - com_alpha)                                (L2P, Eq. 8)
@@ -18,6 +18,7 @@
 // polynomial in x_i, summed over the leaf's chain of ancestors.
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include "kdfmm_internal.cuh"
 
@@ -545,7 +546,7 @@ __device__ __forceinline__ float q_cotangent(const float R[3], const GTerms& G, 
 }
 
 // Mixed mode: coefficients in float32 (as in the forward), r formed in
-// float64, sums in float64 (atomics) or (high, low) float32 pairs.
+// float64, sums in float64.
 template <bool STD>
 __global__ void __launch_bounds__(kM2LWarps * 32) k_vjp_m2l32(VjpArgs V) {
   __shared__ CellBuf s_buf[kM2LWarps];
@@ -559,7 +560,7 @@ __global__ void __launch_bounds__(kM2LWarps * 32) k_vjp_m2l32(VjpArgs V) {
 #pragma unroll
   for (int j = 0; j < 20; ++j) cb[j] = __shfl_sync(0xffffffffu, mine, j);
   const double ax = V.c.cx[a], ay = V.c.cy[a], az = V.c.cz[a];
-  float rh[3] = {0.f, 0.f, 0.f}, rl[3] = {0.f, 0.f, 0.f};
+  double rx = 0.0, ry = 0.0, rz = 0.0;
   const int64_t off = V.far_off[k];
   const int nf = (int)min((int64_t)V.far_cnt[k], V.cap_far);
   for (int e0 = 0; e0 < nf; e0 += 32) {
@@ -578,10 +579,8 @@ __global__ void __launch_bounds__(kM2LWarps * 32) k_vjp_m2l32(VjpArgs V) {
       double* v = B.v + 11 * lane;
       B.cell[lane] = b;
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        df_add(rh[i], rl[i], cr.d[i]);
-        v[1 + i] = -(double)cr.d[i];
-      }
+      for (int i = 0; i < 3; ++i) v[1 + i] = -(double)cr.d[i];
+      rx -= v[1]; ry -= v[2]; rz -= v[3];
       const GTerms G = g_terms(r);
       v[0] = (double)mass_cotangent(r, G, cb);
       v[4] = (double)q_cotangent<0, 0, STD>(r, G, cb);
@@ -593,8 +592,6 @@ __global__ void __launch_bounds__(kM2LWarps * 32) k_vjp_m2l32(VjpArgs V) {
     }
     cell_buf_add(V, B, lane, n);
   }
-  double rx = (double)rh[0] + (double)rl[0], ry = (double)rh[1] + (double)rl[1],
-         rz = (double)rh[2] + (double)rl[2];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     rx += __shfl_xor_sync(0xffffffffu, rx, o);
@@ -944,16 +941,39 @@ __device__ __forceinline__ int stage_chunk(const VjpArgs& V, Chunk& B, int lane,
 
 constexpr int kVjpWarps = 4;
 
+// A sum of float32 terms in three float32 numbers: what the first two lose is
+// carried exactly (two-sums), so n terms of magnitude v are off by some
+// n^2 2^-73 v, where a float64 sum loses up to n^2 2^-54 v.
+struct Sum72 {
+  float h, m, l;
+  __device__ __forceinline__ void add(float v) {
+    float e, e2;
+    two_sum(h, v, h, e);
+    two_sum(m, e, m, e2);
+    l = __fadd_rn(l, e2);
+  }
+  __device__ __forceinline__ double value() const { return (double)h + ((double)m + (double)l); }
+  // false once a term or the sum has left float32
+  __device__ __forceinline__ bool holds() const { return fabsf(h) < __int_as_float(0x7f800000); }
+};
+struct Sum64 {
+  double s;
+  __device__ __forceinline__ void add(float v) { s += float_to_double(v); }
+  __device__ __forceinline__ double value() const { return s; }
+  __device__ __forceinline__ bool holds() const { return true; }
+};
+
 // Mixed mode, target side: warp per target leaf (or segment of a long near
 // list), lanes = (target, slice) as in the forward; a leaf's sources are read
 // by broadcast (a warp instruction touches the slices' few records).  Terms in
-// float32, the same operations as the source side's; each is added to a
-// (high, low) float32 pair, 48 bits, which takes the place of a float64 sum
-// (three float64 additions a pair would keep the 1/64-rate pipe busy for
-// longer than the rest of the pair).  2^20 Plummer sphere, 1.17e9 pairs: 4.7 ms
-// here and 5.7 ms on the source side, against 47.3 ms for the two together
-// when one kernel walked the pairs by target.
-// EXACT: the items of close_t, with float64 differences.
+// float32, the same operations as the source side's; each is added to a sum of
+// three float32 numbers, in the place of a float64 sum (three float64 additions a
+// pair would keep the 1/64-rate pipe busy for longer than the rest of the pair)
+// and with less rounding than it.  2^20 Plummer sphere, 1.17e9 pairs: 5.2 ms
+// here and 5.4 ms on the source side (4.3 and 5.1 with two float32 numbers a sum;
+// one of the three sums in float64: 0.5 ms more), against 47.3 ms for the two
+// together when one kernel walked the pairs by target.
+// EXACT: the items of close_t, with float64 differences and sums.
 template <int SOFT, bool EXACT>
 __device__ __forceinline__ void target32_items(const VjpArgs& V, LeafChunk& B) {
   const unsigned full = 0xffffffffu;
@@ -979,7 +999,7 @@ __device__ __forceinline__ void target32_items(const VjpArgs& V, LeafChunk& B) {
     float eps2 = (float)(eps * eps);
     asm("" : "+f"(eps2));
     float lowest = __int_as_float(0x7f800000);
-    float gxh = 0.f, gxl = 0.f, gyh = 0.f, gyl = 0.f, gzh = 0.f, gzl = 0.f;
+    typename std::conditional<EXACT, Sum64, Sum72>::type sx{}, sy{}, sz{};
     for (int eb = 0; eb < nn;) {
       const int L = stage_chunk(V, B, lane, eb + lane < nn ? V.near_idx[e0 + eb + lane] : -1,
                                 [&](int at, int pj) {
@@ -1012,19 +1032,19 @@ __device__ __forceinline__ void target32_items(const VjpArgs& V, LeafChunk& B) {
           const float jx = jb_term(f, b.x, g, d0, db);
           const float jy = jb_term(f, b.y, g, d1, db);
           const float jz = jb_term(f, b.z, g, d2, db);
-          df_add(gxh, gxl, __fmul_rn(s0.w, jx));
-          df_add(gyh, gyl, __fmul_rn(s0.w, jy));
-          df_add(gzh, gzl, __fmul_rn(s0.w, jz));
+          sx.add(__fmul_rn(s0.w, jx));
+          sy.add(__fmul_rn(s0.w, jy));
+          sz.add(__fmul_rn(s0.w, jz));
         }
       }
       eb += L;
     }
-    if (!EXACT && __any_sync(full, close_pairs(lowest, system_bound(V, k)))) {
+    if (!EXACT && __any_sync(full, close_pairs(lowest, system_bound(V, k)) || !sx.holds() ||
+                                       !sy.holds() || !sz.holds())) {
       if (lane == 0) V.close_t[atomicAdd(&V.tctr[3], 1ull)] = item;
       continue;
     }
-    double gx = (double)gxh + (double)gxl, gy = (double)gyh + (double)gyl,
-           gz = (double)gzh + (double)gzl;
+    double gx = sx.value(), gy = sy.value(), gz = sz.value();
     for (int s = 1; s < K; ++s) {
       const int src = t + s * nt;
       const double ox = __shfl_sync(full, gx, src), oy = __shfl_sync(full, gy, src),
@@ -1047,8 +1067,8 @@ __device__ __forceinline__ void target32_items(const VjpArgs& V, LeafChunk& B) {
 // Mixed mode, source side: warp per source leaf (or piece of a long
 // transposed list), lanes = (source, slice), a slice taking every K-th target
 // leaf.  A leaf's terms are summed over its targets in float32 as a perfect
-// binary tree (four at a time, then a carry stack), then added to a (high,
-// low) float32 pair; one float64 atomic per source and item at the end.
+// binary tree (four at a time, then a carry stack), then added in float64; one
+// float64 atomic per source and item at the end.
 // EXACT: the items of close_s, with float64 differences.
 template <int SOFT, bool EXACT>
 __device__ __forceinline__ void source32_items(const VjpArgs& V, LeafChunk& B, float2* sb) {
@@ -1072,7 +1092,7 @@ __device__ __forceinline__ void source32_items(const VjpArgs& V, LeafChunk& B, f
     float eps2 = (float)(eps * eps);
     asm("" : "+f"(eps2));
     float lowest = __int_as_float(0x7f800000);
-    float sh[4] = {0.f, 0.f, 0.f, 0.f}, slo[4] = {0.f, 0.f, 0.f, 0.f};
+    double g[4] = {0.0, 0.0, 0.0, 0.0};
     const int64_t e0 = V.toff[r] + (int64_t)piece * V.entries;
     const int nn = min(V.tcnt[r] - piece * V.entries, V.entries);
     for (int eb = 0; eb < nn;) {
@@ -1151,7 +1171,7 @@ __device__ __forceinline__ void source32_items(const VjpArgs& V, LeafChunk& B, f
           }
         }
 #pragma unroll
-        for (int c = 0; c < 4; ++c) df_add(sh[c], slo[c], acc[c]);
+        for (int c = 0; c < 4; ++c) g[c] += float_to_double(acc[c]);
       }
       eb += L;
     }
@@ -1159,9 +1179,6 @@ __device__ __forceinline__ void source32_items(const VjpArgs& V, LeafChunk& B, f
       if (lane == 0) V.close_s[atomicAdd(&V.tctr[4], 1ull)] = item;
       continue;
     }
-    double g[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) g[c] = (double)sh[c] + (double)slo[c];
     for (int s = 1; s < K; ++s) {
       const int src = j + s * ns;
 #pragma unroll
