@@ -325,9 +325,11 @@ __device__ __forceinline__ float rsqrt_ftz(float x) {
 // float32 rate here: each costs as much as ~75 float32 or integer ones).  The
 // float32 estimate y of the mantissa's reciprocal root is moved to float64
 // with integer operations, and one step of Householder's third-order
-// iteration, y (1 + e/2 + 3/8 e^2) with e = 1 - v y^2, leaves the rounding of
-// e and of the result (|e| < 2^-21, so the remainder is below 2^-64).  The
-// 3/8 e^2 term, below 2^-43, is formed in float32.  Zero, subnormal, negative,
+// iteration follows, y (1 + e/2 + 3/8 e^2) with e = 1 - v y^2 (|e| < 2^-21).
+// y^2 is exact (48 bits; above the least subnormal even for the largest v), so e
+// has one rounding, of 2^-75; the 3/8 e^2 term, below 2^-43, in float32 is off by
+// 2^-65 and so is the remainder: the result is within 0.501 units in the last
+// place, where the library's function allows one.  Zero, subnormal, negative,
 // infinite and NaN arguments take the library's function.
 __device__ __forceinline__ double rsqrt64(double v) {
   const int hi = __double2hiint(v), lo = __double2loint(v);
@@ -337,7 +339,7 @@ __device__ __forceinline__ double rsqrt64(double v) {
                                  (int)((unsigned)lo >> 29));
   const int yb = __float_as_int(rsqrt_ftz(m));             // in (1/2, 1]
   const double y = __hiloint2double((yb >> 3) + ((896 - (ex >> 1)) << 20), yb << 29);
-  const double e = fma(-(v * y), y, 1.0);
+  const double e = fma(-v, __dmul_rn(y, y), 1.0);
   const float ef = trunc_to_float(e);
   const int cb = __float_as_int(0.375f * ef * ef);         // (0 becomes 2^-127: far below rounding)
   const double c = __hiloint2double((cb >> 3) + (896 << 20), cb << 29);
