@@ -66,14 +66,26 @@ struct P2PArgs {
   double* seg_part;
   int64_t seg_cap;
   const int64_t* sys_off;    // float64: first particle of each system; mixed: null
+  bool grouped;              // a work item is a group of segments (k_p2p_fp64: GROUPS)
 };
 
 // Near entries per segment, by the particles of the leaf's own system alone: an
-// eager evaluation, a replayed graph and a batch that holds the system split
+// eager evaluation, a replayed graph and a batch that holds the system sum
 // alike.  Float64 evaluations of few particles take short segments: their leaves
 // are too few warps for the GPU's 608 float64 pipes (4096 particles: 367 leaves
 // with ~108 near leaves each).  Mixed evaluations keep 256: a shorter segment
 // would move the chunks of 256 sources whose float32 sums are folded at once.
+//
+// A segment's sums start at zero.  Those of a group of 256 entries are added in
+// order, then the groups: (first segment + expansion + rest of the first group)
+// + (second group + third + ...).  So it makes no difference who adds: with few
+// particles in the call each segment is a work item whose sums go to memory
+// (1 KB) for k_seg_combine; from kFullCall on the leaves themselves fill the GPU
+// (16384 warps and more) and a work item is a group, its segments added in
+// registers -- a forest of small systems would take 128 bytes a near entry
+// otherwise, where a group takes 4.  256 systems of 4096, 9.6e6 near entries: 47.9 ms
+// a call and 1.2 GB by segments, 48.1 ms and 38 MB by groups; 64 of 8191: 27.5 and 28.4 ms.
+constexpr int64_t kFullCall = 262144;
 constexpr int kSegSteps = 3;
 __host__ __device__ __forceinline__ int64_t seg_below(int step) {      // particles, exclusive
   return step == 0 ? 8192 : (step == 1 ? 65536 : 262144);
@@ -85,6 +97,10 @@ __host__ __device__ __forceinline__ int seg_step(int64_t n) {
   int step = 0;
   while (step < kSegSteps && n >= seg_below(step)) ++step;
   return step;
+}
+// Entries per work item.
+__device__ __forceinline__ int item_entries(bool grouped, int seglen) {
+  return grouped ? kSegEntries : seglen;
 }
 __device__ __forceinline__ int leaf_segment(const int64_t* __restrict__ sys_off, int sys) {
   return sys_off == nullptr ? kSegEntries : seg_length(seg_step(sys_off[sys + 1] - sys_off[sys]));
@@ -512,8 +528,9 @@ __device__ __forceinline__ void m4_side64(double r, double inv, double inv3, dou
 // supports are float32.  With the library's rsqrt, float64 tests and divisions
 // per kernel pair it was ~45 (M4 binary of 2 x 2^20: 133 ms, now 74; Plummer
 // sphere of 4096: 1.42 ms in long segments, now 0.23).
-template <int SOFT>
-__global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
+template <int SOFT, bool GROUPS>
+__global__ void __launch_bounds__(kP2P64Warps * 32, SOFT == KDFMM_SOFT_PLUMMER && !GROUPS ? 8 : 1)
+k_p2p_fp64(P2PArgs A) {
   constexpr bool M4 = SOFT == KDFMM_SOFT_M4;
   __shared__ double s_x[kP2P64Warps][kStage64], s_y[kP2P64Warps][kStage64];
   __shared__ double s_z[kP2P64Warps][kStage64], s_m[kP2P64Warps][kStage64];
@@ -639,60 +656,79 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
       if (nq > 0) kernel_pairs(nq);
     }
   };
-  if (!seg) {
-    if (lane < nt) stage(lane, (int64_t)fa + lane);
-    __syncwarp();
-    sum_staged(nt, t);
-    __syncwarp();
-  }
   const int64_t nall = min((int64_t)A.near_cnt[k], A.cap_near);
-  const int64_t sidx = seg ? (int64_t)(g - A.seg_first[k] + 1) : 0;
   const int seglen = leaf_segment(A.sys_off, A.leaf_sys[k]);
-  const int64_t e1 = A.near_off[k] + min(nall, (sidx + 1) * seglen);
-  for (int64_t e = A.near_off[k] + sidx * seglen; e < e1;) {
-    const int64_t my = e + lane;
-    int cnt = 0, first = 0;
-    if (my < e1) {
-      const int b = A.near_idx[my];
-      if (b != a) {
-        cnt = A.ccount[b];
-        first = A.cfirst[b];
+  const int64_t sidx = seg ? (int64_t)(g - A.seg_first[k] + 1) : 0;
+  const int64_t entries = item_entries(GROUPS, seglen);
+  const int64_t e_end = A.near_off[k] + min(nall, (sidx + 1) * entries);
+  double bx = 0.0, by = 0.0, bz = 0.0, bp = 0.0;      // GROUPS, slice 0: sums of the leaf's first
+  double rx = 0.0, ry = 0.0, rz = 0.0, rp = 0.0;      // segment, and of the item's others
+  bool lead = !seg;
+  int64_t e = A.near_off[k] + sidx * entries;
+  do {
+    if (lead) {
+      if (lane < nt) stage(lane, (int64_t)fa + lane);
+      __syncwarp();
+      sum_staged(nt, t);
+      __syncwarp();
+    }
+    const int64_t e1 = min(e + seglen, e_end);
+    while (e < e1) {
+      const int64_t my = e + lane;
+      int cnt = 0, first = 0;
+      if (my < e1) {
+        const int b = A.near_idx[my];
+        if (b != a) {
+          cnt = A.ccount[b];
+          first = A.cfirst[b];
+        }
       }
-    }
-    int incl = cnt;
+      int incl = cnt;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int w = __shfl_up_sync(full, incl, o);
-      if (lane >= o) incl += w;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int w = __shfl_up_sync(full, incl, o);
+        if (lane >= o) incl += w;
+      }
+      const int L = __popc(__ballot_sync(full, my < e1 && incl <= kStage64));
+      if (lane < L) {
+        const int beg = incl - cnt;
+        tb[lane] = beg;
+        tf[lane] = first;
+        for (int q = 0; q < cnt; ++q) sl_of[beg + q] = (uint8_t)lane;
+      }
+      __syncwarp();
+      const int total = __shfl_sync(full, incl, L - 1);
+      for (int idx = lane; idx < total; idx += 32) {
+        const int l = sl_of[idx];
+        stage(idx, (int64_t)tf[l] + idx - tb[l]);
+      }
+      __syncwarp();
+      sum_staged(total, -1);
+      __syncwarp();
+      e += L;
     }
-    const int L = __popc(__ballot_sync(full, my < e1 && incl <= kStage64));
-    if (lane < L) {
-      const int beg = incl - cnt;
-      tb[lane] = beg;
-      tf[lane] = first;
-      for (int q = 0; q < cnt; ++q) sl_of[beg + q] = (uint8_t)lane;
+    // the segment's slices, in slice order
+    for (int s = 1; s < K; ++s) {
+      const int src = t + s * nt;
+      const double ox = __shfl_sync(full, fx, src), oy = __shfl_sync(full, fy, src);
+      const double oz = __shfl_sync(full, fz, src), op = __shfl_sync(full, fp, src);
+      if (sl == 0) { fx += ox; fy += oy; fz += oz; fp += op; }
     }
-    __syncwarp();
-    const int total = __shfl_sync(full, incl, L - 1);
-    for (int idx = lane; idx < total; idx += 32) {
-      const int l = sl_of[idx];
-      stage(idx, (int64_t)tf[l] + idx - tb[l]);
+    if constexpr (GROUPS) {
+      if (lead) { bx = fx; by = fy; bz = fz; bp = fp; }
+      else { rx += fx; ry += fy; rz += fz; rp += fp; }
+      fx = fy = fz = fp = 0.0;
+      lead = false;
     }
-    __syncwarp();
-    sum_staged(total, -1);
-    __syncwarp();
-    e += L;
-  }
-  for (int s = 1; s < K; ++s) {
-    const int src = t + s * nt;
-    const double bx = __shfl_sync(full, fx, src), by = __shfl_sync(full, fy, src);
-    const double bz = __shfl_sync(full, fz, src), bp = __shfl_sync(full, fp, src);
-    if (sl == 0) { fx += bx; fy += by; fz += bz; fp += bp; }
+  } while (GROUPS && e < e_end);
+  if constexpr (!GROUPS) {                            // one segment an item
+    if (seg) { rx = fx; ry = fy; rz = fz; rp = fp; }
+    else { bx = fx; by = fy; bz = fz; bp = fp; }
   }
   if (sl != 0 || !act) continue;
   if (seg) {
     double* P = A.seg_part + (int64_t)g * 128 + 4 * t;
-    P[0] = fx; P[1] = fy; P[2] = fz; P[3] = fp;
+    P[0] = rx; P[1] = ry; P[2] = rz; P[3] = rp;
     continue;
   }
   const double* C = A.lexp64 + 20 * (int64_t)k;
@@ -700,10 +736,10 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
   double tx, ty, tz, tp_;
   l2p_tail<double>(C, x, y, z, tx, ty, tz, tp_);
   const int64_t ci = A.tp.idx[it];
-  A.a[3 * ci + 0] = fx + (tx - C[1]);
-  A.a[3 * ci + 1] = fy + (ty - C[2]);
-  A.a[3 * ci + 2] = fz + (tz - C[3]);
-  if (A.phi) A.phi[ci] = fp + (C[0] + tp_);
+  A.a[3 * ci + 0] = (bx + (tx - C[1])) + rx;
+  A.a[3 * ci + 1] = (by + (ty - C[2])) + ry;
+  A.a[3 * ci + 2] = (bz + (tz - C[3])) + rz;
+  if (A.phi) A.phi[ci] = (bp + (C[0] + tp_)) + rp;
   }
 }
 
@@ -714,10 +750,11 @@ __global__ void __launch_bounds__(kP2P64Warps * 32) k_p2p_fp64(P2PArgs A) {
 __global__ void k_seg_plan(const int32_t* __restrict__ near_cnt, int64_t cap_near,
                            int max_leaves, int32_t* counters, int32_t* seg_first,
                            int32_t* seg_leaf, int64_t seg_cap, const int64_t* __restrict__ sys_off,
-                           const int32_t* __restrict__ leaf_sys, int32_t* status) {
+                           const int32_t* __restrict__ leaf_sys, bool grouped, int32_t* status) {
   const int nleaves = min(counters[C_LEAVES], max_leaves);
   KD_GRID_STRIDE(k, nleaves) {
-    const int x = extra_segments(min((int64_t)near_cnt[k], cap_near), leaf_segment(sys_off, leaf_sys[k]));
+    const int x = extra_segments(min((int64_t)near_cnt[k], cap_near),
+                                 item_entries(grouped, leaf_segment(sys_off, leaf_sys[k])));
     int first = -1;
     if (x > 0) {
       const int base = atomicAdd(&counters[C_SEGS], x);
@@ -733,8 +770,9 @@ __global__ void k_seg_plan(const int32_t* __restrict__ near_cnt, int64_t cap_nea
   }
 }
 
-// Adds the extra segments' partial sums to a and phi (caller order), warp
-// per leaf (the warp of its first extra segment), lane per target.
+// Adds the extra items' partial sums to a and phi (caller order): the rest of
+// the first group, then the other groups' sums.  Warp per leaf (the warp of its
+// first extra item), lane per target.
 __global__ void k_seg_combine(P2PArgs A) {
   const int lane = threadIdx.x & 31;
   const int nseg = (int)min((int64_t)A.counters[C_SEGS], A.seg_cap);
@@ -746,21 +784,31 @@ __global__ void k_seg_combine(P2PArgs A) {
     if (g != f) continue;
     const int a = A.leaf_cells[k];
     if (lane >= A.ccount[a]) continue;
-    const int x = extra_segments(min((int64_t)A.near_cnt[k], A.cap_near),
-                                 leaf_segment(A.sys_off, A.leaf_sys[k]));
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    // (a heavy leaf has hundreds of segments: eight pieces' loads in flight)
+    const int entries = item_entries(A.grouped, leaf_segment(A.sys_off, A.leaf_sys[k]));
+    const int x = extra_segments(min((int64_t)A.near_cnt[k], A.cap_near), entries);
+    const int group = kSegEntries / entries;              // items of a group (a power of two)
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;        // of the group
+    double r0 = 0.0, r1 = 0.0, r2 = 0.0, r3 = 0.0;        // of the first group
+    double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;        // of the others
+    // (a heavy leaf has hundreds of items: eight pieces' loads in flight)
 #pragma unroll 8
-    for (int q = 0; q < x; ++q) {
-      const double2* P = reinterpret_cast<const double2*>(A.seg_part + (int64_t)(f + q) * 128 + 4 * lane);
+    for (int q = 1; q <= x; ++q) {
+      const double2* P = reinterpret_cast<const double2*>(A.seg_part + (int64_t)(f + q - 1) * 128 + 4 * lane);
       const double2 p01 = P[0], p23 = P[1];
+      if ((q & (group - 1)) == 0) {
+        if (q == group) { r0 = s0; r1 = s1; r2 = s2; r3 = s3; }
+        else { t0 += s0; t1 += s1; t2 += s2; t3 += s3; }
+        s0 = s1 = s2 = s3 = 0.0;
+      }
       s0 += p01.x; s1 += p01.y; s2 += p23.x; s3 += p23.y;
     }
+    if (x < group) { r0 = s0; r1 = s1; r2 = s2; r3 = s3; }
+    else { t0 += s0; t1 += s1; t2 += s2; t3 += s3; }
     const int64_t ci = A.tp.idx[A.cfirst[a] + lane];
-    A.a[3 * ci + 0] += s0;
-    A.a[3 * ci + 1] += s1;
-    A.a[3 * ci + 2] += s2;
-    if (A.phi) A.phi[ci] += s3;
+    A.a[3 * ci + 0] = (A.a[3 * ci + 0] + r0) + t0;
+    A.a[3 * ci + 1] = (A.a[3 * ci + 1] + r1) + t1;
+    A.a[3 * ci + 2] = (A.a[3 * ci + 2] + r2) + t2;
+    if (A.phi) A.phi[ci] = (A.phi[ci] + r3) + t3;
   }
 }
 
@@ -796,12 +844,18 @@ int ensure_segments(kdfmm_tree_s* t, int64_t need) {
   return KDFMM_OK;
 }
 
-// At most so many extra segments: of each length class the entries of its
-// systems (no more than all, no more than their particles squared) over the length.
+// (Mixed segments and those of one large system are of 256 entries by themselves.)
+static bool grouped_call(const kdfmm_tree_s* t) {
+  return t->p.precision == KDFMM_FP64 && t->n_sys > 1 && t->n >= kFullCall;
+}
+
+// At most so many extra items: by groups, and in mixed evaluations, the entries
+// over 256, else of each length class the entries of its systems (no more than
+// all, no more than their particles squared) over the length.
 int64_t segments_bound(const kdfmm_tree_s* t) {
   const Lists& L = t->L;
   const int64_t entries = L.exact ? L.near_cap : t->host_stats[KDFMM_STAT_NNEAR];
-  if (t->p.precision != KDFMM_FP64) return entries / kSegEntries + 64;
+  if (t->p.precision != KDFMM_FP64 || grouped_call(t)) return entries / kSegEntries + 64;
   if (t->n_sys == 1) return entries / seg_length(seg_step(t->n)) + 64;
   double own[kSegSteps + 1] = {};
   for (int k = 0; k < t->n_sys; ++k) {
@@ -820,7 +874,7 @@ int plan_segments(kdfmm_tree_s* t, cudaStream_t s) {
   k_seg_plan<<<std::min<unsigned>(blocks_for(gl, 256), grid_blocks()), 256, 0, s>>>(
       t->L.near_cnt, t->L.exact ? INT64_MAX : t->L.cap_near, gl, t->counters, t->L.seg_first,
       t->L.seg_leaf, t->L.seg_cap, t->p.precision == KDFMM_FP64 ? t->sys_off : nullptr, t->leaf_sys,
-      t->status);
+      grouped_call(t), t->status);
   t->launches += 1;
   return check_cuda(cudaGetLastError(), "segment plan");
 }
@@ -856,6 +910,7 @@ int run_p2p(kdfmm_tree_s* t, double* a, double* phi, cudaStream_t s) {
   int rc = plan_segments(t, s);
   if (rc) return rc;
   A.sys_off = t->p.precision == KDFMM_FP64 ? t->sys_off : nullptr;
+  A.grouped = grouped_call(t);
   const int gl = std::max(t->grid_leaves, 1);
   const bool m4 = t->p.soft_kind == KDFMM_SOFT_M4;
   if (t->p.precision == KDFMM_MIXED) {
@@ -865,8 +920,13 @@ int run_p2p(kdfmm_tree_s* t, double* a, double* phi, cudaStream_t s) {
   } else {
     // a warp per leaf and per segment that there may be
     const unsigned g64 = blocks_for(gl + t->L.seg_cap, kP2P64Warps);
-    if (m4) k_p2p_fp64<KDFMM_SOFT_M4><<<g64, kP2P64Warps * 32, 0, s>>>(A);
-    else k_p2p_fp64<KDFMM_SOFT_PLUMMER><<<g64, kP2P64Warps * 32, 0, s>>>(A);
+    if (A.grouped) {
+      if (m4) k_p2p_fp64<KDFMM_SOFT_M4, true><<<g64, kP2P64Warps * 32, 0, s>>>(A);
+      else k_p2p_fp64<KDFMM_SOFT_PLUMMER, true><<<g64, kP2P64Warps * 32, 0, s>>>(A);
+    } else {
+      if (m4) k_p2p_fp64<KDFMM_SOFT_M4, false><<<g64, kP2P64Warps * 32, 0, s>>>(A);
+      else k_p2p_fp64<KDFMM_SOFT_PLUMMER, false><<<g64, kP2P64Warps * 32, 0, s>>>(A);
+    }
   }
   k_seg_combine<<<grid_blocks(2), 256, 0, s>>>(A);
   t->launches += 2;
