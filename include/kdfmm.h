@@ -205,8 +205,10 @@ int kdfmm_fmm_accel(kdfmm_tree t, double* a, double* phi, void* stream);
  * (as its evaluation does) from float64 differences, with sums of float64 or wider.  Cell
  * cotangents and the P2P source-side terms are summed with float64 atomics,
  * so the last bits may vary run to run.  Its scratch (at most 112 bytes per
- * particle, 192 per leaf, 80 per cell, 8 per near-list entry, 16 MB) stays with the
- * handle; a call on a capturing stream takes it with cudaMallocAsync.  Errors:
+ * particle, 192 per leaf, 80 per cell, 8 per near-list entry, 16 MB, and an eighth
+ * more) stays with the handle; calls of one handle on several streams follow one
+ * another on the device.  A call on a capturing stream takes its own scratch with
+ * cudaMallocAsync.  Errors:
  * KDFMM_ERR_INVALID_ARG before any evaluation or for non-device pointers,
  * KDFMM_ERR_CUDA on allocation or launch failure. */
 int kdfmm_fmm_accel_vjp(kdfmm_tree t, const double* a_bar, double* x_bar, double* m_bar,

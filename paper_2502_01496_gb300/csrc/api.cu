@@ -431,6 +431,7 @@ void kdfmm_tree_destroy(kdfmm_tree t) {
   cudaFree(t->L.temp);
   cudaFree(t->mom_partial);
   cudaFree(t->vjp_buf);
+  if (t->vjp_done) cudaEventDestroy(t->vjp_done);
   cudaFree(t->sys_off); cudaFree(t->sys_theta); cudaFree(t->sys_eps); cudaFree(t->sys_nleaf);
   cudaFree(t->sys_root);
   if (t->host_sys_off) cudaFreeHost(t->host_sys_off);

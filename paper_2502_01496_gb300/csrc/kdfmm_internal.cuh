@@ -230,6 +230,7 @@ struct kdfmm_tree_s {
 
   void* vjp_buf = nullptr;         // scratch of the adjoint
   size_t vjp_cap = 0;              // its bytes
+  cudaEvent_t vjp_done = nullptr;  // recorded by the last call on it
 
   // captured evaluation (kdfmm_fmm_accel_batched): valid for the arguments
   // and buffers it was captured with

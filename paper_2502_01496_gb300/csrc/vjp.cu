@@ -1528,13 +1528,22 @@ __global__ void __launch_bounds__(128) k_vjp_moments(VjpArgs V, double* __restri
 
 }  // namespace
 
-// Scratch of the adjoint, kept with the handle (grows only; freed with it).
-static int ensure_vjp_scratch(kdfmm_tree_s* t, size_t bytes) {
-  if (t->vjp_cap >= bytes) return KDFMM_OK;
+// Scratch of the adjoint, kept with the handle (grows by an eighth more than
+// asked for: near lists change with the particles; freed with it).  The calls of
+// a handle follow one another on it, whatever streams they are on: each waits for
+// the event that the one before recorded.
+static int ensure_vjp_scratch(kdfmm_tree_s* t, size_t bytes, cudaStream_t s) {
+  int rc;
+  if (!t->vjp_done &&
+      (rc = check_cuda(cudaEventCreateWithFlags(&t->vjp_done, cudaEventDisableTiming), "adjoint event")))
+    return rc;
+  if (t->vjp_cap >= bytes) return check_cuda(cudaStreamWaitEvent(s, t->vjp_done, 0), "adjoint order");
+  if ((rc = check_cuda(cudaEventSynchronize(t->vjp_done), "adjoint order"))) return rc;
   cudaFree(t->vjp_buf);
   t->vjp_buf = nullptr;
   t->vjp_cap = 0;
-  const int rc = check_cuda(cudaMalloc(&t->vjp_buf, bytes), "adjoint scratch");
+  bytes += bytes / 8;
+  rc = check_cuda(cudaMalloc(&t->vjp_buf, bytes), "adjoint scratch");
   if (!rc) t->vjp_cap = bytes;
   else cudaGetLastError();
   return rc;
@@ -1597,7 +1606,7 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
   const bool pooled = capturing != cudaStreamCaptureStatusNone;
   char* buf = nullptr;
   if (pooled) rc = check_cuda(cudaMallocAsync((void**)&buf, at, s), "adjoint scratch");
-  else if (!(rc = ensure_vjp_scratch(t, at))) buf = static_cast<char*>(t->vjp_buf);
+  else if (!(rc = ensure_vjp_scratch(t, at, s))) buf = static_cast<char*>(t->vjp_buf);
   if (rc) return rc;
   V.cell_bar = (double*)(buf + o_cell);
   V.xsrc = (double*)(buf + o_xsrc);
@@ -1665,7 +1674,12 @@ int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, 
   k_vjp_moments<<<blocks_for((int64_t)nl * 16, 128), 128, 0, s>>>(V, x_bar, m_bar);
   t->launches += 11;
   rc = check_cuda(cudaGetLastError(), "adjoint launch");
-  if (pooled) cudaFreeAsync(buf, s);
+  if (pooled) {
+    cudaFreeAsync(buf, s);
+  } else {
+    const int err = check_cuda(cudaEventRecord(t->vjp_done, s), "adjoint order");
+    rc = rc ? rc : err;
+  }
   return rc;
 }
 
