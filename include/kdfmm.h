@@ -97,8 +97,9 @@ typedef struct {
 #define KDFMM_STAT_NFALLBACK 7    /* degenerate cuts split by position */
 #define KDFMM_STAT_NEXACT 8       /* opening decisions settled in float64 */
 #define KDFMM_STAT_LAUNCHES 9     /* kernels launched since the handle was created */
-#define KDFMM_STAT_NHEAVY 10      /* leaves whose walk passed the walk budget and was redone
-                                     block-wide (leaf walk; 0 for the dual walk) */
+#define KDFMM_STAT_NHEAVY 10      /* leaves whose walk was handed on (walk budget; see
+                                     kdfmm_tree_set_walk_budget) and redone block-wide
+                                     (leaf walk; 0 for the dual walk) */
 #define KDFMM_NSTATS 11
 
 /* Phases timed by kdfmm_tree_timing (milliseconds of the most recent call). */
@@ -278,9 +279,13 @@ int kdfmm_tree_export(kdfmm_tree t, int64_t* perm, int64_t* cell_ints, double* c
 /* Tuning (no counterpart in the paper): the number of cells one thread of the
  * leaf walk visits before it hands its leaf to the block-wide walk, which
  * decides every cell of the leaf's system in tiles of 1024 (a leaf in the
- * sparse outskirts of a condensed system can open most of the tree).  budget
- * = 0 restores the default (KDFMM_WALK_BUDGET from the environment, else
- * 4096).  Interaction lists and forces do not depend on it; the arena walk's
+ * sparse outskirts of a condensed system can open most of the tree).  With up
+ * to 80 leaves per SM a warp shares a leaf's walk and the budget counts the
+ * cells of the warp; with up to 320 some threads do, each with the budget to
+ * itself.  budget = 0 restores the default (KDFMM_WALK_BUDGET from the
+ * environment, else 4096; a warp's walk by default hands on the first two
+ * leaves per SM past 40 rounds of 64 cells instead).  A walk that outgrows its
+ * scratch or stack is handed on too.  Interaction lists and forces do not depend on it; the arena walk's
  * scratch grows with it (budget x 4 bytes per walk thread).  Takes effect at
  * the next evaluation (a captured batch graph is captured again).  budget
  * outside [0, 2^20] or a NULL handle gives KDFMM_ERR_INVALID_ARG. */

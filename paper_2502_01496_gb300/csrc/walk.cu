@@ -57,7 +57,8 @@ struct WalkArgs {
   int32_t* heavy;                  // queue of the leaves handed on
   int32_t* heavy_n;                // its length (counters[C_HEAVY])
   int32_t* long_n;                 // long map walks (counters[C_LONG])
-  int sms;
+  int map_budget;                  // cells of a leaf's map walk, where a budget is set
+  int map_long;                    // else: long map walks to hand on
 };
 
 __device__ __forceinline__ bool open_exact(double ax, double ay, double az, double sa, double ha,
@@ -398,10 +399,11 @@ __global__ void __launch_bounds__(128, 10) k_walk_split(WalkArgs W) {
 // and 32 cells a round 0.35.  With 262146 particles (23000 leaves) the maps' zero
 // words and the fewer warps make 8 lanes a leaf the faster (1.88 ms a call
 // against 1.99).
-// A leaf that passes W.budget rounds, or outgrows the stack, goes to k_walk_heavy;
-// so do the first leaves to reach kMapLong rounds, one for each of its blocks: they
-// would end the walk alone (60013 particles: 310 -> 118 us + 38 us of k_walk_heavy;
-// at 64 rounds 136 + 40).
+// A leaf that outgrows the stack goes to k_walk_heavy, and with a budget that the
+// caller has set every leaf whose walk visits more cells than it.  By default the
+// first leaves to reach kMapLong rounds do, one for each of k_walk_heavy's blocks:
+// they would end the walk alone (60013 particles: 310 -> 118 us + 38 us of
+// k_walk_heavy; at 64 rounds, the 4096 cells of the other walks, 136 + 40).
 // With all of them handed over a small theta, where most leaves are long, lost by it
 // (theta = 0.2: 1.55 -> 1.86 ms a call).
 constexpr int kMapLeaves = 12160, kMapLong = 40, kMapHandOver = 2;
@@ -431,7 +433,7 @@ __global__ void __launch_bounds__(32 * kMapWarps, 16) k_walk_map(WalkArgs W, int
   const int i0 = W.sys_root[sys], cells = W.sys_root[sys + 1] - i0;
   const int used = (cells + 31) >> 5;
   bool ok = used <= words && cells <= 65536;              // (at most two cells a leaf: always)
-  int nex = 0, top = ok ? 1 : 0, rounds = 0;
+  int nex = 0, top = ok ? 1 : 0, rounds = 0, visits = 0;
   long long np = 0;
   if (ok) {
     for (int w = lane; w < used; w += 32) map_f[w] = map_n[w] = 0u;
@@ -440,17 +442,18 @@ __global__ void __launch_bounds__(32 * kMapWarps, 16) k_walk_map(WalkArgs W, int
   __syncwarp();
   while (top > 0) {
     ++rounds;
-    bool leave = rounds > W.budget || top > kMapStack - 64 * kMapTake;
-    if (rounds == kMapLong) {
+    bool leave = visits > W.map_budget || top > kMapStack - 64 * kMapTake;
+    if (rounds == kMapLong && W.map_long > 0) {
       int before = 0;
       if (lane == 0) before = atomicAdd(W.long_n, 1);
-      leave = leave || __shfl_sync(full, before, 0) < (int)(kMapHandOver * W.sms);
+      leave = leave || __shfl_sync(full, before, 0) < W.map_long;
     }
     if (leave) {
       ok = false;
       break;
     }
     const int take = min(top, 32 * kMapTake);
+    visits += take;
     int c[kMapTake];
     float4 wb[kMapTake], w2[kMapTake];
     int right[kMapTake];
@@ -494,6 +497,7 @@ __global__ void __launch_bounds__(32 * kMapWarps, 16) k_walk_map(WalkArgs W, int
     }
     __syncwarp();
   }
+  ok = ok && visits <= W.map_budget;
   if (lane == 0) {
     W.far_off[k] = (int64_t)k * W.cap_far;
     W.near_off[k] = (int64_t)k * W.cap_near;
@@ -899,16 +903,20 @@ __global__ void __launch_bounds__(kHeavyThreads, 2) k_walk_heavy(WalkArgs W) {
 inline unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
 // Cells one thread walks before its leaf goes to the block-wide walk: the
-// handle's setting (kdfmm_tree_set_walk_budget), else KDFMM_WALK_BUDGET, else
-// 4096 (the lists do not depend on it).
-static int walk_budget(const kdfmm_tree_s* t) {
+// handle's setting (kdfmm_tree_set_walk_budget), else KDFMM_WALK_BUDGET, else 0.
+static int set_budget(const kdfmm_tree_s* t) {
   if (t->walk_budget > 0) return t->walk_budget;
   const char* v = getenv("KDFMM_WALK_BUDGET");
   if (v != nullptr) {
     const long b = strtol(v, nullptr, 10);
     if (b >= 1 && b <= INT_MAX) return (int)b;
   }
-  return 4096;
+  return 0;
+}
+// The same with the default, 4096 (the lists do not depend on it).
+static int walk_budget(const kdfmm_tree_s* t) {
+  const int b = set_budget(t);
+  return b > 0 ? b : 4096;
 }
 
 }  // namespace
@@ -1019,7 +1027,9 @@ static WalkArgs walk_args(kdfmm_tree_s* t) {
   W.heavy = L.heavy;
   W.heavy_n = t->counters + C_HEAVY;
   W.long_n = t->counters + C_LONG;
-  W.sms = sm_count();
+  const int set = set_budget(t);
+  W.map_budget = set > 0 ? set : INT_MAX;
+  W.map_long = set > 0 ? 0 : kMapHandOver * sm_count();
   return W;
 }
 

@@ -293,8 +293,8 @@ def tree_timing(tree, enable: bool = True, read: bool = True) -> dict | None:
 
 
 def tree_set_walk_budget(tree, budget: int) -> None:
-    """Cells a walk thread visits before its leaf goes to the block-wide walk
-    (0: the default); see kdfmm_tree_set_walk_budget."""
+    """Cells a walk thread (or a warp that shares a leaf's walk) visits before the
+    leaf goes to the block-wide walk (0: the default); see kdfmm_tree_set_walk_budget."""
     _check(lib().kdfmm_tree_set_walk_budget(tree, int(budget)), "tree_set_walk_budget")
 
 
