@@ -1341,7 +1341,7 @@ static int ensure_build_buffers(kdfmm_tree_s* t, int64_t n) {
   KD_ALLOC(t->segB, t->capB);
   KD_ALLOC(t->segL, t->capL);
   // (a later build of fewer particles may take the small chunks)
-  t->cap_chunks = std::max<int64_t>(n / kChunk, std::min<int64_t>(n, kSmallChunkMax) / (8 * 64)) + t->capA + 4;
+  t->cap_chunks = std::max<int64_t>(n / kChunk, std::min<int64_t>(n, small_chunk_max()) / (8 * 64)) + t->capA + 4;
   KD_ALLOC(t->chunk_seg, t->cap_chunks);
   KD_ALLOC(t->chunk_sum, 4 * t->cap_chunks);
   KD_ALLOC(t->chunk_key, 6 * t->cap_chunks);
@@ -1464,7 +1464,7 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
       return set_error(KDFMM_ERR_NONFINITE, "non-finite position or non-positive mass / h");
   }
   // phase A: cells above kSubtreeMax, one level per pass
-  const bool small = n <= kSmallChunkMax;
+  const bool small = n <= small_chunk_max();
   const unsigned maxc = (unsigned)(n / (small ? 8 * 64 : kChunk) + t->capA + 1);
   int cur = 0, level = 0;
   auto run_level = [&](auto threads, const Seg* segs, Seg* next, int src, int dst) {

@@ -15,8 +15,6 @@ namespace kdfmm {
 constexpr int kChunk = 2048;           // phase-A reduction chunk (elements)
 constexpr int kChunkThreads = 256;     // 8 consecutive elements per thread
 static_assert(kChunk == 8 * kChunkThreads, "the chunk reduce sums 8 elements per thread");
-constexpr int kSmallChunkMax = 311296;   // up to here chunks of 512 elements (152 x 2048 elements:
-                                       // one large chunk per SM)
 constexpr int kSubtreeMax = 2048;      // cells this small finish in shared memory
 constexpr int kNumStatus = 4;
 
@@ -59,6 +57,9 @@ enum : int {
 
 // Streaming multiprocessors of the current device (queried once per device).
 int sm_count();
+// Up to here the build takes chunks of 512 elements: one large chunk per SM
+// (152 SMs: 311296 particles).
+inline int64_t small_chunk_max() { return (int64_t)kChunk * sm_count(); }
 // Grid of the grid-stride (persistent) kernels: per_sm blocks on every SM.
 inline unsigned grid_blocks(int per_sm = 8) { return (unsigned)(sm_count() * per_sm); }
 #define KD_GRID_STRIDE(i, n)                                                             \

@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(128, 10) k_walk(WalkArgs W) {
   atomicAdd(&W.stats[3], (unsigned long long)nn);
 }
 
-// Slot mode with 12160 to 48640 leaves: K lanes of a warp (8 or 4) share a leaf's
+// Slot mode with 80 to 320 leaves per SM: K lanes of a warp (8 or 4) share a leaf's
 // walk.  The tree below its first log2 K levels is K runs of pre-order cells;
 // lane s of a leaf descends to run s (deciding the cells on its way: a closed or
 // leaf cell is emitted by the first lane below it) and walks that run alone, into
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(128, 10) k_walk_split(WalkArgs W) {
   }
 }
 
-// Slot mode with at most kMapLeaves leaves: a warp per leaf.  Undecided cells lie
+// Slot mode with at most kMapLeaves leaves per SM: a warp per leaf.  Undecided cells lie
 // on a stack in shared memory; each round the lanes take up to 64 off its top,
 // decide them, and push the children of the opened ones.  The order of the
 // decisions is free: a far or near cell sets its bit in a map over its system's
@@ -406,7 +406,7 @@ __global__ void __launch_bounds__(128, 10) k_walk_split(WalkArgs W) {
 // k_walk_heavy; at 64 rounds, the 4096 cells of the other walks, 136 + 40).
 // With all of them handed over a small theta, where most leaves are long, lost by it
 // (theta = 0.2: 1.55 -> 1.86 ms a call).
-constexpr int kMapLeaves = 12160, kMapLong = 40, kMapHandOver = 2;
+constexpr int kMapLeaves = 80, kMapLong = 40, kMapHandOver = 2;
 constexpr int kMapWarps = 2, kMapStack = 1024, kMapTake = 2;
 __global__ void __launch_bounds__(32 * kMapWarps, 16) k_walk_map(WalkArgs W, int words) {
   extern __shared__ unsigned s_dyn[];
@@ -974,12 +974,13 @@ static int arena_grid_for(int leaves) {
                                                      (int64_t)per_sm * sms));
 }
 
-// Lanes per leaf of the slot-mode walk: 32 (k_walk_map) up to kMapLeaves, else as
-// many as one round of resident threads allows, one beyond 48640 leaves on 152
-// SMs, where the thread walk has the GPU's threads busy by itself.
+// Lanes per leaf of the slot-mode walk: 32 (k_walk_map) up to kMapLeaves a SM,
+// else as many as one round of resident threads (1280 an SM) allows, one beyond
+// 320 leaves a SM, where the thread walk has the GPU's threads busy by itself.
+// (152 SMs: 12160 and 48640 leaves.)
 static int split_lanes(int leaves) {
   const int64_t threads = (int64_t)sm_count() * 10 * 128, n = std::max(leaves, 1);
-  if (n <= kMapLeaves) return 32;
+  if (n <= (int64_t)kMapLeaves * sm_count()) return 32;
   for (int k = 8; k >= 4; k >>= 1)
     if (k * n <= threads) return k;
   return 1;

@@ -1,4 +1,4 @@
-"""The dual walk over forests on both sides of its limit of four systems (one
+"""The dual walk over forests on both sides of its limit of two systems (one
 block for the first levels of the pair recursion and of the downward pass)."""
 import numpy as np
 import pytest
@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("precision", [0, 1])
-@pytest.mark.parametrize("n_sys", [1, 4, 5, 300])
+@pytest.mark.parametrize("n_sys", [1, 2, 3, 4, 5, 300])
 def test_forest_against_the_oracle(oracle, n_sys, precision):
     """Systems of 1 to 400 particles and one of 6000, theta from 0.3 to 0.8, against
     the oracle's dual walk of each; the precisions' bounds, against the system's
