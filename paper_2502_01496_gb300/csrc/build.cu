@@ -1049,22 +1049,25 @@ typedef unsigned long long Starts;
 __device__ __forceinline__ int cells_before(const Starts* off, int64_t p) { return (int)(unsigned)off[p]; }
 __device__ __forceinline__ int leaves_before(const Starts* off, int64_t p) { return (int)(off[p] >> 32); }
 
-// Clears the scan's words.  A build that did not come to its end (too few
-// phase-A levels, a full list, refused input) leaves cells whose links are those
-// of an earlier tree: its cell count becomes 0 here, so that the numbering finds
-// no cells, counts no leaves, and neither the kernels after it nor the walk, M2L
-// and P2P of a captured evaluation touch that tree.  The status word tells the
-// host.
-__global__ void k_number_init(Starts* starts, int32_t* min_depth, int64_t n, int32_t* counters,
-                              const int32_t* __restrict__ status) {
+__global__ void k_number_init(Starts* starts, int32_t* min_depth, int64_t n) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0 && (*status & (ST_UNFINISHED | ST_CAPACITY | ST_NONFINITE))) counters[C_CELLS] = 0;
   if (i < n) { starts[i] = 0; min_depth[i] = INT_MAX; }
+}
+
+// Cells to number.  A build that did not come to its end (too few phase-A levels,
+// a full list, refused input) leaves cells whose links are those of an earlier
+// tree: it counts as without cells, so that the numbering finds none, k_remap
+// leaves no cells and no leaves in the counters, and neither the kernels after it
+// nor the walk, M2L and P2P of a captured evaluation touch that tree.  The status
+// word tells the host.
+__device__ __forceinline__ int cells_to_number(const int32_t* counters) {
+  const int ncells = counters[C_CELLS];
+  return counters[C_STATUS] & (ST_UNFINISHED | ST_CAPACITY | ST_NONFINITE) ? 0 : ncells;
 }
 
 __global__ void k_count_starts(TmpCells tmp, const int32_t* __restrict__ counters, Starts* cnt,
                                int32_t* min_depth) {
-  const int ncells = counters[C_CELLS];
+  const int ncells = cells_to_number(counters);
   KD_GRID_STRIDE(c, ncells) {
     const int f = tmp.first[c];
     atomicAdd(&cnt[f], tmp.left[c] < 0 ? (Starts(1) << 32 | 1) : Starts(1));
@@ -1084,8 +1087,11 @@ __global__ void k_remap(TmpCells tmp, int32_t* counters, const Starts* __restric
                         const int32_t* __restrict__ min_depth, Cells c, int32_t* status, int64_t n,
                         int32_t* leaf_rank, int32_t* leaf_cells, int32_t* leaf_sys,
                         const int64_t* __restrict__ sys_off, int n_sys, int32_t* sys_root) {
-  const int t_n = counters[C_CELLS];
-  if (blockIdx.x == 0 && threadIdx.x == 0) counters[C_LEAVES] = leaves_before(off, n);
+  const int t_n = cells_to_number(counters);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    counters[C_LEAVES] = leaves_before(off, n);
+    if (t_n == 0) counters[C_CELLS] = 0;         // (other blocks go by the status alone then)
+  }
   KD_GRID_STRIDE(k, n_sys + 1) sys_root[k] = cells_before(off, sys_off[k]);
   KD_GRID_STRIDE(t, t_n) {
   const int f = tmp.first[t], cnt = tmp.count[t], d = tmp.depth[t];
@@ -1431,7 +1437,7 @@ static int subtree_setup(kdfmm_tree_s* t, bool fine, size_t smem) {
 // from capacities and reading its count on the device -- so the sequence can
 // be captured in a CUDA graph; a phase A that needed more levels, or any
 // capacity overflow, is left in the status word for the caller to check (the
-// tree then has no cells: k_number_init).
+// tree then has no cells: cells_to_number).
 int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* h, cudaStream_t s,
                int fixed_levels) {
   const int64_t n = t->n;
@@ -1534,7 +1540,7 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
   }
 
   // pre-order numbering, counts read on the device
-  k_number_init<<<blocks_for(n + 1, 256), 256, 0, s>>>(t->starts, t->min_depth, n + 1, t->counters, t->status);
+  k_number_init<<<blocks_for(n + 1, 256), 256, 0, s>>>(t->starts, t->min_depth, n + 1);
   k_count_starts<<<grid_blocks(), 256, 0, s>>>(t->tmp, t->counters, t->starts, t->min_depth);
   scan_u64(t->starts, n, reinterpret_cast<unsigned long long*>(t->scan_tmp), s);
   k_remap<<<grid_blocks(), 256, 0, s>>>(t->tmp, t->counters, t->starts, t->min_depth, t->c, t->status, n,
