@@ -429,7 +429,6 @@ void kdfmm_tree_destroy(kdfmm_tree t) {
   cudaFree(t->L.far_idx); cudaFree(t->L.near_idx);
   cudaFree(t->L.heavy); cudaFree(t->L.seg_first); cudaFree(t->L.seg_leaf); cudaFree(t->L.seg_part);
   cudaFree(t->L.temp);
-  cudaFree(t->mom_partial);
   cudaFree(t->vjp_buf);
   if (t->vjp_done) cudaEventDestroy(t->vjp_done);
   cudaFree(t->sys_off); cudaFree(t->sys_theta); cudaFree(t->sys_eps); cudaFree(t->sys_nleaf);

@@ -28,7 +28,6 @@ namespace kdfmm {
 namespace {
 
 struct BuildArgs {
-  PCols src, dst;
   TmpCells tmp;
   int32_t* counters;
   int32_t* status;
@@ -1489,8 +1488,6 @@ int build_tree(kdfmm_tree_s* t, const double* x, const double* m, const double* 
   };
   while (deferred ? level < fixed_levels : hc[C_NEXT_A] > 0) {
     const int src = level & 1, dst = src ^ 1;
-    A.src = t->buf[src];
-    A.dst = t->buf[dst];
     if (small) run_level(std::integral_constant<int, 64>{}, t->segA[cur], t->segA[cur ^ 1], src, dst);
     else run_level(std::integral_constant<int, kChunkThreads>{}, t->segA[cur], t->segA[cur ^ 1], src, dst);
     t->launches += 4;

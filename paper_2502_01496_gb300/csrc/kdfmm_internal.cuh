@@ -16,7 +16,6 @@ constexpr int kChunk = 2048;           // phase-A reduction chunk (elements)
 constexpr int kChunkThreads = 256;     // 8 consecutive elements per thread
 static_assert(kChunk == 8 * kChunkThreads, "the chunk reduce sums 8 elements per thread");
 constexpr int kSubtreeMax = 2048;      // cells this small finish in shared memory
-constexpr int kNumStatus = 4;
 
 // Device-side status bits (OR-ed into a device word, read after a sync).
 enum : int {
@@ -168,7 +167,7 @@ struct kdfmm_tree_s {
   int32_t* seg_axis = nullptr;
   double* seg_cut = nullptr;
   int32_t* seg_nl = nullptr;
-  int64_t cap_chunks = 0, cap_segA = 0;
+  int64_t cap_chunks = 0;
   kdfmm::TmpCells tmp{};
   unsigned long long* starts = nullptr;  // per particle: cells and leaves starting there, then before it
   int32_t* min_depth = nullptr;
@@ -200,8 +199,6 @@ struct kdfmm_tree_s {
   int32_t* leaf_sys = nullptr;     // device, system of each leaf ordinal
   int64_t* host_sys_off = nullptr; // pinned host copy of sys_off
 
-  double* mom_partial = nullptr;   // total_momentum scratch
-  int64_t cap_mom = 0;
   int64_t* host_stats = nullptr;   // pinned host mirror
   int32_t* host_counters = nullptr;
   int64_t launches = 0;            // kernels launched by this handle
@@ -214,7 +211,6 @@ struct kdfmm_tree_s {
     int2 *q[2] = {nullptr, nullptr}, *far = nullptr, *near = nullptr;
     int64_t q_cap[2] = {0, 0}, far_cap = 0, near_cap = 0;   // entries allocated
     int32_t* ctr = nullptr;              // device: [0] queue out, [1] far pairs, [2] near pairs, [3] overflow
-    int64_t* np2p = nullptr;             // device: particle pairs of the near list
     int32_t* far_cnt = nullptr;          // per cell
     int64_t* far_off = nullptr;          // per cell + 1
     int32_t* far_idx = nullptr;
@@ -379,18 +375,6 @@ __device__ __forceinline__ Sum4 zero4() { return Sum4{0.0, 0.0, 0.0, 0.0}; }
 __device__ __forceinline__ Sum4 add4(const Sum4& a, const Sum4& b) {
   return Sum4{__dadd_rn(a.m, b.m), __dadd_rn(a.x, b.x), __dadd_rn(a.y, b.y), __dadd_rn(a.z, b.z)};
 }
-__device__ __forceinline__ Sum4 shfl_xor4(const Sum4& a, int o) {
-  return Sum4{__shfl_xor_sync(0xffffffffu, a.m, o), __shfl_xor_sync(0xffffffffu, a.x, o),
-              __shfl_xor_sync(0xffffffffu, a.y, o), __shfl_xor_sync(0xffffffffu, a.z, o)};
-}
-// Butterfly over the 32 lanes: lane l holds the sum of an aligned block l;
-// pairing (2j, 2j+1), then pairs of pairs... is the perfect binary tree, and
-// every lane ends with the full sum.
-__device__ __forceinline__ Sum4 warp_tree4(Sum4 v) {
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) v = add4(v, shfl_xor4(v, o));
-  return v;
-}
 // The element (m, m x, m y, m z) of one particle, products correctly rounded.
 __device__ __forceinline__ Sum4 elem4(double m, double x, double y, double z) {
   return Sum4{m, __dmul_rn(m, x), __dmul_rn(m, y), __dmul_rn(m, z)};
@@ -409,32 +393,6 @@ __device__ __forceinline__ Sum4 block_tree(int base, int count, const F& get) {
     Sum4 r = block_tree<LOGB - 1>(base + H, count, get);
     return add4(l, r);
   }
-}
-
-// Canonical pairwise sum of `count` elements (count <= 2048) by one warp: the
-// sequence is padded to P = 2^ceil(log2 count); lane l sums its aligned block
-// of P/32 elements as a perfect tree, the butterfly combines the lanes.
-template <class F>
-__device__ __forceinline__ Sum4 warp_pairwise(int count, const F& get) {
-  const int lane = threadIdx.x & 31;
-  int P = 1;
-  while (P < count) P <<= 1;
-  Sum4 v;
-  if (P <= 32) {
-    v = lane < count ? get(lane) : zero4();
-  } else {
-    const int B = P >> 5;
-    const int base = lane * B;
-    switch (B) {
-      case 2: v = block_tree<1>(base, count, get); break;
-      case 4: v = block_tree<2>(base, count, get); break;
-      case 8: v = block_tree<3>(base, count, get); break;
-      case 16: v = block_tree<4>(base, count, get); break;
-      case 32: v = block_tree<5>(base, count, get); break;
-      default: v = block_tree<6>(base, count, get); break;
-    }
-  }
-  return warp_tree4(v);
 }
 
 __device__ __forceinline__ long long warp_min_ll(long long v) {
@@ -533,7 +491,7 @@ int run_dual_local(kdfmm_tree_s* t, cudaStream_t s);
 void free_dual(kdfmm_tree_s* t);
 int run_p2p(kdfmm_tree_s* t, double* a, double* phi, cudaStream_t s);
 // Extra P2P segments: storage for `need`, an upper bound from the last walk's
-// list sizes, and the plan (run by run_p2p; the adjoint reuses it).
+// list sizes, and the plan (run by run_p2p).
 int ensure_segments(kdfmm_tree_s* t, int64_t need);
 int64_t segments_bound(const kdfmm_tree_s* t);
 int plan_segments(kdfmm_tree_s* t, cudaStream_t s);

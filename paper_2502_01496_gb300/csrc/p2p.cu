@@ -819,7 +819,6 @@ inline unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + thre
 int ensure_segments(kdfmm_tree_s* t, int64_t need) {
   Lists& L = t->L;
   if (L.seg_cap >= need && L.seg_leaf != nullptr) return KDFMM_OK;
-  // the plan of the last evaluation is kept (the adjoint reuses it)
   const int64_t cap = std::max<int64_t>(need, 64);
   int32_t* leaf = nullptr;
   double* part = nullptr;
@@ -828,13 +827,6 @@ int ensure_segments(kdfmm_tree_s* t, int64_t need) {
     cudaFree(leaf);
     cudaGetLastError();
     return set_error(KDFMM_ERR_OOM, "P2P segments (%lld)", (long long)cap);
-  }
-  if (L.seg_leaf != nullptr && L.seg_cap > 0 &&
-      cudaMemcpy(leaf, L.seg_leaf, (size_t)L.seg_cap * sizeof(int32_t), cudaMemcpyDeviceToDevice) !=
-          cudaSuccess) {
-    cudaFree(leaf);
-    cudaFree(part);
-    return check_cuda(cudaGetLastError(), "segment copy");
   }
   cudaFree(L.seg_leaf);
   cudaFree(L.seg_part);

@@ -29,75 +29,47 @@ namespace {
 inline unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
 // ---------------------------------------------------------------------------
-// M2L coefficients (same closed forms as the forward) on a dual-number type
+// M2L coefficients (same closed forms as the forward) on float32 dual numbers
 // ---------------------------------------------------------------------------
-// S: the scalar (double, or float in mixed mode); d holds the derivatives
-// with respect to the three components of r.
-template <class S>
-struct DualT {
-  S v, d[3];
+// d: the derivatives with respect to the three components of r.
+struct Dual {
+  float v, d[3];
 };
-template <class S>
-__device__ __forceinline__ DualT<S> operator+(const DualT<S>& a, const DualT<S>& b) {
-  return DualT<S>{a.v + b.v, {a.d[0] + b.d[0], a.d[1] + b.d[1], a.d[2] + b.d[2]}};
+__device__ __forceinline__ Dual operator+(const Dual& a, const Dual& b) {
+  return Dual{a.v + b.v, {a.d[0] + b.d[0], a.d[1] + b.d[1], a.d[2] + b.d[2]}};
 }
-template <class S>
-__device__ __forceinline__ DualT<S> operator-(const DualT<S>& a, const DualT<S>& b) {
-  return DualT<S>{a.v - b.v, {a.d[0] - b.d[0], a.d[1] - b.d[1], a.d[2] - b.d[2]}};
+__device__ __forceinline__ Dual operator-(const Dual& a, const Dual& b) {
+  return Dual{a.v - b.v, {a.d[0] - b.d[0], a.d[1] - b.d[1], a.d[2] - b.d[2]}};
 }
-template <class S>
-__device__ __forceinline__ DualT<S> operator-(const DualT<S>& a) {
-  return DualT<S>{-a.v, {-a.d[0], -a.d[1], -a.d[2]}};
+__device__ __forceinline__ Dual operator-(const Dual& a) {
+  return Dual{-a.v, {-a.d[0], -a.d[1], -a.d[2]}};
 }
-template <class S>
-__device__ __forceinline__ DualT<S> operator*(const DualT<S>& a, const DualT<S>& b) {
-  return DualT<S>{a.v * b.v,
-                  {a.d[0] * b.v + a.v * b.d[0], a.d[1] * b.v + a.v * b.d[1],
-                   a.d[2] * b.v + a.v * b.d[2]}};
+__device__ __forceinline__ Dual operator*(const Dual& a, const Dual& b) {
+  return Dual{a.v * b.v,
+              {a.d[0] * b.v + a.v * b.d[0], a.d[1] * b.v + a.v * b.d[1], a.d[2] * b.v + a.v * b.d[2]}};
 }
-template <class S>
-__device__ __forceinline__ DualT<S>& operator+=(DualT<S>& a, const DualT<S>& b) { return a = a + b; }
+__device__ __forceinline__ Dual& operator+=(Dual& a, const Dual& b) { return a = a + b; }
 
 __device__ __forceinline__ float rsq(float v) { return rsqrtf(v); }
 
-template <class S>
-__device__ __forceinline__ DualT<S> rsqrt_dual(const DualT<S>& a) {
-  const S r = rsq(a.v);
-  const S dr = S(-0.5) * r / a.v;
-  return DualT<S>{r, {dr * a.d[0], dr * a.d[1], dr * a.d[2]}};
+__device__ __forceinline__ Dual rsqrt_dual(const Dual& a) {
+  const float r = rsq(a.v);
+  const float dr = -0.5f * r / a.v;
+  return Dual{r, {dr * a.d[0], dr * a.d[1], dr * a.d[2]}};
 }
+// A constant.
+__device__ __forceinline__ Dual lift(float v) { return Dual{v, {0.f, 0.f, 0.f}}; }
 
-// A scalar as the coefficients' type (a dual number with zero derivatives).
-template <class T>
-struct Lift {
-  __device__ static __forceinline__ T of(T v) { return v; }
-  using Scalar = T;
-};
-template <class S>
-struct Lift<DualT<S>> {
-  __device__ static __forceinline__ DualT<S> of(S v) { return DualT<S>{v, {S(0), S(0), S(0)}}; }
-  using Scalar = S;
-};
-template <class T>
-__device__ __forceinline__ T tc(double v) {
-  return Lift<T>::of((typename Lift<T>::Scalar)v);
-}
-
-template <class S>
-__device__ __forceinline__ DualT<S> rs(const DualT<S>& v) { return rsqrt_dual(v); }
-
-template <class T>
-__device__ __forceinline__ T c2e(int a, int b, const T R[3], const T u[3], const T Qm[3][3], T s1,
-                                 T s2, T t2, T t3) {
-  T v = s2 * R[a] * R[b] + t3 * (R[a] * u[b] + R[b] * u[a]) + t2 * Qm[a][b];
+__device__ __forceinline__ Dual c2e(int a, int b, const Dual R[3], const Dual u[3],
+                                    const Dual Qm[3][3], Dual s1, Dual s2, Dual t2, Dual t3) {
+  Dual v = s2 * R[a] * R[b] + t3 * (R[a] * u[b] + R[b] * u[a]) + t2 * Qm[a][b];
   if (a == b) v += s1;
   return v;
 }
 
-template <class T>
-__device__ __forceinline__ T c3e(int a, int b, int c, const T R[3], const T u[3], const T Qm[3][3],
-                                 T s2, T s3, T t3, T t4) {
-  T d = tc<T>(0.0), du = tc<T>(0.0);
+__device__ __forceinline__ Dual c3e(int a, int b, int c, const Dual R[3], const Dual u[3],
+                                    const Dual Qm[3][3], Dual s2, Dual s3, Dual t3, Dual t4) {
+  Dual d = lift(0.0f), du = lift(0.0f);
   if (a == b) { d += R[c]; du += u[c]; }
   if (a == c) { d += R[b]; du += u[b]; }
   if (b == c) { d += R[a]; du += u[a]; }
@@ -112,46 +84,42 @@ __device__ __forceinline__ T c3e(int a, int b, int c, const T R[3], const T u[3]
 // keeps one accumulator instead of twenty.
 // STD: the standard p = 3 series -- the quadrupole keeps only its C0 and C1
 // terms (as in m2l.cu).
-template <class T, bool STD>
-__device__ T m2l_contract(const T R[3], typename Lift<T>::Scalar M,
-                          const typename Lift<T>::Scalar Q[6],
-                          const typename Lift<T>::Scalar w[20]) {
-  using L = Lift<T>;
-  const T Qm[3][3] = {{L::of(Q[0]), L::of(Q[1]), L::of(Q[2])},
-                      {L::of(Q[1]), L::of(Q[3]), L::of(Q[4])},
-                      {L::of(Q[2]), L::of(Q[4]), L::of(Q[5])}};
-  const T R2 = R[0] * R[0] + R[1] * R[1] + R[2] * R[2];
-  const T g0 = rs(R2);
-  const T i2 = g0 * g0;
-  const T g1 = -(g0 * i2);
-  const T g2 = tc<T>(-3.0) * g1 * i2;
-  const T g3 = tc<T>(-5.0) * g2 * i2;
-  const T g4 = tc<T>(-7.0) * g3 * i2;
-  const T g5 = tc<T>(-9.0) * g4 * i2;
-  T u[3];
+template <bool STD>
+__device__ Dual m2l_contract(const Dual R[3], float M, const float Q[6], const float w[20]) {
+  const Dual Qm[3][3] = {{lift(Q[0]), lift(Q[1]), lift(Q[2])},
+                         {lift(Q[1]), lift(Q[3]), lift(Q[4])},
+                         {lift(Q[2]), lift(Q[4]), lift(Q[5])}};
+  const Dual R2 = R[0] * R[0] + R[1] * R[1] + R[2] * R[2];
+  const Dual g0 = rsqrt_dual(R2);
+  const Dual i2 = g0 * g0;
+  const Dual g1 = -(g0 * i2);
+  const Dual g2 = lift(-3.0f) * g1 * i2;
+  const Dual g3 = lift(-5.0f) * g2 * i2;
+  const Dual g4 = lift(-7.0f) * g3 * i2;
+  const Dual g5 = lift(-9.0f) * g4 * i2;
+  Dual u[3];
   for (int i = 0; i < 3; ++i) u[i] = Qm[i][0] * R[0] + Qm[i][1] * R[1] + Qm[i][2] * R[2];
-  const T q = R[0] * u[0] + R[1] * u[1] + R[2] * u[2];
-  const T qs = q * tc<T>(1.0 / 6.0);
-  const T Mt = L::of(M);
-  const T s1 = -(Mt * g1) - g3 * qs;
-  const T t2 = g2 * tc<T>(-1.0 / 3.0);
-  T acc = L::of(w[0]) * (-(Mt * g0) - g2 * qs);
-  for (int i = 0; i < 3; ++i) acc += L::of(w[1 + i]) * (s1 * R[i] + t2 * u[i]);
-  const T s1h = STD ? -(Mt * g1) : s1;
-  const T s2 = STD ? -(Mt * g2) : -(Mt * g2) - g4 * qs;
-  const T s3 = STD ? -(Mt * g3) : -(Mt * g3) - g5 * qs;
-  const T t2h = STD ? tc<T>(0.0) : t2;
-  const T t3 = STD ? tc<T>(0.0) : g3 * tc<T>(-1.0 / 3.0);
-  const T t4 = STD ? tc<T>(0.0) : g4 * tc<T>(-1.0 / 3.0);
+  const Dual q = R[0] * u[0] + R[1] * u[1] + R[2] * u[2];
+  const Dual qs = q * lift((float)(1.0 / 6.0));
+  const Dual Mt = lift(M);
+  const Dual s1 = -(Mt * g1) - g3 * qs;
+  const Dual t2 = g2 * lift((float)(-1.0 / 3.0));
+  Dual acc = lift(w[0]) * (-(Mt * g0) - g2 * qs);
+  for (int i = 0; i < 3; ++i) acc += lift(w[1 + i]) * (s1 * R[i] + t2 * u[i]);
+  const Dual s1h = STD ? -(Mt * g1) : s1;
+  const Dual s2 = STD ? -(Mt * g2) : -(Mt * g2) - g4 * qs;
+  const Dual s3 = STD ? -(Mt * g3) : -(Mt * g3) - g5 * qs;
+  const Dual t2h = STD ? lift(0.0f) : t2;
+  const Dual t3 = STD ? lift(0.0f) : g3 * lift((float)(-1.0 / 3.0));
+  const Dual t4 = STD ? lift(0.0f) : g4 * lift((float)(-1.0 / 3.0));
   const int c2a[6] = {0, 0, 0, 1, 1, 2}, c2b[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
-  for (int k = 0; k < 6; ++k)
-    acc += L::of(w[4 + k]) * c2e<T>(c2a[k], c2b[k], R, u, Qm, s1h, s2, t2h, t3);
+  for (int k = 0; k < 6; ++k) acc += lift(w[4 + k]) * c2e(c2a[k], c2b[k], R, u, Qm, s1h, s2, t2h, t3);
   const int c3a[10] = {0, 0, 0, 0, 0, 0, 1, 1, 1, 2}, c3b[10] = {0, 0, 0, 1, 1, 2, 1, 1, 2, 2},
             c3c[10] = {0, 1, 2, 1, 2, 2, 1, 2, 2, 2};
 #pragma unroll
   for (int k = 0; k < 10; ++k)
-    acc += L::of(w[10 + k]) * c3e<T>(c3a[k], c3b[k], c3c[k], R, u, Qm, s2, s3, t3, t4);
+    acc += lift(w[10 + k]) * c3e(c3a[k], c3b[k], c3c[k], R, u, Qm, s2, s3, t3, t4);
   return acc;
 }
 
@@ -572,10 +540,8 @@ __global__ void __launch_bounds__(kM2LWarps * 32) k_vjp_m2l32(VjpArgs V) {
       const float4 q0 = V.c.src32[4 * (int64_t)b + 2], q1 = V.c.src32[4 * (int64_t)b + 3];
       const float Qb[6] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y};
       // r-derivatives of sum_j cb_j C_j by dual numbers; M and Q enter linearly
-      const DualT<float> R[3] = {DualT<float>{r[0], {1.f, 0.f, 0.f}}, DualT<float>{r[1], {0.f, 1.f, 0.f}},
-                                 DualT<float>{r[2], {0.f, 0.f, 1.f}}};
-      const DualT<float> cr =
-          m2l_contract<DualT<float>, STD>(R, V.c.src32[4 * (int64_t)b].w, Qb, cb);
+      const Dual R[3] = {Dual{r[0], {1.f, 0.f, 0.f}}, Dual{r[1], {0.f, 1.f, 0.f}}, Dual{r[2], {0.f, 0.f, 1.f}}};
+      const Dual cr = m2l_contract<STD>(R, V.c.src32[4 * (int64_t)b].w, Qb, cb);
       double* v = B.v + 11 * lane;
       B.cell[lane] = b;
 #pragma unroll

@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(128, 10) k_walk_split(WalkArgs W) {
   }
   __syncwarp();
   // the group's lists: prefixes, totals, statistics
-  const unsigned group = (K == 32 ? full : (1u << K) - 1u) << (lane - gl);
+  const unsigned group = ((1u << K) - 1u) << (lane - gl);
   const bool queued = (__ballot_sync(full, !ok) & group) != 0u;
   if (queued) nf = nn = 0;
   int pf = nf, pn = nn;
