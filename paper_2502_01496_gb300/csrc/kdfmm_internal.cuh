@@ -115,13 +115,13 @@ struct Lists {
   int32_t arena_grid;              // blocks of the arena walk
   int64_t* near_np;                // in the counter block: statistics of the walk (4)
   int32_t* heavy;                  // leaves queued for the block-wide walk (nleaves)
-  // near lists longer than a segment are split: segment 0 stays with the
-  // leaf, the others are work items of their own whose partial sums
-  // (seg_part, 32 targets x 4 doubles each) are added in segment order
-  int32_t* seg_first;              // per leaf: first extra segment, or -1
-  int32_t* seg_leaf;               // per extra segment: its leaf
-  double* seg_part;                // per extra segment: partial sums
-  int64_t seg_cap;                 // extra segments allocated
+  // near lists longer than a work item (a segment, or a group of them) are
+  // split: the first item stays with the leaf, the others are items of their own
+  // whose partial sums (seg_part, 32 targets x 4 doubles each) are added in order
+  int32_t* seg_first;              // per leaf: first extra item, or -1
+  int32_t* seg_leaf;               // per extra item: its leaf
+  double* seg_part;                // per extra item: partial sums
+  int64_t seg_cap;                 // extra items allocated
 };
 
 // Near entries per P2P segment (float64 evaluations of few particles take

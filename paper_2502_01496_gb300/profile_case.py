@@ -5,7 +5,7 @@ eagerly, later ones replay its captured graph).
 
   python -m paper_2502_01496_gb300.profile_case [--workload binary|plummer|batch]
       [--n-per-star 262144] [--n 1048576] [--theta 0.5] [--n-leaf 16]
-      [--precision mixed|fp64] [--evals 1]
+      [--precision mixed|fp64] [--evals 1] [--adjoint]
 """
 from __future__ import annotations
 
@@ -21,6 +21,7 @@ def main():
     ap.add_argument("--n-leaf", type=int, default=16)
     ap.add_argument("--precision", choices=["mixed", "fp64"], default="mixed")
     ap.add_argument("--evals", type=int, default=1, help="build + evaluation repetitions")
+    ap.add_argument("--adjoint", action="store_true", help="binary, plummer: an adjoint after each evaluation")
     args = ap.parse_args()
     import torch
     from . import native
@@ -54,7 +55,9 @@ def main():
                      precision=prec)
     for _ in range(args.evals):
         f.build(x, m, h)
-        f.accel()
+        a, _ = f.accel()
+        if args.adjoint:
+            f.vjp(a)
     torch.cuda.synchronize()
     print(f.stats())
 
