@@ -187,8 +187,9 @@ int kdfmm_tree_moments(kdfmm_tree t, const double* x, const double* m, const dou
  * when that cannot be allocated, in two passes: count, then fill).  The slot
  * walk of some 10^4 to 5 10^4 leaves keeps a scratch of at most 0.4 GB, and
  * works without it where it cannot be allocated.  Long near lists are summed
- * in pieces whose partial sums are kept: 4 bytes per near-list entry, at most 128
- * in float64 evaluations of fewer than 262144 particles in all.
+ * in pieces whose partial sums are kept: 4 bytes per near-list entry; in float64
+ * evaluations of fewer than 262144 particles in all up to 128, while that is no
+ * more than some 1 GB.
  * Synchronises `stream` once (list sizes), again when the lists outgrew their
  * buffers and the walk is repeated. */
 int kdfmm_fmm_accel(kdfmm_tree t, double* a, double* phi, void* stream);

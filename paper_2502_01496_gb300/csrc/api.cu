@@ -321,7 +321,7 @@ static void graph_capture(kdfmm_tree_s* t, const double* x, const double* m, con
   t->graph_levels = std::max(t->levels_used, 0) + 2;
   t->graph_leaves = (int32_t)std::min<int64_t>(t->n, (int64_t)t->nleaves + t->nleaves / 4 + 64);
   if (t->L.arena ? ensure_arena(t, t->graph_leaves, 1.25) : ensure_slots(t, t->graph_leaves)) return;
-  if (ensure_segments(t, segments_bound(t) + segments_bound(t) / 4)) return;
+  if (ensure_segments(t, 0.25)) return;
   const int32_t grid_eager = t->grid_leaves;
   const int64_t launches0 = t->launches;
   const bool timing = t->timing;
@@ -547,7 +547,7 @@ int kdfmm_fmm_accel(kdfmm_tree t, double* a, double* phi, void* stream) {
   if ((rc = dual ? run_dual_local(t, s) : run_m2l(t, s))) return rc;
   phase_end(t, KDFMM_PHASE_M2L, s);
   phase_begin(t, KDFMM_PHASE_P2P, s);
-  if ((rc = ensure_segments(t, segments_bound(t)))) return rc;
+  if ((rc = ensure_segments(t, 0.0))) return rc;
   if ((rc = run_p2p(t, a, phi, s))) return rc;
   phase_end(t, KDFMM_PHASE_P2P, s);
   t->evaluated = true;

@@ -122,6 +122,7 @@ struct Lists {
   int32_t* seg_leaf;               // per extra item: its leaf
   double* seg_part;                // per extra item: partial sums
   int64_t seg_cap;                 // extra items allocated
+  bool seg_grouped;                // float64: an item is a group of segments
 };
 
 // Near entries per P2P segment (float64 evaluations of few particles take
@@ -490,10 +491,9 @@ int run_dual_walk(kdfmm_tree_s* t, cudaStream_t s);
 int run_dual_local(kdfmm_tree_s* t, cudaStream_t s);
 void free_dual(kdfmm_tree_s* t);
 int run_p2p(kdfmm_tree_s* t, double* a, double* phi, cudaStream_t s);
-// Extra P2P segments: storage for `need`, an upper bound from the last walk's
-// list sizes, and the plan (run by run_p2p).
-int ensure_segments(kdfmm_tree_s* t, int64_t need);
-int64_t segments_bound(const kdfmm_tree_s* t);
+// Extra P2P segments: storage for an upper bound from the last walk's list sizes
+// (and `spare` of it more), and the plan (run by run_p2p).
+int ensure_segments(kdfmm_tree_s* t, double spare);
 int plan_segments(kdfmm_tree_s* t, cudaStream_t s);
 int run_vjp(kdfmm_tree_s* t, const double* a_bar, double* x_bar, double* m_bar, cudaStream_t s);
 int momentum(const double* m, const double* v, int64_t n, double* out, double* scratch,

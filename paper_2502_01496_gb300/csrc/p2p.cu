@@ -84,12 +84,15 @@ struct P2PArgs {
 // order, then the groups: (first segment + expansion + rest of the first group)
 // + (second group + third + ...).  So it makes no difference who adds: with few
 // particles in the call each segment is a work item whose sums go to memory
-// (1 KB) for k_seg_combine; from kFullCall on the leaves themselves fill the GPU
-// (16384 warps and more) and a work item is a group, its segments added in
-// registers -- a forest of small systems would take 128 bytes a near entry
-// otherwise, where a group takes 4.  256 systems of 4096, 9.6e6 near entries: 47.9 ms
-// a call and 1.2 GB by segments, 48.1 ms and 38 MB by groups; 64 of 8191: 27.5 and 28.4 ms.
-constexpr int64_t kFullCall = 262144;
+// (1 KB) for k_seg_combine; a work item is a group, its segments added in
+// registers, in forests from kFullCall particles on, whose leaves themselves fill
+// the GPU (16384 warps and more), and in calls of more than kShortItems segments
+// (32768 groups and more; 1 GB), whose near lists are long: segments would take
+// 128 bytes a near entry, where groups take 4.  256 systems of 4096, 9.6e6 near
+// entries: 47.9 ms a call and 1.2 GB by segments, 48.1 ms and 38 MB by groups; 64 of
+// 8191: 27.5 and 28.4 ms.  One system with each leaf near all others: 3000 particles
+// 10.8 ms and 1.2 GB, 10.4 and 36 MB; 8000 74.7 and 8.2 GB, 72.8 and 0.25.
+constexpr int64_t kFullCall = 262144, kShortItems = int64_t(1) << 20;
 constexpr int kSegSteps = 3;
 __host__ __device__ __forceinline__ int64_t seg_below(int step) {      // particles, exclusive
   return step == 0 ? 8192 : (step == 1 ? 65536 : 262144);
@@ -820,8 +823,42 @@ inline unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + thre
 
 }  // namespace
 
-int ensure_segments(kdfmm_tree_s* t, int64_t need) {
+// Near entries of the last walk (exact lists: those allocated).
+static int64_t near_entries(const kdfmm_tree_s* t) {
+  return t->L.exact ? t->L.near_cap : t->host_stats[KDFMM_STAT_NNEAR];
+}
+
+// At most so many extra items if each segment is one: of each length class the
+// entries of its systems (no more than all, no more than their particles
+// squared) over the length.  *shorter: those of short segments.
+static int64_t segment_items(const kdfmm_tree_s* t, int64_t* shorter) {
+  const int64_t entries = near_entries(t);
+  *shorter = 0;
+  if (t->p.precision != KDFMM_FP64) return entries / kSegEntries + 64;
+  double own[kSegSteps + 1] = {};
+  for (int k = 0; k < t->n_sys; ++k) {
+    const double n = (double)(t->host_sys_off[k + 1] - t->host_sys_off[k]);
+    own[seg_step((int64_t)n)] += n * n;
+  }
+  int64_t items = 64;
+  for (int q = 0; q <= kSegSteps; ++q) {
+    items += (int64_t)std::min((double)entries, own[q]) / seg_length(q);
+    if (q < kSegSteps) *shorter = items;
+  }
+  return items;
+}
+
+// What the extra items of the evaluation are (L.seg_grouped), with room for them
+// and, for later evaluations of other particles, `spare` of that more.
+int ensure_segments(kdfmm_tree_s* t, double spare) {
   Lists& L = t->L;
+  int64_t shorter;
+  int64_t need = segment_items(t, &shorter);
+  // (Mixed segments and those of one large system are of 256 entries by themselves.)
+  L.seg_grouped = t->p.precision == KDFMM_FP64 &&
+                  ((t->n_sys > 1 && t->n >= kFullCall) || shorter > kShortItems);
+  if (L.seg_grouped) need = near_entries(t) / kSegEntries + 64;
+  need += (int64_t)(spare * (double)need);
   if (L.seg_cap >= need && L.seg_leaf != nullptr) return KDFMM_OK;
   const int64_t cap = std::max<int64_t>(need, 64);
   int32_t* leaf = nullptr;
@@ -840,37 +877,13 @@ int ensure_segments(kdfmm_tree_s* t, int64_t need) {
   return KDFMM_OK;
 }
 
-// (Mixed segments and those of one large system are of 256 entries by themselves.)
-static bool grouped_call(const kdfmm_tree_s* t) {
-  return t->p.precision == KDFMM_FP64 && t->n_sys > 1 && t->n >= kFullCall;
-}
-
-// At most so many extra items: by groups, and in mixed evaluations, the entries
-// over 256, else of each length class the entries of its systems (no more than
-// all, no more than their particles squared) over the length.
-int64_t segments_bound(const kdfmm_tree_s* t) {
-  const Lists& L = t->L;
-  const int64_t entries = L.exact ? L.near_cap : t->host_stats[KDFMM_STAT_NNEAR];
-  if (t->p.precision != KDFMM_FP64 || grouped_call(t)) return entries / kSegEntries + 64;
-  if (t->n_sys == 1) return entries / seg_length(seg_step(t->n)) + 64;
-  double own[kSegSteps + 1] = {};
-  for (int k = 0; k < t->n_sys; ++k) {
-    const int64_t n = t->host_sys_off[k + 1] - t->host_sys_off[k];
-    own[seg_step(n)] += (double)n * (double)n;
-  }
-  int64_t bound = 64;
-  for (int q = 0; q <= kSegSteps; ++q)
-    bound += (int64_t)std::min((double)entries, own[q]) / seg_length(q);
-  return bound;
-}
-
 int plan_segments(kdfmm_tree_s* t, cudaStream_t s) {
   const int gl = std::max(t->grid_leaves, 1);
   cudaMemsetAsync(t->counters + C_SEGS, 0, sizeof(int32_t), s);
   k_seg_plan<<<std::min<unsigned>(blocks_for(gl, 256), grid_blocks()), 256, 0, s>>>(
       t->L.near_cnt, t->L.exact ? INT64_MAX : t->L.cap_near, gl, t->counters, t->L.seg_first,
       t->L.seg_leaf, t->L.seg_cap, t->p.precision == KDFMM_FP64 ? t->sys_off : nullptr, t->leaf_sys,
-      grouped_call(t), t->status);
+      t->L.seg_grouped, t->status);
   t->launches += 1;
   return check_cuda(cudaGetLastError(), "segment plan");
 }
@@ -906,7 +919,7 @@ int run_p2p(kdfmm_tree_s* t, double* a, double* phi, cudaStream_t s) {
   int rc = plan_segments(t, s);
   if (rc) return rc;
   A.sys_off = t->p.precision == KDFMM_FP64 ? t->sys_off : nullptr;
-  A.grouped = grouped_call(t);
+  A.grouped = t->L.seg_grouped;
   const int gl = std::max(t->grid_leaves, 1);
   const bool m4 = t->p.soft_kind == KDFMM_SOFT_M4;
   if (t->p.precision == KDFMM_MIXED) {
