@@ -204,7 +204,8 @@ int kdfmm_fmm_accel(kdfmm_tree t, double* a, double* phi, void* stream);
  * a_bar: N x 3 cotangent (caller order, device); x_bar: N x 3 and m_bar: N
  * outputs (device, overwritten).  FP64 mode runs every step in float64;
  * mixed mode forms the M2L r-derivatives and the P2P pair terms in float32
- * (as its evaluation does) from float64 differences, with sums of float64 or wider.  Cell
+ * (as its evaluation does) from float64 differences, with sums of float64 or wider
+ * (a source's terms over the particles of one target leaf are added in float32 first).  Cell
  * cotangents and the P2P source-side terms are summed with float64 atomics,
  * so the last bits may vary run to run.  Its scratch (at most 112 bytes per
  * particle, 192 per leaf, 80 per cell, 8 per near-list entry, 16 MB, and an eighth

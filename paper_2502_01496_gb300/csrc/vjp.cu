@@ -3,7 +3,8 @@
 // and smoothing lengths held fixed).  The paper has no adjoint; this is the
 // derivative of the evaluation of Sec. 2 (Eqs. 3, 6, 7, 8, 13).  FP64 mode
 // runs every step in float64; mixed mode runs the M2L and P2P reverses with
-// float32 terms (as its forward does) and sums of float64 or wider.
+// float32 terms (as its forward does) and sums of float64 or wider (a source's
+// terms over the particles of one target leaf are added in float32 first).
 //
 // a_i = sum_{j in near(leaf i), j != i} m_j K(x_i - x_j)            (P2P)
 //     + L(C_alpha, x_i - com_alpha)                                (L2P, Eq. 8)
@@ -336,7 +337,7 @@ __global__ void __launch_bounds__(kL2PWarps * 32) k_vjp_l2p(const double* __rest
 // M2L reverse: warp per sink leaf, lanes over its far cells.  Mixed mode is bound
 // by float32 issue (some 2500 instructions a pair, three quarters of them the
 // dual numbers): the cotangents of M and Q, which needed seven contractions with
-// mostly zero terms (15.8 ms on the 2^20 Plummer sphere, 1.32e8 pairs; 12.4 now), are
+// mostly zero terms (15.8 ms on the 2^20 Plummer sphere, 1.32e8 pairs; 12.5 now), are
 // written without those terms.  A far cell's ten
 // cotangents (M_bar, com_bar, Q_bar) go to float64 atomics through shared
 // memory, so that a warp instruction adds 32 consecutive values (about three
